@@ -201,7 +201,12 @@ int alloc_buffers(sdc_ctx* c) {
     if (ok) ok = dalloc(&B.part, 12 * (size_t)B.max_blocks);
     if (ok && c->opt.cg_scaled) {
         B.sval_width = c->K.K.width;
-        ok = dalloc(&B.sv, ld) && dalloc(&B.sval, (size_t)std::max(B.sval_width, 1) * ld);
+        ulonglong2* pub = nullptr;
+        ok = dalloc(&B.sv, ld) && dalloc(&B.sval, (size_t)std::max(B.sval_width, 1) * ld) &&
+             dalloc(&B.flow, kFlowWords) && dalloc(&pub, 2 * ld);
+        B.pub = pub;
+        // tags of no launch
+        if (ok) cudaMemsetAsync(B.pub, 0, 2 * ld * sizeof(ulonglong2), c->stream);
     }
     if (!ok) return SDC_E_NOMEM;
     // pinned: [0] count, [1] err, then kMaxM node energies at byte 16
@@ -222,6 +227,8 @@ void free_all(sdc_ctx* c) {
                  B.seg_iters};
     for (int* p : ip) cudaFree(p);
     cudaFree(B.bars);
+    cudaFree(B.pub);
+    cudaFree(B.flow);
     cudaFree(B.seg_relres);
     if (c->h_bounds) cudaFreeHost(c->h_bounds);
     c->h_bounds = nullptr;

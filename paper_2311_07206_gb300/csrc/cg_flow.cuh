@@ -1,0 +1,696 @@
+// Node solves with every vector on chip and no grid barrier in the iteration.
+//
+// The solves of a step are bound by FP64 issue where a CTA owns many rows and by the
+// latency of the iteration's synchronisation chain where it owns few.  Three things
+// replace the barrier, the per-block records and their two passes of the other kernels:
+//
+// 1. Neighbour values travel with their version.  A row's published value and a tag
+//    (launch id, iteration) are one 16-byte word, stored and loaded as a single relaxed
+//    128-bit access; a consumer re-reads the few words that are not there yet.  No fence
+//    and no barrier separate the update from the next product, and the columns a CTA
+//    owns itself are read from its shared memory.
+// 2. The two dot products are summed in place.  Against an exponent window known from the
+//    previous iteration's total a value becomes four signed 26-bit limbs: a warp adds
+//    limbs with the integer warp reduction, a CTA adds the warps' limbs, and eight lanes
+//    add the CTA's limbs to eight 64-bit words with one relaxed reduction.  A word's top
+//    byte counts the arrivals, so the poll that finds all of them has the sum in hand:
+//    one store-and-poll round trip for barrier and sum together.  Two sets of words
+//    alternate and are never reset: a CTA knows the previous total of a set and takes the
+//    difference.  Measured for 152 CTAs: 1,510 cycles for the exchange of eight words,
+//    against 2,900 for the release/acquire barrier alone and 8,500 for barrier, block sums
+//    and totals of 152 records.
+// 3. p and x, which nothing waits for, are updated after the sums are posted.
+//
+// Integer addition is exact, so a total does not depend on the order of the arrivals, and
+// every CTA reads the same total.  The window holds 103 bits from kFlowHead bits above
+// the previous gamma down; a partial sum above it, or a total more than kFlowDrop bits
+// below the previous one, repeats the exchange with the exact largest exponents (the
+// start of a solve finds its window the same way).
+#pragma once
+
+#include "device_common.cuh"
+
+namespace sdc {
+namespace {
+
+typedef unsigned long long u64;
+
+constexpr int kFlowHead = 10;    // growth of gamma over one iteration that fits the window
+constexpr int kFlowDrop = 22;    // fall of gamma up to which the sum keeps 2^-54 of its value
+
+// relaxed single-copy-atomic 128-bit access: (value bits, tag)
+__device__ __forceinline__ void pub_store(ulonglong2* p, double v, u64 tag) {
+    asm volatile("{ .reg .b128 t; mov.b128 t, {%1, %2}; st.relaxed.gpu.global.b128 [%0], t; }" ::"l"(p),
+                 "l"((u64)__double_as_longlong(v)), "l"(tag)
+                 : "memory");
+}
+__device__ __forceinline__ void pub_load_if(bool on, const ulonglong2* p, u64& v, u64& tag) {
+    asm volatile(
+        "{ .reg .pred q; .reg .b128 t; setp.ne.u32 q, %3, 0; mov.b128 t, {%0, %1};\n\t"
+        "@q ld.relaxed.gpu.global.b128 t, [%2]; mov.b128 {%0, %1}, t; }"
+        : "+l"(v), "+l"(tag)
+        : "l"(p), "r"((unsigned)on)
+        : "memory");
+}
+__device__ __forceinline__ u64 ld_relaxed64(const u64* p) {
+    u64 v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void red_add64(u64* p, u64 v) {
+    asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+// Shared state of one CTA.
+struct FlowShared {
+    alignas(16) int lim[32][8];   // limb sums of each warp: 4 of a, 4 of b
+    double alpha, beta;
+    int topa, topb;               // window tops (largest exponent field) of the next sums
+    int ovf, ok, state;           // state: 0 go on, 1 converged, 2 non-finite, 3 repeat the sum
+    int next;                     // next chunk of rows of the product
+    int fmax[64];
+};
+
+// v against a window whose largest exponent field is `top`: |v| = sum_k l[k] 2^(26 k) units
+// of 2^(top - 1125), truncated; false when v lies above the window.
+__device__ __forceinline__ bool flow_limbs(double v, int top, int (&l)[4]) {
+    const u64 bits = (u64)__double_as_longlong(v);
+    const int f = (int)(bits >> 52) & 0x7ff;
+    const u64 mant = (bits & 0xfffffffffffffull) | (f > 0 ? (1ull << 52) : 0ull);
+    const int sh = min(max(f, 1) - top + 50, 50);
+    const u64 lo = sh >= 0 ? mant << sh : mant >> min(-sh, 63);
+    const u64 hi = sh > 0 ? mant >> (64 - sh) : 0ull;
+    const int s = (int)((long long)bits >> 63);   // 0 or -1
+    constexpr unsigned m = (1u << 26) - 1u;
+    l[0] = ((int)((unsigned)lo & m) ^ s) - s;
+    l[1] = ((int)((unsigned)(lo >> 26) & m) ^ s) - s;
+    l[2] = ((int)((unsigned)((lo >> 52) | (hi << 12)) & m) ^ s) - s;
+    l[3] = ((int)(unsigned)(hi >> 14) ^ s) - s;
+    return f <= top;
+}
+
+// Post the CTA's sums of a and b to the words acc[0..7]: every thread calls it; it holds
+// one CTA barrier, after which warp 0 adds the warps' limbs and posts them.
+__device__ __forceinline__ void flow_post(double a, double b, FlowShared& S, u64* acc) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    int la[4], lb[4];
+    bool in = flow_limbs(a, S.topa, la);
+    in = flow_limbs(b, S.topb, lb) && in;
+    const bool out = __any_sync(0xffffffffu, !in);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        la[k] = __reduce_add_sync(0xffffffffu, la[k]);
+        lb[k] = __reduce_add_sync(0xffffffffu, lb[k]);
+    }
+    if (lane == 0) {
+        *reinterpret_cast<int4*>(&S.lim[wid][0]) = make_int4(la[0], la[1], la[2], la[3]);
+        *reinterpret_cast<int4*>(&S.lim[wid][4]) = make_int4(lb[0], lb[1], lb[2], lb[3]);
+        if (out) S.ovf = 1;
+    }
+    __syncthreads();
+    if (wid == 0) {
+        long long s = 0;
+        for (int w = lane >> 3; w < nw; w += 4) s += S.lim[w][lane & 7];
+        s += __shfl_xor_sync(0xffffffffu, s, 8);
+        s += __shfl_xor_sync(0xffffffffu, s, 16);
+        // top byte: arrivals; next byte: CTAs with a value above the window
+        if (lane < 8) red_add64(acc + lane, (1ull << 56) + ((u64)(S.ovf != 0) << 48) + (u64)s);
+    }
+}
+
+// Quotient by Newton's iteration from the hardware's reciprocal estimate (relative error
+// 2^-20): 1/d (1 + e + e^2) with e = 1 - d y, then one residual correction of the quotient.
+// Divisors outside the normal range with a margin take the division.
+__device__ __forceinline__ double flow_quot(double n, double d) {
+    const int f = (int)((u64)__double_as_longlong(d) >> 52) & 0x7ff;
+    const int fn = (int)((u64)__double_as_longlong(n) >> 52) & 0x7ff;
+    if (f < 100 || f > 1946 || fn < 100 || fn > 1946 || abs(fn - f) > 900) return n / d;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+    const double e = fma(-d, y, 1.0), q0 = n * y;
+    const double e2 = fma(e, e, e);
+    const double q = fma(q0, e2, q0);
+    const double r = fma(-d, q, n);
+    return fma(r, y, q);
+}
+
+// What warp 0 carries from sum to sum (the same in every lane but prev).
+struct FlowScalars {
+    u64 prev[2];              // lane's word of each set before the running sum (lanes 0..7)
+    double inv_g, inv_a;      // 1 / gamma and 1 / alpha of the last sum (0 before the first)
+    double thresh, lo, hi;    // stopping test: bound on sqrt(gamma) and a band around its square
+    double gamma0, energy, rn;
+    int nsum;
+};
+
+__device__ __forceinline__ void flow_scalars_init(FlowScalars& Z) {
+    Z.prev[0] = Z.prev[1] = 0;
+    Z.inv_g = Z.inv_a = 0.0;
+    Z.thresh = Z.lo = Z.hi = 0.0;
+    Z.gamma0 = Z.energy = Z.rn = 0.0;
+    Z.nsum = 0;
+}
+
+// Warp 0: wait for the sums posted as number `npub`, derive alpha and beta (cg_scalars'
+// recurrences, den_t = delta_t - beta_t gamma_t / alpha_{t-1}) and the next windows.
+// exact: the windows came from the exact exponents (no repeat for a fall of gamma).
+__device__ __forceinline__ void flow_totals(FlowShared& S, FlowScalars& Z, const u64* acc, int set,
+                                            int G, bool exact, double rtol, long long budget,
+                                            int* err) {
+    const int lane = threadIdx.x & 31;
+    u64 v = 0, d = 0;
+    const u64 prev = set ? Z.prev[1] : Z.prev[0];
+    const long long t0 = clock64();
+    int ok = 1;
+    while (true) {
+        bool here = true;
+        if (lane < 8) {
+            v = ld_relaxed64(acc + lane);
+            d = v - prev + (1ull << 47);
+            here = (d >> 56) == (u64)G;
+        }
+        if (__all_sync(0xffffffffu, here)) break;
+        if (clock64() - t0 > budget) {
+            ok = 0;
+            break;
+        }
+    }
+    ok = __all_sync(0xffffffffu, ok);
+    if (!ok) {
+        if (lane == 0) {
+            raise_error(err, SDC_E_TIMEOUT);
+            S.ok = 0;
+        }
+        return;
+    }
+    if (set) Z.prev[1] = v; else Z.prev[0] = v;
+    const bool above = __any_sync(0xffffffffu, lane < 8 && ((d >> 48) & 0xff) != 0);
+    if (lane == 0) S.ovf = 0;
+    // the totals: lanes 0-3 assemble gamma, lanes 4-7 delta (the other lanes repeat them)
+    const long long part = (long long)(d & 0xffffffffffffull) - (1ll << 47);
+    __int128 q = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        q += (__int128)__shfl_sync(0xffffffffu, part, (lane & 4) + k) << (26 * k);
+    const double tot = xs_to_double(q, ((lane & 4) ? S.topb : S.topa) - 2);
+    const double g = __shfl_sync(0xffffffffu, tot, 0), dl = __shfl_sync(0xffffffffu, tot, 4);
+    const int fg = xs_field(g);
+    // the decisions compare bit patterns (g >= 0): an FP64 comparison has 64 cycles latency
+    const long long gb = __double_as_longlong(g);
+    int state = 0;
+    if (above) {
+        state = 3;
+    } else if (Z.nsum == 0) {
+        if (gb == 0) state = 1;
+    } else if (gb <= __double_as_longlong(Z.lo)) {
+        state = 1;
+    } else if (gb < __double_as_longlong(Z.hi) && sqrt(g) <= Z.thresh) {
+        state = 1;
+    } else if (!exact && fg < S.topa - kFlowHead - kFlowDrop) {
+        state = 3;
+    }
+    if (state != 3) {
+        Z.rn = g;
+        if (Z.nsum == 0) Z.gamma0 = g;
+    }
+    if (state == 0) {
+        const double beta = g * Z.inv_g;
+        const double den = fma(-beta, g * Z.inv_a, dl);
+        // lane 0: alpha = gamma / den, lane 1: 1 / gamma, lane 2: 1 / alpha
+        const double num = lane == 0 ? g : lane == 1 ? 1.0 : den;
+        const double quo = flow_quot(num, lane == 0 ? den : g);
+        const double alpha = __shfl_sync(0xffffffffu, quo, 0);
+        Z.inv_g = __shfl_sync(0xffffffffu, quo, 1);
+        Z.inv_a = __shfl_sync(0xffffffffu, quo, 2);
+        if (lane == 0) {
+            S.alpha = alpha;
+            S.beta = beta;
+            S.topa = S.topb = min(fg + kFlowHead, 2046);
+        }
+        Z.energy = fma(alpha, g, Z.energy);   // x' A x = sum of alpha_t gamma_t
+        if (xs_field(alpha) == 2047) state = 2;
+        ++Z.nsum;
+    }
+    if (lane == 0) S.state = state;
+}
+// Once, after the first sum's scalars are out: sqrt(gamma) <= rtol sqrt(gamma_0) is decided by
+// comparing gamma with a band of 2^-50 around the squared bound and by the square root
+// itself inside it.  Squares that leave the normal range always take the square root.
+__device__ __forceinline__ void flow_first_bound(FlowScalars& Z, double rtol) {
+    Z.thresh = rtol * sqrt(Z.gamma0);
+    const double q = Z.thresh * Z.thresh;
+    const bool normal = q > 1e-280 && q < 1e280;
+    Z.lo = normal ? q * (1.0 - 0x1p-50) : 0.0;
+    Z.hi = normal ? q * (1.0 + 0x1p-50) : INFINITY;
+}
+
+// Windows from the exact largest exponents of the CTAs' partial sums, with a release /
+// acquire grid barrier that also publishes every global write before it.  emax words hold
+// (generation << 32) | field and only grow.  Returns false after a timeout.
+__device__ __forceinline__ bool flow_window(double a, double b, FlowShared& S, u64* emax,
+                                            unsigned* bar, int G, unsigned& epoch, unsigned gen,
+                                            int headb, long long budget, int* err) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int fa = __reduce_max_sync(0xffffffffu, xs_field(a));
+    const int fb = __reduce_max_sync(0xffffffffu, xs_field(b));
+    if (lane == 0) {
+        S.fmax[wid] = fa;
+        S.fmax[32 + wid] = fb;
+    }
+    __syncthreads();
+    epoch += G;
+    if (wid == 0) {
+        const int ma = __reduce_max_sync(0xffffffffu, lane < nw ? S.fmax[lane] : 1);
+        const int mb = __reduce_max_sync(0xffffffffu, lane < nw ? S.fmax[32 + lane] : 1);
+        if (lane == 0) {
+            atomicMax(emax, ((u64)gen << 32) | (unsigned)ma);
+            atomicMax(emax + 1, ((u64)gen << 32) | (unsigned)mb);
+            S.ok = barrier_arrive_wait(bar, epoch, budget, err);
+            const int ga = (int)(unsigned)ld_relaxed64(emax), gb = (int)(unsigned)ld_relaxed64(emax + 1);
+            S.state = ga >= 2047 || gb >= 2047 ? 2 : 0;
+            S.topa = ga;
+            S.topb = min(gb + headb, 2046);
+            S.ovf = 0;
+        }
+    }
+    __syncthreads();
+    return S.ok != 0;
+}
+
+// Off-diagonal product of row i: acc + sum_k val(k) x(col(k)) in slot order.  Columns of this
+// CTA (rows [r0, r0 + nl)) come from shared memory (own), the others from their published
+// words, read again until they carry `tag`.  All loads of CH slots are issued before the
+// first is used.
+template <int CH, class Val>
+__device__ __forceinline__ double flow_row_dot(double acc, int len, size_t i, int ld,
+                                               const int* __restrict__ col, int ncol, int r0, int nl,
+                                               const double* own, const ulonglong2* pub, u64 tag,
+                                               int site, FlowShared& S, long long budget, int* err,
+                                               Val&& val) {
+    for (int k0 = 0; k0 < len; k0 += CH) {
+        int j[CH];
+        double a[CH];
+        u64 x[CH], g[CH];
+#pragma unroll
+        for (int k = 0; k < CH; ++k) {
+            j[k] = r0;
+            a[k] = 0.0;
+            if (k0 + k < len) {
+                const size_t q = (size_t)(k0 + k) * ld + i;
+                j[k] = sdc_idx(__ldg(col + q), ncol, site);
+                a[k] = val(q);
+            }
+        }
+        unsigned pend = 0;
+#pragma unroll
+        for (int k = 0; k < CH; ++k) {
+            const int l = j[k] - r0;
+            const bool mine = (unsigned)l < (unsigned)nl;
+            x[k] = mine ? (u64)__double_as_longlong(own[l]) : 0ull;
+            g[k] = k0 + k < len && !mine ? ~tag : tag;
+            pub_load_if(g[k] != tag, pub + j[k], x[k], g[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < CH; ++k) pend |= (g[k] != tag ? 1u : 0u) << k;
+        if (pend) {
+            const long long t0 = clock64();
+            do {
+#pragma unroll
+                for (int k = 0; k < CH; ++k) pub_load_if((pend >> k) & 1u, pub + j[k], x[k], g[k]);
+#pragma unroll
+                for (int k = 0; k < CH; ++k)
+                    if (g[k] == tag) pend &= ~(1u << k);
+                if (pend && clock64() - t0 > budget) {
+                    raise_error(err, SDC_E_TIMEOUT);
+                    S.ok = 0;
+                }
+                if (!*(volatile int*)&S.ok) pend = 0;   // a wait of the CTA has run out
+            } while (pend);
+        }
+#pragma unroll
+        for (int k = 0; k < CH; ++k)
+            if (k0 + k < len) acc += a[k] * __longlong_as_double((long long)x[k]);
+    }
+    return acc;
+}
+
+template <int MAXT>
+struct FlowChunk {
+    static constexpr int value = MAXT > 512 ? 3 : 6;
+};
+
+// First phase of a solve on the CTA's rows: s = diag^-1/2, r = s b (and zero vectors), both
+// published plainly, then a grid barrier that also finds the first windows, then the scaled
+// off-diagonals c s_i a_ij s_j and w = (I + c S K_off S) r.  f(l, r) receives a row's r,
+// g(l, w) its w; gamma and delta partial sums in ga, de.  Returns false to leave the kernel.
+template <int MAXT, class F, class H>
+__device__ __forceinline__ bool flow_start(const CgParams& P, const FlowParams& Q, FlowShared& S,
+                                           int r0, int nl, unsigned& epoch, double& ga, double& de,
+                                           F&& f, H&& h) {
+    const int t = threadIdx.x, B = blockDim.x, G = gridDim.x, ld = P.ld;
+    const double c = P.c;
+    ga = de = 0.0;
+    if (t == 0) {
+        S.ok = 1;
+        S.ovf = 0;
+        S.next = 0;
+    }
+    for (int l = t; l < nl; l += B) {
+        const int i = r0 + l;
+        const double d = P.mc[i] * (1.0 + c * P.J[i]) + c * P.kdc[i];
+        double si = 0.0;
+        if (!isfinite(d)) raise_error(P.err, SDC_E_NONFINITE);
+        else if (!(d > 0.0)) raise_error(P.err, SDC_E_DOMAIN);
+        else si = rsqrt(d);
+        P.sv[i] = si;
+        const double r = si * P.b[i];
+        P.u[i] = r;
+        ga += r * r;
+        f(l, r);
+    }
+    if (P.inject_fault && blockIdx.x == G - 1) {
+        // leave without arriving: every other CTA's bounded wait runs out
+        if (G == 1 && t == 0) raise_error(P.err, SDC_E_TIMEOUT);
+        return false;
+    }
+    // delta's partial sums: |w.r| of a thread <= |A| gamma, gamma <= 2^17 largest partial
+    if (!flow_window(ga, ga, S, Q.emax, Q.bar, G, epoch, 1u, 21, P.budget, P.err)) return false;
+    if (S.state == 2) {
+        if (blockIdx.x == 0 && t == 0) raise_error(P.err, SDC_E_NONFINITE);
+        return false;
+    }
+    constexpr int CH = FlowChunk<MAXT>::value;
+    for (int l = t; l < nl; l += B) {
+        const int i = r0 + l;
+        const int len = __ldg(P.alen + i);
+        const double csi = c * __ldcg(P.sv + i);
+        const double ri = __ldcg(P.u + i);
+        double acc = ri;
+        for (int k0 = 0; k0 < len; k0 += CH) {
+            int j[CH];
+            double av[CH], sj[CH], uj[CH];
+#pragma unroll
+            for (int k = 0; k < CH; ++k)
+                if (k0 + k < len) {
+                    const size_t q = (size_t)(k0 + k) * ld + i;
+                    j[k] = sdc_idx(__ldg(P.acol + q), P.n, 44);
+                    av[k] = __ldg(P.aval + q);
+                }
+#pragma unroll
+            for (int k = 0; k < CH; ++k)
+                if (k0 + k < len) {
+                    sj[k] = __ldcg(P.sv + j[k]);
+                    uj[k] = __ldcg(P.u + j[k]);
+                }
+#pragma unroll
+            for (int k = 0; k < CH; ++k)
+                if (k0 + k < len) {
+                    const double a = csi * av[k] * sj[k];
+                    P.sval[(size_t)(k0 + k) * ld + i] = a;
+                    acc += a * uj[k];
+                }
+        }
+        h(l, acc);
+        de += acc * ri;
+    }
+    return true;
+}
+
+// End of a solve: statistics, x = S x~ on the CTA's rows and the LU-trick coupling, whose
+// neighbours' x travel as tagged words.  xt(l): the CTA's x~.
+template <int MAXT, class X>
+__device__ __forceinline__ void flow_finish(const CgParams& P, const FlowParams& Q, FlowShared& S,
+                                            const FlowScalars& Z, int r0, int nl, int it, X&& xt) {
+    const int t = threadIdx.x, B = blockDim.x, ld = P.ld;
+    const bool lead = blockIdx.x == 0 && t == 0;
+    if (S.state == 2) {
+        if (lead) raise_error(P.err, SDC_E_NONFINITE);
+        return;
+    }
+    if (lead) {
+        *P.iters_out = it;
+        *P.relres_out = Z.gamma0 > 0.0 ? sqrt(fabs(Z.rn) / Z.gamma0) : 0.0;
+        if (P.energy_out) *P.energy_out = Z.energy;
+    }
+    // the words of iteration it - 1, whose readers are done: their CTAs posted sum `it`
+    ulonglong2* const pub = Q.pub + (size_t)((it + 1) & 1) * ld;
+    const u64 tag = Q.id + (u64)it + 2;
+    const bool couple = P.epi_lo < P.epi_hi;
+    for (int l = t; l < nl; l += B) {
+        const int i = r0 + l;
+        const double x = __ldcg(P.sv + i) * xt(l);
+        P.x[i] = x;
+        if (couple) pub_store(pub + i, x, tag);
+    }
+    if (!couple) return;
+    for (int l = t; l < nl; l += B) {
+        const int i = r0 + l;
+        const int len = __ldg(P.alen + i);
+        const double kx = flow_row_dot<FlowChunk<MAXT>::value>(
+            0.0, len, (size_t)i, ld, P.acol, P.n, 0, 0, nullptr, pub, tag, 47, S, P.budget, P.err,
+            [&](size_t q) { return __ldg(P.aval + q); });
+        cg_couple_row(P, i, P.x[i], kx);
+    }
+}
+
+// ---- pipelined arrangement (see pcg_group), scaled form ------------------------------
+// Per iteration: update of z, s, w, r and the two dot products (w published); sums posted;
+// p, x (r_old is kept in the other of two r buffers until then); the product
+// n = (I + c S K_off S) w on every warp but warp 0, which waits for the sums and derives the
+// scalars.  The product's 32-row chunks beyond the first per warp are handed out by a
+// counter, so warp 0 takes what is left when it joins.
+template <int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) {
+    extern __shared__ double sm[];
+    __shared__ FlowShared S;
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5, nw = blockDim.x >> 5;
+    const int G = gridDim.x, L = P.L, ld = P.ld;
+    const int r0 = blockIdx.x * L;
+    const int nl = max(0, min(P.n - r0, L));
+    const int nch = (nl + 31) >> 5;
+    double* rc = sm;             // r, and the r before it
+    double* ro = sm + L;
+    double* const sw = sm + 2 * L;
+    double* const sp = sm + 3 * L;
+    double* const ss = sm + 4 * L;
+    double* const sz = sm + 5 * L;
+    double* const sn = sm + 6 * L;
+    double* const xs = Q.x_smem ? sm + 7 * L : P.x + r0;
+    const int wrow = wid == 0 ? nw - 1 : wid - 1;   // the warps' order over the chunks
+    unsigned epoch = 0, gen = 1;
+    double ga, de, alpha = 0.0, beta = 0.0;
+    FlowScalars Z;
+    flow_scalars_init(Z);
+    if (!flow_start<MAXT>(
+            P, Q, S, r0, nl, epoch, ga, de,
+            [&](int l, double r) {
+                rc[l] = r;
+                sp[l] = ss[l] = sz[l] = 0.0;
+                xs[l] = 0.0;
+            },
+            [&](int l, double w) {
+                sw[l] = w;
+                pub_store(Q.pub + r0 + l, w, Q.id + 1);
+            }))
+        return;
+    int it = 0;
+    unsigned npub = 0;
+    bool exact = true, redo = false;
+    auto update_px = [&]() {
+        for (int c = wrow; c < nch; c += nw) {
+            const int l = 32 * c + lane;
+            if (l < nl) {
+                const double p = ro[l] + beta * sp[l];
+                sp[l] = p;
+                xs[l] += alpha * p;
+            }
+        }
+    };
+    while (true) {
+        u64* const acc = Q.acc + 8 * (npub & 1);
+        flow_post(ga, de, S, acc);
+        if (wid == 0)
+            flow_totals(S, Z, acc, npub & 1, G, exact, P.rtol, P.budget, P.err);
+        ++npub;
+        if (!redo) {
+            if (it > 0) update_px();
+            const u64 tag = Q.id + (u64)it + 1;
+            const ulonglong2* const pub = Q.pub + (size_t)(it & 1) * ld;
+            int c = wid - 1;
+            while (true) {
+                if (c < 0) {
+                    if (lane == 0) c = atomicAdd(&S.next, 1) + nw - 1;
+                    c = __shfl_sync(0xffffffffu, c, 0);
+                }
+                if (c >= nch) break;
+                const int l = 32 * c + lane;
+                if (l < nl) {
+                    const int i = r0 + l;
+                    sn[l] = flow_row_dot<FlowChunk<MAXT>::value>(
+                        sw[l], __ldg(P.alen + i), (size_t)i, ld, P.acol, P.n, r0, nl, sw, pub, tag, 42,
+                        S, P.budget, P.err, [&](size_t q) { return P.sval[q]; });
+                }
+                c = -1;
+                __syncwarp();
+            }
+        }
+        __syncthreads();
+        if (!S.ok) return;
+        if (S.state == 3) {
+            if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, 0, P.budget, P.err)) return;
+            if (S.state == 0) {
+                exact = redo = true;
+                continue;
+            }
+        }
+        exact = redo = false;
+        if (S.state != 0) break;
+        if (it >= P.maxit) {
+            if (blockIdx.x == 0 && t == 0) raise_error(P.err, SDC_E_CG_NOCONV);
+            break;
+        }
+        ++it;
+        alpha = S.alpha;
+        beta = S.beta;
+        if (t == 0) S.next = 0;
+        if (wid == 0 && it == 1) flow_first_bound(Z, P.rtol);
+        const u64 tag = Q.id + (u64)it + 1;
+        ulonglong2* const pub = Q.pub + (size_t)(it & 1) * ld + r0;
+        ga = de = 0.0;
+        for (int c = wrow; c < nch; c += nw) {
+            const int l = 32 * c + lane;
+            if (l < nl) {
+                const double w0 = sw[l];
+                const double z = sn[l] + beta * sz[l];
+                const double s = w0 + beta * ss[l];
+                const double w = w0 - alpha * z;
+                const double r = rc[l] - alpha * s;
+                pub_store(pub + l, w, tag);
+                sw[l] = w;
+                ro[l] = r;
+                sz[l] = z;
+                ss[l] = s;
+                ga += r * r;
+                de += w * r;
+            }
+        }
+        double* const q = rc;
+        rc = ro;
+        ro = q;
+    }
+    flow_finish<MAXT>(P, Q, S, Z, r0, nl, it, [&](int l) { return xs[l]; });
+}
+
+// ---- classical arrangement (see pcgc_group), scaled form -----------------------------
+// Per iteration: update of s and r (r published), the product w = (I + c S K_off S) r and the
+// dot products, the sums posted, and while they are summed p and x.  r_new goes into w's
+// place, which s has used up; with three buffers (nbuf = 3) the next w goes into a third, so
+// that r_old is still there for p after the product; with two, p and x come before it.
+template <int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) {
+    extern __shared__ double sm[];
+    __shared__ FlowShared S;
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5, nw = blockDim.x >> 5;
+    const int G = gridDim.x, L = P.L, ld = P.ld;
+    const int r0 = blockIdx.x * L;
+    const int nl = max(0, min(P.n - r0, L));
+    const int nch = (nl + 31) >> 5;
+    const bool late = Q.nbuf == 3;
+    double* rb = sm;
+    double* wb = sm + L;
+    double* const sp = sm + 2 * L;
+    double* const ss = sm + 3 * L;
+    double* fb = late ? sm + 4 * L : rb;
+    double* const xs = Q.x_smem ? sm + 5 * L : P.x + r0;
+    const int wrow = wid == 0 ? nw - 1 : wid - 1;
+    unsigned epoch = 0, gen = 1;
+    double ga, de, alpha = 0.0, beta = 0.0;
+    FlowScalars Z;
+    flow_scalars_init(Z);
+    if (!flow_start<MAXT>(
+            P, Q, S, r0, nl, epoch, ga, de,
+            [&](int l, double r) {
+                rb[l] = r;
+                sp[l] = ss[l] = 0.0;
+                xs[l] = 0.0;
+            },
+            [&](int l, double w) { wb[l] = w; }))
+        return;
+    int it = 0;
+    unsigned npub = 0;
+    bool exact = true, redo = false;
+    auto update_px = [&](const double* r) {
+        for (int c = wrow; c < nch; c += nw) {
+            const int l = 32 * c + lane;
+            if (l < nl) {
+                const double p = r[l] + beta * sp[l];
+                sp[l] = p;
+                xs[l] += alpha * p;
+            }
+        }
+    };
+    while (true) {
+        u64* const acc = Q.acc + 8 * (npub & 1);
+        flow_post(ga, de, S, acc);
+        if (wid == 0)
+            flow_totals(S, Z, acc, npub & 1, G, exact, P.rtol, P.budget, P.err);
+        ++npub;
+        if (late && it > 0 && !redo) update_px(fb);
+        __syncthreads();
+        if (!S.ok) return;
+        if (S.state == 3) {
+            if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, 0, P.budget, P.err)) return;
+            if (S.state == 0) {
+                exact = redo = true;
+                continue;
+            }
+        }
+        exact = redo = false;
+        if (S.state != 0) break;
+        if (it >= P.maxit) {
+            if (blockIdx.x == 0 && t == 0) raise_error(P.err, SDC_E_CG_NOCONV);
+            break;
+        }
+        ++it;
+        alpha = S.alpha;
+        beta = S.beta;
+        const u64 tag = Q.id + (u64)it + 1;
+        ulonglong2* const pub = Q.pub + (size_t)(it & 1) * ld;
+        for (int c = wrow; c < nch; c += nw) {
+            const int l = 32 * c + lane;
+            if (l < nl) {
+                const double s = wb[l] + beta * ss[l];
+                const double r = rb[l] - alpha * s;
+                pub_store(pub + r0 + l, r, tag);
+                wb[l] = r;
+                ss[l] = s;
+            }
+        }
+        __syncthreads();
+        if (wid == 0 && it == 1) flow_first_bound(Z, P.rtol);
+        if (!late) update_px(rb);
+        ga = de = 0.0;
+        for (int c = wrow; c < nch; c += nw) {
+            const int l = 32 * c + lane;
+            if (l < nl) {
+                const int i = r0 + l;
+                const double r = wb[l];
+                const double w = flow_row_dot<FlowChunk<MAXT>::value>(
+                    r, __ldg(P.alen + i), (size_t)i, ld, P.acol, P.n, r0, nl, wb, pub, tag, 46, S,
+                    P.budget, P.err, [&](size_t q) { return P.sval[q]; });
+                fb[l] = w;
+                ga += r * r;
+                de += w * r;
+            }
+        }
+        // r <- w's place, w <- the product's, and r_old's is free (two buffers: the same one)
+        double* const q = rb;
+        rb = wb;
+        wb = fb;
+        fb = late ? q : rb;
+    }
+    flow_finish<MAXT>(P, Q, S, Z, r0, nl, it, [&](int l) { return xs[l]; });
+}
+
+}  // namespace
+}  // namespace sdc

@@ -127,6 +127,9 @@ struct StepBuffers {
     double* sv = nullptr;     // [ld] diag^-1/2 of the scaled solve
     double* sval = nullptr;   // [sval_width][ld] scaled off-diagonal values of the scaled solve
     int sval_width = 0;
+    void* pub = nullptr;      // [2][ld] 16-byte words of the flow kernels: published value, tag
+    unsigned long long* flow = nullptr;   // [kFlowWords] their sums and barrier, zeroed per launch
+    unsigned long long flow_id = 0;       // launches so far (tags)
     int max_blocks = 0;
     int* flag = nullptr;      // [ld]
     int* map = nullptr;       // [ld] old compact row -> new compact row or -1
@@ -163,9 +166,9 @@ void launch_residual(int M, int n, const int* act, const Ell& K, const double* k
                      const Coll& co, int reaction_implicit, StepBuffers& B, cudaStream_t s,
                      const int* n_dev = nullptr);
 // Launch configuration of the restricted PCG solves.
-constexpr int kSmemVectorsS = 6;    // the same for the symmetrically scaled variant
-constexpr int kSmemVectorsCS = 4;   // the scaled classical shared-memory variant (kSmemRowsC rows)
-constexpr int kSmemRowsS = 4800;    // rows per block of the symmetrically scaled variant
+constexpr int kFlowSmemBytes = 225 * 1024;   // dynamic shared memory of the flow kernels
+constexpr int kFlowWords = 34;      // 64-bit words of their grid-wide state
+constexpr int kFlowClassicalRows = 250000;   // automatic arrangement: classical above
 constexpr int kSmemVectors = 8;     // per-row doubles in shared memory, shared-memory variant
 constexpr int kSmemRows = 3584;     // rows per block of the shared-memory variant
 // target rows per block of the shared-memory variants below their capacity: one row

@@ -185,6 +185,25 @@ __device__ __forceinline__ void cg_couple_row(const CgParams& P, int i, double x
     }
 }
 
+// Grid-wide state of the flow kernels (cg_flow.cuh).
+struct FlowParams {
+    ulonglong2* pub;            // published words (value, tag) per row, two buffers of ld
+    unsigned long long* acc;    // two sets of eight words of the running sums
+    unsigned long long* emax;   // largest exponents of gamma's and delta's partial sums
+    unsigned* bar;              // arrivals of the barriers outside the iteration
+    unsigned long long id;      // launch id << 32: tags of different launches differ
+    int x_smem;                 // x in shared memory (else in P.x)
+    int nbuf;                   // classical: buffers shared by r and w (2 or 3)
+};
+
+}  // namespace
+}  // namespace sdc
+
+#include "cg_flow.cuh"
+
+namespace sdc {
+namespace {
+
 // Off-diagonal product of row i over its ELL slots, acc + sum_k val(k) x(col(k))
 // in slot order (the same FMAs, in the same order, as a plain slot loop).  The
 // column and value loads of CH slots, and then their gathers, are all issued
@@ -807,191 +826,6 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_smem(CgParams P) {
 #undef SZ
 #undef SN
 #undef SI
-
-// Symmetrically scaled form of the pipelined shared-memory solve.  Jacobi-PCG
-// on A = diag(d) + c K_off is CG on S A S = I + c S K_off S with S = diag(d)^-1/2,
-// x = S x~, b~ = S b: the same iterates, the same stopping quantity
-// (r~.r~ = r.D^-1 r) and the same energy (x~' S A S x~ = x' A x).  Per
-// row-iteration it saves the two preconditioner products (u = D^-1 r, m = D^-1 w)
-// and the scaling of the product by c, and keeps six vectors on chip instead of
-// eight (4800 rows per block).  The scaled off-diagonals c s_i a_ij s_j are
-// written once per solve to P.sval (each block its own rows, after a grid barrier
-// that publishes s).  Per row-iteration: len FMAs of the product (started from
-// w_i, the unit diagonal), six recurrence FMAs, two dot FMAs.
-template <int MAXT>
-__global__ void __launch_bounds__(MAXT, 1) k_pcg_scaled(CgParams P) {
-    extern __shared__ double sm[];
-    __shared__ CgShared S;
-    const int G = gridDim.x, B = blockDim.x, t = threadIdx.x;
-    const int L = P.L, ld = P.ld;
-    const int r0 = blockIdx.x * L;
-    const int nl = max(0, min(P.n - r0, L));
-    const int sp0 = B >= 256 ? 64 : 0;
-#define SR(l) sm[(l)]
-#define SW(l) sm[L + (l)]
-#define SP(l) sm[2 * L + (l)]
-#define SS(l) sm[3 * L + (l)]
-#define SZ(l) sm[4 * L + (l)]
-#define SN(l) sm[5 * L + (l)]
-    double* __restrict__ ug = P.u;
-    double* __restrict__ xg = P.x;
-    double* __restrict__ sg = P.sv;
-    double* __restrict__ sval = P.sval;
-    const double* __restrict__ aval = P.aval;
-    const int* __restrict__ acol = P.acol;
-    const int* __restrict__ alen = P.alen;
-    const double c = P.c;
-    XsRecord* const rec = reinterpret_cast<XsRecord*>(P.part);
-    unsigned epoch = 0;
-    int buf = 0;
-
-    for (int l = t; l < nl; l += B) {
-        const int i = r0 + l;
-        const double d = P.mc[i] * (1.0 + c * P.J[i]) + c * P.kdc[i];
-        double si = 0.0;
-        if (!isfinite(d)) raise_error(P.err, SDC_E_NONFINITE);
-        else if (!(d > 0.0)) raise_error(P.err, SDC_E_DOMAIN);
-        else si = rsqrt(d);
-        sg[i] = si;
-        const double r = si * P.b[i];
-        SR(l) = r;
-        ug[i] = r;
-        SP(l) = 0.0;
-        SS(l) = 0.0;
-        SZ(l) = 0.0;
-        xg[i] = 0.0;
-    }
-    if (P.inject_fault && blockIdx.x == G - 1) {
-        if (G == 1 && t == 0) raise_error(P.err, SDC_E_TIMEOUT);
-        return;
-    }
-    if (!grid_barrier(P.bar, epoch, P.budget, P.err, &S.ok)) return;
-    // scaled rows of this block, and w = (I + c S K_off S) r~
-    double ga = 0.0, de = 0.0;
-    for (int l = t; l < nl; l += B) {
-        const int i = r0 + l;
-        const int len = __ldg(alen + i);
-        const double csi = c * __ldcg(sg + i);
-        const double ri = SR(l);
-        double acc = ri;
-        for (int k0 = 0; k0 < len; k0 += EllChunk<MAXT>::value) {
-            int j[EllChunk<MAXT>::value];
-            double av[EllChunk<MAXT>::value], sj[EllChunk<MAXT>::value], uj[EllChunk<MAXT>::value];
-#pragma unroll
-            for (int k = 0; k < EllChunk<MAXT>::value; ++k) {
-                if (k0 + k < len) {
-                    const size_t q = (size_t)(k0 + k) * ld + i;
-                    j[k] = sdc_idx(__ldg(acol + q), P.n, 44);
-                    av[k] = __ldg(aval + q);
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < EllChunk<MAXT>::value; ++k) {
-                if (k0 + k < len) {
-                    sj[k] = __ldcg(sg + j[k]);
-                    uj[k] = __ldcg(ug + j[k]);
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < EllChunk<MAXT>::value; ++k) {
-                if (k0 + k < len) {
-                    const double a = csi * av[k] * sj[k];
-                    sval[(size_t)(k0 + k) * ld + i] = a;
-                    acc += a * uj[k];
-                }
-            }
-        }
-        SW(l) = acc;
-        ga += ri * ri;
-        de += acc * ri;
-        P.m[i] = acc;
-    }
-    int it = 0, nsum = 0;
-    while (true) {
-        if (!cg_publish_arrive(ga, de, S, rec + buf * G, P.bar, G, (int)blockIdx.x, epoch,
-                               P.budget, P.err))
-            return;
-        const double* mc = P.m + (nsum & 1) * (size_t)ld;
-        auto totals = [&]() {
-            double g, d;
-            xs_group_total(G, [&](int k) { return xs_load_cg(rec + buf * G + k); }, S.xs, g, d);
-            if ((t & 31) == 0) cg_scalars(S, t >> 5, nsum, g, d, P.rtol);
-        };
-        if (sp0 > 0 && t < 64) totals();
-        if (t >= sp0) {
-            for (int l = t - sp0; l < nl; l += B - sp0) {
-                const int i = r0 + l;
-                const int len = __ldg(alen + i);
-                SN(l) = ell_row_dot<EllChunk<MAXT>::value>(SW(l), len, (size_t)i, ld, acol, P.n,
-                                    [&](size_t q) { return __ldcg(sval + q); },
-                                    [&](int j) { return __ldcg(mc + j); });
-            }
-        }
-        if (sp0 == 0 && t < 64) totals();
-        __syncthreads();
-        ++nsum;
-        buf ^= 1;
-        if (S.state != 0) break;
-        if (it >= P.maxit) {
-            if (blockIdx.x == 0 && t == 0) raise_error(P.err, SDC_E_CG_NOCONV);
-            break;
-        }
-        ++it;
-        const double alpha = S.alpha, beta = S.beta;
-        double* mn = P.m + (nsum & 1) * (size_t)ld;
-        ga = de = 0.0;
-        for (int l = t; l < nl; l += B) {
-            const int i = r0 + l;
-            const double wi = SW(l), ri = SR(l);
-            const double zi = SN(l) + beta * SZ(l);
-            const double s_i = wi + beta * SS(l);
-            const double pi = ri + beta * SP(l);
-            SZ(l) = zi;
-            SS(l) = s_i;
-            SP(l) = pi;
-            xg[i] += alpha * pi;
-            const double r2 = ri - alpha * s_i;
-            const double w2 = wi - alpha * zi;
-            SR(l) = r2;
-            SW(l) = w2;
-            ga += r2 * r2;
-            de += w2 * r2;
-            mn[i] = w2;
-        }
-    }
-    if (S.state == 2) {
-        if (blockIdx.x == 0 && t == 0) raise_error(P.err, SDC_E_NONFINITE);
-        return;
-    }
-    if (blockIdx.x == 0 && t == 0) {
-        *P.iters_out = it;
-        *P.relres_out = cg_relres(S);
-        if (P.energy_out) *P.energy_out = S.energy;
-    }
-    // x = S x~ on this block's rows; the epilogue gathers neighbours' x after a barrier
-    for (int l = t; l < nl; l += B) {
-        const int i = r0 + l;
-        xg[i] = __ldcg(sg + i) * __ldcg(xg + i);
-    }
-    if (P.epi_lo < P.epi_hi) {
-        if (!grid_barrier(P.bar, epoch, P.budget, P.err, &S.ok)) return;
-        for (int l = t; l < nl; l += B) {
-            const int i = r0 + l;
-            const int len = __ldg(alen + i);
-            const double xi = __ldcg(xg + i);
-            const double acc = ell_row_dot<EllChunk<MAXT>::value>(0.0, len, (size_t)i, ld, acol, P.n,
-                                           [&](size_t q) { return __ldg(aval + q); },
-                                           [&](int j) { return __ldcg(xg + j); });
-            cg_couple_row(P, i, xi, acc);
-        }
-    }
-}
-#undef SR
-#undef SW
-#undef SP
-#undef SS
-#undef SZ
-#undef SN
 
 // Thread-block-cluster variant for small active sets (n <= C * L rows, one
 // cluster of C CTAs).  The same iteration as k_pcg_smem; m of other CTAs is
@@ -1741,136 +1575,6 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcgc_batch(CgParams P, const SegBlo
 
 // Shared-memory form of the classical arrangement (rows as in k_pcg_smem;
 // r, u, p, s, w and the reciprocal diagonal on chip, u published).
-// Shared-memory form of pcgc_group_scaled: rows as in k_pcgc_smem, r, p, s, w on
-// chip (four vectors), r published for the neighbours' products.
-template <int MAXT>
-__global__ void __launch_bounds__(MAXT, 1) k_pcgc_scaled(CgParams P) {
-    extern __shared__ double sm[];
-    __shared__ CgShared S;
-    const int G = gridDim.x, B = blockDim.x, t = threadIdx.x;
-    const int L = P.L, ld = P.ld;
-    const int r0 = blockIdx.x * L;
-    const int nl = max(0, min(P.n - r0, L));
-    double* __restrict__ sr = sm;
-    double* __restrict__ sp = sm + L;
-    double* __restrict__ ss = sm + 2 * L;
-    double* __restrict__ sw = sm + 3 * L;
-    double* __restrict__ ug = P.u;
-    double* __restrict__ xg = P.x;
-    double* __restrict__ sg = P.sv;
-    double* __restrict__ sval = P.sval;
-    const double* __restrict__ aval = P.aval;
-    const int* __restrict__ acol = P.acol;
-    const int* __restrict__ alen = P.alen;
-    const double c = P.c;
-    unsigned epoch = 0;
-    int buf = 0;
-
-    for (int l = t; l < nl; l += B) {
-        const int i = r0 + l;
-        const double d = P.mc[i] * (1.0 + c * P.J[i]) + c * P.kdc[i];
-        double si = 0.0;
-        if (!isfinite(d)) raise_error(P.err, SDC_E_NONFINITE);
-        else if (!(d > 0.0)) raise_error(P.err, SDC_E_DOMAIN);
-        else si = rsqrt(d);
-        sg[i] = si;
-        const double r = si * P.b[i];
-        sr[l] = r;
-        ug[i] = r;
-        sp[l] = 0.0;
-        ss[l] = 0.0;
-        xg[i] = 0.0;
-    }
-    if (P.inject_fault && blockIdx.x == G - 1) {
-        if (G == 1 && t == 0) raise_error(P.err, SDC_E_TIMEOUT);
-        return;
-    }
-    if (!grid_barrier(P.bar, epoch, P.budget, P.err, &S.ok)) return;
-    // scaled rows: written and read back by the same thread (same row mapping in every loop)
-    for (int l = t; l < nl; l += B) {
-        const int i = r0 + l;
-        const int len = __ldg(alen + i);
-        const double csi = c * __ldcg(sg + i);
-        for (int k = 0; k < len; ++k) {
-            const size_t q = (size_t)k * ld + i;
-            sval[q] = csi * __ldg(aval + q) * __ldcg(sg + sdc_idx(__ldg(acol + q), P.n, 45));
-        }
-    }
-    XsRecord* const rec = reinterpret_cast<XsRecord*>(P.part);
-    int it = 0, nsum = 0;
-    while (true) {
-        double ga = 0.0, de = 0.0;
-        for (int l = t; l < nl; l += B) {
-            const int i = r0 + l;
-            const int len = __ldg(alen + i);
-            const double ri = sr[l];
-            double acc = ri;
-            for (int k = 0; k < len; ++k) {
-                const size_t q = (size_t)k * ld + i;
-                acc += sval[q] * __ldcg(ug + sdc_idx(__ldg(acol + q), P.n, 46));
-            }
-            sw[l] = acc;
-            ga += ri * ri;
-            de += acc * ri;
-        }
-        if (!cg_publish_arrive(ga, de, S, rec + buf * G, P.bar, G, (int)blockIdx.x, epoch,
-                               P.budget, P.err))
-            return;
-        if (t < 64) {
-            double g, d;
-            xs_group_total(G, [&](int k) { return xs_load_cg(rec + buf * G + k); }, S.xs, g, d);
-            if ((t & 31) == 0) cg_scalars(S, t >> 5, nsum, g, d, P.rtol);
-        }
-        __syncthreads();
-        ++nsum;
-        buf ^= 1;
-        if (S.state != 0) break;
-        if (it >= P.maxit) {
-            if (blockIdx.x == 0 && t == 0) raise_error(P.err, SDC_E_CG_NOCONV);
-            break;
-        }
-        ++it;
-        const double alpha = S.alpha, beta = S.beta;
-        for (int l = t; l < nl; l += B) {
-            const double ri = sr[l];
-            const double pi = ri + beta * sp[l];
-            const double s_i = sw[l] + beta * ss[l];
-            sp[l] = pi;
-            ss[l] = s_i;
-            xg[r0 + l] += alpha * pi;
-            const double r = ri - alpha * s_i;
-            sr[l] = r;
-            ug[r0 + l] = r;
-        }
-        if (!grid_barrier(P.bar, epoch, P.budget, P.err, &S.ok)) return;
-    }
-    if (S.state == 2) {
-        if (blockIdx.x == 0 && t == 0) raise_error(P.err, SDC_E_NONFINITE);
-        return;
-    }
-    if (blockIdx.x == 0 && t == 0) {
-        *P.iters_out = it;
-        *P.relres_out = cg_relres(S);
-        if (P.energy_out) *P.energy_out = S.energy;
-    }
-    for (int l = t; l < nl; l += B) {
-        const int i = r0 + l;
-        xg[i] = __ldcg(sg + i) * __ldcg(xg + i);
-    }
-    if (P.epi_lo < P.epi_hi) {
-        if (!grid_barrier(P.bar, epoch, P.budget, P.err, &S.ok)) return;
-        for (int l = t; l < nl; l += B) {
-            const int i = r0 + l;
-            const int len = __ldg(alen + i);
-            const double xi = __ldcg(xg + i);
-            double acc = 0.0;
-            for (int k = 0; k < len; ++k)
-                acc += __ldg(aval + (size_t)k * ld + i) * __ldcg(xg + sdc_idx(__ldg(acol + (size_t)k * ld + i), P.n, 47));
-            cg_couple_row(P, i, xi, acc);
-        }
-    }
-}
-
 template <int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) k_pcgc_smem(CgParams P) {
     extern __shared__ double sm[];
@@ -2237,17 +1941,16 @@ PcgKernel pcg_general_kernel(int block) {
     return block > 512 ? k_pcg<1024> : block > 256 ? k_pcg<512> : k_pcg<256>;
 }
 PcgKernel pcg_smem_kernel(int block) { return block > 512 ? k_pcg_smem<1024> : k_pcg_smem<512>; }
-PcgKernel pcgc_scaled_kernel(int block) {
-    return block > 512 ? k_pcgc_scaled<1024> : k_pcgc_scaled<512>;
+using FlowKernel = void (*)(CgParams, FlowParams);
+FlowKernel flow_kernel(int block, bool classical) {
+    if (classical) return block > 512 ? k_cgc_flow<1024> : k_cgc_flow<512>;
+    return block > 512 ? k_pcg_flow<1024> : k_pcg_flow<512>;
 }
 PcgKernel pcgcs_general_kernel(int block) {
     return block > 512 ? k_pcgcs<1024> : block > 256 ? k_pcgcs<512> : k_pcgcs<256>;
 }
 PcgKernel pcgs_general_kernel(int block) {
     return block > 512 ? k_pcgs<1024> : block > 256 ? k_pcgs<512> : k_pcgs<256>;
-}
-PcgKernel pcg_scaled_kernel(int block) {
-    return block > 512 ? k_pcg_scaled<1024> : k_pcg_scaled<512>;
 }
 PcgKernel pcg_cluster_kernel(int block) {
     return block > 512 ? k_pcg_cluster<1024> : k_pcg_cluster<512>;
@@ -2272,12 +1975,9 @@ void pcg_smem_attrs() {
     for (PcgKernel k : {k_pcgc_smem<512>, k_pcgc_smem<1024>})
         cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(kSmemVectorsC * kSmemRowsC * sizeof(double)));
-    for (PcgKernel k : {k_pcg_scaled<512>, k_pcg_scaled<1024>})
+    for (FlowKernel k : {k_pcg_flow<512>, k_pcg_flow<1024>, k_cgc_flow<512>, k_cgc_flow<1024>})
         cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(kSmemVectorsS * kSmemRowsS * sizeof(double)));
-    for (PcgKernel k : {k_pcgc_scaled<512>, k_pcgc_scaled<1024>})
-        cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(kSmemVectorsCS * kSmemRowsC * sizeof(double)));
+                             kFlowSmemBytes);
     for (PcgKernel k : {k_pcg_cluster<512>, k_pcg_cluster<1024>}) {
         cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(kClusterVectors * kClusterRows * sizeof(double)));
@@ -2488,10 +2188,65 @@ int launch_pcg_role(int n, const Ell& A, const PcgRole& role, double dt, int M, 
     return launch_pcg_params(P, c2, B, s);
 }
 
+// Shape of a flow launch: rows per CTA, CTAs, threads, shared memory; false when the rows
+// do not fit on chip.  Up to 28 chunks of 32 rows a CTA has one row per thread, warp 0 apart,
+// and its rows are a multiple of 128: FP64 issue is what a full warp per sub-partition
+// takes whatever its active lanes, so fewer CTAs with full warps are never slower.
+struct FlowShape {
+    int L, grid, block, x_smem, nbuf;
+    size_t smem;
+};
+bool flow_shape(int n, bool classical, const PcgConfig& cfg, FlowShape& f) {
+    const int rows = kFlowSmemBytes / 8;                // doubles on chip
+    const int cap = (classical ? rows / 4 : rows / 7) / 32 * 32;
+    int gm = std::min(cfg.sms, 255);                    // arrivals are counted in a byte
+    if (n > (long long)gm * cap) return false;
+    if (cfg.max_blocks > 0) gm = std::min(gm, std::max(cfg.max_blocks, nblk(n, cap)));
+    int l = nblk(n, gm);
+    if (cfg.rows_per_block > 0) l = std::max(l, std::min(cfg.rows_per_block, cap));
+    const int maxb = n >= cfg.big_rows ? 1024 : std::min(std::max(cfg.smem_block, 64), 1024);
+    f.L = std::min(l <= 896 ? (l + 127) / 128 * 128 : (l + 31) / 32 * 32, cap);
+    f.grid = nblk(n, f.L);
+    f.block = std::min(32 + std::min(f.L, (n + 31) / 32 * 32), maxb);
+    if (classical) {
+        f.nbuf = 5 * f.L <= rows ? 3 : 2;
+        f.x_smem = f.nbuf == 3 && 6 * f.L <= rows;
+    } else {
+        f.nbuf = 2;
+        f.x_smem = 8 * f.L <= rows;
+    }
+    f.smem = (size_t)((classical ? 2 + f.nbuf : 7) + f.x_smem) * f.L * sizeof(double);
+    return true;
+}
+
+int launch_flow(CgParams& P, bool classical, const FlowShape& f, StepBuffers& B, cudaStream_t s) {
+    pcg_smem_attrs();
+    FlowParams Q;
+    Q.pub = reinterpret_cast<ulonglong2*>(B.pub);
+    Q.acc = B.flow;
+    Q.emax = B.flow + 16;
+    Q.bar = reinterpret_cast<unsigned*>(B.flow + 32);
+    Q.id = ++B.flow_id << 32;
+    Q.x_smem = f.x_smem;
+    Q.nbuf = f.nbuf;
+    P.L = f.L;
+    cudaMemsetAsync(B.flow, 0, kFlowWords * sizeof(unsigned long long), s);
+    void* args[] = {&P, &Q};
+    cudaError_t e = cudaLaunchCooperativeKernel((const void*)flow_kernel(f.block, classical),
+                                                dim3(f.grid), dim3(f.block), args, f.smem, s);
+    return e == cudaSuccess ? SDC_OK : SDC_E_CUDA;
+}
+
 int launch_pcg_params(CgParams& P, const PcgConfig& cfg, StepBuffers& B, cudaStream_t s) {
     const int n = P.n;
     // the exact-sum records are read with 16-byte loads
     if (reinterpret_cast<uintptr_t>(P.part) % 16 != 0) return SDC_E_INVALID;
+    FlowShape fs;
+    const bool flow_classical =
+        !cfg.pipelined || (cfg.general_classical && n > kFlowClassicalRows);
+    if (cfg.variant != 1 && cfg.scaled && P.sv && P.sval && B.pub &&
+        flow_shape(n, flow_classical, cfg, fs))
+        return launch_flow(P, flow_classical, fs, B, s);
     cudaMemsetAsync(&B.sc->bar, 0, sizeof(unsigned), s);
     void* args[] = {&P};
     // automatic arrangement: the pipelined form pays off where the vectors live on chip;
@@ -2509,11 +2264,9 @@ int launch_pcg_params(CgParams& P, const PcgConfig& cfg, StepBuffers& B, cudaStr
             P.L = nblk(n, grid);
             const int blk = n >= cfg.big_rows ? 1024 : cfg.smem_block;
             pcg_smem_attrs();
-            const bool sc = cfg.scaled && P.sv && P.sval;
             cudaError_t e = cudaLaunchCooperativeKernel(
-                (const void*)(sc ? pcgc_scaled_kernel(blk) : pcgc_smem_kernel(blk)), dim3(grid),
-                dim3(blk), args,
-                (size_t)(sc ? kSmemVectorsCS : kSmemVectorsC) * P.L * sizeof(double), s);
+                (const void*)pcgc_smem_kernel(blk), dim3(grid), dim3(blk), args,
+                (size_t)kSmemVectorsC * P.L * sizeof(double), s);
             return e == cudaSuccess ? SDC_OK : SDC_E_CUDA;
         }
         int grid = std::min(cfg.max_blocks_general, nblk(n, cfg.block));
@@ -2546,24 +2299,6 @@ int launch_pcg_params(CgParams& P, const PcgConfig& cfg, StepBuffers& B, cudaStr
         lc.attrs = at;
         lc.numAttrs = 1;
         cudaError_t e = cudaLaunchKernelEx(&lc, pcg_cluster_kernel(cfg.smem_block), P);
-        return e == cudaSuccess ? SDC_OK : SDC_E_CUDA;
-    }
-    // symmetrically scaled shared-memory form: one block per SM at most.  Up to the Jacobi
-    // form's capacity only: above it (the 686k-row tissue mesh) 4,500 on-chip rows per block
-    // leave too little L1 for the irregular gathers and the global-vector kernel is faster
-    // (16.1 against 18.9 ms of PCG per step)
-    if (cfg.variant != 1 && cfg.scaled && P.sv && P.sval && n <= cfg.sms * kSmemRows) {
-        const int rpb = cfg.rows_per_block > 0 ? cfg.rows_per_block : kSmemRowsDefault;
-        int grid = std::max(nblk(n, kSmemRowsS), nblk(n, rpb));
-        grid = std::min(grid, cfg.sms);
-        if (cfg.max_blocks > 0) grid = std::min(grid, cfg.max_blocks);
-        grid = std::max(std::max(grid, nblk(n, kSmemRowsS)), 1);
-        P.L = nblk(n, grid);
-        const size_t smem = (size_t)kSmemVectorsS * P.L * sizeof(double);
-        const int blk = n >= cfg.big_rows ? 1024 : cfg.smem_block;
-        pcg_smem_attrs();
-        cudaError_t e = cudaLaunchCooperativeKernel((const void*)pcg_scaled_kernel(blk),
-                                                    dim3(grid), dim3(blk), args, smem, s);
         return e == cudaSuccess ? SDC_OK : SDC_E_CUDA;
     }
     // shared-memory variant: one block per SM at most, each owning <= kSmemRows rows

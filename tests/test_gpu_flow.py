@@ -1,0 +1,101 @@
+"""The node-solve kernels that keep every vector on chip (cg_flow.cuh) against the oracle at
+the edges of their launch rule: chunks of 32 rows, CTAs of 128 rows, one or more rows per
+thread, x in shared or global memory, two or three buffers for r and w; and solves whose
+gamma leaves the window of the fixed-point sums in one iteration, downwards and upwards.
+
+Tolerance: that of the parity tests, 1e-10 relative in the max norm and CG counts to one
+(both sides stop at rtol = 1e-10).
+"""
+
+import numpy as np
+import pytest
+
+import oracle
+import workloads as W
+from workloads.configs import AP_BENCH, Workload
+from workloads.meshes import grid2d
+
+pytestmark = pytest.mark.gpu
+
+RTOL = 1e-10
+
+
+@pytest.fixture(scope="module")
+def torch_dev():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2311_07206_gb300 import build as b
+    b.build()
+    return torch, torch.device("cuda:0")
+
+
+def _workload(nx, ny, h, dt, M=2, sweeps=2, tol=0.0, v=None):
+    mesh = grid2d(nx, ny, h)
+    rng = np.random.default_rng(nx * 1000 + ny)
+    v0 = rng.uniform(0.0, 1.0, mesh.n_nodes) if v is None else v(rng, mesh.n_nodes)
+    return Workload("grid", mesh, np.diag([1.0, 0.5, 1.0]), dict(AP_BENCH), M=M, dt=dt,
+                    sweeps=sweeps, tol=tol, steps=1, v0=v0, w0=np.zeros(mesh.n_nodes))
+
+
+def _check(wl, torch, dev, **opts):
+    from paper_2311_07206_gb300 import Context, default_options
+    ctx = Context.from_workload(wl, options=default_options(cg_maxit=20000, **opts),
+                                stream=torch.cuda.current_stream(dev).cuda_stream)
+    v = torch.tensor(wl.v0, dtype=torch.float64, device=dev)
+    w = torch.tensor(wl.w0, dtype=torch.float64, device=dev)
+    st = ctx.step(v, w, 0.0, wl.dt, wl.sweeps, wl.tol)
+    ctx.close()
+    r = oracle.System.from_mesh(wl.mesh, wl.sigma).step(wl.ionic, wl.M, wl.v0, wl.w0, wl.dt,
+                                                        wl.sweeps, wl.tol, cg_maxit=20000)
+    assert r["status"] == 0
+    for a, b in ((v, r["v"]), (w, r["w"])):
+        assert np.abs(a.cpu().numpy() - b).max() <= RTOL * max(1.0, np.abs(b).max())
+    for k in range(wl.sweeps):
+        for m in range(wl.M):
+            a, b = st.cg_iters[k][m], r["stats"].cg_iters[k * 8 + m]
+            # ill-conditioned solves: counts differ by rounding, within 10 %
+            assert abs(a - b) <= max(1, b // 10), (k, m, a, b)
+    return st
+
+
+@pytest.mark.parametrize("pipelined", [0, 1])
+@pytest.mark.parametrize("nx,ny,blocks", [
+    (2, 2, 0), (4, 8, 0), (3, 11, 0), (8, 16, 0), (3, 43, 0),    # one chunk, one CTA, and one more
+    (139, 140, 0),                                               # 152 CTAs of 128 rows, and more
+    (28, 32, 1), (23, 39, 1),                                    # one row per thread, then more
+    (61, 63, 1), (64, 65, 1),                                    # x on chip, then in global memory
+    (64, 90, 1), (67, 86, 1),                                    # three buffers, then two
+])
+def test_edges_of_the_launch_rule(torch_dev, nx, ny, blocks, pipelined):
+    torch, dev = torch_dev
+    _check(_workload(nx, ny, 0.3, 0.1), torch, dev, cg_pipelined=pipelined, cg_max_blocks=blocks)
+
+
+@pytest.mark.parametrize("pipelined", [0, 1])
+def test_gamma_falls_below_the_window(torch_dev, pipelined):
+    """c K / m ~ 1e-5: gamma falls by about 1e-10 (2^-33) per iteration."""
+    torch, dev = torch_dev
+    st = _check(_workload(40, 37, 0.3, 1e-6), torch, dev, cg_pipelined=pipelined)
+    assert st.cg_iters[0][0] <= 4
+
+
+def test_gamma_rises_above_the_window(torch_dev):
+    """The right-hand side is the lowest mode with a trace of high modes: the first step of
+    CG, exact for the low mode, lifts the others by (lambda_high / lambda_low)^2 > 2^10."""
+    torch, dev = torch_dev
+    wl = _workload(40, 37, 2e-3, 0.1, sweeps=1,
+                   v=lambda rng, n: 0.5 + 1e-8 * rng.standard_normal(n))
+    # gamma_1 / gamma_0 of the same CG on the host: the case does what it says
+    S = oracle.System.from_mesh(wl.mesh, wl.sigma)
+    K, m = S.dense()
+    c = wl.dt * oracle.collocation(wl.M)[2][0, 0]
+    v = wl.v0
+    J = 8.0 * (3.0 * v * v - 2.0 * 1.15 * v + 0.15)
+    f = -K @ v - m * 8.0 * v * (v - 0.15) * (v - 1.0)
+    b = wl.dt * oracle.collocation(wl.M)[1][0].sum() * f
+    A = np.diag(m * (1.0 + c * J)) + c * K
+    d = np.diag(A)
+    r1 = b - (b @ (b / d)) / ((b / d) @ A @ (b / d)) * (A @ (b / d))
+    assert (r1 @ (r1 / d)) / (b @ (b / d)) > 2.0 ** 11
+    _check(wl, torch, dev, cg_pipelined=0)
