@@ -36,6 +36,7 @@ namespace {
 typedef unsigned long long u64;
 
 constexpr int kFlowHead = 10;    // growth of gamma over one iteration that fits the window
+constexpr int kFlowSumHead = 18; // total over largest partial sum (155,648 threads, 2^103 units)
 constexpr int kFlowDrop = 22;    // fall of gamma up to which the sum keeps 2^-54 of its value
 
 // relaxed single-copy-atomic 128-bit access: (value bits, tag)
@@ -57,13 +58,27 @@ __device__ __forceinline__ u64 ld_relaxed64(const u64* p) {
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
+__device__ __forceinline__ void ld_relaxed64x2(const u64* p, u64& a, u64& b) {
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+}
 __device__ __forceinline__ void red_add64(u64* p, u64 v) {
     asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
+// What warp 0 carries from sum to sum.
+struct FlowScalars {
+    u64 prev[2][8];           // each set's words before the running sum
+    double g, den;            // gamma and gamma / alpha of the last sum
+    double inv_g, inv_a;      // 1 / gamma and 1 / alpha of it (0 before the first)
+    double thresh, lo, hi;    // stopping test: bound on sqrt(gamma) and a band around its square
+    double gamma0, energy;
+    int nsum;
+};
+
 // Shared state of one CTA.
 struct FlowShared {
     alignas(16) int lim[32][8];   // limb sums of each warp: 4 of a, 4 of b
+    FlowScalars z;
     double alpha, beta;
     int topa, topb;               // window tops (largest exponent field) of the next sums
     int ovf, ok, state;           // state: 0 go on, 1 converged, 2 non-finite, 3 repeat the sum
@@ -109,65 +124,106 @@ __device__ __forceinline__ void flow_post(double a, double b, FlowShared& S, u64
     }
     __syncthreads();
     if (wid == 0) {
+        // lane: limb lane & 7 of warps lane >> 3, + 4, ...; every load before the first add
+        const int out0 = S.ovf;
+        int x[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int w = (lane >> 3) + 4 * k;
+            x[k] = w < nw ? S.lim[w][lane & 7] : 0;
+        }
         long long s = 0;
-        for (int w = lane >> 3; w < nw; w += 4) s += S.lim[w][lane & 7];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s += x[k];
         s += __shfl_xor_sync(0xffffffffu, s, 8);
         s += __shfl_xor_sync(0xffffffffu, s, 16);
         // top byte: arrivals; next byte: CTAs with a value above the window
-        if (lane < 8) red_add64(acc + lane, (1ull << 56) + ((u64)(S.ovf != 0) << 48) + (u64)s);
+        if (lane < 8) red_add64(acc + lane, (1ull << 56) + ((u64)(out0 != 0) << 48) + (u64)s);
     }
 }
 
-// Quotient by Newton's iteration from the hardware's reciprocal estimate (relative error
-// 2^-20): 1/d (1 + e + e^2) with e = 1 - d y, then one residual correction of the quotient.
-// Divisors outside the normal range with a margin take the division.
+// The rare ends of the paths below, kept out of line so that none of their long sequences is
+// executed speculatively.
+__device__ __noinline__ double flow_divide(double n, double d) { return n / d; }
+__device__ __noinline__ double flow_ldexp(double v, int e) { return ldexp(v, e); }
+__device__ __noinline__ bool flow_sqrt_at_most(double g, double thresh) { return sqrt(g) <= thresh; }
+
+// Quotient by Newton's iteration from the hardware's reciprocal estimate y (relative error
+// 2^-20): n y (1 + e + e^2), e = 1 - d y, within an ulp of n / d.  Operands near the ends of
+// the exponent range take the division.  Four FP64 operations (65 cycles each) where the
+// division takes 570 cycles.
 __device__ __forceinline__ double flow_quot(double n, double d) {
     const int f = (int)((u64)__double_as_longlong(d) >> 52) & 0x7ff;
     const int fn = (int)((u64)__double_as_longlong(n) >> 52) & 0x7ff;
-    if (f < 100 || f > 1946 || fn < 100 || fn > 1946 || abs(fn - f) > 900) return n / d;
+    if (min(f, fn) < 200 || max(f, fn) > 1846 || abs(fn - f) > 800) return flow_divide(n, d);
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
     const double e = fma(-d, y, 1.0), q0 = n * y;
     const double e2 = fma(e, e, e);
-    const double q = fma(q0, e2, q0);
-    const double r = fma(-d, q, n);
-    return fma(r, y, q);
+    return fma(q0, e2, q0);
 }
 
-// What warp 0 carries from sum to sum (the same in every lane but prev).
-struct FlowScalars {
-    u64 prev[2];              // lane's word of each set before the running sum (lanes 0..7)
-    double inv_g, inv_a;      // 1 / gamma and 1 / alpha of the last sum (0 before the first)
-    double thresh, lo, hi;    // stopping test: bound on sqrt(gamma) and a band around its square
-    double gamma0, energy, rn;
-    int nsum;
-};
+// Total of a value's four limb sums in units of 2^(top - 1125), rounded once: the digits are
+// carried into A 2^52 + B with |A| < 2^51 and 0 <= B < 2^52, which integer additions place in
+// the significands of 1.5 2^52 + A and 2^52 + B.  in: false when the total has grown out of
+// that range (2^103 units).
+__device__ __forceinline__ double flow_value(long long s0, long long s1, long long s2, long long s3,
+                                             int top, bool& in) {
+    constexpr long long m = (1ll << 26) - 1;
+    s1 += s0 >> 26;
+    s2 += s1 >> 26;
+    s3 += s2 >> 26;
+    in = s3 < (1ll << 24) && s3 >= -(1ll << 24);
+    const double a = __longlong_as_double(0x4338000000000000ll + ((s3 << 26) + (s2 & m)));
+    const double b = __longlong_as_double(0x4330000000000000ll + (((s1 & m) << 26) + (s0 & m)));
+    const double v = fma(a - 0x1.8p52, 0x1p52, b - 0x1p52);
+    // times 2^(top - 1125), in the exponent field where the result is normal
+    const long long w = __double_as_longlong(v);
+    const int f = (int)(w >> 52) & 0x7ff, g = f + top - 1125;
+    if (f == 0) return 0.0;
+    if (g >= 1 && g <= 2046) return __longlong_as_double(w + ((long long)(top - 1125) << 52));
+    return flow_ldexp(v, top - 1125);
+}
 
 __device__ __forceinline__ void flow_scalars_init(FlowScalars& Z) {
-    Z.prev[0] = Z.prev[1] = 0;
-    Z.inv_g = Z.inv_a = 0.0;
-    Z.thresh = Z.lo = Z.hi = 0.0;
-    Z.gamma0 = Z.energy = Z.rn = 0.0;
-    Z.nsum = 0;
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) Z.prev[0][k] = Z.prev[1][k] = 0;
+        Z.g = Z.den = 1.0;
+        Z.inv_g = Z.inv_a = 0.0;
+        Z.thresh = Z.lo = Z.hi = 0.0;
+        Z.gamma0 = Z.energy = 0.0;
+        Z.nsum = 0;
+    }
 }
 
-// Warp 0: wait for the sums posted as number `npub`, derive alpha and beta (cg_scalars'
+// Warp 0: wait for the sums posted to set `set`, derive alpha and beta (cg_scalars'
 // recurrences, den_t = delta_t - beta_t gamma_t / alpha_{t-1}) and the next windows.
 // exact: the windows came from the exact exponents (no repeat for a fall of gamma).
-__device__ __forceinline__ void flow_totals(FlowShared& S, FlowScalars& Z, const u64* acc, int set,
-                                            int G, bool exact, double rtol, long long budget,
-                                            int* err) {
+__device__ __forceinline__ void flow_totals(FlowShared& S, const u64* acc, int set, int G, bool exact,
+                                            long long budget, int* err) {
     const int lane = threadIdx.x & 31;
-    u64 v = 0, d = 0;
-    const u64 prev = set ? Z.prev[1] : Z.prev[0];
+    FlowScalars& Z = S.z;
+    const double inv_g = Z.inv_g, inv_a = Z.inv_a;
+    const long long lo = __double_as_longlong(Z.lo), hi = __double_as_longlong(Z.hi);
+    const int nsum = Z.nsum, topa = S.topa, topb = S.topb;
+    // lane 0 reads gamma's words, lane 1 delta's: a word with all its arrivals is final
+    u64 v[4], d[4];
+    u64* const prev = Z.prev[set] + 4 * (lane & 1);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        d[k] = (1ull << 47) - prev[k];
+        v[k] = 0;
+    }
     const long long t0 = clock64();
     int ok = 1;
     while (true) {
         bool here = true;
-        if (lane < 8) {
-            v = ld_relaxed64(acc + lane);
-            d = v - prev + (1ull << 47);
-            here = (d >> 56) == (u64)G;
+        if (lane < 2) {
+            ld_relaxed64x2(acc + 4 * lane, v[0], v[1]);
+            ld_relaxed64x2(acc + 4 * lane + 2, v[2], v[3]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) here = here && ((v[k] + d[k]) >> 56) == (u64)G;
         }
         if (__all_sync(0xffffffffu, here)) break;
         if (clock64() - t0 > budget) {
@@ -183,70 +239,86 @@ __device__ __forceinline__ void flow_totals(FlowShared& S, FlowScalars& Z, const
         }
         return;
     }
-    if (set) Z.prev[1] = v; else Z.prev[0] = v;
-    const bool above = __any_sync(0xffffffffu, lane < 8 && ((d >> 48) & 0xff) != 0);
-    if (lane == 0) S.ovf = 0;
-    // the totals: lanes 0-3 assemble gamma, lanes 4-7 delta (the other lanes repeat them)
-    const long long part = (long long)(d & 0xffffffffffffull) - (1ll << 47);
-    __int128 q = 0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-        q += (__int128)__shfl_sync(0xffffffffu, part, (lane & 4) + k) << (26 * k);
-    const double tot = xs_to_double(q, ((lane & 4) ? S.topb : S.topa) - 2);
-    const double g = __shfl_sync(0xffffffffu, tot, 0), dl = __shfl_sync(0xffffffffu, tot, 4);
+    for (int k = 0; k < 4; ++k) d[k] += v[k];
+    bool in;
+    const double tot = flow_value((long long)(d[0] & 0xffffffffffffull) - (1ll << 47),
+                                  (long long)(d[1] & 0xffffffffffffull) - (1ll << 47),
+                                  (long long)(d[2] & 0xffffffffffffull) - (1ll << 47),
+                                  (long long)(d[3] & 0xffffffffffffull) - (1ll << 47),
+                                  lane ? topb : topa, in);
+    const bool above = __any_sync(0xffffffffu, lane < 2 && (!in || ((d[0] >> 48) & 0xff) != 0));
+    const double g = __shfl_sync(0xffffffffu, tot, 0), dl = __shfl_sync(0xffffffffu, tot, 1);
     const int fg = xs_field(g);
-    // the decisions compare bit patterns (g >= 0): an FP64 comparison has 64 cycles latency
+    // the decisions compare bit patterns (g >= 0): an FP64 comparison has 65 cycles latency
     const long long gb = __double_as_longlong(g);
     int state = 0;
     if (above) {
         state = 3;
-    } else if (Z.nsum == 0) {
-        if (gb == 0) state = 1;
-    } else if (gb <= __double_as_longlong(Z.lo)) {
-        state = 1;
-    } else if (gb < __double_as_longlong(Z.hi) && sqrt(g) <= Z.thresh) {
-        state = 1;
-    } else if (!exact && fg < S.topa - kFlowHead - kFlowDrop) {
-        state = 3;
+    } else if (nsum == 0) {
+        state = gb == 0 ? 1 : 0;
+    } else if (gb < hi) {
+        state = gb <= lo || flow_sqrt_at_most(g, Z.thresh) ? 1 : 0;
     }
-    if (state != 3) {
-        Z.rn = g;
-        if (Z.nsum == 0) Z.gamma0 = g;
-    }
-    if (state == 0) {
-        const double beta = g * Z.inv_g;
-        const double den = fma(-beta, g * Z.inv_a, dl);
-        // lane 0: alpha = gamma / den, lane 1: 1 / gamma, lane 2: 1 / alpha
-        const double num = lane == 0 ? g : lane == 1 ? 1.0 : den;
-        const double quo = flow_quot(num, lane == 0 ? den : g);
-        const double alpha = __shfl_sync(0xffffffffu, quo, 0);
-        Z.inv_g = __shfl_sync(0xffffffffu, quo, 1);
-        Z.inv_a = __shfl_sync(0xffffffffu, quo, 2);
-        if (lane == 0) {
+    if (state == 0 && !exact && fg < topa - kFlowHead - kFlowDrop) state = 3;
+    const double beta = g * inv_g;
+    const double den = fma(-beta, g * inv_a, dl);
+    const double alpha = flow_quot(g, den);
+    if (state == 0 && xs_field(alpha) == 2047) state = 2;
+    if (lane == 0) {
+        S.state = state;
+        S.ovf = 0;
+        if (state != 3) Z.g = g;
+        if (state == 0) {
             S.alpha = alpha;
             S.beta = beta;
+            Z.den = den;
             S.topa = S.topb = min(fg + kFlowHead, 2046);
         }
-        Z.energy = fma(alpha, g, Z.energy);   // x' A x = sum of alpha_t gamma_t
-        if (xs_field(alpha) == 2047) state = 2;
-        ++Z.nsum;
     }
-    if (lane == 0) S.state = state;
+    if (lane < 2) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) prev[k] = v[k];
+    }
 }
+
 // Once, after the first sum's scalars are out: sqrt(gamma) <= rtol sqrt(gamma_0) is decided by
 // comparing gamma with a band of 2^-50 around the squared bound and by the square root
 // itself inside it.  Squares that leave the normal range always take the square root.
-__device__ __forceinline__ void flow_first_bound(FlowScalars& Z, double rtol) {
-    Z.thresh = rtol * sqrt(Z.gamma0);
-    const double q = Z.thresh * Z.thresh;
+__device__ __noinline__ void flow_first_bound(FlowScalars& Z, double g, double rtol) {
+    const double thresh = rtol * sqrt(g), q = thresh * thresh;
     const bool normal = q > 1e-280 && q < 1e280;
-    Z.lo = normal ? q * (1.0 - 0x1p-50) : 0.0;
-    Z.hi = normal ? q * (1.0 + 0x1p-50) : INFINITY;
+    if ((threadIdx.x & 31) == 0) {
+        Z.gamma0 = g;
+        Z.thresh = thresh;
+        Z.lo = normal ? q * (1.0 - 0x1p-50) : 0.0;
+        Z.hi = normal ? q * (1.0 + 0x1p-50) : INFINITY;
+    }
+}
+
+// Warp 0, off the critical path (the other warps are at the update): what the next sum needs.
+__device__ __forceinline__ void flow_next(FlowShared& S, double rtol) {
+    const int lane = threadIdx.x & 31;
+    FlowScalars& Z = S.z;
+    const double g = Z.g, den = Z.den;
+    const double q = flow_quot(lane == 0 ? 1.0 : den, g);   // lane 0: 1 / gamma, lane 1: 1 / alpha
+    const double e = fma(S.alpha, g, Z.energy);             // x' A x = sum of alpha_t gamma_t
+    const int nsum = Z.nsum;
+    __syncwarp();
+    if (lane == 0) {
+        Z.inv_g = q;
+        Z.energy = e;
+        Z.nsum = nsum + 1;
+    }
+    if (lane == 1) Z.inv_a = q;
+    if (nsum == 0) flow_first_bound(Z, g, rtol);
+    __syncwarp();
 }
 
 // Windows from the exact largest exponents of the CTAs' partial sums, with a release /
 // acquire grid barrier that also publishes every global write before it.  emax words hold
-// (generation << 32) | field and only grow.  Returns false after a timeout.
+// (generation << 32) | field and only grow.  The windows leave room for the
+// total over the largest partial sum.  Returns false after a timeout.
 __device__ __forceinline__ bool flow_window(double a, double b, FlowShared& S, u64* emax,
                                             unsigned* bar, int G, unsigned& epoch, unsigned gen,
                                             int headb, long long budget, int* err) {
@@ -268,7 +340,7 @@ __device__ __forceinline__ bool flow_window(double a, double b, FlowShared& S, u
             S.ok = barrier_arrive_wait(bar, epoch, budget, err);
             const int ga = (int)(unsigned)ld_relaxed64(emax), gb = (int)(unsigned)ld_relaxed64(emax + 1);
             S.state = ga >= 2047 || gb >= 2047 ? 2 : 0;
-            S.topa = ga;
+            S.topa = min(ga + kFlowSumHead, 2046);
             S.topb = min(gb + headb, 2046);
             S.ovf = 0;
         }
@@ -373,8 +445,8 @@ __device__ __forceinline__ bool flow_start(const CgParams& P, const FlowParams& 
         if (G == 1 && t == 0) raise_error(P.err, SDC_E_TIMEOUT);
         return false;
     }
-    // delta's partial sums: |w.r| of a thread <= |A| gamma, gamma <= 2^17 largest partial
-    if (!flow_window(ga, ga, S, Q.emax, Q.bar, G, epoch, 1u, 21, P.budget, P.err)) return false;
+    // delta's partial sums: |w.r| of a thread <= |A| gamma, gamma <= 2^17.3 largest partial
+    if (!flow_window(ga, ga, S, Q.emax, Q.bar, G, epoch, 1u, 22, P.budget, P.err)) return false;
     if (S.state == 2) {
         if (blockIdx.x == 0 && t == 0) raise_error(P.err, SDC_E_NONFINITE);
         return false;
@@ -420,7 +492,7 @@ __device__ __forceinline__ bool flow_start(const CgParams& P, const FlowParams& 
 // neighbours' x travel as tagged words.  xt(l): the CTA's x~.
 template <int MAXT, class X>
 __device__ __forceinline__ void flow_finish(const CgParams& P, const FlowParams& Q, FlowShared& S,
-                                            const FlowScalars& Z, int r0, int nl, int it, X&& xt) {
+                                            int r0, int nl, int it, X&& xt) {
     const int t = threadIdx.x, B = blockDim.x, ld = P.ld;
     const bool lead = blockIdx.x == 0 && t == 0;
     if (S.state == 2) {
@@ -429,8 +501,8 @@ __device__ __forceinline__ void flow_finish(const CgParams& P, const FlowParams&
     }
     if (lead) {
         *P.iters_out = it;
-        *P.relres_out = Z.gamma0 > 0.0 ? sqrt(fabs(Z.rn) / Z.gamma0) : 0.0;
-        if (P.energy_out) *P.energy_out = Z.energy;
+        *P.relres_out = S.z.gamma0 > 0.0 ? sqrt(fabs(S.z.g) / S.z.gamma0) : 0.0;
+        if (P.energy_out) *P.energy_out = S.z.energy;
     }
     // the words of iteration it - 1, whose readers are done: their CTAs posted sum `it`
     ulonglong2* const pub = Q.pub + (size_t)((it + 1) & 1) * ld;
@@ -479,8 +551,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
     const int wrow = wid == 0 ? nw - 1 : wid - 1;   // the warps' order over the chunks
     unsigned epoch = 0, gen = 1;
     double ga, de, alpha = 0.0, beta = 0.0;
-    FlowScalars Z;
-    flow_scalars_init(Z);
+    flow_scalars_init(S.z);
     if (!flow_start<MAXT>(
             P, Q, S, r0, nl, epoch, ga, de,
             [&](int l, double r) {
@@ -510,7 +581,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
         u64* const acc = Q.acc + 8 * (npub & 1);
         flow_post(ga, de, S, acc);
         if (wid == 0)
-            flow_totals(S, Z, acc, npub & 1, G, exact, P.rtol, P.budget, P.err);
+            flow_totals(S, acc, npub & 1, G, exact, P.budget, P.err);
         ++npub;
         if (!redo) {
             if (it > 0) update_px();
@@ -537,7 +608,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
         __syncthreads();
         if (!S.ok) return;
         if (S.state == 3) {
-            if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, 0, P.budget, P.err)) return;
+            if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, kFlowSumHead, P.budget, P.err)) return;
             if (S.state == 0) {
                 exact = redo = true;
                 continue;
@@ -553,7 +624,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
         alpha = S.alpha;
         beta = S.beta;
         if (t == 0) S.next = 0;
-        if (wid == 0 && it == 1) flow_first_bound(Z, P.rtol);
+        if (wid == 0) flow_next(S, P.rtol);
         const u64 tag = Q.id + (u64)it + 1;
         ulonglong2* const pub = Q.pub + (size_t)(it & 1) * ld + r0;
         ga = de = 0.0;
@@ -578,7 +649,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
         rc = ro;
         ro = q;
     }
-    flow_finish<MAXT>(P, Q, S, Z, r0, nl, it, [&](int l) { return xs[l]; });
+    flow_finish<MAXT>(P, Q, S, r0, nl, it, [&](int l) { return xs[l]; });
 }
 
 // ---- classical arrangement (see pcgc_group), scaled form -----------------------------
@@ -605,8 +676,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) 
     const int wrow = wid == 0 ? nw - 1 : wid - 1;
     unsigned epoch = 0, gen = 1;
     double ga, de, alpha = 0.0, beta = 0.0;
-    FlowScalars Z;
-    flow_scalars_init(Z);
+    flow_scalars_init(S.z);
     if (!flow_start<MAXT>(
             P, Q, S, r0, nl, epoch, ga, de,
             [&](int l, double r) {
@@ -633,13 +703,13 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) 
         u64* const acc = Q.acc + 8 * (npub & 1);
         flow_post(ga, de, S, acc);
         if (wid == 0)
-            flow_totals(S, Z, acc, npub & 1, G, exact, P.rtol, P.budget, P.err);
+            flow_totals(S, acc, npub & 1, G, exact, P.budget, P.err);
         ++npub;
         if (late && it > 0 && !redo) update_px(fb);
         __syncthreads();
         if (!S.ok) return;
         if (S.state == 3) {
-            if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, 0, P.budget, P.err)) return;
+            if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, kFlowSumHead, P.budget, P.err)) return;
             if (S.state == 0) {
                 exact = redo = true;
                 continue;
@@ -666,8 +736,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) 
                 ss[l] = s;
             }
         }
+        if (wid == 0) flow_next(S, P.rtol);
         __syncthreads();
-        if (wid == 0 && it == 1) flow_first_bound(Z, P.rtol);
         if (!late) update_px(rb);
         ga = de = 0.0;
         for (int c = wrow; c < nch; c += nw) {
@@ -689,7 +759,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) 
         wb = fb;
         fb = late ? q : rb;
     }
-    flow_finish<MAXT>(P, Q, S, Z, r0, nl, it, [&](int l) { return xs[l]; });
+    flow_finish<MAXT>(P, Q, S, r0, nl, it, [&](int l) { return xs[l]; });
 }
 
 }  // namespace

@@ -2205,7 +2205,7 @@ bool flow_shape(int n, bool classical, const PcgConfig& cfg, FlowShape& f) {
     int l = nblk(n, gm);
     if (cfg.rows_per_block > 0) l = std::max(l, std::min(cfg.rows_per_block, cap));
     const int maxb = n >= cfg.big_rows ? 1024 : std::min(std::max(cfg.smem_block, 64), 1024);
-    f.L = std::min(l <= 896 ? (l + 127) / 128 * 128 : (l + 31) / 32 * 32, cap);
+    f.L = std::min(l <= 96 ? 96 : l <= 896 ? (l + 127) / 128 * 128 : (l + 31) / 32 * 32, cap);
     f.grid = nblk(n, f.L);
     f.block = std::min(32 + std::min(f.L, (n + 31) / 32 * 32), maxb);
     if (classical) {
