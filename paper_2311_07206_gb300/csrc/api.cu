@@ -10,6 +10,7 @@
 #include <cstring>
 #include <string>
 #include <functional>
+#include <mutex>
 #include <vector>
 
 #include "sdc_internal.h"
@@ -1297,6 +1298,67 @@ sdc_status sdc_get_matrix(const sdc_ctx* cc, int* row_ptr, int* col, double* val
     return SDC_OK;
 }
 
+// Workspace of one stand-alone solve, from a stream-ordered pool of this library: cudaMalloc
+// and cudaFree take 150 us of a call whose solve takes 80.  One pool per device, made on first
+// use (and again after cudaDeviceReset, known by the context's id); it keeps at most kSolvePool
+// bytes between calls and sdc_destroy gives those back.  The driver's pools are safe with
+// several threads and streams.  Where none can be had the workspace is allocated as such.
+constexpr unsigned long long kSolvePool = 64ull << 20;
+struct SolvePools {
+    std::mutex mu;
+    cudaMemPool_t pool[64] = {};
+    unsigned long long ctx[64] = {};
+    cudaMemPool_t get() {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+        std::lock_guard<std::mutex> lock(mu);
+        const unsigned long long id = current_context_id();
+        if (id == 0) return nullptr;
+        if (!pool[dev] || ctx[dev] != id) {
+            cudaMemPoolProps props = {};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            cudaMemPool_t q = nullptr;
+            unsigned long long keep = kSolvePool;
+            if (cudaMemPoolCreate(&q, &props) != cudaSuccess ||
+                cudaMemPoolSetAttribute(q, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+                cudaGetLastError();
+                return nullptr;
+            }
+            pool[dev] = q;
+            ctx[dev] = id;
+        }
+        return pool[dev];
+    }
+    void trim() {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return;
+        std::lock_guard<std::mutex> lock(mu);
+        if (pool[dev] && ctx[dev] == current_context_id()) cudaMemPoolTrimTo(pool[dev], 0);
+    }
+};
+static SolvePools g_solve_pools;
+struct SolveWorkspace {
+    void* p = nullptr;
+    cudaStream_t s;
+    bool pooled = false;
+    SolveWorkspace(size_t bytes, cudaStream_t stream) : s(stream) {
+        if (cudaMemPool_t q = g_solve_pools.get())
+            pooled = cudaMallocFromPoolAsync(&p, bytes, q, s) == cudaSuccess;
+        if (!pooled) {
+            cudaGetLastError();
+            if (cudaMalloc(&p, bytes) != cudaSuccess) p = nullptr;
+        }
+    }
+    ~SolveWorkspace() {
+        if (pooled) cudaFreeAsync(p, s);
+        else cudaFree(p);
+    }
+    SolveWorkspace(const SolveWorkspace&) = delete;
+    SolveWorkspace& operator=(const SolveWorkspace&) = delete;
+};
+
 static sdc_status pcg_solve_body(int n, const double* d_val, const int* d_col, const int* d_len,
                                  int ld, int width, const double* d_kdiag, const double* d_mass,
                                  const double* d_J, double c, const double* d_b, double* d_x,
@@ -1321,6 +1383,40 @@ static sdc_status pcg_solve_body(int n, const double* d_val, const int* d_col, c
         (width > 0 && (!d_val || !d_col)) || !(rtol > 0.0) || maxit < 1 || !std::isfinite(c))
         return fail(nullptr, SDC_E_INVALID, "sdc_pcg_solve: invalid arguments");
     cudaStream_t s = (cudaStream_t)stream;
+    Ell A;
+    A.val = const_cast<double*>(d_val);
+    A.col = const_cast<int*>(d_col);
+    A.len = const_cast<int*>(d_len);
+    A.ld = ld;
+    A.width = width;
+    int status = SDC_OK;
+    int h[3] = {0, 0, 0};   // -, error, iterations
+    double hr = 0.0;
+    const size_t fd = pcg_standalone_flow_doubles(n, ld, width);
+    if (fd > 0) {
+        SolveWorkspace ws(fd * sizeof(double), s);
+        if (!ws.p) return fail(nullptr, SDC_E_NOMEM, "sdc_pcg_solve: workspace allocation failed");
+        double r[kStandaloneResults];
+        if (launch_pcg_standalone_flow(n, A, d_kdiag, d_mass, d_J, c, d_b, d_x, rtol, maxit,
+                                       4000000000LL, (double*)ws.p, s) != SDC_OK) {
+            status = cuda_fail(nullptr, "sdc_pcg_solve launch");
+        } else {
+            cudaMemcpyAsync(r, (double*)ws.p + fd - kStandaloneResults, sizeof r,
+                            cudaMemcpyDeviceToHost, s);
+            if (cudaStreamSynchronize(s) != cudaSuccess) {
+                status = cuda_fail(nullptr, "sdc_pcg_solve");
+            } else {
+                hr = r[0];
+                std::memcpy(h + 1, r + 1, 2 * sizeof(int));
+                if (h[1] != 0)
+                    status = fail(nullptr, (sdc_status)h[1], "sdc_pcg_solve: %s",
+                                  sdc_status_string(h[1]));
+            }
+        }
+        if (iters) *iters = h[2];
+        if (relres) *relres = hr;
+        return (sdc_status)status;
+    }
     const int block = 256;
     const int maxb = pcg_max_blocks(block);
     // workspace: 8 vectors of n, the published m in two buffers ld apart (the kernels
@@ -1343,15 +1439,6 @@ static sdc_status pcg_solve_body(int n, const double* d_val, const int* d_col, c
     w.bar = sc;
     w.err = (int*)(sc + 1);
     w.iters = (int*)(sc + 2);
-    Ell A;
-    A.val = const_cast<double*>(d_val);
-    A.col = const_cast<int*>(d_col);
-    A.len = const_cast<int*>(d_len);
-    A.ld = ld;
-    A.width = width;
-    int status = SDC_OK;
-    int h[3] = {0, 0, 0};
-    double hr = 0.0;
     cudaMemsetAsync(w.relres, 0, sizeof(double) + 3 * sizeof(unsigned), s);
     if (launch_pcg_standalone(n, A, d_kdiag, d_mass, d_J, c, d_b, d_x, rtol, maxit, 4000000000LL,
                               block, w, s) != SDC_OK) {
@@ -1654,6 +1741,7 @@ void sdc_destroy(sdc_ctx* c) {
     cudaStreamSynchronize(c->stream);
     free_all(c);
     delete c;
+    g_solve_pools.trim();
 }
 
 }  // extern "C"

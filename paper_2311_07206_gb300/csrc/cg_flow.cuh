@@ -105,36 +105,38 @@ __device__ __forceinline__ bool flow_limbs(double v, int top, int (&l)[4]) {
 }
 
 // Post the CTA's sums of a and b to the words acc[0..7]: every thread calls it; it holds
-// one CTA barrier, after which warp 0 adds the warps' limbs and posts them.
-__device__ __forceinline__ void flow_post(double a, double b, FlowShared& S, u64* acc) {
+// one CTA barrier, after which warp 0 adds the warps' limbs and posts them.  A warp without
+// rows (warp 0 of a CTA with one row per thread) leaves its zeros of flow_scalars_init.
+__device__ __forceinline__ void flow_post(double a, double b, bool rows, FlowShared& S, u64* acc) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    int la[4], lb[4];
-    bool in = flow_limbs(a, S.topa, la);
-    in = flow_limbs(b, S.topb, lb) && in;
-    const bool out = __any_sync(0xffffffffu, !in);
+    if (rows) {
+        int la[4], lb[4];
+        bool in = flow_limbs(a, S.topa, la);
+        in = flow_limbs(b, S.topb, lb) && in;
+        const bool out = __any_sync(0xffffffffu, !in);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        la[k] = __reduce_add_sync(0xffffffffu, la[k]);
-        lb[k] = __reduce_add_sync(0xffffffffu, lb[k]);
-    }
-    if (lane == 0) {
-        *reinterpret_cast<int4*>(&S.lim[wid][0]) = make_int4(la[0], la[1], la[2], la[3]);
-        *reinterpret_cast<int4*>(&S.lim[wid][4]) = make_int4(lb[0], lb[1], lb[2], lb[3]);
-        if (out) S.ovf = 1;
+        for (int k = 0; k < 4; ++k) {
+            la[k] = __reduce_add_sync(0xffffffffu, la[k]);
+            lb[k] = __reduce_add_sync(0xffffffffu, lb[k]);
+        }
+        if (lane == 0) {
+            *reinterpret_cast<int4*>(&S.lim[wid][0]) = make_int4(la[0], la[1], la[2], la[3]);
+            *reinterpret_cast<int4*>(&S.lim[wid][4]) = make_int4(lb[0], lb[1], lb[2], lb[3]);
+            if (out) S.ovf = 1;
+        }
     }
     __syncthreads();
     if (wid == 0) {
         // lane: limb lane & 7 of warps lane >> 3, + 4, ...; every load before the first add
         const int out0 = S.ovf;
-        int x[8];
+        long long s = S.lim[lane >> 3][lane & 7];   // (rows of warps beyond the block: zero)
+        if (nw > 4) {
+            int x[7];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int w = (lane >> 3) + 4 * k;
-            x[k] = w < nw ? S.lim[w][lane & 7] : 0;
+            for (int k = 0; k < 7; ++k) x[k] = S.lim[(lane >> 3) + 4 * k + 4][lane & 7];
+#pragma unroll
+            for (int k = 0; k < 7; ++k) s += x[k];
         }
-        long long s = 0;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) s += x[k];
         s += __shfl_xor_sync(0xffffffffu, s, 8);
         s += __shfl_xor_sync(0xffffffffu, s, 16);
         // top byte: arrivals; next byte: CTAs with a value above the window
@@ -155,12 +157,13 @@ __device__ __noinline__ bool flow_sqrt_at_most(double g, double thresh) { return
 __device__ __forceinline__ double flow_quot(double n, double d) {
     const int f = (int)((u64)__double_as_longlong(d) >> 52) & 0x7ff;
     const int fn = (int)((u64)__double_as_longlong(n) >> 52) & 0x7ff;
-    if (min(f, fn) < 200 || max(f, fn) > 1846 || abs(fn - f) > 800) return flow_divide(n, d);
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
     const double e = fma(-d, y, 1.0), q0 = n * y;
     const double e2 = fma(e, e, e);
-    return fma(q0, e2, q0);
+    const double q = fma(q0, e2, q0);
+    if (min(f, fn) < 200 || max(f, fn) > 1846 || abs(fn - f) > 800) return flow_divide(n, d);
+    return q;
 }
 
 // Total of a value's four limb sums in units of 2^(top - 1125), rounded once: the digits are
@@ -185,7 +188,9 @@ __device__ __forceinline__ double flow_value(long long s0, long long s1, long lo
     return flow_ldexp(v, top - 1125);
 }
 
-__device__ __forceinline__ void flow_scalars_init(FlowScalars& Z) {
+__device__ __forceinline__ void flow_scalars_init(FlowShared& S) {
+    FlowScalars& Z = S.z;
+    for (int k = threadIdx.x; k < 256; k += blockDim.x) S.lim[k >> 3][k & 7] = 0;
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < 8; ++k) Z.prev[0][k] = Z.prev[1][k] = 0;
@@ -264,7 +269,7 @@ __device__ __forceinline__ void flow_totals(FlowShared& S, const u64* acc, int s
     const double beta = g * inv_g;
     const double den = fma(-beta, g * inv_a, dl);
     const double alpha = flow_quot(g, den);
-    if (state == 0 && xs_field(alpha) == 2047) state = 2;
+    // (a non-finite alpha shows in the next sums, whose exact exponents end the solve)
     if (lane == 0) {
         S.state = state;
         S.ovf = 0;
@@ -351,8 +356,8 @@ __device__ __forceinline__ bool flow_window(double a, double b, FlowShared& S, u
 
 // Off-diagonal product of row i: acc + sum_k val(k) x(col(k)) in slot order.  Columns of this
 // CTA (rows [r0, r0 + nl)) come from shared memory (own), the others from their published
-// words, read again until they carry `tag`.  All loads of CH slots are issued before the
-// first is used.
+// words, read again until they carry `tag`.  val(k) is the value of slot k.  All loads of CH
+// slots are issued before the first is used.
 template <int CH, class Val>
 __device__ __forceinline__ double flow_row_dot(double acc, int len, size_t i, int ld,
                                                const int* __restrict__ col, int ncol, int r0, int nl,
@@ -370,7 +375,7 @@ __device__ __forceinline__ double flow_row_dot(double acc, int len, size_t i, in
             if (k0 + k < len) {
                 const size_t q = (size_t)(k0 + k) * ld + i;
                 j[k] = sdc_idx(__ldg(col + q), ncol, site);
-                a[k] = val(q);
+                a[k] = val(k0 + k);
             }
         }
         unsigned pend = 0;
@@ -406,20 +411,43 @@ __device__ __forceinline__ double flow_row_dot(double acc, int len, size_t i, in
     return acc;
 }
 
+// f(l) for the thread's local rows: 32-row chunks over the warps, warp 0 last (a CTA with one
+// row per thread leaves it none); the passes that feed the sums use this order.
+template <class F>
+__device__ __forceinline__ void flow_rows(int nl, F&& f) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int c = wid == 0 ? nw - 1 : wid - 1; 32 * c < nl; c += nw) {
+        const int l = 32 * c + lane;
+        if (l < nl) f(l);
+    }
+}
+
+// The same over the warps but warp 0: p and x, while warp 0 sees to the sums.
+template <class F>
+__device__ __forceinline__ void flow_rows_px(int nl, F&& f) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if (wid == 0) return;
+    for (int c = wid - 1; 32 * c < nl; c += nw - 1) {
+        const int l = 32 * c + lane;
+        if (l < nl) f(l);
+    }
+}
+
 template <int MAXT>
 struct FlowChunk {
-    static constexpr int value = MAXT > 512 ? 3 : 6;
+    static constexpr int value = MAXT > 768 ? 3 : MAXT > 512 ? 4 : 7;
 };
 
 // First phase of a solve on the CTA's rows: s = diag^-1/2, r = s b (and zero vectors), both
 // published plainly, then a grid barrier that also finds the first windows, then the scaled
-// off-diagonals c s_i a_ij s_j and w = (I + c S K_off S) r.  f(l, r) receives a row's r,
+// off-diagonals c s_i a_ij s_j (slot k of local row l at vb[k vs + l]) and
+// w = (I + c S K_off S) r.  f(l, r) receives a row's r,
 // g(l, w) its w; gamma and delta partial sums in ga, de.  Returns false to leave the kernel.
 template <int MAXT, class F, class H>
 __device__ __forceinline__ bool flow_start(const CgParams& P, const FlowParams& Q, FlowShared& S,
-                                           int r0, int nl, unsigned& epoch, double& ga, double& de,
-                                           F&& f, H&& h) {
-    const int t = threadIdx.x, B = blockDim.x, G = gridDim.x, ld = P.ld;
+                                           int r0, int nl, double* vb, int vs, unsigned& epoch,
+                                           double& ga, double& de, F&& f, H&& h) {
+    const int t = threadIdx.x, G = gridDim.x, ld = P.ld;
     const double c = P.c;
     ga = de = 0.0;
     if (t == 0) {
@@ -427,7 +455,7 @@ __device__ __forceinline__ bool flow_start(const CgParams& P, const FlowParams& 
         S.ovf = 0;
         S.next = 0;
     }
-    for (int l = t; l < nl; l += B) {
+    flow_rows(nl, [&](int l) {
         const int i = r0 + l;
         const double d = P.mc[i] * (1.0 + c * P.J[i]) + c * P.kdc[i];
         double si = 0.0;
@@ -439,7 +467,7 @@ __device__ __forceinline__ bool flow_start(const CgParams& P, const FlowParams& 
         P.u[i] = r;
         ga += r * r;
         f(l, r);
-    }
+    });
     if (P.inject_fault && blockIdx.x == G - 1) {
         // leave without arriving: every other CTA's bounded wait runs out
         if (G == 1 && t == 0) raise_error(P.err, SDC_E_TIMEOUT);
@@ -452,7 +480,7 @@ __device__ __forceinline__ bool flow_start(const CgParams& P, const FlowParams& 
         return false;
     }
     constexpr int CH = FlowChunk<MAXT>::value;
-    for (int l = t; l < nl; l += B) {
+    flow_rows(nl, [&](int l) {
         const int i = r0 + l;
         const int len = __ldg(P.alen + i);
         const double csi = c * __ldcg(P.sv + i);
@@ -478,13 +506,13 @@ __device__ __forceinline__ bool flow_start(const CgParams& P, const FlowParams& 
             for (int k = 0; k < CH; ++k)
                 if (k0 + k < len) {
                     const double a = csi * av[k] * sj[k];
-                    P.sval[(size_t)(k0 + k) * ld + i] = a;
+                    vb[(size_t)(k0 + k) * vs + l] = a;
                     acc += a * uj[k];
                 }
         }
         h(l, acc);
         de += acc * ri;
-    }
+    });
     return true;
 }
 
@@ -493,8 +521,8 @@ __device__ __forceinline__ bool flow_start(const CgParams& P, const FlowParams& 
 template <int MAXT, class X>
 __device__ __forceinline__ void flow_finish(const CgParams& P, const FlowParams& Q, FlowShared& S,
                                             int r0, int nl, int it, X&& xt) {
-    const int t = threadIdx.x, B = blockDim.x, ld = P.ld;
-    const bool lead = blockIdx.x == 0 && t == 0;
+    const int ld = P.ld;
+    const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
     if (S.state == 2) {
         if (lead) raise_error(P.err, SDC_E_NONFINITE);
         return;
@@ -508,21 +536,21 @@ __device__ __forceinline__ void flow_finish(const CgParams& P, const FlowParams&
     ulonglong2* const pub = Q.pub + (size_t)((it + 1) & 1) * ld;
     const u64 tag = Q.id + (u64)it + 2;
     const bool couple = P.epi_lo < P.epi_hi;
-    for (int l = t; l < nl; l += B) {
+    flow_rows(nl, [&](int l) {
         const int i = r0 + l;
         const double x = __ldcg(P.sv + i) * xt(l);
         P.x[i] = x;
         if (couple) pub_store(pub + i, x, tag);
-    }
+    });
     if (!couple) return;
-    for (int l = t; l < nl; l += B) {
+    flow_rows(nl, [&](int l) {
         const int i = r0 + l;
         const int len = __ldg(P.alen + i);
         const double kx = flow_row_dot<FlowChunk<MAXT>::value>(
             0.0, len, (size_t)i, ld, P.acol, P.n, 0, 0, nullptr, pub, tag, 47, S, P.budget, P.err,
-            [&](size_t q) { return __ldg(P.aval + q); });
+            [&](int k) { return __ldg(P.aval + (size_t)k * ld + i); });
         cg_couple_row(P, i, P.x[i], kx);
-    }
+    });
 }
 
 // ---- pipelined arrangement (see pcg_group), scaled form ------------------------------
@@ -548,12 +576,15 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
     double* const sz = sm + 5 * L;
     double* const sn = sm + 6 * L;
     double* const xs = Q.x_smem ? sm + 7 * L : P.x + r0;
-    const int wrow = wid == 0 ? nw - 1 : wid - 1;   // the warps' order over the chunks
+    // scaled off-diagonals: behind the vectors, or in global memory
+    double* const vb = Q.v_smem ? sm + (size_t)(7 + Q.x_smem) * L : P.sval + r0;
+    const int vs = Q.v_smem ? L : ld;
+    const bool has_rows = wid != 0 || nw <= nch;   // (warps beyond the rows add zeros)
     unsigned epoch = 0, gen = 1;
     double ga, de, alpha = 0.0, beta = 0.0;
-    flow_scalars_init(S.z);
+    flow_scalars_init(S);
     if (!flow_start<MAXT>(
-            P, Q, S, r0, nl, epoch, ga, de,
+            P, Q, S, r0, nl, vb, vs, epoch, ga, de,
             [&](int l, double r) {
                 rc[l] = r;
                 sp[l] = ss[l] = sz[l] = 0.0;
@@ -568,18 +599,15 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
     unsigned npub = 0;
     bool exact = true, redo = false;
     auto update_px = [&]() {
-        for (int c = wrow; c < nch; c += nw) {
-            const int l = 32 * c + lane;
-            if (l < nl) {
-                const double p = ro[l] + beta * sp[l];
-                sp[l] = p;
-                xs[l] += alpha * p;
-            }
-        }
+        flow_rows_px(nl, [&](int l) {
+            const double p = ro[l] + beta * sp[l];
+            sp[l] = p;
+            xs[l] += alpha * p;
+        });
     };
     while (true) {
         u64* const acc = Q.acc + 8 * (npub & 1);
-        flow_post(ga, de, S, acc);
+        flow_post(ga, de, has_rows, S, acc);
         if (wid == 0)
             flow_totals(S, acc, npub & 1, G, exact, P.budget, P.err);
         ++npub;
@@ -599,7 +627,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
                     const int i = r0 + l;
                     sn[l] = flow_row_dot<FlowChunk<MAXT>::value>(
                         sw[l], __ldg(P.alen + i), (size_t)i, ld, P.acol, P.n, r0, nl, sw, pub, tag, 42,
-                        S, P.budget, P.err, [&](size_t q) { return P.sval[q]; });
+                        S, P.budget, P.err, [&](int k) { return vb[(size_t)k * vs + l]; });
                 }
                 c = -1;
                 __syncwarp();
@@ -628,23 +656,20 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
         const u64 tag = Q.id + (u64)it + 1;
         ulonglong2* const pub = Q.pub + (size_t)(it & 1) * ld + r0;
         ga = de = 0.0;
-        for (int c = wrow; c < nch; c += nw) {
-            const int l = 32 * c + lane;
-            if (l < nl) {
-                const double w0 = sw[l];
-                const double z = sn[l] + beta * sz[l];
-                const double s = w0 + beta * ss[l];
-                const double w = w0 - alpha * z;
-                const double r = rc[l] - alpha * s;
-                pub_store(pub + l, w, tag);
-                sw[l] = w;
-                ro[l] = r;
-                sz[l] = z;
-                ss[l] = s;
-                ga += r * r;
-                de += w * r;
-            }
-        }
+        flow_rows(nl, [&](int l) {
+            const double w0 = sw[l];
+            const double z = sn[l] + beta * sz[l];
+            const double s = w0 + beta * ss[l];
+            const double w = w0 - alpha * z;
+            const double r = rc[l] - alpha * s;
+            pub_store(pub + l, w, tag);
+            sw[l] = w;
+            ro[l] = r;
+            sz[l] = z;
+            ss[l] = s;
+            ga += r * r;
+            de += w * r;
+        });
         double* const q = rc;
         rc = ro;
         ro = q;
@@ -661,7 +686,7 @@ template <int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) {
     extern __shared__ double sm[];
     __shared__ FlowShared S;
-    const int t = threadIdx.x, lane = t & 31, wid = t >> 5, nw = blockDim.x >> 5;
+    const int t = threadIdx.x, wid = t >> 5, nw = blockDim.x >> 5;
     const int G = gridDim.x, L = P.L, ld = P.ld;
     const int r0 = blockIdx.x * L;
     const int nl = max(0, min(P.n - r0, L));
@@ -673,12 +698,14 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) 
     double* const ss = sm + 3 * L;
     double* fb = late ? sm + 4 * L : rb;
     double* const xs = Q.x_smem ? sm + 5 * L : P.x + r0;
-    const int wrow = wid == 0 ? nw - 1 : wid - 1;
+    double* const vb = Q.v_smem ? sm + (size_t)(2 + Q.nbuf + Q.x_smem) * L : P.sval + r0;
+    const int vs = Q.v_smem ? L : ld;
+    const bool has_rows = wid != 0 || nw <= nch;
     unsigned epoch = 0, gen = 1;
     double ga, de, alpha = 0.0, beta = 0.0;
-    flow_scalars_init(S.z);
+    flow_scalars_init(S);
     if (!flow_start<MAXT>(
-            P, Q, S, r0, nl, epoch, ga, de,
+            P, Q, S, r0, nl, vb, vs, epoch, ga, de,
             [&](int l, double r) {
                 rb[l] = r;
                 sp[l] = ss[l] = 0.0;
@@ -689,23 +716,18 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) 
     int it = 0;
     unsigned npub = 0;
     bool exact = true, redo = false;
-    auto update_px = [&](const double* r) {
-        for (int c = wrow; c < nch; c += nw) {
-            const int l = 32 * c + lane;
-            if (l < nl) {
-                const double p = r[l] + beta * sp[l];
-                sp[l] = p;
-                xs[l] += alpha * p;
-            }
-        }
+    auto px_row = [&](const double* r, int l) {
+        const double p = r[l] + beta * sp[l];
+        sp[l] = p;
+        xs[l] += alpha * p;
     };
     while (true) {
         u64* const acc = Q.acc + 8 * (npub & 1);
-        flow_post(ga, de, S, acc);
+        flow_post(ga, de, has_rows, S, acc);
         if (wid == 0)
             flow_totals(S, acc, npub & 1, G, exact, P.budget, P.err);
         ++npub;
-        if (late && it > 0 && !redo) update_px(fb);
+        if (late && it > 0 && !redo) flow_rows_px(nl, [&](int l) { px_row(fb, l); });
         __syncthreads();
         if (!S.ok) return;
         if (S.state == 3) {
@@ -726,33 +748,28 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) 
         beta = S.beta;
         const u64 tag = Q.id + (u64)it + 1;
         ulonglong2* const pub = Q.pub + (size_t)(it & 1) * ld;
-        for (int c = wrow; c < nch; c += nw) {
-            const int l = 32 * c + lane;
-            if (l < nl) {
-                const double s = wb[l] + beta * ss[l];
-                const double r = rb[l] - alpha * s;
-                pub_store(pub + r0 + l, r, tag);
-                wb[l] = r;
-                ss[l] = s;
-            }
-        }
+        flow_rows(nl, [&](int l) {
+            const double s = wb[l] + beta * ss[l];
+            const double r = rb[l] - alpha * s;
+            pub_store(pub + r0 + l, r, tag);
+            wb[l] = r;
+            ss[l] = s;
+        });
         if (wid == 0) flow_next(S, P.rtol);
         __syncthreads();
-        if (!late) update_px(rb);
+        // (the thread that writes the row's product over r_old)
+        if (!late) flow_rows(nl, [&](int l) { px_row(rb, l); });
         ga = de = 0.0;
-        for (int c = wrow; c < nch; c += nw) {
-            const int l = 32 * c + lane;
-            if (l < nl) {
-                const int i = r0 + l;
-                const double r = wb[l];
-                const double w = flow_row_dot<FlowChunk<MAXT>::value>(
-                    r, __ldg(P.alen + i), (size_t)i, ld, P.acol, P.n, r0, nl, wb, pub, tag, 46, S,
-                    P.budget, P.err, [&](size_t q) { return P.sval[q]; });
-                fb[l] = w;
-                ga += r * r;
-                de += w * r;
-            }
-        }
+        flow_rows(nl, [&](int l) {
+            const int i = r0 + l;
+            const double r = wb[l];
+            const double w = flow_row_dot<FlowChunk<MAXT>::value>(
+                r, __ldg(P.alen + i), (size_t)i, ld, P.acol, P.n, r0, nl, wb, pub, tag, 46, S,
+                P.budget, P.err, [&](int k) { return vb[(size_t)k * vs + l]; });
+            fb[l] = w;
+            ga += r * r;
+            de += w * r;
+        });
         // r <- w's place, w <- the product's, and r_old's is free (two buffers: the same one)
         double* const q = rb;
         rb = wb;

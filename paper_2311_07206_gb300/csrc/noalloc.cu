@@ -5,9 +5,10 @@
 // every byte of device memory through its own pool and forbids raw cudaMalloc
 // (it would bypass the pool's budget or fragment it), and time-critical loops
 // in which cudaMalloc/cudaFree may block or synchronise the device.  They pass
-// inputs and outputs as usual; the solver's workspace (ten vectors, per-block
-// partial sums, the barrier counter and status words) lives in the file-scope
-// array below instead of a per-call allocation.
+// inputs and outputs as usual; the solver's workspace (the published words and
+// two vectors of the on-chip kernels; for wide matrices, whose scaled values do not
+// fit in shared memory, ten vectors, per-block partial sums, the barrier counter and
+// status words) lives in the file-scope array below instead of a per-call allocation.
 //
 // Costs and limits of that choice:
 //   * every GPU that loads the library reserves the array (about 5.6 MB) until
@@ -24,6 +25,7 @@
 //     in the new context, and the first call there looks it up again.
 
 #include <cstdio>
+#include <cstring>
 #include <mutex>
 
 #include "sdc_internal.h"
@@ -43,6 +45,14 @@ std::mutex g_mu;
 double* g_scratch_addr[kMaxDevices] = {};
 unsigned long long g_scratch_ctx[kMaxDevices] = {};   // context id the address belongs to
 
+sdc_status reject(sdc_status st, const char* msg) {
+    sdc::set_thread_error(msg);
+    return st;
+}
+
+}  // namespace
+
+namespace sdc {
 // Unique id of the calling thread's current context (cuCtxGetId through the
 // runtime's driver entry point, so the library needs no link to libcuda);
 // 0 when there is none yet or the query is unavailable.
@@ -61,13 +71,9 @@ unsigned long long current_context_id() {
     if (!fn || fn(nullptr, &id) != 0) return 0;
     return id;
 }
+}  // namespace sdc
 
-sdc_status reject(sdc_status st, const char* msg) {
-    sdc::set_thread_error(msg);
-    return st;
-}
-
-}  // namespace
+using sdc::current_context_id;
 
 extern "C" sdc_status sdc_pcg_solve_noalloc(int n, const double* d_val, const int* d_col,
                                             const int* d_len, int ld, int width,
@@ -120,41 +126,55 @@ extern "C" sdc_status sdc_pcg_solve_noalloc(int n, const double* d_val, const in
         base = g_scratch_addr[dev];
     }
     cudaStream_t s = (cudaStream_t)stream;
-    sdc::PcgScratch w;
-    w.r = base;
-    w.u = base + (size_t)n;
-    w.p = base + 2 * (size_t)n;
-    w.s = base + 3 * (size_t)n;
-    w.w = base + 4 * (size_t)n;
-    w.idA = base + 5 * (size_t)n;
-    w.z = base + 6 * (size_t)n;
-    w.nv = base + 7 * (size_t)n;
-    w.m = base + 8 * (size_t)n;
-    w.part = base + kVecDoubles;
-    w.max_blocks = kMaxBlocks;
-    w.relres = base + kVecDoubles + 12 * (size_t)kMaxBlocks;
-    unsigned* sc = (unsigned*)(w.relres + 1);
-    w.bar = sc;
-    w.err = (int*)(sc + 1);
-    w.iters = (int*)(sc + 2);
     sdc::Ell A;
     A.val = const_cast<double*>(d_val);
     A.col = const_cast<int*>(d_col);
     A.len = const_cast<int*>(d_len);
     A.ld = ld;
     A.width = width;
-    // the barrier counter, error word and outputs must start at zero on every call
-    if (cudaMemsetAsync(w.relres, 0, kScalarDoubles * sizeof(double), s) != cudaSuccess)
-        return reject(SDC_E_CUDA, "sdc_pcg_solve_noalloc: clearing the status words failed");
-    if (sdc::launch_pcg_standalone(n, A, d_kdiag, d_mass, d_J, c, d_b, d_x, rtol, maxit,
-                                   4000000000LL, 256, w, s) != SDC_OK)
-        return reject(SDC_E_CUDA, "sdc_pcg_solve_noalloc: launch failed");
-    int h[3] = {0, 0, 0};
+    int h[3] = {0, 0, 0};   // -, error, iterations
     double hr = 0.0;
-    if (cudaMemcpyAsync(h, sc, 3 * sizeof(unsigned), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaMemcpyAsync(&hr, w.relres, sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-        return reject(SDC_E_CUDA, "sdc_pcg_solve_noalloc: reading the status failed");
+    const size_t fd = sdc::pcg_standalone_flow_doubles(n, ld, width);
+    if (fd > 0 && fd <= kScratchDoubles) {
+        if (sdc::launch_pcg_standalone_flow(n, A, d_kdiag, d_mass, d_J, c, d_b, d_x, rtol, maxit,
+                                            4000000000LL, base, s) != SDC_OK)
+            return reject(SDC_E_CUDA, "sdc_pcg_solve_noalloc: launch failed");
+        double r[sdc::kStandaloneResults];
+        if (cudaMemcpyAsync(r, base + fd - sdc::kStandaloneResults, sizeof r, cudaMemcpyDeviceToHost,
+                            s) != cudaSuccess ||
+            cudaStreamSynchronize(s) != cudaSuccess)
+            return reject(SDC_E_CUDA, "sdc_pcg_solve_noalloc: reading the status failed");
+        hr = r[0];
+        memcpy(h + 1, r + 1, 2 * sizeof(int));
+    } else {
+        sdc::PcgScratch w;
+        w.r = base;
+        w.u = base + (size_t)n;
+        w.p = base + 2 * (size_t)n;
+        w.s = base + 3 * (size_t)n;
+        w.w = base + 4 * (size_t)n;
+        w.idA = base + 5 * (size_t)n;
+        w.z = base + 6 * (size_t)n;
+        w.nv = base + 7 * (size_t)n;
+        w.m = base + 8 * (size_t)n;
+        w.part = base + kVecDoubles;
+        w.max_blocks = kMaxBlocks;
+        w.relres = base + kVecDoubles + 12 * (size_t)kMaxBlocks;
+        unsigned* sc = (unsigned*)(w.relres + 1);
+        w.bar = sc;
+        w.err = (int*)(sc + 1);
+        w.iters = (int*)(sc + 2);
+        // the barrier counter, error word and outputs must start at zero on every call
+        if (cudaMemsetAsync(w.relres, 0, kScalarDoubles * sizeof(double), s) != cudaSuccess)
+            return reject(SDC_E_CUDA, "sdc_pcg_solve_noalloc: clearing the status words failed");
+        if (sdc::launch_pcg_standalone(n, A, d_kdiag, d_mass, d_J, c, d_b, d_x, rtol, maxit,
+                                       4000000000LL, 256, w, s) != SDC_OK)
+            return reject(SDC_E_CUDA, "sdc_pcg_solve_noalloc: launch failed");
+        if (cudaMemcpyAsync(h, sc, 3 * sizeof(unsigned), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+            cudaMemcpyAsync(&hr, w.relres, sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+            cudaStreamSynchronize(s) != cudaSuccess)
+            return reject(SDC_E_CUDA, "sdc_pcg_solve_noalloc: reading the status failed");
+    }
     if (iters) *iters = h[2];
     if (relres) *relres = hr;
     {

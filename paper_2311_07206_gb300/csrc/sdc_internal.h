@@ -168,7 +168,7 @@ void launch_residual(int M, int n, const int* act, const Ell& K, const double* k
 // Launch configuration of the restricted PCG solves.
 constexpr int kFlowSmemBytes = 225 * 1024;   // dynamic shared memory of the flow kernels
 constexpr int kFlowWords = 34;      // 64-bit words of their grid-wide state
-constexpr int kFlowClassicalRows = 250000;   // automatic arrangement: classical above
+constexpr int kFlowClassicalRows = 130000;   // automatic arrangement: classical above
 constexpr int kSmemVectors = 8;     // per-row doubles in shared memory, shared-memory variant
 constexpr int kSmemRows = 3584;     // rows per block of the shared-memory variant
 // target rows per block of the shared-memory variants below their capacity: one row
@@ -212,6 +212,8 @@ void launch_nodes_out_perm(int N, int M, const int* perm, const double* X, doubl
                            cudaStream_t s);
 // Message returned by sdc_last_error(NULL) on the calling thread.
 void set_thread_error(const char* msg);
+// Id of the calling thread's current CUDA context, 0 when unknown (noalloc.cu).
+unsigned long long current_context_id();
 
 // One node solve with caller-chosen right-hand side, solution, J and
 // coupling targets (the reverse sweep of the adjoint uses it).
@@ -364,6 +366,14 @@ int launch_pcg_standalone(int n, const Ell& A, const double* kdiag, const double
                           const double* J, double c, const double* b, double* x, double rtol,
                           int maxit, long long budget, int block, const PcgScratch& w,
                           cudaStream_t s);
+// The same solve in the flow kernels: doubles of workspace (256-byte aligned), 0 when the
+// rows do not fit on chip; the last kStandaloneResults of them are the results: relres, then
+// error code and iterations (ints).
+constexpr int kStandaloneResults = 2;
+size_t pcg_standalone_flow_doubles(int n, int ld, int width, size_t* zero_at = nullptr);
+int launch_pcg_standalone_flow(int n, const Ell& A, const double* kdiag, const double* mass,
+                               const double* J, double c, const double* b, double* x, double rtol,
+                               int maxit, long long budget, double* ws, cudaStream_t s);
 int pcg_cluster_size(int block);
 // tol_drop_dev: when set, the selection reads TOL_drop there instead of tol_drop
 void launch_update(int M, int n, const int* act, const double* w0, double dt, const Ionic& ion,

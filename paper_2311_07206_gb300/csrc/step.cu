@@ -12,6 +12,7 @@
 //   select   : stable compaction of the flagged rows (warp ballot + block scan)
 //   extract  : K[I_{k+1}, I_{k+1}] from K[I_k, I_k] through the old->new row map
 
+#include <atomic>
 #include <cfloat>
 #include <cstdint>
 
@@ -194,6 +195,7 @@ struct FlowParams {
     unsigned long long id;      // launch id << 32: tags of different launches differ
     int x_smem;                 // x in shared memory (else in P.x)
     int nbuf;                   // classical: buffers shared by r and w (2 or 3)
+    int v_smem;                 // scaled off-diagonals in shared memory (else in P.sval)
 };
 
 }  // namespace
@@ -1943,8 +1945,9 @@ PcgKernel pcg_general_kernel(int block) {
 PcgKernel pcg_smem_kernel(int block) { return block > 512 ? k_pcg_smem<1024> : k_pcg_smem<512>; }
 using FlowKernel = void (*)(CgParams, FlowParams);
 FlowKernel flow_kernel(int block, bool classical) {
-    if (classical) return block > 512 ? k_cgc_flow<1024> : k_cgc_flow<512>;
-    return block > 512 ? k_pcg_flow<1024> : k_pcg_flow<512>;
+    if (classical)
+        return block > 768 ? k_cgc_flow<1024> : block > 512 ? k_cgc_flow<768> : k_cgc_flow<512>;
+    return block > 768 ? k_pcg_flow<1024> : block > 512 ? k_pcg_flow<768> : k_pcg_flow<512>;
 }
 PcgKernel pcgcs_general_kernel(int block) {
     return block > 512 ? k_pcgcs<1024> : block > 256 ? k_pcgcs<512> : k_pcgcs<256>;
@@ -1965,17 +1968,20 @@ PcgBatchKernel pcg_batch_kernel(int, bool pipelined, bool scaled = false) {
     return pipelined ? k_pcg_batch<1024> : scaled ? k_pcgcs_batch<1024> : k_pcgc_batch<1024>;
 }
 
-// opt-in dynamic shared memory of the on-chip variants (set once per instantiation)
+// opt-in dynamic shared memory of the on-chip variants: set once per context (the attributes
+// go with it, on cudaDeviceReset and from device to device)
 void pcg_smem_attrs() {
-    static bool done = false;
-    if (done) return;
+    static std::atomic<unsigned long long> done{0};
+    const unsigned long long ctx = current_context_id();
+    if (ctx != 0 && done.load() == ctx) return;
     for (PcgKernel k : {k_pcg_smem<512>, k_pcg_smem<1024>})
         cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(kSmemVectors * kSmemRows * sizeof(double)));
     for (PcgKernel k : {k_pcgc_smem<512>, k_pcgc_smem<1024>})
         cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(kSmemVectorsC * kSmemRowsC * sizeof(double)));
-    for (FlowKernel k : {k_pcg_flow<512>, k_pcg_flow<1024>, k_cgc_flow<512>, k_cgc_flow<1024>})
+    for (FlowKernel k : {k_pcg_flow<512>, k_pcg_flow<768>, k_pcg_flow<1024>, k_cgc_flow<512>,
+                         k_cgc_flow<768>, k_cgc_flow<1024>})
         cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kFlowSmemBytes);
     for (PcgKernel k : {k_pcg_cluster<512>, k_pcg_cluster<1024>}) {
@@ -1983,7 +1989,7 @@ void pcg_smem_attrs() {
                              (int)(kClusterVectors * kClusterRows * sizeof(double)));
         cudaFuncSetAttribute((const void*)k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     }
-    done = true;
+    done.store(current_context_id());
 }
 
 int pcg_max_blocks(int block) {
@@ -2193,7 +2199,7 @@ int launch_pcg_role(int n, const Ell& A, const PcgRole& role, double dt, int M, 
 // and its rows are a multiple of 128: FP64 issue is what a full warp per sub-partition
 // takes whatever its active lanes, so fewer CTAs with full warps are never slower.
 struct FlowShape {
-    int L, grid, block, x_smem, nbuf;
+    int L, grid, block, x_smem, nbuf, v_smem;
     size_t smem;
 };
 bool flow_shape(int n, bool classical, const PcgConfig& cfg, FlowShape& f) {
@@ -2204,7 +2210,8 @@ bool flow_shape(int n, bool classical, const PcgConfig& cfg, FlowShape& f) {
     if (cfg.max_blocks > 0) gm = std::min(gm, std::max(cfg.max_blocks, nblk(n, cap)));
     int l = nblk(n, gm);
     if (cfg.rows_per_block > 0) l = std::max(l, std::min(cfg.rows_per_block, cap));
-    const int maxb = n >= cfg.big_rows ? 1024 : std::min(std::max(cfg.smem_block, 64), 1024);
+    // (a block size below the default caps the threads; below big_rows only)
+    const int maxb = n >= cfg.big_rows || cfg.smem_block >= 512 ? 1024 : std::max(cfg.smem_block, 64);
     f.L = std::min(l <= 96 ? 96 : l <= 896 ? (l + 127) / 128 * 128 : (l + 31) / 32 * 32, cap);
     f.grid = nblk(n, f.L);
     f.block = std::min(32 + std::min(f.L, (n + 31) / 32 * 32), maxb);
@@ -2215,22 +2222,35 @@ bool flow_shape(int n, bool classical, const PcgConfig& cfg, FlowShape& f) {
         f.nbuf = 2;
         f.x_smem = 8 * f.L <= rows;
     }
+    f.v_smem = 0;
     f.smem = (size_t)((classical ? 2 + f.nbuf : 7) + f.x_smem) * f.L * sizeof(double);
     return true;
 }
+// The scaled off-diagonals of `width` slots in shared memory as well, if there is room: for
+// callers without a global array for them (measured no faster than through L1: 4.1 us per
+// iteration either way on 58k rows).
+bool flow_values_on_chip(int width, FlowShape& f) {
+    const size_t v = (size_t)width * f.L * sizeof(double);
+    if (f.smem + v > (size_t)kFlowSmemBytes) return false;
+    f.v_smem = 1;
+    f.smem += v;
+    return true;
+}
 
-int launch_flow(CgParams& P, bool classical, const FlowShape& f, StepBuffers& B, cudaStream_t s) {
+// words: kFlowWords words, zero; pub: tags of other launches only
+int launch_flow(CgParams& P, bool classical, const FlowShape& f, void* pub,
+                unsigned long long* words, unsigned long long id, cudaStream_t s) {
     pcg_smem_attrs();
     FlowParams Q;
-    Q.pub = reinterpret_cast<ulonglong2*>(B.pub);
-    Q.acc = B.flow;
-    Q.emax = B.flow + 16;
-    Q.bar = reinterpret_cast<unsigned*>(B.flow + 32);
-    Q.id = ++B.flow_id << 32;
+    Q.pub = reinterpret_cast<ulonglong2*>(pub);
+    Q.acc = words;
+    Q.emax = words + 16;
+    Q.bar = reinterpret_cast<unsigned*>(words + 32);
+    Q.id = id << 32;
     Q.x_smem = f.x_smem;
     Q.nbuf = f.nbuf;
+    Q.v_smem = f.v_smem;
     P.L = f.L;
-    cudaMemsetAsync(B.flow, 0, kFlowWords * sizeof(unsigned long long), s);
     void* args[] = {&P, &Q};
     cudaError_t e = cudaLaunchCooperativeKernel((const void*)flow_kernel(f.block, classical),
                                                 dim3(f.grid), dim3(f.block), args, f.smem, s);
@@ -2245,8 +2265,10 @@ int launch_pcg_params(CgParams& P, const PcgConfig& cfg, StepBuffers& B, cudaStr
     const bool flow_classical =
         !cfg.pipelined || (cfg.general_classical && n > kFlowClassicalRows);
     if (cfg.variant != 1 && cfg.scaled && P.sv && P.sval && B.pub &&
-        flow_shape(n, flow_classical, cfg, fs))
-        return launch_flow(P, flow_classical, fs, B, s);
+        flow_shape(n, flow_classical, cfg, fs)) {
+        cudaMemsetAsync(B.flow, 0, kFlowWords * sizeof(unsigned long long), s);
+        return launch_flow(P, flow_classical, fs, B.pub, B.flow, ++B.flow_id, s);
+    }
     cudaMemsetAsync(&B.sc->bar, 0, sizeof(unsigned), s);
     void* args[] = {&P};
     // automatic arrangement: the pipelined form pays off where the vectors live on chip;
@@ -2526,6 +2548,67 @@ int launch_pcg_batch_planned(const Ell& A, int m, double dt, const Coll& co, dou
                                       cfg.scaled && P.sv && P.sval),
         dim3(G), dim3(cfg.batch_block), args, 0, s);
     return e == cudaSuccess ? SDC_OK : SDC_E_CUDA;
+}
+
+// Stand-alone solves run in the flow kernels while the rows fit on chip.
+bool pcg_standalone_shape(int n, int width, FlowShape& f, bool& classical) {
+    PcgConfig cfg;
+    cfg.sms = pcg_sm_count();
+    cfg.smem_block = 512;
+    classical = n > kFlowClassicalRows;
+    if (cfg.sms < 1 || !flow_shape(n, classical, cfg, f)) return false;
+    flow_values_on_chip(width, f);
+    return true;
+}
+
+size_t pcg_standalone_flow_doubles(int n, int ld, int width, size_t* zero_at) {
+    FlowShape f;
+    bool classical;
+    if (!pcg_standalone_shape(n, width, f, classical)) return 0;
+    // u, diag^-1/2, [scaled values], then from a 256-byte boundary on what starts at zero:
+    // the published words, the sums, the results
+    const size_t z = (2 * (size_t)n + (f.v_smem ? 0 : (size_t)width * ld) + 31) / 32 * 32;
+    if (zero_at) *zero_at = z;
+    return z + (4 * (size_t)ld + 31) / 32 * 32 + kFlowWords + kStandaloneResults;
+}
+
+int launch_pcg_standalone_flow(int n, const Ell& A, const double* kdiag, const double* mass,
+                               const double* J, double c, const double* b, double* x, double rtol,
+                               int maxit, long long budget, double* ws, cudaStream_t s) {
+    FlowShape f;
+    bool classical;
+    size_t z = 0;
+    const size_t total = pcg_standalone_flow_doubles(n, A.ld, A.width, &z);
+    if (!total || !pcg_standalone_shape(n, A.width, f, classical) ||
+        reinterpret_cast<uintptr_t>(ws) % 256 != 0)
+        return SDC_E_INVALID;
+    if (cudaMemsetAsync(ws + z, 0, (total - z) * sizeof(double), s) != cudaSuccess)
+        return SDC_E_CUDA;
+    double* const words = ws + z + (4 * (size_t)A.ld + 31) / 32 * 32;
+    double* const res = words + kFlowWords;
+    CgParams P{};
+    P.n = n;
+    P.ld = A.ld;
+    P.aval = A.val;
+    P.acol = A.col;
+    P.alen = A.len;
+    P.mc = mass;
+    P.kdc = kdiag;
+    P.J = J;
+    P.c = c;
+    P.b = b;
+    P.x = x;
+    P.u = ws;
+    P.sv = ws + n;
+    P.sval = f.v_smem ? nullptr : ws + 2 * (size_t)n;
+    P.relres_out = res;
+    P.err = reinterpret_cast<int*>(res + 1);
+    P.iters_out = P.err + 1;
+    P.rtol = rtol;
+    P.maxit = maxit;
+    P.budget = budget;
+    P.M = 1;            // no coupling into other nodes
+    return launch_flow(P, classical, f, ws + z, reinterpret_cast<unsigned long long*>(words), 1, s);
 }
 
 int launch_pcg_standalone(int n, const Ell& A, const double* kdiag, const double* mass,
