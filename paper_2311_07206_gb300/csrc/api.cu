@@ -1392,7 +1392,7 @@ static sdc_status pcg_solve_body(int n, const double* d_val, const int* d_col, c
     int status = SDC_OK;
     int h[3] = {0, 0, 0};   // -, error, iterations
     double hr = 0.0;
-    const size_t fd = pcg_standalone_flow_doubles(n, ld, width);
+    const size_t fd = pcg_standalone_flow_doubles(n, ld, width, maxit);
     if (fd > 0) {
         SolveWorkspace ws(fd * sizeof(double), s);
         if (!ws.p) return fail(nullptr, SDC_E_NOMEM, "sdc_pcg_solve: workspace allocation failed");
@@ -1720,8 +1720,8 @@ sdc_status sdc_set_coarse_blocks(sdc_ctx* c, const int* block_of_dof, int n_bloc
         return SDC_OK;
     }
     std::string why;
-    const int rc = coarse_setup(c->coarse, block_of_dof, c->N, n_blocks, c->B.ld, &c->B.sc->err,
-                                c->stream, why);
+    const int rc = coarse_setup(c->coarse, block_of_dof, c->N, n_blocks, c->B.ld, c->emi.A.width,
+                                &c->B.sc->err, c->stream, why);
     if (rc != SDC_OK) return fail(c, (sdc_status)rc, "%s", why.c_str());
     return SDC_OK;
 }

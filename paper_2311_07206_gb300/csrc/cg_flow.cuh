@@ -39,19 +39,37 @@ constexpr int kFlowHead = 10;    // growth of gamma over one iteration that fits
 constexpr int kFlowSumHead = 18; // total over largest partial sum (155,648 threads, 2^103 units)
 constexpr int kFlowDrop = 22;    // fall of gamma up to which the sum keeps 2^-54 of its value
 
-// relaxed single-copy-atomic 128-bit access: (value bits, tag)
-__device__ __forceinline__ void pub_store(ulonglong2* p, double v, u64 tag) {
+// A published word: value, tag (12 bits of launch, 20 of iteration; the host clears the words
+// when the launch count wraps), 32 spare bits.  Stored and loaded as one relaxed
+// single-copy-atomic 128-bit access.
+__device__ __forceinline__ void pub_store(ulonglong2* p, double v, unsigned tag) {
     asm volatile("{ .reg .b128 t; mov.b128 t, {%1, %2}; st.relaxed.gpu.global.b128 [%0], t; }" ::"l"(p),
-                 "l"((u64)__double_as_longlong(v)), "l"(tag)
+                 "l"((u64)__double_as_longlong(v)), "l"((u64)tag)
                  : "memory");
 }
-__device__ __forceinline__ void pub_load_if(bool on, const ulonglong2* p, u64& v, u64& tag) {
-    asm volatile(
-        "{ .reg .pred q; .reg .b128 t; setp.ne.u32 q, %3, 0; mov.b128 t, {%0, %1};\n\t"
-        "@q ld.relaxed.gpu.global.b128 t, [%2]; mov.b128 {%0, %1}, t; }"
-        : "+l"(v), "+l"(tag)
-        : "l"(p), "r"((unsigned)on)
-        : "memory");
+__device__ __forceinline__ void pub_load(const ulonglong2* p, u64& v, unsigned& tag) {
+    u64 t;
+    asm volatile("{ .reg .b128 t; ld.relaxed.gpu.global.b128 t, [%2]; mov.b128 {%0, %1}, t; }"
+                 : "=l"(v), "=l"(t)
+                 : "l"(p)
+                 : "memory");
+    tag = (unsigned)t;
+}
+// Value of column j: from the CTA's shared memory (32-bit shared address `own` of local row 0)
+// when l = j - r0 < nl, else the published word; tag is left alone in the first case.
+__device__ __forceinline__ void flow_fetch(unsigned l, unsigned nl, unsigned own, const ulonglong2* p,
+                                           u64& v, unsigned& tag) {
+    if (l < nl) {
+        asm volatile("ld.shared.u64 %0, [%1];" : "=l"(v) : "r"(own + 8u * l) : "memory");
+    } else {
+        unsigned __int128 w;
+        asm volatile("ld.relaxed.gpu.global.b128 %0, [%1];" : "=q"(w) : "l"(p) : "memory");
+        v = (u64)w;
+        tag = (unsigned)(w >> 64);
+    }
+}
+__device__ __forceinline__ unsigned smem_addr(const double* p) {
+    return (unsigned)__cvta_generic_to_shared(p);
 }
 __device__ __forceinline__ u64 ld_relaxed64(const u64* p) {
     u64 v;
@@ -205,8 +223,10 @@ __device__ __forceinline__ void flow_scalars_init(FlowShared& S) {
 // Warp 0: wait for the sums posted to set `set`, derive alpha and beta (cg_scalars'
 // recurrences, den_t = delta_t - beta_t gamma_t / alpha_{t-1}) and the next windows.
 // exact: the windows came from the exact exponents (no repeat for a fall of gamma).
+// HEAD, DROP: kFlowHead and kFlowDrop.  arrived() runs once the wait is over.
+template <int HEAD, int DROP, class A>
 __device__ __forceinline__ void flow_totals(FlowShared& S, const u64* acc, int set, int G, bool exact,
-                                            long long budget, int* err) {
+                                            long long budget, int* err, A&& arrived) {
     const int lane = threadIdx.x & 31;
     FlowScalars& Z = S.z;
     const double inv_g = Z.inv_g, inv_a = Z.inv_a;
@@ -237,13 +257,12 @@ __device__ __forceinline__ void flow_totals(FlowShared& S, const u64* acc, int s
         }
     }
     ok = __all_sync(0xffffffffu, ok);
-    if (!ok) {
-        if (lane == 0) {
-            raise_error(err, SDC_E_TIMEOUT);
-            S.ok = 0;
-        }
-        return;
+    if (!ok && lane == 0) {
+        raise_error(err, SDC_E_TIMEOUT);
+        S.ok = 0;
     }
+    arrived();
+    if (!ok) return;
 #pragma unroll
     for (int k = 0; k < 4; ++k) d[k] += v[k];
     bool in;
@@ -265,7 +284,7 @@ __device__ __forceinline__ void flow_totals(FlowShared& S, const u64* acc, int s
     } else if (gb < hi) {
         state = gb <= lo || flow_sqrt_at_most(g, Z.thresh) ? 1 : 0;
     }
-    if (state == 0 && !exact && fg < topa - kFlowHead - kFlowDrop) state = 3;
+    if (state == 0 && !exact && fg < topa - HEAD - DROP) state = 3;
     const double beta = g * inv_g;
     const double den = fma(-beta, g * inv_a, dl);
     const double alpha = flow_quot(g, den);
@@ -278,7 +297,7 @@ __device__ __forceinline__ void flow_totals(FlowShared& S, const u64* acc, int s
             S.alpha = alpha;
             S.beta = beta;
             Z.den = den;
-            S.topa = S.topb = min(fg + kFlowHead, 2046);
+            S.topa = S.topb = min(fg + HEAD, 2046);
         }
     }
     if (lane < 2) {
@@ -354,55 +373,47 @@ __device__ __forceinline__ bool flow_window(double a, double b, FlowShared& S, u
     return S.ok != 0;
 }
 
-// Off-diagonal product of row i: acc + sum_k val(k) x(col(k)) in slot order.  Columns of this
-// CTA (rows [r0, r0 + nl)) come from shared memory (own), the others from their published
-// words, read again until they carry `tag`.  val(k) is the value of slot k.  All loads of CH
-// slots are issued before the first is used.
-template <int CH, class Val>
-__device__ __forceinline__ double flow_row_dot(double acc, int len, size_t i, int ld,
-                                               const int* __restrict__ col, int ncol, int r0, int nl,
-                                               const double* own, const ulonglong2* pub, u64 tag,
-                                               int site, FlowShared& S, long long budget, int* err,
-                                               Val&& val) {
+// Off-diagonal product of a row: acc + sum_k v[k vs] x(c[k ld]) over its len slots, in order.
+// Columns of this CTA (rows [r0, r0 + nl)) come from shared memory (own), the others from their
+// published words, fetched again until they carry `tag`.  All loads of CH slots are issued
+// before the first is used.  The product of a CTA with many rows is bound by instruction
+// issue, not by FP64 or latency (two padded slots more per row: 442k rows 13.5 -> 15.2 us per
+// iteration), so a slot is kept to a dozen instructions.
+template <int CH>
+__device__ __forceinline__ double flow_row_dot(double acc, int len, const int* __restrict__ c, int ld,
+                                               const double* v, int vs, int ncol, int r0, int nl,
+                                               unsigned own, const ulonglong2* pub, unsigned tag,
+                                               int site, FlowShared& S, long long budget, int* err) {
     for (int k0 = 0; k0 < len; k0 += CH) {
         int j[CH];
         double a[CH];
-        u64 x[CH], g[CH];
 #pragma unroll
         for (int k = 0; k < CH; ++k) {
             j[k] = r0;
-            a[k] = 0.0;
             if (k0 + k < len) {
-                const size_t q = (size_t)(k0 + k) * ld + i;
-                j[k] = sdc_idx(__ldg(col + q), ncol, site);
-                a[k] = val(k0 + k);
+                j[k] = sdc_idx(__ldg(c + (size_t)k * ld), ncol, site);
+                a[k] = v[(size_t)k * vs];
             }
         }
-        unsigned pend = 0;
+        c += (size_t)CH * ld;
+        v += (size_t)CH * vs;
+        u64 x[CH];
+        long long t0 = 0;
+        while (true) {
+            unsigned bad = 0;
 #pragma unroll
-        for (int k = 0; k < CH; ++k) {
-            const int l = j[k] - r0;
-            const bool mine = (unsigned)l < (unsigned)nl;
-            x[k] = mine ? (u64)__double_as_longlong(own[l]) : 0ull;
-            g[k] = k0 + k < len && !mine ? ~tag : tag;
-            pub_load_if(g[k] != tag, pub + j[k], x[k], g[k]);
-        }
-#pragma unroll
-        for (int k = 0; k < CH; ++k) pend |= (g[k] != tag ? 1u : 0u) << k;
-        if (pend) {
-            const long long t0 = clock64();
-            do {
-#pragma unroll
-                for (int k = 0; k < CH; ++k) pub_load_if((pend >> k) & 1u, pub + j[k], x[k], g[k]);
-#pragma unroll
-                for (int k = 0; k < CH; ++k)
-                    if (g[k] == tag) pend &= ~(1u << k);
-                if (pend && clock64() - t0 > budget) {
-                    raise_error(err, SDC_E_TIMEOUT);
-                    S.ok = 0;
-                }
-                if (!*(volatile int*)&S.ok) pend = 0;   // a wait of the CTA has run out
-            } while (pend);
+            for (int k = 0; k < CH; ++k) {
+                unsigned g = tag;
+                flow_fetch((unsigned)(j[k] - r0), (unsigned)nl, own, pub + j[k], x[k], g);
+                bad |= g ^ tag;
+            }
+            if (!bad) break;
+            if (t0 == 0) t0 = clock64();
+            if (clock64() - t0 > budget) {
+                raise_error(err, SDC_E_TIMEOUT);
+                S.ok = 0;
+            }
+            if (!*(volatile int*)&S.ok) break;   // a wait of the CTA has run out
         }
 #pragma unroll
         for (int k = 0; k < CH; ++k)
@@ -445,7 +456,8 @@ struct FlowChunk {
 // g(l, w) its w; gamma and delta partial sums in ga, de.  Returns false to leave the kernel.
 template <int MAXT, class F, class H>
 __device__ __forceinline__ bool flow_start(const CgParams& P, const FlowParams& Q, FlowShared& S,
-                                           int r0, int nl, double* vb, int vs, unsigned& epoch,
+                                           int r0, int nl, unsigned short* plen, double* vb, int vs,
+                                           unsigned& epoch,
                                            double& ga, double& de, F&& f, H&& h) {
     const int t = threadIdx.x, G = gridDim.x, ld = P.ld;
     const double c = P.c;
@@ -483,6 +495,7 @@ __device__ __forceinline__ bool flow_start(const CgParams& P, const FlowParams& 
     flow_rows(nl, [&](int l) {
         const int i = r0 + l;
         const int len = __ldg(P.alen + i);
+        plen[l] = (unsigned short)len;
         const double csi = c * __ldcg(P.sv + i);
         const double ri = __ldcg(P.u + i);
         double acc = ri;
@@ -534,7 +547,7 @@ __device__ __forceinline__ void flow_finish(const CgParams& P, const FlowParams&
     }
     // the words of iteration it - 1, whose readers are done: their CTAs posted sum `it`
     ulonglong2* const pub = Q.pub + (size_t)((it + 1) & 1) * ld;
-    const u64 tag = Q.id + (u64)it + 2;
+    const unsigned tag = Q.id + (unsigned)it + 2;
     const bool couple = P.epi_lo < P.epi_hi;
     flow_rows(nl, [&](int l) {
         const int i = r0 + l;
@@ -547,8 +560,7 @@ __device__ __forceinline__ void flow_finish(const CgParams& P, const FlowParams&
         const int i = r0 + l;
         const int len = __ldg(P.alen + i);
         const double kx = flow_row_dot<FlowChunk<MAXT>::value>(
-            0.0, len, (size_t)i, ld, P.acol, P.n, 0, 0, nullptr, pub, tag, 47, S, P.budget, P.err,
-            [&](int k) { return __ldg(P.aval + (size_t)k * ld + i); });
+            0.0, len, P.acol + i, ld, P.aval + i, ld, P.n, 0, 0, 0u, pub, tag, 47, S, P.budget, P.err);
         cg_couple_row(P, i, P.x[i], kx);
     });
 }
@@ -577,14 +589,16 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
     double* const sn = sm + 6 * L;
     double* const xs = Q.x_smem ? sm + 7 * L : P.x + r0;
     // scaled off-diagonals: behind the vectors, or in global memory
-    double* const vb = Q.v_smem ? sm + (size_t)(7 + Q.x_smem) * L : P.sval + r0;
+    unsigned short* const plen =
+        reinterpret_cast<unsigned short*>(sm + (size_t)(7 + Q.x_smem) * L);   // row lengths
+    double* const vb = Q.v_smem ? sm + (size_t)(7 + Q.x_smem) * L + L / 4 : P.sval + r0;
     const int vs = Q.v_smem ? L : ld;
     const bool has_rows = wid != 0 || nw <= nch;   // (warps beyond the rows add zeros)
     unsigned epoch = 0, gen = 1;
     double ga, de, alpha = 0.0, beta = 0.0;
     flow_scalars_init(S);
     if (!flow_start<MAXT>(
-            P, Q, S, r0, nl, vb, vs, epoch, ga, de,
+            P, Q, S, r0, nl, plen, vb, vs, epoch, ga, de,
             [&](int l, double r) {
                 rc[l] = r;
                 sp[l] = ss[l] = sz[l] = 0.0;
@@ -609,11 +623,11 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
         u64* const acc = Q.acc + 8 * (npub & 1);
         flow_post(ga, de, has_rows, S, acc);
         if (wid == 0)
-            flow_totals(S, acc, npub & 1, G, exact, P.budget, P.err);
+            flow_totals<kFlowHead, kFlowDrop>(S, acc, npub & 1, G, exact, P.budget, P.err, [] {});
         ++npub;
         if (!redo) {
             if (it > 0) update_px();
-            const u64 tag = Q.id + (u64)it + 1;
+            const unsigned tag = Q.id + (unsigned)it + 1;
             const ulonglong2* const pub = Q.pub + (size_t)(it & 1) * ld;
             int c = wid - 1;
             while (true) {
@@ -626,8 +640,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
                 if (l < nl) {
                     const int i = r0 + l;
                     sn[l] = flow_row_dot<FlowChunk<MAXT>::value>(
-                        sw[l], __ldg(P.alen + i), (size_t)i, ld, P.acol, P.n, r0, nl, sw, pub, tag, 42,
-                        S, P.budget, P.err, [&](int k) { return vb[(size_t)k * vs + l]; });
+                        sw[l], plen[l], P.acol + i, ld, vb + l, vs, P.n, r0, nl, smem_addr(sw), pub, tag,
+                        42, S, P.budget, P.err);
                 }
                 c = -1;
                 __syncwarp();
@@ -653,7 +667,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
         beta = S.beta;
         if (t == 0) S.next = 0;
         if (wid == 0) flow_next(S, P.rtol);
-        const u64 tag = Q.id + (u64)it + 1;
+        const unsigned tag = Q.id + (unsigned)it + 1;
         ulonglong2* const pub = Q.pub + (size_t)(it & 1) * ld + r0;
         ga = de = 0.0;
         flow_rows(nl, [&](int l) {
@@ -698,14 +712,16 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) 
     double* const ss = sm + 3 * L;
     double* fb = late ? sm + 4 * L : rb;
     double* const xs = Q.x_smem ? sm + 5 * L : P.x + r0;
-    double* const vb = Q.v_smem ? sm + (size_t)(2 + Q.nbuf + Q.x_smem) * L : P.sval + r0;
+    unsigned short* const plen =
+        reinterpret_cast<unsigned short*>(sm + (size_t)(2 + Q.nbuf + Q.x_smem) * L);
+    double* const vb = Q.v_smem ? sm + (size_t)(2 + Q.nbuf + Q.x_smem) * L + L / 4 : P.sval + r0;
     const int vs = Q.v_smem ? L : ld;
     const bool has_rows = wid != 0 || nw <= nch;
     unsigned epoch = 0, gen = 1;
     double ga, de, alpha = 0.0, beta = 0.0;
     flow_scalars_init(S);
     if (!flow_start<MAXT>(
-            P, Q, S, r0, nl, vb, vs, epoch, ga, de,
+            P, Q, S, r0, nl, plen, vb, vs, epoch, ga, de,
             [&](int l, double r) {
                 rb[l] = r;
                 sp[l] = ss[l] = 0.0;
@@ -725,7 +741,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) 
         u64* const acc = Q.acc + 8 * (npub & 1);
         flow_post(ga, de, has_rows, S, acc);
         if (wid == 0)
-            flow_totals(S, acc, npub & 1, G, exact, P.budget, P.err);
+            flow_totals<kFlowHead, kFlowDrop>(S, acc, npub & 1, G, exact, P.budget, P.err, [] {});
         ++npub;
         if (late && it > 0 && !redo) flow_rows_px(nl, [&](int l) { px_row(fb, l); });
         __syncthreads();
@@ -746,7 +762,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) 
         ++it;
         alpha = S.alpha;
         beta = S.beta;
-        const u64 tag = Q.id + (u64)it + 1;
+        const unsigned tag = Q.id + (unsigned)it + 1;
         ulonglong2* const pub = Q.pub + (size_t)(it & 1) * ld;
         flow_rows(nl, [&](int l) {
             const double s = wb[l] + beta * ss[l];
@@ -760,12 +776,13 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) 
         // (the thread that writes the row's product over r_old)
         if (!late) flow_rows(nl, [&](int l) { px_row(rb, l); });
         ga = de = 0.0;
+        const unsigned own = smem_addr(wb);
         flow_rows(nl, [&](int l) {
             const int i = r0 + l;
             const double r = wb[l];
             const double w = flow_row_dot<FlowChunk<MAXT>::value>(
-                r, __ldg(P.alen + i), (size_t)i, ld, P.acol, P.n, r0, nl, wb, pub, tag, 46, S,
-                P.budget, P.err, [&](int k) { return vb[(size_t)k * vs + l]; });
+                r, plen[l], P.acol + i, ld, vb + l, vs, P.n, r0, nl, own, pub, tag, 46, S, P.budget,
+                P.err);
             fb[l] = w;
             ga += r * r;
             de += w * r;
@@ -777,6 +794,392 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) 
         fb = late ? q : rb;
     }
     flow_finish<MAXT>(P, Q, S, r0, nl, it, [&](int l) { return xs[l]; });
+}
+
+// ---- classical arrangement with the two-level preconditioner --------------------------
+// u = r + Y y, y = E^-1 t, t = Y' r, in place of u = r (see k_pcgcs_coarse, whose recurrences for
+// t and Y' s this kernel shares: Y' s <- Y' w + beta Y' s, t <- t - alpha Y' s).  The rows are the
+// positions of the block order: CTA b owns positions [b L, b L + L), cut at the block boundaries
+// into pieces; columns are translated to positions once per solve.  (Carrying y by the same
+// recurrences, which would take E^-1 off the critical path, stalls: the rounding of E^-1 Y' w
+// is not small against y once the residual has fallen by the condition of E.)
+// A piece's sum of Y w is exact: every warp adds its rows of a piece as limbs in a window
+// known from the piece's largest term of the iteration before, one warp adds the warps' limbs
+// (terms outside the window: that warp adds the rows again, from their largest exponent); the sum travels to
+// the other CTAs as a tagged word.  Per iteration: t; y of the own pieces' blocks, s, r; u
+// (published); the product, the dot products and the pieces' limbs; while the dot products are
+// summed the pieces' sums, p, x and the words of all pieces.
+// Before (k_pcgcs_coarse, two grid barriers and vectors in global memory): 16.0 us per
+// iteration on 131k rows.
+struct CoarseFlowParams {
+    int q, qn, ptot, npmax;   // blocks, blocks with active rows, pieces, most pieces of a CTA
+    const int* crow;          // [n] compact row of each position
+    const int* ipos;          // [n] position of each compact row
+    int* pcol;                // [width][ld] columns as positions, in position order
+    const int* tp;            // [G + 1] first piece of each CTA
+    const int* piece;         // [3 ptot]: block, first and end position
+    const int* blk_ptr;       // [q + 1] pieces of each block
+    const int* nzb;           // [qn] the blocks with active rows, ascending
+    const double* Einv;       // [q][q]
+    ulonglong2* words;        // [2][pstride] published piece sums
+    int pstride;
+};
+
+// gamma = r.u is a sum of terms that cancel against each other within a block, so its window
+// leaves more room above (and repeats for smaller falls).
+constexpr int kCoarseHead = 24, kCoarseDrop = 8;
+// A piece's window: room of the sum over its largest term, growth of the largest term since
+// the last sum, and its fall up to which the window keeps 57 bits of it.
+constexpr int kPieceHead = 16, kPieceGrow = 10, kPieceFall = 20;
+
+__host__ __device__ inline size_t coarse_flow_smem(int L, int vectors, int qn, int ptot, int npmax) {
+    return (size_t)vectors * L * 8 + (size_t)(3 * qn + ptot + npmax) * 8 +
+           (size_t)((L + 31) / 32 + npmax) * 16 + 16 + (size_t)(2 * qn + 1 + 5 * npmax) * 4 +
+           (size_t)L * 4;
+}
+
+__device__ __forceinline__ void flow_bar_sync(int id, int n) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+__device__ __forceinline__ void flow_bar_arrive(int id, int n) {
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+
+template <int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) k_cgc2_flow(CgParams P, FlowParams Q, CoarseFlowParams C) {
+    extern __shared__ __align__(16) double sm[];
+    __shared__ FlowShared S;
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5, nw = blockDim.x >> 5, B = blockDim.x;
+    const int G = gridDim.x, L = P.L, ld = P.ld;
+    const int r0 = blockIdx.x * L;
+    const int nl = max(0, min(P.n - r0, L));
+    const int nch = (nl + 31) >> 5;
+    const double c = P.c;
+    const bool late = Q.nbuf == 3;
+    double* ub = sm;
+    double* wb = sm + L;
+    double* const sr = sm + 2 * L;
+    double* const sp = sm + 3 * L;
+    double* const ss = sm + 4 * L;
+    double* const sy = sm + 5 * L;
+    double* ob = late ? sm + 6 * L : nullptr;   // u_old, until p has it
+    const int nv = (late ? 7 : 6) + Q.x_smem;
+    double* const sx = sm + (size_t)(nv - 1) * L;          // (x_smem)
+    double* const tw = sm + (size_t)nv * L;                // [qn] Y' w of the blocks with rows
+    double* const ts = tw + C.qn;                          // [qn] Y' s
+    double* const tr = ts + C.qn;                          // [qn] t = Y' r
+    double* const stp = tr + C.qn;                         // [ptot] the pieces' sums
+    double* const ysh = stp + C.ptot;                      // [npmax] y of the own pieces
+    int4* const recs = reinterpret_cast<int4*>(
+        (reinterpret_cast<uintptr_t>(ysh + C.npmax) + 15) & ~(uintptr_t)15);   // [nch + npmax] limbs
+    int* const snz = reinterpret_cast<int*>(recs + (L + 31) / 32 + C.npmax);   // [qn]
+    int* const sbp = snz + C.qn;                           // [qn + 1]
+    int* const pbeg = sbp + C.qn + 1;                      // [npmax] own pieces: local range, block,
+    int* const pend = pbeg + C.npmax;
+    int* const pblk = pend + C.npmax;
+    int* const ptop = pblk + C.npmax;                      // window, largest exponent of the terms
+    int* const pmax = ptop + C.npmax;
+    unsigned short* const pid = reinterpret_cast<unsigned short*>(pmax + C.npmax);   // [L]
+    unsigned short* const plen = pid + L;                                            // [L]
+    const bool has_rows = wid != 0 || nw <= nch;
+    const int e0 = C.tp[blockIdx.x], np = C.tp[blockIdx.x + 1] - e0;
+    double* const vb = P.sval + r0;
+    unsigned epoch = 0, gen = 0;
+    flow_scalars_init(S);
+    if (t == 0) {
+        S.ok = 1;
+        S.ovf = 0;
+    }
+    for (int m = t; m < C.qn; m += B) {
+        const int a = sdc_idx(C.nzb[m], C.q, 73);
+        snz[m] = a;
+        sbp[m] = C.blk_ptr[a];
+    }
+    if (t == 0) sbp[C.qn] = C.blk_ptr[C.q];
+    for (int a = t; a < np; a += B) {
+        const int e = sdc_idx(e0 + a, C.ptot, 74);
+        pblk[a] = sdc_idx(C.piece[3 * e], C.q, 75);
+        pbeg[a] = C.piece[3 * e + 1] - r0;
+        pend[a] = C.piece[3 * e + 2] - r0;
+        ptop[a] = 0;         // no window yet: every term lies above it
+        pmax[a] = 0;
+    }
+    __syncthreads();
+    for (int l = t; l < nl; l += B) {
+        int lo = 0, hi = np - 1;      // the piece that holds position l
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (pend[mid] > l) hi = mid; else lo = mid + 1;
+        }
+        pid[l] = (unsigned short)lo;
+    }
+    double* const xs = Q.x_smem ? sx : nullptr;
+    auto row_of = [&](int l) { return sdc_idx(C.crow[r0 + l], P.n, 70); };
+    flow_rows(nl, [&](int l) {
+        const int i = row_of(l);
+        const double d = P.mc[i] * (1.0 + c * P.J[i]) + c * P.kdc[i];
+        double si = 0.0;
+        if (!isfinite(d)) raise_error(P.err, SDC_E_NONFINITE);
+        else if (!(d > 0.0)) raise_error(P.err, SDC_E_DOMAIN);
+        else si = rsqrt(d);
+        P.sv[r0 + l] = si;
+        sy[l] = d * si;
+        sr[l] = si * P.b[i];
+        sp[l] = ss[l] = 0.0;
+        plen[l] = (unsigned short)P.alen[i];
+        if (xs) xs[l] = 0.0; else P.x[i] = 0.0;
+    });
+    __syncthreads();
+    // a warp's limbs of v over the pieces of chunk k (every lane of the warp calls it)
+    auto piece_limbs = [&](int k, double v) {
+        const int l = 32 * k + lane;
+        const int a0 = pid[32 * k], a1 = pid[min(32 * k + 31, nl - 1)];
+        const int mine = l < nl ? (int)pid[l] : -1;
+        for (int a = a0; a <= a1; ++a) {
+            int q[4];
+            const double x = mine == a ? v : 0.0;
+            const int top = ptop[a];
+            flow_limbs(x, top, q);
+            const int f = __reduce_max_sync(0xffffffffu, xs_field(x));
+#pragma unroll
+            for (int m = 0; m < 4; ++m) q[m] = __reduce_add_sync(0xffffffffu, q[m]);
+            if (lane == 0) {
+                recs[a + k] = make_int4(q[0], q[1], q[2], q[3]);
+                atomicMax(&pmax[a], f);
+            }
+        }
+    };
+    // sum of a lane's 64-bit limbs over the warp (each below 2^46)
+    auto warp_value = [&](const long long (&x)[4], int top) {
+        long long r[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+            r[m] = ((long long)__reduce_add_sync(0xffffffffu, (int)(x[m] >> 20)) << 20) +
+                   __reduce_add_sync(0xffffffffu, (int)(x[m] & 0xfffff));
+        bool in;
+        return flow_value(r[0], r[1], r[2], r[3], top, in);
+    };
+    // warps 1..: the own pieces' sums, published with `tag`; term(l): the rows' values
+    auto piece_post = [&](ulonglong2* out, unsigned tag, auto&& term) {
+        if (wid == 0) return;
+        for (int a = wid - 1; a < np; a += nw - 1) {
+            long long x[4] = {0, 0, 0, 0};
+            const int f = pmax[a], d = ptop[a] - kPieceHead - f;
+            int top = ptop[a];
+            if (d < 0 || d > kPieceGrow + kPieceFall) {
+                top = f + kPieceHead;
+                for (int l = pbeg[a] + lane; l < pend[a]; l += 32) {
+                    int q[4];
+                    flow_limbs(term(l), top, q);
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) x[m] += q[m];
+                }
+            } else {
+                for (int k = (pbeg[a] >> 5) + lane; k <= (pend[a] - 1) >> 5; k += 32) {
+                    const int4 q = recs[a + k];
+                    x[0] += q.x;
+                    x[1] += q.y;
+                    x[2] += q.z;
+                    x[3] += q.w;
+                }
+            }
+            const double v = warp_value(x, top);
+            if (lane == 0) {
+                pub_store(out + e0 + a, v, tag);
+                pmax[a] = 0;
+                ptop[a] = f + kPieceGrow + kPieceHead;
+            }
+        }
+    };
+    // warps 1..: every piece's sum, then Y' w of the blocks with active rows
+    auto coarse_in = [&](const ulonglong2* in, unsigned tag) {
+        const long long t0 = clock64();
+        for (int e = t - 32; e < C.ptot; e += B - 32) {
+            u64 v = 0;
+            unsigned g = ~tag;
+            while (true) {
+                pub_load(in + e, v, g);
+                if (g == tag) break;
+                if (clock64() - t0 > P.budget) {
+                    raise_error(P.err, SDC_E_TIMEOUT);
+                    S.ok = 0;
+                }
+                if (!*(volatile int*)&S.ok) break;
+            }
+            stp[e] = __longlong_as_double((long long)v);
+        }
+        flow_bar_sync(3, B - 32);
+        for (int m = t - 32; m < C.qn; m += B - 32) {
+            double a = 0.0;
+            for (int e = sbp[m]; e < sbp[m + 1]; ++e) a += stp[e];
+            tw[m] = a;
+        }
+    };
+    // y = E^-1 t of the own pieces' blocks, a warp per piece
+    auto coarse_y = [&]() {
+        for (int a = nw - 1 - wid; a < np; a += nw) {
+            const double* row = C.Einv + (size_t)pblk[a] * C.q;
+            double pa = 0.0;
+            for (int m = lane; m < C.qn; m += 32) pa += __ldg(row + snz[m]) * tr[m];
+            const int top = __reduce_max_sync(0xffffffffu, xs_field(pa)) + kPieceHead;
+            int q[4];
+            flow_limbs(pa, top, q);
+            const long long x[4] = {q[0], q[1], q[2], q[3]};
+            const double v = warp_value(x, top);
+            if (lane == 0) ysh[a] = v;
+        }
+    };
+    // t = Y' r of the initial residual
+    for (int k = wid == 0 ? nw - 1 : wid - 1; k < nch; k += nw) {
+        const int l = 32 * k + lane;
+        piece_limbs(k, l < nl ? sy[l] * sr[l] : 0.0);
+    }
+    if (!group_barrier(Q.bar, G, epoch, P.budget, P.err, &S.ok)) return;   // diag^-1/2 is out
+    piece_post(C.words, Q.id + 1, [&](int l) { return sy[l] * sr[l]; });
+    flow_rows(nl, [&](int l) {
+        const int i = row_of(l);
+        const double csi = c * P.sv[r0 + l];
+        const int len = plen[l];
+        for (int k = 0; k < len; ++k) {
+            const size_t e = (size_t)k * ld;
+            const int j = sdc_idx(C.ipos[sdc_idx(P.acol[e + i], P.n, 71)], P.n, 72);
+            C.pcol[e + r0 + l] = j;
+            vb[e + l] = csi * P.aval[e + i] * __ldcg(P.sv + j);
+        }
+    });
+    if (wid != 0) coarse_in(C.words, Q.id + 1);
+    __syncthreads();
+    if (!S.ok) return;
+    for (int m = t; m < C.qn; m += B) {
+        tr[m] = tw[m];
+        ts[m] = 0.0;
+    }
+    __syncthreads();
+    coarse_y();
+    __syncthreads();
+    flow_rows(nl, [&](int l) {
+        const double u = sr[l] + sy[l] * ysh[pid[l]];
+        ub[l] = u;
+        pub_store(Q.pub + r0 + l, u, Q.id + 1);
+    });
+    __syncthreads();
+    int it = 0;
+    unsigned npub = 0;
+    bool exact = true, redo = false;
+    double ga, de, alpha = 0.0, beta = 0.0;
+    auto px_row = [&](const double* u, int l) {
+        const double p = u[l] + beta * sp[l];
+        sp[l] = p;
+        if (xs) xs[l] += alpha * p; else P.x[row_of(l)] += alpha * p;
+    };
+    while (true) {
+        const unsigned wtag = Q.id + (unsigned)it + 2;
+        ulonglong2* const words = C.words + (size_t)((it + 1) & 1) * C.pstride;
+        if (!redo) {
+            // w = (I + c S K_off S) u, r.u, w.u, Y' w
+            const unsigned tag = Q.id + (unsigned)it + 1;
+            const ulonglong2* const pub = Q.pub + (size_t)(it & 1) * ld;
+            ga = de = 0.0;
+            for (int k = wid == 0 ? nw - 1 : wid - 1; k < nch; k += nw) {
+                const int l = 32 * k + lane;
+                double v = 0.0;
+                if (l < nl) {
+                    const double u = ub[l];
+                    const double w = flow_row_dot<FlowChunk<MAXT>::value>(
+                        u, plen[l], C.pcol + r0 + l, ld, vb + l, ld, P.n, r0, nl, smem_addr(ub), pub,
+                        tag, 76, S, P.budget, P.err);
+                    wb[l] = w;
+                    ga += sr[l] * u;
+                    de += w * u;
+                    v = sy[l] * w;
+                }
+                __syncwarp();
+                piece_limbs(k, v);
+            }
+            if (it == 0) {
+                // the windows of the first sums, from the exact exponents
+                if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, kFlowSumHead, P.budget,
+                                 P.err))
+                    return;
+                if (S.state == 2) break;
+            }
+        }
+        u64* const acc = Q.acc + 8 * (npub & 1);
+        flow_post(ga, de, has_rows, S, acc);
+        if (wid == 0) {
+            flow_totals<kCoarseHead, kCoarseDrop>(S, acc, npub & 1, G, exact, P.budget, P.err,
+                                                  [&] { flow_bar_arrive(2, B); });
+        } else {
+            if (!redo) {
+                piece_post(words, wtag, [&](int l) { return sy[l] * wb[l]; });
+                if (late && it > 0) flow_rows_px(nl, [&](int l) { px_row(ob, l); });
+            }
+            // the words of all pieces follow close on the sums
+            flow_bar_sync(2, B);
+            if (!redo) coarse_in(words, wtag);
+        }
+        ++npub;
+        __syncthreads();
+        if (!S.ok) return;
+        if (S.state == 3) {
+            if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, kFlowSumHead, P.budget, P.err))
+                return;
+            if (S.state == 0) {
+                exact = redo = true;
+                continue;
+            }
+        }
+        exact = redo = false;
+        if (S.state != 0) break;
+        if (it >= P.maxit) {
+            if (blockIdx.x == 0 && t == 0) raise_error(P.err, SDC_E_CG_NOCONV);
+            break;
+        }
+        ++it;
+        alpha = S.alpha;
+        beta = S.beta;
+        for (int m = B - 1 - t; m < C.qn; m += B) {
+            const double sa = tw[m] + beta * ts[m];
+            ts[m] = sa;
+            tr[m] -= alpha * sa;
+        }
+        __syncthreads();
+        coarse_y();
+        flow_rows(nl, [&](int l) {
+            const double s = wb[l] + beta * ss[l];
+            ss[l] = s;
+            sr[l] -= alpha * s;
+        });
+        if (wid == 0) flow_next(S, P.rtol);
+        __syncthreads();
+        const unsigned utag = Q.id + (unsigned)it + 1;
+        ulonglong2* const pub = Q.pub + (size_t)(it & 1) * ld + r0;
+        flow_rows(nl, [&](int l) {
+            const double u = sr[l] + sy[l] * ysh[pid[l]];
+            wb[l] = u;
+            pub_store(pub + l, u, utag);
+        });
+        __syncthreads();
+        if (!late) flow_rows(nl, [&](int l) { px_row(ub, l); });
+        // u <- w's place; the next w goes into the third buffer (two: u_old's place)
+        double* const o = ub;
+        ub = wb;
+        wb = late ? ob : o;
+        if (late) ob = o;
+    }
+    if (S.state == 2) {
+        if (blockIdx.x == 0 && t == 0) raise_error(P.err, SDC_E_NONFINITE);
+        return;
+    }
+    if (blockIdx.x == 0 && t == 0) {
+        *P.iters_out = it;
+        *P.relres_out = S.z.gamma0 > 0.0 ? sqrt(fabs(S.z.g) / S.z.gamma0) : 0.0;
+        if (P.energy_out) *P.energy_out = S.z.energy;
+    }
+    flow_rows(nl, [&](int l) {
+        const int i = row_of(l);
+        P.x[i] = P.sv[r0 + l] * (xs ? xs[l] : P.x[i]);
+    });
 }
 
 }  // namespace

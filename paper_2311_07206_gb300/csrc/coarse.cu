@@ -84,9 +84,10 @@ __global__ void k_coarse_scan(int nc, const int* __restrict__ cnt, int* __restri
     }
 }
 
-// crow[off + rank] = compact row of each active dof of gperm, in gperm order
+// crow[off + rank] = compact row of each active dof of gperm, in gperm order; ipos its inverse
 __global__ void k_coarse_scatter(int N, const int* __restrict__ gperm, const int* __restrict__ pos,
-                                 const int* __restrict__ off, int n, int* __restrict__ crow) {
+                                 const int* __restrict__ off, int n, int* __restrict__ crow,
+                                 int* __restrict__ ipos) {
     __shared__ int woff[32];
     const int k = blockIdx.x * kChunk + threadIdx.x;
     const int g = k < N ? sdc_idx(gperm[k], N, 82) : 0;
@@ -110,6 +111,7 @@ __global__ void k_coarse_scatter(int N, const int* __restrict__ gperm, const int
     if (on) {
         const int at = off[blockIdx.x] + woff[wid] + __popc(bal & ((1u << lane) - 1u));
         crow[sdc_idx(at, n, 83)] = p;
+        ipos[sdc_idx(p, n, 84)] = at;
     }
 }
 
@@ -299,8 +301,8 @@ __global__ void __launch_bounds__(kInvThreads) k_coarse_invert(int q, double* __
 
 }  // namespace
 
-int coarse_setup(CoarseDev& C, const int* h_lab, int N, int q, int ld, int* err, cudaStream_t s,
-                 std::string& why) {
+int coarse_setup(CoarseDev& C, const int* h_lab, int N, int q, int ld, int width, int* err,
+                 cudaStream_t s, std::string& why) {
     coarse_free(C);
     if (!h_lab || q < 1 || q > kMaxCoarseBlocks) {
         why = "coarse blocks: n_blocks must lie in [1, " + std::to_string(kMaxCoarseBlocks) + "]";
@@ -320,13 +322,17 @@ int coarse_setup(CoarseDev& C, const int* h_lab, int N, int q, int ld, int* err,
     for (int i = 0; i < N; ++i) gperm[cnt[h_lab[i]]++] = i;
     const int nc = nb(N, kChunk);
     const int G = pcg_sm_count();
-    const int P = (ld + kCoarseTile - 1) / kCoarseTile + q;   // pieces: tiles + block boundaries
+    // tiles of either form (kCoarseTile positions, or one tile per CTA); pieces: tiles + block
+    // boundaries
+    const int tiles = std::max((ld + kCoarseTile - 1) / kCoarseTile, G);
+    const int P = tiles + q;
     auto al = [&](void** p, size_t bytes) { return cudaMalloc(p, std::max<size_t>(bytes, 8)); };
     if (al((void**)&C.lab, (size_t)N * 4) || al((void**)&C.gperm, (size_t)N * 4) ||
         al((void**)&C.lab_c, (size_t)ld * 4) || al((void**)&C.crow, (size_t)ld * 4) ||
         al((void**)&C.boff, (size_t)(q + 1) * 4) || al((void**)&C.chunk_cnt, (size_t)nc * 4) ||
         al((void**)&C.chunk_off, (size_t)nc * 4) ||
-        al((void**)&C.tp, (size_t)((ld + kCoarseTile - 1) / kCoarseTile + 1) * 4) ||
+        al((void**)&C.tp, (size_t)(tiles + 1) * 4) || al((void**)&C.ipos, (size_t)ld * 4) ||
+        al((void**)&C.pcol, (size_t)width * ld * 4) || al(&C.words, (size_t)2 * P * 16) ||
         al((void**)&C.nzb, (size_t)q * 4) || al((void**)&C.piece, (size_t)3 * P * 4) ||
         al((void**)&C.blk_ptr, (size_t)(q + 1) * 4) || al((void**)&C.tpiece, (size_t)P * 8) ||
         al((void**)&C.Eacc, (size_t)q * q * 8) ||
@@ -336,6 +342,7 @@ int coarse_setup(CoarseDev& C, const int* h_lab, int N, int q, int ld, int* err,
         why = "coarse blocks: device allocation failed";
         return SDC_E_NOMEM;
     }
+    cudaMemsetAsync(C.words, 0, (size_t)2 * P * 16, s);   // tags of no launch
     cudaMemcpyAsync(C.lab, h_lab, (size_t)N * 4, cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(C.gperm, gperm.data(), (size_t)N * 4, cudaMemcpyHostToDevice, s);
     if (cudaStreamSynchronize(s) != cudaSuccess) {
@@ -344,6 +351,8 @@ int coarse_setup(CoarseDev& C, const int* h_lab, int N, int q, int ld, int* err,
         return SDC_E_CUDA;
     }
     C.q = q;
+    C.width = width;
+    C.pstride = P;
     C.N = N;
     C.Gmax = G;
     C.G = G;
@@ -356,48 +365,64 @@ void coarse_free(CoarseDev& C) {
                     (void*)C.chunk_cnt, (void*)C.chunk_off, (void*)C.tp, (void*)C.piece,
                     (void*)C.blk_ptr, (void*)C.tpiece, (void*)C.nzb,
                     (void*)C.Eacc, (void*)C.Einv, (void*)C.piv, (void*)C.dmax,
-                    (void*)C.bar})
+                    (void*)C.bar, (void*)C.ipos, (void*)C.pcol, C.words})
         if (p) cudaFree(p);
     C = CoarseDev{};
 }
 
-int coarse_sweep(CoarseDev& C, int n, const int* act, const int* pos, int G, cudaStream_t s) {
+int coarse_sweep(CoarseDev& C, int n, const int* act, const int* pos, int maxit,
+                 const PcgConfig& cfg, cudaStream_t s) {
     const int N = C.N, q = C.q, nc = nb(N, kChunk);
     if (n < 1) return SDC_OK;
-    const int T = kCoarseTile, ntiles = nb(n, T);
-    G = std::max(1, std::min({G, C.Gmax, ntiles}));
     k_coarse_labels<<<nb(n, 256), 256, 0, s>>>(n, act, C.lab, N, C.lab_c);
     k_coarse_count<<<nc, kChunk, 0, s>>>(N, C.gperm, pos, C.chunk_cnt);
     k_coarse_scan<<<1, 1024, 0, s>>>(nc, C.chunk_cnt, C.chunk_off);
-    k_coarse_scatter<<<nc, kChunk, 0, s>>>(N, C.gperm, pos, C.chunk_off, n, C.crow);
+    k_coarse_scatter<<<nc, kChunk, 0, s>>>(N, C.gperm, pos, C.chunk_off, n, C.crow,
+                                         C.ipos);
     k_coarse_bounds<<<nb(q + 1, 256), 256, 0, s>>>(q, n, C.crow, C.lab_c, C.boff);
     C.h_boff.resize(q + 1);
     cudaMemcpyAsync(C.h_boff.data(), C.boff, (size_t)(q + 1) * 4, cudaMemcpyDeviceToHost, s);
     if (cudaStreamSynchronize(s) != cudaSuccess) return SDC_E_CUDA;
     if (C.h_boff[q] != n) return SDC_E_INVALID;   // every active row carries a block
     // pieces: the tiles cut at the block boundaries, in position order (so in block
-    // order too, crow being sorted by block)
-    C.h_tp.assign(ntiles + 1, 0);
-    C.h_piece.clear();
-    C.h_blk_ptr.assign(q + 1, 0);
-    int a = 0;
-    for (int j = 0; j < ntiles; ++j) {
-        const int k0 = j * T, k1 = std::min(n, k0 + T);
-        for (int k = k0; k < k1;) {
-            while (C.h_boff[a + 1] <= k) ++a;
-            const int e = std::min(k1, C.h_boff[a + 1]);
-            C.h_piece.insert(C.h_piece.end(), {a, k, e});
-            ++C.h_blk_ptr[a + 1];
-            k = e;
+    // order too, crow being sorted by block); tile j on CTA j mod G
+    int G = 1, ntiles = 0;
+    auto cut = [&](int T, int gmax) {
+        ntiles = nb(n, T);
+        G = std::max(1, std::min(gmax, ntiles));
+        C.h_tp.assign(ntiles + 1, 0);
+        C.h_piece.clear();
+        C.h_blk_ptr.assign(q + 1, 0);
+        int a = 0;
+        for (int j = 0; j < ntiles; ++j) {
+            const int k0 = j * T, k1 = std::min(n, k0 + T);
+            for (int k = k0; k < k1;) {
+                while (C.h_boff[a + 1] <= k) ++a;
+                const int e = std::min(k1, C.h_boff[a + 1]);
+                C.h_piece.insert(C.h_piece.end(), {a, k, e});
+                ++C.h_blk_ptr[a + 1];
+                k = e;
+            }
+            C.h_tp[j + 1] = (int)(C.h_piece.size() / 3);
         }
-        C.h_tp[j + 1] = (int)(C.h_piece.size() / 3);
+        C.pmax = 0;
+        for (int b = 0; b < G; ++b) {
+            int np = 0;
+            for (int j = b; j < ntiles; j += G) np += C.h_tp[j + 1] - C.h_tp[j];
+            C.pmax = std::max(C.pmax, np);
+        }
+        C.ptot = (int)(C.h_piece.size() / 3);
+        C.qn = 0;
+        for (int b = 0; b < q; ++b) C.qn += C.h_blk_ptr[b + 1] > 0;
+    };
+    // on chip, one tile per CTA, where the rows and the coarse data fit
+    C.L = coarse_flow_rows(n, maxit, cfg);
+    C.flow = 0;
+    if (C.L > 0) {
+        cut(C.L, C.Gmax);
+        C.flow = ntiles == G && coarse_flow_fit(C);
     }
-    int pmax = 0;
-    for (int b = 0; b < G; ++b) {
-        int np = 0;
-        for (int j = b; j < ntiles; j += G) np += C.h_tp[j + 1] - C.h_tp[j];
-        pmax = std::max(pmax, np);
-    }
+    if (!C.flow) cut(kCoarseTile, std::min(cfg.sms, C.Gmax));
     C.h_nzb.clear();
     for (int b = 0; b < q; ++b)
         if (C.h_blk_ptr[b + 1]) C.h_nzb.push_back(b);
@@ -410,9 +435,6 @@ int coarse_sweep(CoarseDev& C, int n, const int* act, const int* pos, int G, cud
     C.G = G;
     C.ntiles = ntiles;
     C.tmax = nb(ntiles, G);
-    C.qn = (int)C.h_nzb.size();
-    C.pmax = pmax;
-    C.ptot = (int)(C.h_piece.size() / 3);
     // the host vectors must outlive the copies
     return cudaStreamSynchronize(s) == cudaSuccess ? SDC_OK : SDC_E_CUDA;
 }

@@ -129,7 +129,8 @@ struct StepBuffers {
     int sval_width = 0;
     void* pub = nullptr;      // [2][ld] 16-byte words of the flow kernels: published value, tag
     unsigned long long* flow = nullptr;   // [kFlowWords] their sums and barrier, zeroed per launch
-    unsigned long long flow_id = 0;       // launches so far (tags)
+    unsigned flow_id = 0;     // launches since the words were cleared (tags), and how often
+    unsigned flow_wraps = 0;
     int max_blocks = 0;
     int* flag = nullptr;      // [ld]
     int* map = nullptr;       // [ld] old compact row -> new compact row or -1
@@ -167,6 +168,7 @@ void launch_residual(int M, int n, const int* act, const Ell& K, const double* k
                      const int* n_dev = nullptr);
 // Launch configuration of the restricted PCG solves.
 constexpr int kFlowSmemBytes = 225 * 1024;   // dynamic shared memory of the flow kernels
+constexpr int kFlowMaxit = 1000000;   // iterations a tag can count
 constexpr int kFlowWords = 34;      // 64-bit words of their grid-wide state
 constexpr int kFlowClassicalRows = 130000;   // automatic arrangement: classical above
 constexpr int kSmemVectors = 8;     // per-row doubles in shared memory, shared-memory variant
@@ -270,23 +272,38 @@ struct CoarseDev {
     int ptot = 0;                        // pieces of the sweep
     int ntiles = 0;                      // tiles of the sweep
     int tmax = 0;                        // most tiles of one CTA
+    // on-chip form (k_cgc2_flow): tiles of L positions, one per CTA
+    int width = 0;                       // slots of the node operator
+    int* ipos = nullptr;                 // [ld] position of each compact row
+    int* pcol = nullptr;                 // [width][ld] columns as positions
+    void* words = nullptr;               // [2][pstride] 16-byte words of the pieces' sums
+    int pstride = 0;
+    unsigned wraps = 0;                  // the flow_wraps the words were last cleared at
+    int flow = 0;                        // this sweep's solves run in it
+    int L = 0, block = 0, nbuf = 0, x_smem = 0;
+    size_t smem = 0;
 };
+// Shape of the on-chip form for n rows: rows per CTA (0: none); then, with the pieces known,
+// its buffers and shared memory (false: no room).
+int coarse_flow_rows(int n, int maxit, const PcgConfig& cfg);
+bool coarse_flow_fit(CoarseDev& C);
 // labels: host, N entries in [0, q).  Allocates and uploads; returns an sdc_status.
-int coarse_setup(CoarseDev& C, const int* h_lab, int N, int q, int ld, int* err, cudaStream_t s,
-                 std::string& why);
+int coarse_setup(CoarseDev& C, const int* h_lab, int N, int q, int ld, int width, int* err,
+                 cudaStream_t s, std::string& why);
 void coarse_free(CoarseDev& C);
 // Per sweep: block of each compact row, rows sorted by block, block ranges and the
 // pieces of the CG launch (tiles of kCoarseTile positions, round robin over the CTAs,
 // cut at blocks).  pos: dof -> compact row (-1 outside the active set).  Synchronises
 // the stream (reads the block ranges).
-int coarse_sweep(CoarseDev& C, int n, const int* act, const int* pos, int G, cudaStream_t s);
+int coarse_sweep(CoarseDev& C, int n, const int* act, const int* pos, int maxit,
+                 const PcgConfig& cfg, cudaStream_t s);
 // Per node solve: E = Z' A Z of the operator diag(mc (1 + c J) + c kdc) + c A_off on the
 // active rows (exact fixed-point accumulation) and its inverse.
 int coarse_factor(CoarseDev& C, int n, const Ell& A, const double* mc, const double* J,
                   const double* kdc, double c, long long budget, cudaStream_t s);
 // The node solve with the two-level preconditioner (classical scaled arrangement).
 int launch_pcg_coarse(int n, const Ell& A, const PcgRole& role, double rtol, int maxit,
-                      const CoarseDev& C, const PcgConfig& cfg, StepBuffers& B, cudaStream_t s);
+                      CoarseDev& C, const PcgConfig& cfg, StepBuffers& B, cudaStream_t s);
 
 // Batched PCG: independent solves of the instances whose compact rows are
 // [bounds[s], bounds[s+1]); empty instances are skipped.
@@ -370,7 +387,7 @@ int launch_pcg_standalone(int n, const Ell& A, const double* kdiag, const double
 // rows do not fit on chip; the last kStandaloneResults of them are the results: relres, then
 // error code and iterations (ints).
 constexpr int kStandaloneResults = 2;
-size_t pcg_standalone_flow_doubles(int n, int ld, int width, size_t* zero_at = nullptr);
+size_t pcg_standalone_flow_doubles(int n, int ld, int width, int maxit, size_t* zero_at = nullptr);
 int launch_pcg_standalone_flow(int n, const Ell& A, const double* kdiag, const double* mass,
                                const double* J, double c, const double* b, double* x, double rtol,
                                int maxit, long long budget, double* ws, cudaStream_t s);

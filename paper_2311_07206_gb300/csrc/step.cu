@@ -192,7 +192,7 @@ struct FlowParams {
     unsigned long long* acc;    // two sets of eight words of the running sums
     unsigned long long* emax;   // largest exponents of gamma's and delta's partial sums
     unsigned* bar;              // arrivals of the barriers outside the iteration
-    unsigned long long id;      // launch id << 32: tags of different launches differ
+    unsigned id;                // launch id << 20: tags of different launches differ
     int x_smem;                 // x in shared memory (else in P.x)
     int nbuf;                   // classical: buffers shared by r and w (2 or 3)
     int v_smem;                 // scaled off-diagonals in shared memory (else in P.sval)
@@ -1984,6 +1984,9 @@ void pcg_smem_attrs() {
                          k_cgc_flow<768>, k_cgc_flow<1024>})
         cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kFlowSmemBytes);
+    for (const void* k : {(const void*)k_cgc2_flow<512>, (const void*)k_cgc2_flow<768>,
+                          (const void*)k_cgc2_flow<1024>})
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kFlowSmemBytes);
     for (PcgKernel k : {k_pcg_cluster<512>, k_pcg_cluster<1024>}) {
         cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(kClusterVectors * kClusterRows * sizeof(double)));
@@ -2097,8 +2100,41 @@ int launch_pcg(int n, const Ell& A, int m, double dt, const Coll& co, double rto
     return launch_pcg_params(P, cfg, B, s);
 }
 
+// Launch id of the next flow launch on a context's buffers: 12 bits, the published words
+// cleared when they wrap (0 is no launch's).
+unsigned next_flow_id(StepBuffers& B, cudaStream_t s) {
+    if (++B.flow_id >= 4096) {
+        cudaMemsetAsync(B.pub, 0, (size_t)2 * B.ld * 16, s);
+        B.flow_id = 1;
+        ++B.flow_wraps;
+    }
+    return B.flow_id;
+}
+
+int coarse_flow_rows(int n, int maxit, const PcgConfig& cfg) {
+    if (cfg.variant == 1 || !cfg.scaled || maxit >= kFlowMaxit) return 0;
+    int gm = std::min(cfg.sms, 255);
+    if (cfg.max_blocks > 0) gm = std::min(gm, cfg.max_blocks);
+    const int l = nblk(n, gm);
+    const int L = l <= 96 ? 96 : l <= 896 ? (l + 127) / 128 * 128 : (l + 31) / 32 * 32;
+    return 6 * L <= kFlowSmemBytes / 8 ? L : 0;
+}
+bool coarse_flow_fit(CoarseDev& C) {
+    // one row per thread up to 736 rows; above, 512 threads with 128 registers each (us per
+    // iteration with 512 / 768 / 1024 threads: 131k rows 9.4 / 10.9 / 10.5, 250k 14.9 / 16.2 /
+    // 15.5, 505k 23.8 / 25.2 / 26.4; in one row per thread 83k 8.4 against 8.9)
+    C.block = C.L <= 736 ? 32 + C.L : 512;
+    for (int v = 8; v >= 6; --v) {   // with x and the third buffer, with the buffer, with neither
+        C.nbuf = v >= 7 ? 3 : 2;
+        C.x_smem = v == 8;
+        C.smem = coarse_flow_smem(C.L, v, C.qn, C.ptot, C.pmax);
+        if (C.smem <= (size_t)kFlowSmemBytes) return true;
+    }
+    return false;
+}
+
 int launch_pcg_coarse(int n, const Ell& A, const PcgRole& role, double rtol, int maxit,
-                      const CoarseDev& C, const PcgConfig& cfg, StepBuffers& B, cudaStream_t s) {
+                      CoarseDev& C, const PcgConfig& cfg, StepBuffers& B, cudaStream_t s) {
     CgParams P{};
     P.n = n;
     P.ld = B.ld;
@@ -2126,6 +2162,46 @@ int launch_pcg_coarse(int n, const Ell& A, const PcgRole& role, double rtol, int
     P.relres_out = role.relres_out;
     P.energy_out = role.energy_out;
     P.M = 1;
+    if (C.flow) {
+        if (!B.pub || C.width > B.sval_width || A.width > C.width) return SDC_E_INVALID;
+        pcg_smem_attrs();
+        FlowParams Q{};
+        Q.pub = reinterpret_cast<ulonglong2*>(B.pub);
+        Q.acc = B.flow;
+        Q.emax = B.flow + 16;
+        Q.bar = reinterpret_cast<unsigned*>(B.flow + 32);
+        Q.id = next_flow_id(B, s) << 20;
+        if (C.wraps != B.flow_wraps) {
+            cudaMemsetAsync(C.words, 0, (size_t)2 * C.pstride * 16, s);
+            C.wraps = B.flow_wraps;
+        }
+        Q.x_smem = C.x_smem;
+        Q.nbuf = C.nbuf;
+        P.L = C.L;
+        CoarseFlowParams F;
+        F.q = C.q;
+        F.qn = C.qn;
+        F.ptot = C.ptot;
+        F.npmax = C.pmax;
+        F.crow = C.crow;
+        F.ipos = C.ipos;
+        F.pcol = C.pcol;
+        F.tp = C.tp;
+        F.piece = C.piece;
+        F.blk_ptr = C.blk_ptr;
+        F.nzb = C.nzb;
+        F.Einv = C.Einv;
+        F.words = reinterpret_cast<ulonglong2*>(C.words);
+        F.pstride = C.pstride;
+        cudaMemsetAsync(B.flow, 0, kFlowWords * sizeof(unsigned long long), s);
+        void* fa[] = {&P, &Q, &F};
+        const void* k = C.block > 768   ? (const void*)k_cgc2_flow<1024>
+                        : C.block > 512 ? (const void*)k_cgc2_flow<768>
+                                        : (const void*)k_cgc2_flow<512>;
+        return cudaLaunchCooperativeKernel(k, dim3(C.G), dim3(C.block), fa, C.smem, s) == cudaSuccess
+                   ? SDC_OK
+                   : SDC_E_CUDA;
+    }
     cudaMemsetAsync(&B.sc->bar, 0, sizeof(unsigned), s);
     CoarseParams CP;
     CP.q = C.q;
@@ -2204,7 +2280,8 @@ struct FlowShape {
 };
 bool flow_shape(int n, bool classical, const PcgConfig& cfg, FlowShape& f) {
     const int rows = kFlowSmemBytes / 8;                // doubles on chip
-    const int cap = (classical ? rows / 4 : rows / 7) / 32 * 32;
+    // (4 or 7 vectors and 2 bytes of row length)
+    const int cap = (classical ? rows * 4 / 17 : rows * 4 / 29) / 32 * 32;
     int gm = std::min(cfg.sms, 255);                    // arrivals are counted in a byte
     if (n > (long long)gm * cap) return false;
     if (cfg.max_blocks > 0) gm = std::min(gm, std::max(cfg.max_blocks, nblk(n, cap)));
@@ -2216,14 +2293,14 @@ bool flow_shape(int n, bool classical, const PcgConfig& cfg, FlowShape& f) {
     f.grid = nblk(n, f.L);
     f.block = std::min(32 + std::min(f.L, (n + 31) / 32 * 32), maxb);
     if (classical) {
-        f.nbuf = 5 * f.L <= rows ? 3 : 2;
-        f.x_smem = f.nbuf == 3 && 6 * f.L <= rows;
+        f.nbuf = 5 * f.L + f.L / 4 <= rows ? 3 : 2;
+        f.x_smem = f.nbuf == 3 && 6 * f.L + f.L / 4 <= rows;
     } else {
         f.nbuf = 2;
-        f.x_smem = 8 * f.L <= rows;
+        f.x_smem = 8 * f.L + f.L / 4 <= rows;
     }
     f.v_smem = 0;
-    f.smem = (size_t)((classical ? 2 + f.nbuf : 7) + f.x_smem) * f.L * sizeof(double);
+    f.smem = (size_t)((classical ? 2 + f.nbuf : 7) + f.x_smem) * f.L * sizeof(double) + 2 * f.L;
     return true;
 }
 // The scaled off-diagonals of `width` slots in shared memory as well, if there is room: for
@@ -2239,14 +2316,14 @@ bool flow_values_on_chip(int width, FlowShape& f) {
 
 // words: kFlowWords words, zero; pub: tags of other launches only
 int launch_flow(CgParams& P, bool classical, const FlowShape& f, void* pub,
-                unsigned long long* words, unsigned long long id, cudaStream_t s) {
+                unsigned long long* words, unsigned id, cudaStream_t s) {
     pcg_smem_attrs();
     FlowParams Q;
     Q.pub = reinterpret_cast<ulonglong2*>(pub);
     Q.acc = words;
     Q.emax = words + 16;
     Q.bar = reinterpret_cast<unsigned*>(words + 32);
-    Q.id = id << 32;
+    Q.id = id << 20;
     Q.x_smem = f.x_smem;
     Q.nbuf = f.nbuf;
     Q.v_smem = f.v_smem;
@@ -2264,10 +2341,10 @@ int launch_pcg_params(CgParams& P, const PcgConfig& cfg, StepBuffers& B, cudaStr
     FlowShape fs;
     const bool flow_classical =
         !cfg.pipelined || (cfg.general_classical && n > kFlowClassicalRows);
-    if (cfg.variant != 1 && cfg.scaled && P.sv && P.sval && B.pub &&
+    if (cfg.variant != 1 && cfg.scaled && P.sv && P.sval && B.pub && P.maxit < kFlowMaxit &&
         flow_shape(n, flow_classical, cfg, fs)) {
         cudaMemsetAsync(B.flow, 0, kFlowWords * sizeof(unsigned long long), s);
-        return launch_flow(P, flow_classical, fs, B.pub, B.flow, ++B.flow_id, s);
+        return launch_flow(P, flow_classical, fs, B.pub, B.flow, next_flow_id(B, s), s);
     }
     cudaMemsetAsync(&B.sc->bar, 0, sizeof(unsigned), s);
     void* args[] = {&P};
@@ -2561,10 +2638,10 @@ bool pcg_standalone_shape(int n, int width, FlowShape& f, bool& classical) {
     return true;
 }
 
-size_t pcg_standalone_flow_doubles(int n, int ld, int width, size_t* zero_at) {
+size_t pcg_standalone_flow_doubles(int n, int ld, int width, int maxit, size_t* zero_at) {
     FlowShape f;
     bool classical;
-    if (!pcg_standalone_shape(n, width, f, classical)) return 0;
+    if (maxit >= kFlowMaxit || !pcg_standalone_shape(n, width, f, classical)) return 0;
     // u, diag^-1/2, [scaled values], then from a 256-byte boundary on what starts at zero:
     // the published words, the sums, the results
     const size_t z = (2 * (size_t)n + (f.v_smem ? 0 : (size_t)width * ld) + 31) / 32 * 32;
@@ -2578,7 +2655,7 @@ int launch_pcg_standalone_flow(int n, const Ell& A, const double* kdiag, const d
     FlowShape f;
     bool classical;
     size_t z = 0;
-    const size_t total = pcg_standalone_flow_doubles(n, A.ld, A.width, &z);
+    const size_t total = pcg_standalone_flow_doubles(n, A.ld, A.width, maxit, &z);
     if (!total || !pcg_standalone_shape(n, A.width, f, classical) ||
         reinterpret_cast<uintptr_t>(ws) % 256 != 0)
         return SDC_E_INVALID;

@@ -99,3 +99,31 @@ def test_gamma_rises_above_the_window(torch_dev):
     r1 = b - (b @ (b / d)) / ((b / d) @ A @ (b / d)) * (A @ (b / d))
     assert (r1 @ (r1 / d)) / (b @ (b / d)) > 2.0 ** 11
     _check(wl, torch, dev, cg_pipelined=0)
+
+
+@pytest.mark.parametrize("blocks", [0, 1, 3])
+def test_two_level_edges(torch_dev, blocks):
+    """Cell-by-cell bricks of 4,176 dofs in 72 blocks: on many CTAs (pieces of one warp and
+    less), on one CTA (two buffers, x in global memory, rows many times the threads) and on
+    three (pieces across CTAs).  Counts to 5 %, as the two-level parity tests have them."""
+    torch, dev = torch_dev
+    from paper_2311_07206_gb300 import Context, default_options
+    from workloads.emi import coarse_blocks, emi_bricks
+    wl = emi_bricks(cells=(2, 1, 1), cell_um=(24.0, 14.0, 10.0), h=2.0, margin=2, sweeps=2)
+    lab = coarse_blocks(wl, split=(6, 2, 2), min_dofs=300)
+    assert (wl.n, lab.max() + 1) == (4176, 72)
+    ctx = Context.from_emi(wl, options=default_options(cg_max_blocks=blocks),
+                           stream=torch.cuda.current_stream(dev).cuda_stream)
+    ctx.set_coarse_blocks(lab)
+    u = torch.tensor(wl.u0, dtype=torch.float64, device=dev)
+    w = torch.tensor(wl.w0, dtype=torch.float64, device=dev)
+    st = ctx.step(u, w, 0.0, wl.dt, wl.sweeps, wl.tol)
+    ctx.close()
+    r = oracle.System.from_mesh(wl.mesh).step_emi(wl, wl.u0, wl.w0, coarse=lab)
+    assert r["status"] == 0
+    for a, b in ((u, r["u"]), (w, r["w"])):
+        assert np.abs(a.cpu().numpy() - b).max() <= RTOL * max(1.0, np.abs(b).max())
+    for k in range(wl.sweeps):
+        for m in range(wl.M):
+            a, b = st.cg_iters[k][m], r["stats"].cg_iters[k * 8 + m]
+            assert abs(a - b) <= max(2, b // 20), (k, m, a, b)
