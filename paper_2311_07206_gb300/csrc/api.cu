@@ -181,6 +181,8 @@ int alloc_buffers(sdc_ctx* c) {
     if (ok && !c->inst_off.empty()) {
         const int nseg = (int)c->inst_off.size() - 1;
         B.nseg = nseg;
+        for (int g = 0; g < nseg; ++g)
+            B.seg_max = std::max(B.seg_max, c->inst_off[g + 1] - c->inst_off[g]);
         P.batch_block = std::min(P.block, 256);
         P.batch_pipelined = c->opt.cg_pipelined == 1;
         P.max_blocks_batch = pcg_batch_max_blocks(P.batch_block);
@@ -188,8 +190,9 @@ int alloc_buffers(sdc_ctx* c) {
             P.max_blocks_batch = std::min(P.max_blocks_batch, c->opt.cg_max_blocks);
         B.max_blocks = std::max(B.max_blocks, P.max_blocks_batch);
         ok = dalloc(&B.inst_off, nseg + 1) && dalloc(&B.bounds, nseg + 1) &&
-             dalloc(&B.segtab, 5 * (size_t)P.max_blocks_batch) && dalloc(&B.bars, nseg) &&
-             (B.segtab_cap = P.max_blocks_batch) > 0 &&
+             (B.segtab_cap = std::max(P.max_blocks_batch, 4 * P.sms)) > 0 &&
+             dalloc(&B.segtab, 5 * (size_t)B.segtab_cap) && dalloc(&B.bars, nseg) &&
+             dalloc(&B.bflow_words, (size_t)nseg * kFlowWords) &&
              dalloc(&B.seg_iters, (size_t)SDC_MAX_SWEEPS * kMaxM * nseg) &&
              dalloc(&B.seg_relres, (size_t)SDC_MAX_SWEEPS * kMaxM * nseg) &&
              dalloc(&B.plan, 2 * (size_t)nseg) && dalloc(&B.nk, SDC_MAX_SWEEPS + 1) &&
@@ -229,6 +232,7 @@ void free_all(sdc_ctx* c) {
     for (int* p : ip) cudaFree(p);
     cudaFree(B.bars);
     cudaFree(B.pub);
+    cudaFree(B.bflow_words);
     cudaFree(B.flow);
     cudaFree(B.seg_relres);
     if (c->h_bounds) cudaFreeHost(c->h_bounds);
@@ -759,6 +763,8 @@ sdc_status step_batch_graph(sdc_ctx* c, double* d_v, double* d_w, double dt, int
         cudaMemsetAsync(B.sc, 0, sizeof(DevScalars), s);
         cudaMemsetAsync(B.seg_iters, 0, cnt * sizeof(int), s);
         cudaMemsetAsync(B.seg_relres, 0, cnt * sizeof(double), s);
+        // the replays' launches carry the same ids: no word of an earlier step may remain
+        if (batch_on_chip(c->pcg, B)) cudaMemsetAsync(B.pub, 0, (size_t)2 * B.ld * 16, s);
         launch_graph_init(B, s);
         launch_spread(N, M, d_v, d_w, B.V, B.W, s);
         L += 2;
@@ -946,6 +952,8 @@ sdc_status step_core(sdc_ctx* c, double* d_v, double* d_w, double t, double dt, 
         const size_t cnt = (size_t)SDC_MAX_SWEEPS * kMaxM * B.nseg;
         cudaMemsetAsync(B.seg_iters, 0, cnt * sizeof(int), s);
         cudaMemsetAsync(B.seg_relres, 0, cnt * sizeof(double), s);
+        // a captured step counts its launches from 1 as well
+        if (batch_on_chip(c->pcg, B)) cudaMemsetAsync(B.pub, 0, (size_t)2 * B.ld * 16, s);
     }
     const double big = 1.7976931348623157e308;
     cudaMemcpyAsync(&B.sc->margin, &big, sizeof(double), cudaMemcpyHostToDevice, s);

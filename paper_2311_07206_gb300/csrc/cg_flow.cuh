@@ -375,7 +375,8 @@ __device__ __forceinline__ bool flow_window(double a, double b, FlowShared& S, u
 
 // Off-diagonal product of a row: acc + sum_k v[k vs] x(c[k ld]) over its len slots, in order.
 // Columns of this CTA (rows [r0, r0 + nl)) come from shared memory (own), the others from their
-// published words, fetched again until they carry `tag`.  All loads of CH slots are issued
+// published words, fetched again until they carry `tag` (slots past the row's end fetch row r0:
+// with nl = 0 the caller passes a row of its own, whose word is there).  All loads of CH slots are issued
 // before the first is used.  The product of a CTA with many rows is bound by instruction
 // issue, not by FP64 or latency (two padded slots more per row: 442k rows 13.5 -> 15.2 us per
 // iteration), so a slot is kept to a dozen instructions.
@@ -454,12 +455,12 @@ struct FlowChunk {
 // off-diagonals c s_i a_ij s_j (slot k of local row l at vb[k vs + l]) and
 // w = (I + c S K_off S) r.  f(l, r) receives a row's r,
 // g(l, w) its w; gamma and delta partial sums in ga, de.  Returns false to leave the kernel.
-template <int MAXT, class F, class H>
+template <int CH, class F, class H>
 __device__ __forceinline__ bool flow_start(const CgParams& P, const FlowParams& Q, FlowShared& S,
                                            int r0, int nl, unsigned short* plen, double* vb, int vs,
                                            unsigned& epoch,
                                            double& ga, double& de, F&& f, H&& h) {
-    const int t = threadIdx.x, G = gridDim.x, ld = P.ld;
+    const int t = threadIdx.x, G = Q.G, ld = P.ld;
     const double c = P.c;
     ga = de = 0.0;
     if (t == 0) {
@@ -480,7 +481,7 @@ __device__ __forceinline__ bool flow_start(const CgParams& P, const FlowParams& 
         ga += r * r;
         f(l, r);
     });
-    if (P.inject_fault && blockIdx.x == G - 1) {
+    if (P.inject_fault && Q.bidx == G - 1) {
         // leave without arriving: every other CTA's bounded wait runs out
         if (G == 1 && t == 0) raise_error(P.err, SDC_E_TIMEOUT);
         return false;
@@ -488,10 +489,9 @@ __device__ __forceinline__ bool flow_start(const CgParams& P, const FlowParams& 
     // delta's partial sums: |w.r| of a thread <= |A| gamma, gamma <= 2^17.3 largest partial
     if (!flow_window(ga, ga, S, Q.emax, Q.bar, G, epoch, 1u, 22, P.budget, P.err)) return false;
     if (S.state == 2) {
-        if (blockIdx.x == 0 && t == 0) raise_error(P.err, SDC_E_NONFINITE);
+        if (Q.bidx == 0 && t == 0) raise_error(P.err, SDC_E_NONFINITE);
         return false;
     }
-    constexpr int CH = FlowChunk<MAXT>::value;
     flow_rows(nl, [&](int l) {
         const int i = r0 + l;
         const int len = __ldg(P.alen + i);
@@ -531,18 +531,18 @@ __device__ __forceinline__ bool flow_start(const CgParams& P, const FlowParams& 
 
 // End of a solve: statistics, x = S x~ on the CTA's rows and the LU-trick coupling, whose
 // neighbours' x travel as tagged words.  xt(l): the CTA's x~.
-template <int MAXT, class X>
+template <int CH, class X>
 __device__ __forceinline__ void flow_finish(const CgParams& P, const FlowParams& Q, FlowShared& S,
                                             int r0, int nl, int it, X&& xt) {
     const int ld = P.ld;
-    const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
+    const bool lead = Q.bidx == 0 && threadIdx.x == 0;
     if (S.state == 2) {
         if (lead) raise_error(P.err, SDC_E_NONFINITE);
         return;
     }
     if (lead) {
-        *P.iters_out = it;
-        *P.relres_out = S.z.gamma0 > 0.0 ? sqrt(fabs(S.z.g) / S.z.gamma0) : 0.0;
+        *Q.iters_out = it;
+        *Q.relres_out = S.z.gamma0 > 0.0 ? sqrt(fabs(S.z.g) / S.z.gamma0) : 0.0;
         if (P.energy_out) *P.energy_out = S.z.energy;
     }
     // the words of iteration it - 1, whose readers are done: their CTAs posted sum `it`
@@ -559,8 +559,8 @@ __device__ __forceinline__ void flow_finish(const CgParams& P, const FlowParams&
     flow_rows(nl, [&](int l) {
         const int i = r0 + l;
         const int len = __ldg(P.alen + i);
-        const double kx = flow_row_dot<FlowChunk<MAXT>::value>(
-            0.0, len, P.acol + i, ld, P.aval + i, ld, P.n, 0, 0, 0u, pub, tag, 47, S, P.budget, P.err);
+        const double kx = flow_row_dot<CH>(
+            0.0, len, P.acol + i, ld, P.aval + i, ld, P.n, i, 0, 0u, pub, tag, 47, S, P.budget, P.err);
         cg_couple_row(P, i, P.x[i], kx);
     });
 }
@@ -575,8 +575,11 @@ template <int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) {
     extern __shared__ double sm[];
     __shared__ FlowShared S;
+    constexpr int CH = FlowChunk<MAXT>::value;
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5, nw = blockDim.x >> 5;
     const int G = gridDim.x, L = P.L, ld = P.ld;
+    Q.G = G;
+    Q.bidx = blockIdx.x;
     const int r0 = blockIdx.x * L;
     const int nl = max(0, min(P.n - r0, L));
     const int nch = (nl + 31) >> 5;
@@ -597,7 +600,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
     unsigned epoch = 0, gen = 1;
     double ga, de, alpha = 0.0, beta = 0.0;
     flow_scalars_init(S);
-    if (!flow_start<MAXT>(
+    if (!flow_start<CH>(
             P, Q, S, r0, nl, plen, vb, vs, epoch, ga, de,
             [&](int l, double r) {
                 rc[l] = r;
@@ -639,7 +642,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
                 const int l = 32 * c + lane;
                 if (l < nl) {
                     const int i = r0 + l;
-                    sn[l] = flow_row_dot<FlowChunk<MAXT>::value>(
+                    sn[l] = flow_row_dot<CH>(
                         sw[l], plen[l], P.acol + i, ld, vb + l, vs, P.n, r0, nl, smem_addr(sw), pub, tag,
                         42, S, P.budget, P.err);
                 }
@@ -688,7 +691,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
         rc = ro;
         ro = q;
     }
-    flow_finish<MAXT>(P, Q, S, r0, nl, it, [&](int l) { return xs[l]; });
+    flow_finish<CH>(P, Q, S, r0, nl, it, [&](int l) { return xs[l]; });
 }
 
 // ---- classical arrangement (see pcgc_group), scaled form -----------------------------
@@ -696,14 +699,13 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
 // dot products, the sums posted, and while they are summed p and x.  r_new goes into w's
 // place, which s has used up; with three buffers (nbuf = 3) the next w goes into a third, so
 // that r_old is still there for p after the product; with two, p and x come before it.
-template <int MAXT>
-__global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) {
-    extern __shared__ double sm[];
-    __shared__ FlowShared S;
+// One group of Q.G CTAs (the launch, or one instance of a batched launch); this CTA, number
+// Q.bidx of it, owns rows [r0, r0 + nl), at most P.L.
+template <int CH>
+__device__ __forceinline__ void cgc_flow(const CgParams& P, const FlowParams& Q, FlowShared& S, double* sm,
+                                         int r0, int nl) {
     const int t = threadIdx.x, wid = t >> 5, nw = blockDim.x >> 5;
-    const int G = gridDim.x, L = P.L, ld = P.ld;
-    const int r0 = blockIdx.x * L;
-    const int nl = max(0, min(P.n - r0, L));
+    const int G = Q.G, L = P.L, ld = P.ld;
     const int nch = (nl + 31) >> 5;
     const bool late = Q.nbuf == 3;
     double* rb = sm;
@@ -720,7 +722,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) 
     unsigned epoch = 0, gen = 1;
     double ga, de, alpha = 0.0, beta = 0.0;
     flow_scalars_init(S);
-    if (!flow_start<MAXT>(
+    if (!flow_start<CH>(
             P, Q, S, r0, nl, plen, vb, vs, epoch, ga, de,
             [&](int l, double r) {
                 rb[l] = r;
@@ -756,7 +758,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) 
         exact = redo = false;
         if (S.state != 0) break;
         if (it >= P.maxit) {
-            if (blockIdx.x == 0 && t == 0) raise_error(P.err, SDC_E_CG_NOCONV);
+            if (Q.bidx == 0 && t == 0) raise_error(P.err, SDC_E_CG_NOCONV);
             break;
         }
         ++it;
@@ -780,7 +782,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) 
         flow_rows(nl, [&](int l) {
             const int i = r0 + l;
             const double r = wb[l];
-            const double w = flow_row_dot<FlowChunk<MAXT>::value>(
+            const double w = flow_row_dot<CH>(
                 r, plen[l], P.acol + i, ld, vb + l, vs, P.n, r0, nl, own, pub, tag, 46, S, P.budget,
                 P.err);
             fb[l] = w;
@@ -793,7 +795,39 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) 
         wb = fb;
         fb = late ? q : rb;
     }
-    flow_finish<MAXT>(P, Q, S, r0, nl, it, [&](int l) { return xs[l]; });
+    flow_finish<CH>(P, Q, S, r0, nl, it, [&](int l) { return xs[l]; });
+}
+
+template <int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) {
+    extern __shared__ double sm[];
+    __shared__ FlowShared S;
+    Q.G = gridDim.x;
+    Q.bidx = blockIdx.x;
+    const int r0 = blockIdx.x * P.L;
+    cgc_flow<FlowChunk<MAXT>::value>(P, Q, S, sm, r0, max(0, min(P.n - r0, P.L)));
+}
+
+// Batched form: the blocks of an instance are a group with its own sums, barrier and
+// iteration count.  Several CTAs share an SM, so that one works while another waits.
+template <int MAXT>
+__global__ void __launch_bounds__(MAXT, 1024 / MAXT)
+    k_cgc_flow_batch(CgParams P, FlowParams Q, const SegBlock* __restrict__ tab,
+                     int* __restrict__ seg_iters, double* __restrict__ seg_relres) {
+    extern __shared__ double sm[];
+    __shared__ FlowShared S;
+    const SegBlock g = tab[blockIdx.x];
+    if (g.nblk == 0) return;   // no group: a planned launch's spare block
+    Q.G = g.nblk;
+    Q.bidx = (int)blockIdx.x - g.blk0;
+    Q.acc += (size_t)g.seg * kFlowWords;
+    Q.emax = Q.acc + 16;
+    Q.bar = reinterpret_cast<unsigned*>(Q.acc + 32);
+    Q.iters_out = seg_iters + g.seg;
+    Q.relres_out = seg_relres + g.seg;
+    const int Lg = ((g.row1 - g.row0 + g.nblk - 1) / g.nblk + 31) & ~31;
+    const int r0 = g.row0 + Q.bidx * Lg;
+    cgc_flow<4>(P, Q, S, sm, r0, max(0, min(g.row1 - r0, Lg)));
 }
 
 // ---- classical arrangement with the two-level preconditioner --------------------------
@@ -1172,8 +1206,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc2_flow(CgParams P, FlowParams Q,
         return;
     }
     if (blockIdx.x == 0 && t == 0) {
-        *P.iters_out = it;
-        *P.relres_out = S.z.gamma0 > 0.0 ? sqrt(fabs(S.z.g) / S.z.gamma0) : 0.0;
+        *Q.iters_out = it;
+        *Q.relres_out = S.z.gamma0 > 0.0 ? sqrt(fabs(S.z.g) / S.z.gamma0) : 0.0;
         if (P.energy_out) *P.energy_out = S.z.energy;
     }
     flow_rows(nl, [&](int l) {

@@ -105,6 +105,14 @@ unsigned long long check_take_coarse(void* stream, unsigned* count);
 // calling thread when ctx is NULL); otherwise st unchanged.
 sdc_status check_outcome(sdc_ctx* ctx, void* stream, sdc_status st);
 
+// Shape of the batched on-chip solves and the configuration it was found for.
+struct BatchFlow {
+    int block = 0, rpb = 0, max_blocks = -1;
+    bool on = false;
+    int grid = 0, L = 0, nbuf = 0, x_smem = 0;   // grid 0: not on chip
+    size_t smem = 0;
+};
+
 struct StepBuffers {
     int N = 0, M = 0, ld = 0;
     double* V = nullptr;      // [N][M] node-interleaved collocation iterates of v
@@ -151,6 +159,9 @@ struct StepBuffers {
     int* nk = nullptr;            // [SDC_MAX_SWEEPS + 1] |I_k| of a captured step
     int* bounds_k = nullptr;      // [(SDC_MAX_SWEEPS + 1) (nseg + 1)] boundaries per sweep
     unsigned* bars = nullptr;     // [nseg] barrier counters
+    int seg_max = 0;              // dofs of the largest instance
+    BatchFlow bflow;
+    unsigned long long* bflow_words = nullptr;   // [nseg][kFlowWords]
     int* seg_iters = nullptr;     // [SDC_MAX_SWEEPS * kMaxM * nseg]
     double* seg_relres = nullptr; // same shape
 };
@@ -321,6 +332,8 @@ int launch_pcg_batch_planned(const Ell& A, int m, double dt, const Coll& co, dou
                              int maxit, int sweep, const PcgConfig& cfg, const int* bounds_dev,
                              bool plan, StepBuffers& B, cudaStream_t s);
 int pcg_batch_max_blocks(int block);
+// Whether the batched solves run on chip (and so use the published words).
+bool batch_on_chip(const PcgConfig& cfg, StepBuffers& B);
 
 // ---- adjoint (adjoint.cu) ----
 struct AdjointArgs {

@@ -196,6 +196,9 @@ struct FlowParams {
     int x_smem;                 // x in shared memory (else in P.x)
     int nbuf;                   // classical: buffers shared by r and w (2 or 3)
     int v_smem;                 // scaled off-diagonals in shared memory (else in P.sval)
+    int G, bidx;                // CTAs of the group, this CTA's number (set by the kernels)
+    int* iters_out;             // results of the group's solve
+    double* relres_out;
 };
 
 }  // namespace
@@ -2177,6 +2180,8 @@ int launch_pcg_coarse(int n, const Ell& A, const PcgRole& role, double rtol, int
         }
         Q.x_smem = C.x_smem;
         Q.nbuf = C.nbuf;
+        Q.iters_out = P.iters_out;
+        Q.relres_out = P.relres_out;
         P.L = C.L;
         CoarseFlowParams F;
         F.q = C.q;
@@ -2327,6 +2332,8 @@ int launch_flow(CgParams& P, bool classical, const FlowShape& f, void* pub,
     Q.x_smem = f.x_smem;
     Q.nbuf = f.nbuf;
     Q.v_smem = f.v_smem;
+    Q.iters_out = P.iters_out;
+    Q.relres_out = P.relres_out;
     P.L = f.L;
     void* args[] = {&P, &Q};
     cudaError_t e = cudaLaunchCooperativeKernel((const void*)flow_kernel(f.block, classical),
@@ -2443,6 +2450,120 @@ int pcg_batch_max_blocks(int block) {
     return sms * per;
 }
 
+// Batched solves on chip.  A CTA takes at least batch_rows_per_block / 8 rows and, in a sweep of
+// `total` rows, enough that every instance's CTAs fit the grid of `grid` resident ones:
+// sum of ceil(rows / rpb) <= total / rpb + nseg.  An instance has at most 255 CTAs (arrivals are
+// counted in a byte).
+__host__ __device__ inline int batch_flow_rows(long long total, int grid, int nseg, int floor_rows) {
+    const long long r = (total + (grid - nseg) - 1) / (grid - nseg);
+    const int rpb = (int)((r + 31) / 32 * 32);
+    return rpb > floor_rows ? rpb : floor_rows;
+}
+__host__ __device__ inline int batch_flow_blocks(int rows, int rpb) {
+    const int b = (rows + rpb - 1) / rpb;
+    return b < 255 ? b : 255;
+}
+int batch_flow_floor(const PcgConfig& cfg) {
+    return std::max(32, cfg.batch_rows_per_block / 8 / 32 * 32);
+}
+const void* batch_flow_kernel(int block) {
+    return block > 512 ? (const void*)k_cgc_flow_batch<1024>
+           : block > 256 ? (const void*)k_cgc_flow_batch<512>
+                         : (const void*)k_cgc_flow_batch<256>;
+}
+
+// Grid, rows and shared memory per CTA for the whole batch (the largest sweep), from the most
+// CTAs per SM down; grid 0 when the rows do not fit.  Kept per launch configuration.
+const BatchFlow& batch_flow_shape(const PcgConfig& cfg, StepBuffers& B) {
+    BatchFlow& f = B.bflow;
+    const bool on = cfg.variant != 1 && cfg.scaled && !cfg.batch_pipelined && B.pub && B.sval;
+    if (f.block == cfg.batch_block && f.rpb == cfg.batch_rows_per_block &&
+        f.max_blocks == cfg.max_blocks && f.on == on)
+        return f;
+    f = BatchFlow{};
+    f.block = cfg.batch_block;
+    f.rpb = cfg.batch_rows_per_block;
+    f.max_blocks = cfg.max_blocks;
+    f.on = on;
+    if (!on || cfg.batch_block > 1024 || cfg.batch_block < 64) return f;
+    const void* k = batch_flow_kernel(cfg.batch_block);
+    for (int per = 1024 / std::max(cfg.batch_block, 256); per >= 1; --per) {
+        int grid = cfg.sms * per;
+        if (cfg.max_blocks > 0) grid = std::min(grid, cfg.max_blocks);
+        grid = std::min(grid, B.segtab_cap);
+        if (grid <= B.nseg) continue;
+        const int floor_rows = batch_flow_floor(cfg);
+        int L = batch_flow_rows(B.N, grid, B.nseg, floor_rows);
+        L = std::max(L, (nblk(B.seg_max, 255) + 31) / 32 * 32);
+        for (int v = 6; v >= 4; --v) {   // with x and the third buffer, the buffer, neither
+            const size_t smem = (size_t)v * L * sizeof(double) + 2 * L;
+            if (smem > (size_t)kFlowSmemBytes) continue;
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kFlowSmemBytes);
+            int occ = 0;
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, cfg.batch_block, smem) !=
+                    cudaSuccess ||
+                occ < per)
+                continue;
+            f.grid = grid;
+            f.L = L;
+            f.smem = smem;
+            f.nbuf = v >= 5 ? 3 : 2;
+            f.x_smem = v == 6;
+            return f;
+        }
+    }
+    return f;
+}
+
+bool batch_on_chip(const PcgConfig& cfg, StepBuffers& B) { return batch_flow_shape(cfg, B).grid > 0; }
+
+// Block table of a batched on-chip solve from the device boundaries (one block).
+__global__ void k_batch_plan_flow(int nseg, const int* __restrict__ bounds, int G, int floor_rows,
+                                  SegBlock* __restrict__ tab, int* __restrict__ first) {
+    __shared__ int total_s, rpb_s;
+    if (threadIdx.x == 0) {
+        rpb_s = batch_flow_rows(bounds[nseg] - bounds[0], G, nseg, floor_rows);
+        int run = 0;
+        for (int g = 0; g < nseg; ++g) {
+            first[g] = run;
+            run += batch_flow_blocks(bounds[g + 1] - bounds[g], rpb_s);
+        }
+        total_s = run;
+    }
+    __syncthreads();
+    for (int b = threadIdx.x; b < G; b += blockDim.x) {
+        SegBlock e{0, 0, 0, 0, 0};
+        if (b < total_s) {
+            // the last instance whose first block is <= b: a non-empty one
+            int lo = 0, hi = nseg - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (first[mid] <= b) lo = mid; else hi = mid - 1;
+            }
+            e = SegBlock{bounds[lo], bounds[lo + 1], first[lo],
+                         batch_flow_blocks(bounds[lo + 1] - bounds[lo], rpb_s), lo};
+        }
+        tab[b] = e;
+    }
+}
+
+int launch_batch_flow(CgParams& P, const BatchFlow& f, int grid, unsigned id, int* seg_iters,
+                      double* seg_relres, StepBuffers& B, cudaStream_t s) {
+    FlowParams Q{};
+    Q.pub = reinterpret_cast<ulonglong2*>(B.pub);
+    Q.acc = B.bflow_words;
+    Q.id = id << 20;
+    Q.x_smem = f.x_smem;
+    Q.nbuf = f.nbuf;
+    P.L = f.L;
+    cudaMemsetAsync(B.bflow_words, 0, (size_t)B.nseg * kFlowWords * sizeof(unsigned long long), s);
+    const SegBlock* tab = reinterpret_cast<const SegBlock*>(B.segtab);
+    void* args[] = {&P, &Q, (void*)&tab, &seg_iters, &seg_relres};
+    const cudaError_t e = cudaLaunchCooperativeKernel(batch_flow_kernel(f.block), dim3(grid),
+                                                      dim3(f.block), args, f.smem, s);
+    return e == cudaSuccess ? SDC_OK : SDC_E_CUDA;
+}
+
 void launch_seg_bounds(const int* act, const int* count, StepBuffers& B, cudaStream_t s,
                        int* bounds_out) {
     k_seg_bounds<<<nblk(B.nseg + 1, 128), 128, 0, s>>>(count, act, B.nseg, B.inst_off,
@@ -2557,6 +2678,23 @@ int launch_pcg_batch(int n, const Ell& A, int m, double dt, const Coll& co, doub
                      int maxit, int sweep, const PcgConfig& cfg, const std::vector<int>& bounds,
                      StepBuffers& B, cudaStream_t s) {
     const int nseg = (int)bounds.size() - 1;
+    const BatchFlow& bf = batch_flow_shape(cfg, B);
+    if (bf.grid > 0 && maxit < kFlowMaxit) {
+        const int rpb = batch_flow_rows(bounds[nseg] - bounds[0], bf.grid, nseg, batch_flow_floor(cfg));
+        std::vector<SegBlock> tab;
+        for (int g = 0; g < nseg; ++g) {
+            const int nb = batch_flow_blocks(bounds[g + 1] - bounds[g], rpb), b0 = (int)tab.size();
+            for (int b = 0; b < nb; ++b) tab.push_back({bounds[g], bounds[g + 1], b0, nb, g});
+        }
+        if (tab.empty()) return SDC_OK;
+        if (cudaMemcpyAsync(B.segtab, tab.data(), tab.size() * sizeof(SegBlock),
+                            cudaMemcpyHostToDevice, s) != cudaSuccess)
+            return SDC_E_CUDA;
+        CgParams P = batch_params(n, A, m, dt, co, rtol, maxit, cfg, B);
+        return launch_batch_flow(P, bf, (int)tab.size(), next_flow_id(B, s),
+                                 B.seg_iters + (size_t)(sweep * kMaxM + m) * nseg,
+                                 B.seg_relres + (size_t)(sweep * kMaxM + m) * nseg, B, s);
+    }
     const int Gmax = cfg.max_blocks_batch;
     // blocks per instance: proportional to its active rows, at least one
     std::vector<int> want(nseg, 0);
@@ -2611,6 +2749,17 @@ int launch_pcg_batch_planned(const Ell& A, int m, double dt, const Coll& co, dou
     const int G = cfg.max_blocks_batch;
     if (nseg < 1 || nseg > G || G > B.segtab_cap) return SDC_E_INVALID;
     SegBlock* tab = reinterpret_cast<SegBlock*>(B.segtab);
+    const BatchFlow& bf = batch_flow_shape(cfg, B);
+    if (bf.grid > 0 && maxit < kFlowMaxit) {
+        if (plan)
+            k_batch_plan_flow<<<1, 256, 0, s>>>(nseg, bounds_dev, bf.grid, batch_flow_floor(cfg), tab,
+                                                B.plan);
+        CgParams P = batch_params(B.N, A, m, dt, co, rtol, maxit, cfg, B);
+        // (the step clears the published words, so its launches count from 1)
+        return launch_batch_flow(P, bf, bf.grid, (unsigned)(sweep * co.M + m + 1),
+                                 B.seg_iters + (size_t)(sweep * kMaxM + m) * nseg,
+                                 B.seg_relres + (size_t)(sweep * kMaxM + m) * nseg, B, s);
+    }
     if (plan)
         k_batch_plan<<<1, 256, 0, s>>>(nseg, bounds_dev, G, cfg.batch_rows_per_block, tab, B.plan,
                                        B.plan + nseg);
