@@ -71,13 +71,37 @@ __global__ void k_nodes_out_perm(int N, int M, const int* __restrict__ perm,
     for (int m = 0; m < M; ++m) out[(size_t)m * N + o] = X[(size_t)i * M + m];
 }
 
+// Constants of the Aliev-Panfilov model folded on the host.  The residual and update kernels
+// are bound by FP64 issue (M = 4 on the slab: 112 and 165 operations per row before, 92 and 107
+// now; 442k rows 119 and 155 us before), so nothing uniform is computed per thread and
+// comparisons are made on the bits.
+struct IonicFold {
+    double ga, a, gs, mu2;
+    double d2, d1, d0;        // dI/dv = v (d2 v + d1) + d0 + w
+    double a1;                // 1 + a
+    double cmu1, ceps;        // cw mu1, cw eps
+};
+inline IonicFold fold_ionic(const Ionic& p) {
+    return IonicFold{p.ga, p.a, p.gs, p.mu2, 3.0 * p.ga, -2.0 * p.ga * (1.0 + p.a), p.ga * p.a,
+                     1.0 + p.a, p.cw * p.mu1, p.cw * p.eps};
+}
+// Q and Qhat times dt
+inline Coll fold_dt(const Coll& co, double dt) {
+    Coll c = co;
+    for (int k = 0; k < kMaxM * kMaxM; ++k) {
+        c.Q[k] = dt * co.Q[k];
+        c.Qh[k] = dt * co.Qh[k];
+    }
+    return c;
+}
+
 template <int M>
 __global__ void k_residual(int n, const int* __restrict__ act, const double* __restrict__ kval,
                            const int* __restrict__ kcol, const int* __restrict__ klen, int ldk,
                            const double* __restrict__ kdiag, const double* __restrict__ mass,
                            const double* __restrict__ stim, double stim_on,
                            const double* __restrict__ V, const double* __restrict__ W,
-                           const double* __restrict__ v0, double dt, Ionic ion, Coll co,
+                           const double* __restrict__ v0, IonicFold ion, Coll co,
                            int reaction_implicit, int ld, double* __restrict__ R,
                            double* __restrict__ Jout, double* __restrict__ mc,
                            double* __restrict__ kdc, const int* __restrict__ n_dev, int N) {
@@ -105,16 +129,20 @@ __global__ void k_residual(int n, const int* __restrict__ act, const double* __r
 #pragma unroll
     for (int m = 0; m < M; ++m) {
         const double wm = W[(size_t)g * M + m];
-        f[m] = -kv[m] - mi * (ap_I(ion, vm[m], wm) - s);
-        Jout[(size_t)m * ld + p] = reaction_implicit ? ap_dIdv(ion, vm[m], wm) : 0.0;
+        const double v = vm[m];
+        // I - s = v (ga (v - a) (v - 1) + w) - s
+        const double I = fma(v, fma(ion.ga * (v - ion.a), v - 1.0, wm), -s);
+        f[m] = fma(-mi, I, -kv[m]);
+        Jout[(size_t)m * ld + p] =
+            reaction_implicit ? fma(v, fma(ion.d2, v, ion.d1), ion.d0 + wm) : 0.0;
     }
-    const double base = mi * v0[g];
+    const double vz = v0[g];
 #pragma unroll
     for (int m = 0; m < M; ++m) {
-        double q = 0.0;
+        double q = mi * (vz - vm[m]);
 #pragma unroll
-        for (int j = 0; j < M; ++j) q += co.Q[m * kMaxM + j] * f[j];
-        R[(size_t)m * ld + p] = base + dt * q - mi * vm[m];
+        for (int j = 0; j < M; ++j) q += co.Q[m * kMaxM + j] * f[j];   // (dt Q)
+        R[(size_t)m * ld + p] = q;
     }
     mc[p] = mi;
     kdc[p] = kd;
@@ -1698,7 +1726,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcgc_smem(CgParams P) {
 template <int M>
 __global__ void k_update(int n, const int* __restrict__ act, const double* __restrict__ D, int ld,
                          double* __restrict__ V, double* __restrict__ W,
-                         const double* __restrict__ w0, double dt, Ionic ion, Coll co,
+                         const double* __restrict__ w0, IonicFold ion, Coll co,
                          double tol_drop, int w_frozen, int* __restrict__ flag,
                          int* __restrict__ blockcnt, double* __restrict__ blockmarg,
                          int* __restrict__ err, const double* __restrict__ tol_drop_dev,
@@ -1713,14 +1741,16 @@ __global__ void k_update(int n, const int* __restrict__ act, const double* __res
     if (p < n) {
         const int g = act ? sdc_idx(act[p], N, 61) : p;
         double vm[M];
-        double amax = 0.0;
+        long long abits = 0;   // max |d| on the bits, NaN left out (fmax)
 #pragma unroll
         for (int m = 0; m < M; ++m) {
             const double d = D[(size_t)m * ld + p];
             vm[m] = V[(size_t)g * M + m] + d;
             V[(size_t)g * M + m] = vm[m];
-            amax = fmax(amax, fabs(d));
+            const long long b = __double_as_longlong(d) & 0x7fffffffffffffffll;
+            if (b > abits && b <= 0x7ff0000000000000ll) abits = b;
         }
+        const double amax = __longlong_as_double(abits);
         if (!w_frozen) {
             // two divisions per row instead of 2 M (FP64 division is a long sequence on this
             // part): the M reciprocals 1 / (v + mu2), then the M reciprocals of the denominators
@@ -1730,36 +1760,41 @@ __global__ void k_update(int n, const int* __restrict__ act, const double* __res
             for (int m = 0; m < M; ++m) {
                 wm[m] = W[(size_t)g * M + m];
                 xs[m] = vm[m] + ion.mu2;
-                if (!(xs[m] > 0.0)) raise_error(err, SDC_E_DOMAIN);
+                if (!positive(xs[m])) raise_error(err, SDC_E_DOMAIN);
             }
             batch_reciprocal<M>(xs, inv);
 #pragma unroll
             for (int m = 0; m < M; ++m) {
-                ap_R_dRdw_inv(ion, vm[m], wm[m], inv[m], gR[m], dR[m]);
-                xs[m] = 1.0 - dt * co.Qh[m * kMaxM + m] * dR[m];
-                if (!(xs[m] > 0.0)) raise_error(err, SDC_E_DOMAIN);
+                // R = cw (eps + mu1 w / (v + mu2)) (-w - gs v (v - a - 1)) and dR/dw
+                const double v = vm[m];
+                const double E = fma(ion.cmu1 * wm[m], inv[m], ion.ceps);
+                const double G = fma(-ion.gs * v, v - ion.a1, -wm[m]);
+                gR[m] = E * G;
+                dR[m] = fma(ion.cmu1 * inv[m], G, -E);
+                xs[m] = fma(-co.Qh[m * kMaxM + m], dR[m], 1.0);   // (dt Qhat)
+                if (!positive(xs[m])) raise_error(err, SDC_E_DOMAIN);
             }
             batch_reciprocal<M>(xs, inv);
 #pragma unroll
             for (int m = 0; m < M; ++m) {
-                double q = 0.0;
+                double acc = wz - wm[m];
 #pragma unroll
-                for (int j = 0; j < M; ++j) q += co.Q[m * kMaxM + j] * gR[j];
-                double acc = wz + dt * q - wm[m];
+                for (int j = 0; j < M; ++j) acc += co.Q[m * kMaxM + j] * gR[j];
 #pragma unroll
-                for (int j = 0; j < m; ++j) acc += dt * co.Qh[m * kMaxM + j] * dR[j] * e[j];
-                e[m] = acc * inv[m];
+                for (int j = 0; j < m; ++j) acc += co.Qh[m * kMaxM + j] * e[j];
+                const double em = acc * inv[m];
+                W[(size_t)g * M + m] = wm[m] + em;
+                e[m] = dR[m] * em;
             }
-#pragma unroll
-            for (int m = 0; m < M; ++m) W[(size_t)g * M + m] = wm[m] + e[m];
         }
-        if (!isfinite(amax)) raise_error(err, SDC_E_NONFINITE);
-        keep = amax >= tol_drop ? 1 : 0;
+        if (abits == 0x7ff0000000000000ll) raise_error(err, SDC_E_NONFINITE);
+        // amax >= tol_drop (both >= 0, tol_drop not NaN)
+        keep = abits >= __double_as_longlong(tol_drop) ? 1 : 0;
         if (tol_drop > 0.0) margin = fabs(amax - tol_drop);
         flag[p] = keep;
     }
     const unsigned bal = __ballot_sync(0xffffffffu, keep);
-    margin = warp_min(margin);
+    margin = warp_min_positive(margin);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     if (lane == 0) {
         wc[wid] = __popc(bal);
@@ -1771,7 +1806,7 @@ __global__ void k_update(int n, const int* __restrict__ act, const double* __res
         double mg = lane < nw ? wmg[lane] : DBL_MAX;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-        mg = warp_min(mg);
+        mg = warp_min_positive(mg);
         if (lane == 0) {
             blockcnt[blockIdx.x] = c;
             blockmarg[blockIdx.x] = mg;
@@ -1930,7 +1965,8 @@ void launch_residual(int M, int n, const int* act, const Ell& K, const double* k
     dispatch_M(M, [&](auto mc) {
         constexpr int MM = decltype(mc)::value;
         k_residual<MM><<<nblk(n, 128), 128, 0, s>>>(n, act, K.val, K.col, K.len, K.ld, kdiag, mass,
-                                                      stim, stim_on, V, W, v0, dt, ion, co,
+                                                      stim, stim_on, V, W, v0, fold_ionic(ion),
+                                                      fold_dt(co, dt),
                                                       reaction_implicit, B.ld, B.R, B.J, B.mc, B.kdc,
                                                       n_dev, B.N);
     });
@@ -2898,7 +2934,8 @@ void launch_update(int M, int n, const int* act, const double* w0, double dt, co
     dispatch_M(M, [&](auto mc) {
         constexpr int MM = decltype(mc)::value;
         k_update<MM><<<nblk(n, kUpdateBlock), kUpdateBlock, 0, s>>>(
-            n, act, B.D, B.ld, B.V, B.W, w0, dt, ion, co, tol_drop, w_frozen, B.flag, B.blockcnt,
+            n, act, B.D, B.ld, B.V, B.W, w0, fold_ionic(ion), fold_dt(co, dt), tol_drop, w_frozen,
+            B.flag, B.blockcnt,
             B.blockmarg, &B.sc->err, tol_drop_dev, n_dev, B.N);
     });
 }
