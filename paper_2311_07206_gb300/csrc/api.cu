@@ -207,10 +207,11 @@ int alloc_buffers(sdc_ctx* c) {
         B.sval_width = c->K.K.width;
         ulonglong2* pub = nullptr;
         ok = dalloc(&B.sv, ld) && dalloc(&B.sval, (size_t)std::max(B.sval_width, 1) * ld) &&
-             dalloc(&B.flow, kFlowWords) && dalloc(&pub, 2 * ld);
+             dalloc(&B.flow, 2 * kFlowWords) && dalloc(&pub, 2 * ld);
         B.pub = pub;
         // tags of no launch
         if (ok) cudaMemsetAsync(B.pub, 0, 2 * ld * sizeof(ulonglong2), c->stream);
+        if (ok) cudaMemsetAsync(B.flow, 0, 2 * kFlowWords * sizeof(*B.flow), c->stream);
     }
     if (!ok) return SDC_E_NOMEM;
     // pinned: [0] count, [1] err, then kMaxM node energies at byte 16

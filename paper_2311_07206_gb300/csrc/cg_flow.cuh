@@ -468,6 +468,8 @@ __device__ __forceinline__ bool flow_start(const CgParams& P, const FlowParams& 
         S.ovf = 0;
         S.next = 0;
     }
+    if (Q.zero && Q.bidx == 0)
+        for (int k = t; k < kFlowWords; k += blockDim.x) Q.zero[k] = 0;
     flow_rows(nl, [&](int l) {
         const int i = r0 + l;
         const double d = P.mc[i] * (1.0 + c * P.J[i]) + c * P.kdc[i];
@@ -924,6 +926,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc2_flow(CgParams P, FlowParams Q,
         S.ok = 1;
         S.ovf = 0;
     }
+    if (Q.zero && blockIdx.x == 0)
+        for (int k = t; k < kFlowWords; k += B) Q.zero[k] = 0;
     for (int m = t; m < C.qn; m += B) {
         const int a = sdc_idx(C.nzb[m], C.q, 73);
         snz[m] = a;

@@ -136,7 +136,8 @@ struct StepBuffers {
     double* sval = nullptr;   // [sval_width][ld] scaled off-diagonal values of the scaled solve
     int sval_width = 0;
     void* pub = nullptr;      // [2][ld] 16-byte words of the flow kernels: published value, tag
-    unsigned long long* flow = nullptr;   // [kFlowWords] their sums and barrier, zeroed per launch
+    unsigned long long* flow = nullptr;   // [2][kFlowWords] their sums and barrier, two sets in turn
+    int flow_set = 0;         // the next launch's set (zero)
     unsigned flow_id = 0;     // launches since the words were cleared (tags), and how often
     unsigned flow_wraps = 0;
     int max_blocks = 0;

@@ -220,6 +220,9 @@ struct FlowParams {
     unsigned long long* acc;    // two sets of eight words of the running sums
     unsigned long long* emax;   // largest exponents of gamma's and delta's partial sums
     unsigned* bar;              // arrivals of the barriers outside the iteration
+    unsigned long long* zero;   // the next launch's words, cleared by this one (or null): the
+                                // launches of a stream alternate between two sets, which spares
+                                // a memset per solve
     unsigned id;                // launch id << 20: tags of different launches differ
     int x_smem;                 // x in shared memory (else in P.x)
     int nbuf;                   // classical: buffers shared by r and w (2 or 3)
@@ -2206,9 +2209,10 @@ int launch_pcg_coarse(int n, const Ell& A, const PcgRole& role, double rtol, int
         pcg_smem_attrs();
         FlowParams Q{};
         Q.pub = reinterpret_cast<ulonglong2*>(B.pub);
-        Q.acc = B.flow;
-        Q.emax = B.flow + 16;
-        Q.bar = reinterpret_cast<unsigned*>(B.flow + 32);
+        Q.acc = B.flow + (size_t)B.flow_set * kFlowWords;
+        Q.emax = Q.acc + 16;
+        Q.bar = reinterpret_cast<unsigned*>(Q.acc + 32);
+        Q.zero = B.flow + (size_t)(B.flow_set ^ 1) * kFlowWords;
         Q.id = next_flow_id(B, s) << 20;
         if (C.wraps != B.flow_wraps) {
             cudaMemsetAsync(C.words, 0, (size_t)2 * C.pstride * 16, s);
@@ -2234,14 +2238,14 @@ int launch_pcg_coarse(int n, const Ell& A, const PcgRole& role, double rtol, int
         F.Einv = C.Einv;
         F.words = reinterpret_cast<ulonglong2*>(C.words);
         F.pstride = C.pstride;
-        cudaMemsetAsync(B.flow, 0, kFlowWords * sizeof(unsigned long long), s);
         void* fa[] = {&P, &Q, &F};
         const void* k = C.block > 768   ? (const void*)k_cgc2_flow<1024>
                         : C.block > 512 ? (const void*)k_cgc2_flow<768>
                                         : (const void*)k_cgc2_flow<512>;
-        return cudaLaunchCooperativeKernel(k, dim3(C.G), dim3(C.block), fa, C.smem, s) == cudaSuccess
-                   ? SDC_OK
-                   : SDC_E_CUDA;
+        if (cudaLaunchCooperativeKernel(k, dim3(C.G), dim3(C.block), fa, C.smem, s) != cudaSuccess)
+            return SDC_E_CUDA;
+        B.flow_set ^= 1;
+        return SDC_OK;
     }
     cudaMemsetAsync(&B.sc->bar, 0, sizeof(unsigned), s);
     CoarseParams CP;
@@ -2355,11 +2359,13 @@ bool flow_values_on_chip(int width, FlowShape& f) {
     return true;
 }
 
-// words: kFlowWords words, zero; pub: tags of other launches only
+// words: kFlowWords words, zero; zero: the next launch's, to be cleared (or null); pub: tags
+// of other launches only
 int launch_flow(CgParams& P, bool classical, const FlowShape& f, void* pub,
-                unsigned long long* words, unsigned id, cudaStream_t s) {
+                unsigned long long* words, unsigned long long* zero, unsigned id, cudaStream_t s) {
     pcg_smem_attrs();
-    FlowParams Q;
+    FlowParams Q{};
+    Q.zero = zero;
     Q.pub = reinterpret_cast<ulonglong2*>(pub);
     Q.acc = words;
     Q.emax = words + 16;
@@ -2386,8 +2392,11 @@ int launch_pcg_params(CgParams& P, const PcgConfig& cfg, StepBuffers& B, cudaStr
         !cfg.pipelined || (cfg.general_classical && n > kFlowClassicalRows);
     if (cfg.variant != 1 && cfg.scaled && P.sv && P.sval && B.pub && P.maxit < kFlowMaxit &&
         flow_shape(n, flow_classical, cfg, fs)) {
-        cudaMemsetAsync(B.flow, 0, kFlowWords * sizeof(unsigned long long), s);
-        return launch_flow(P, flow_classical, fs, B.pub, B.flow, next_flow_id(B, s), s);
+        unsigned long long* words = B.flow + (size_t)B.flow_set * kFlowWords;
+        unsigned long long* other = B.flow + (size_t)(B.flow_set ^ 1) * kFlowWords;
+        const int rc = launch_flow(P, flow_classical, fs, B.pub, words, other, next_flow_id(B, s), s);
+        if (rc == SDC_OK) B.flow_set ^= 1;
+        return rc;
     }
     cudaMemsetAsync(&B.sc->bar, 0, sizeof(unsigned), s);
     void* args[] = {&P};
@@ -2870,7 +2879,8 @@ int launch_pcg_standalone_flow(int n, const Ell& A, const double* kdiag, const d
     P.maxit = maxit;
     P.budget = budget;
     P.M = 1;            // no coupling into other nodes
-    return launch_flow(P, classical, f, ws + z, reinterpret_cast<unsigned long long*>(words), 1, s);
+    return launch_flow(P, classical, f, ws + z, reinterpret_cast<unsigned long long*>(words), nullptr,
+                       1, s);
 }
 
 int launch_pcg_standalone(int n, const Ell& A, const double* kdiag, const double* mass,
