@@ -32,47 +32,25 @@ constexpr int kAdjBlock = 256;
 
 inline int nb(int n, int b) { return (n + b - 1) / b; }
 
-// Aliev-Panfilov derivatives needed by the adjoint.  p = (ga, gs, a).
-struct ApDer {
-    double I, Iv, Iw, Ivv, Ivw, I_ga, I_a, Iv_ga, Iv_a;
-    double R, Rv, Rw, Rwv, Rww, R_gs, R_a, Rw_gs, Rw_a;
+// Every kernel below is bound by the FP64 pipe (two operations per cycle and SM) or by its
+// launch, not by memory: products of constants are folded on the host (dt into Q and Qhat),
+// divisions are the three-operation reciprocal, and what several kernels used is computed once.
+struct AdjIonic {
+    double ga, gs, a, mu2;
+    double ga3, gaq, ga6, a1;   // 3 ga, -2 ga (1 + a), 6 ga, 1 + a
+    double cmu1, ceps;          // cw mu1, cw eps
 };
 
-__device__ __forceinline__ ApDer ap_der(const Ionic& p, double v, double w) {
-    ApDer d;
-    const double vm1 = v - 1.0, vma = v - p.a;
-    d.I = p.ga * v * vma * vm1 + v * w;
-    d.Iv = p.ga * (3.0 * v * v - 2.0 * (1.0 + p.a) * v + p.a) + w;
-    d.Iw = v;
-    d.Ivv = p.ga * (6.0 * v - 2.0 * (1.0 + p.a));
-    d.Ivw = 1.0;
-    d.I_ga = v * vma * vm1;
-    d.I_a = -p.ga * v * vm1;
-    d.Iv_ga = 3.0 * v * v - 2.0 * (1.0 + p.a) * v + p.a;
-    d.Iv_a = p.ga * (1.0 - 2.0 * v);
-    const double inv = 1.0 / (v + p.mu2);
-    const double E = p.eps + p.mu1 * w * inv;
-    const double Ew = p.mu1 * inv;
-    const double Ev = -p.mu1 * w * inv * inv;
-    const double Ewv = -p.mu1 * inv * inv;
-    const double G = -w - p.gs * v * (v - p.a - 1.0);
-    const double Gv = -p.gs * (2.0 * v - p.a - 1.0);
-    const double G_gs = -v * (v - p.a - 1.0);
-    const double G_a = p.gs * v;
-    d.R = p.cw * E * G;
-    d.Rv = p.cw * (Ev * G + E * Gv);
-    d.Rw = p.cw * (Ew * G - E);
-    d.Rwv = p.cw * (Ewv * G + Ew * Gv - Ev);
-    d.Rww = -2.0 * p.cw * Ew;
-    d.R_gs = p.cw * E * G_gs;
-    d.R_a = p.cw * E * G_a;
-    d.Rw_gs = p.cw * Ew * G_gs;
-    d.Rw_a = p.cw * Ew * G_a;
-    return d;
+inline AdjIonic fold_adjoint(const Ionic& p) {
+    return AdjIonic{p.ga,       p.gs,           p.a,          p.mu2,         3.0 * p.ga,
+                    -2.0 * p.ga * (1.0 + p.a), 6.0 * p.ga, 1.0 + p.a, p.cw * p.mu1,
+                    p.cw * p.eps};
 }
 
-// per-block partial sums of the three ionic-parameter gradients
-__device__ __forceinline__ void block_sum3(double a, double b, double c, double* out3) {
+// Sums of (a, b, c) over the block, added to the block's own three partials: the launches of
+// one adjoint follow one another, so a block's partials have one writer at a time and one
+// final sum in a fixed order is enough.
+__device__ __forceinline__ void block_add3(double a, double b, double c, double* part) {
     __shared__ double sh[3][32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     a = warp_sum(a);
@@ -84,33 +62,22 @@ __device__ __forceinline__ void block_sum3(double a, double b, double c, double*
         sh[2][wid] = c;
     }
     __syncthreads();
-    if (wid == 0) {
-        double x = lane < nw ? sh[0][lane] : 0.0;
-        double y = lane < nw ? sh[1][lane] : 0.0;
-        double z = lane < nw ? sh[2][lane] : 0.0;
-        x = warp_sum(x);
-        y = warp_sum(y);
-        z = warp_sum(z);
-        if (lane == 0) {
-            out3[3 * blockIdx.x + 0] = x;
-            out3[3 * blockIdx.x + 1] = y;
-            out3[3 * blockIdx.x + 2] = z;
-        }
+    if (wid < 3) {
+        const double x = warp_sum(lane < nw ? sh[wid][lane] : 0.0);
+        if (lane == 0) part[3 * blockIdx.x + wid] += x;
     }
 }
 
-// fixed-order sum of nblk block partials into the running accumulator acc[3]
-__global__ void k_sum3(int nblk, const double* __restrict__ part, double* __restrict__ acc) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// The blocks' partials in a fixed order: 256 strided sums, then the tree of block_add3
+// (acc zeroed before).
+__global__ void k_sum3(int nblk, const double* __restrict__ part, double* acc) {
     double a = 0.0, b = 0.0, c = 0.0;
-    for (int i = 0; i < nblk; ++i) {
+    for (int i = threadIdx.x; i < nblk; i += blockDim.x) {
         a += part[3 * i];
         b += part[3 * i + 1];
         c += part[3 * i + 2];
     }
-    acc[0] += a;
-    acc[1] += b;
-    acc[2] += c;
+    block_add3(a, b, c, acc);
 }
 
 __global__ void k_adj_init(int N, int M, const double* __restrict__ lv,
@@ -127,221 +94,285 @@ __global__ void k_adj_init(int N, int M, const double* __restrict__ lv,
     lw0[i] = 0.0;
 }
 
-// Reverse of the pointwise w sweep on the active rows.  Vn: v after the sweep,
-// Wo / Wn: w before / after; Wb is replaced by the adjoint of w before the
-// sweep, Vb (adjoint of v after the sweep) and lw0 accumulate.
-template <int M>
-__global__ void k_adj_wsweep(int n, const int* __restrict__ act, const double* __restrict__ Vn,
-                             const double* __restrict__ Wo, const double* __restrict__ Wn,
-                             double dt, Ionic ion, Coll co, double* __restrict__ Vb,
-                             double* __restrict__ Wb, double* __restrict__ lw0,
-                             double* __restrict__ part3, int N) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    double gga = 0.0, ggs = 0.0, ga_ = 0.0;
-    if (p < n) {
-        const int g = act ? sdc_idx(act[p], N, 201) : p;
-        ApDer d[M];
-        double eps[M], den[M], eb[M], Nb[M], sb[M], gb[M], db[M];
-#pragma unroll
-        for (int m = 0; m < M; ++m) {
-            d[m] = ap_der(ion, Vn[(size_t)g * M + m], Wo[(size_t)g * M + m]);
-            eps[m] = Wn[(size_t)g * M + m] - Wo[(size_t)g * M + m];
-            den[m] = 1.0 - dt * co.Qh[m * kMaxM + m] * d[m].Rw;
-            eb[m] = Wb[(size_t)g * M + m];     // adjoint of W' = W + eps
-            gb[m] = 0.0;
-            db[m] = 0.0;
-        }
-        // eps_m = N_m / den_m,  N_m = s_m + dt sum_{j<m} Qh_mj d_j eps_j
-#pragma unroll
-        for (int m = M - 1; m >= 0; --m) {
-            Nb[m] = eb[m] / den[m];
-            const double denb = -eb[m] * eps[m] / den[m];
-            db[m] += denb * (-dt * co.Qh[m * kMaxM + m]);
-            sb[m] = Nb[m];
-#pragma unroll
-            for (int j = 0; j < m; ++j) {
-                db[j] += Nb[m] * dt * co.Qh[m * kMaxM + j] * eps[j];
-                eb[j] += Nb[m] * dt * co.Qh[m * kMaxM + j] * d[j].Rw;
-            }
-        }
-        // s_m = w0 + dt sum_j Q_mj g_j - W_m
-        double w0b = 0.0;
-#pragma unroll
-        for (int m = 0; m < M; ++m) {
-            w0b += sb[m];
-#pragma unroll
-            for (int j = 0; j < M; ++j) gb[j] += dt * co.Q[m * kMaxM + j] * sb[m];
-        }
-        lw0[g] += w0b;
-#pragma unroll
-        for (int m = 0; m < M; ++m) {
-            // W' = W + eps: adjoint of W is eb (direct) - sb (via s) + chain through g, d
-            const double wb = Wb[(size_t)g * M + m] - sb[m] + gb[m] * d[m].Rw + db[m] * d[m].Rww;
-            Wb[(size_t)g * M + m] = wb;
-            Vb[(size_t)g * M + m] += gb[m] * d[m].Rv + db[m] * d[m].Rwv;
-            ggs += gb[m] * d[m].R_gs + db[m] * d[m].Rw_gs;
-            ga_ += gb[m] * d[m].R_a + db[m] * d[m].Rw_a;
-        }
-    }
-    block_sum3(gga, ggs, ga_, part3);
-}
-
-// Per-sweep quantities of the active rows (compact): J, dv, mass, K_ii, and the
-// adjoint of dv gathered from Vb.
+// Before the reverse solves of a sweep, on its active rows: the reverse of the pointwise w
+// sweep (unless w is frozen), then the compact right-hand sides (Vb), J, mass and K_ii of the
+// node solves.  Vo, Wo: state before the sweep, Vn, Wn: after it; Wb is replaced by the adjoint
+// of w before the sweep, Vb (adjoint of v after the sweep) and lw0 accumulate.
+//   eps_m = N_m / den_m,  N_m = s_m + dt sum_{j<m} Qh_mj R_w,j eps_j,
+//   den_m = 1 - dt Qh_mm R_w,m,  s_m = w0 + dt sum_j Q_mj R_j - W_m,  R = cw E G
 template <int M>
 __global__ void k_adj_prep(int n, const int* __restrict__ act, const double* __restrict__ Vo,
                            const double* __restrict__ Wo, const double* __restrict__ Vn,
-                           const double* __restrict__ kdiag, const double* __restrict__ mass,
-                           const double* __restrict__ Vb, Ionic ion, int reaction_implicit,
-                           int ld, double* __restrict__ J, double* __restrict__ D,
+                           const double* __restrict__ Wn, const double* __restrict__ kdiag,
+                           const double* __restrict__ mass, AdjIonic ion, Coll co, int w_frozen,
+                           int reaction_implicit, int ld, double* __restrict__ Vb,
+                           double* __restrict__ Wb, double* __restrict__ lw0,
+                           double* __restrict__ part3, double* __restrict__ J,
                            double* __restrict__ mc, double* __restrict__ kdc,
-                           double* __restrict__ Db, double* __restrict__ Jb, int N) {
+                           double* __restrict__ Db, int N) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const int g = act ? sdc_idx(act[p], N, 202) : p;
+    double ggs = 0.0, ga_ = 0.0;
+    if (p < n) {
+        const int g = act ? sdc_idx(act[p], N, 201) : p;
+        double wo[M], vb[M];
 #pragma unroll
-    for (int m = 0; m < M; ++m) {
-        const double v = Vo[(size_t)g * M + m], w = Wo[(size_t)g * M + m];
-        J[(size_t)m * ld + p] = reaction_implicit ? ap_dIdv(ion, v, w) : 0.0;
-        D[(size_t)m * ld + p] = Vn[(size_t)g * M + m] - v;
-        Db[(size_t)m * ld + p] = Vb[(size_t)g * M + m];
-        Jb[(size_t)m * ld + p] = 0.0;
+        for (int m = 0; m < M; ++m) {
+            wo[m] = Wo[(size_t)g * M + m];
+            vb[m] = Vb[(size_t)g * M + m];
+        }
+        if (!w_frozen) {
+            double E[M], u[M], Rv[M], Rw[M], Rwv[M], eps[M], eb[M], sb[M], gb[M], db[M], wb0[M];
+#pragma unroll
+            for (int m = 0; m < M; ++m) {
+                const double v = Vn[(size_t)g * M + m], w = wo[m];
+                const double inv = recip(v + ion.mu2);
+                u[m] = ion.cmu1 * inv;                       // cw dE/dw
+                E[m] = fma(u[m], w, ion.ceps);               // cw E
+                const double ui = u[m] * inv;                // - cw d2E/dwdv
+                const double Ev = -ui * w;
+                const double x = v - ion.a1;
+                const double G = fma(-ion.gs * v, x, -w);
+                const double Gv = -ion.gs * (x + v);
+                Rv[m] = fma(Ev, G, E[m] * Gv);
+                Rw[m] = fma(u[m], G, -E[m]);
+                Rwv[m] = fma(-ui, G, fma(u[m], Gv, -Ev));
+                eps[m] = Wn[(size_t)g * M + m] - w;
+                wb0[m] = Wb[(size_t)g * M + m];              // adjoint of W' = W + eps
+                eb[m] = wb0[m];
+                gb[m] = 0.0;
+                db[m] = 0.0;
+            }
+#pragma unroll
+            for (int m = M - 1; m >= 0; --m) {
+                const double q = co.Qh[m * kMaxM + m];
+                sb[m] = eb[m] * recip(fma(-q, Rw[m], 1.0));   // N_m's and s_m's adjoint
+                db[m] = fma(sb[m] * eps[m], q, db[m]);
+#pragma unroll
+                for (int j = 0; j < m; ++j) {
+                    const double sq = sb[m] * co.Qh[m * kMaxM + j];
+                    db[j] = fma(sq, eps[j], db[j]);
+                    eb[j] = fma(sq, Rw[j], eb[j]);
+                }
+            }
+            double w0b = 0.0;
+#pragma unroll
+            for (int m = 0; m < M; ++m) {
+                w0b += sb[m];
+#pragma unroll
+                for (int j = 0; j < M; ++j) gb[j] = fma(co.Q[m * kMaxM + j], sb[m], gb[j]);
+            }
+            lw0[g] += w0b;
+#pragma unroll
+            for (int m = 0; m < M; ++m) {
+                // W' = W + eps: direct, - sb (via s), and the chain through R and R_w
+                const double v = Vn[(size_t)g * M + m];
+                Wb[(size_t)g * M + m] =
+                    fma(db[m], -2.0 * u[m], fma(gb[m], Rw[m], wb0[m] - sb[m]));
+                vb[m] = fma(db[m], Rwv[m], fma(gb[m], Rv[m], vb[m]));
+                Vb[(size_t)g * M + m] = vb[m];
+                // dR/dgs = -cw E v (v - a - 1), dR/da = cw E gs v; the same with dE/dw for R_w
+                const double t = v * fma(db[m], u[m], gb[m] * E[m]);
+                ggs = fma(ion.a1 - v, t, ggs);
+                ga_ += t;
+            }
+        }
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+            const double v = Vo[(size_t)g * M + m];
+            J[(size_t)m * ld + p] =
+                reaction_implicit
+                    ? fma(v, fma(ion.ga3, v, ion.gaq), fma(ion.ga, ion.a, wo[m])) : 0.0;
+            Db[(size_t)m * ld + p] = vb[m];
+        }
+        mc[p] = mass[g];
+        kdc[p] = kdiag[g];
     }
-    mc[p] = mass[g];
-    kdc[p] = kdiag[g];
+    if (!w_frozen) block_add3(0.0, ggs, ion.gs * ga_, part3);
 }
 
-// After the reverse solve of node m (x = bbar_m): adjoint of J through A_m and
-// through the couplings b_m uses for j < m; the conductivity pairs; and the
-// full-length copy of bbar_m.
+// After the reverse solves (X_m = bbar_m = rbar_m), on the active rows: the reverse of the
+// residual and the adjoint of J, which reaches A_m and the couplings of every node m >= j:
+//   Jbar_j = - mass D_j sum_{m>=j} dt Qh_mj bbar_m,  D = V' - V
+// (one expression over the M solutions: as one pass after each of the M solves it cost four
+// microseconds and two launch gaps a node).  Full-length copies of bbar and fbar, node-major.
 template <int M>
-__global__ void k_adj_node_post(int n, const int* __restrict__ act, int m, double dt, Coll co,
-                                int ld, int N, const double* __restrict__ x,
-                                const double* __restrict__ D, const double* __restrict__ mc,
-                                double* __restrict__ Jb, double* __restrict__ bfull,
-                                double* __restrict__ vkfull) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const int g = act ? sdc_idx(act[p], N, 203) : p;
-    const double xb = x[p];
-    const double cm = dt * co.Qh[m * kMaxM + m];
-    const double dm = D[(size_t)m * ld + p];
-    Jb[(size_t)m * ld + p] += -mc[p] * cm * xb * dm;
-    double vk = -cm * dm;
-    for (int j = 0; j < m; ++j) {
-        const double dj = D[(size_t)j * ld + p];
-        Jb[(size_t)j * ld + p] += -dt * co.Qh[m * kMaxM + j] * mc[p] * dj * xb;
-        vk += -dt * co.Qh[m * kMaxM + j] * dj;
-    }
-    bfull[(size_t)m * N + g] = xb;
-    vkfull[(size_t)m * N + g] = vk;
-}
-
-// Reverse of the residual on the active rows: rbar_m = bbar_m.
-template <int M>
-__global__ void k_adj_residual(int n, const int* __restrict__ act, int ld, int N, double dt,
-                               Coll co, Ionic ion, int reaction_implicit,
-                               const double* __restrict__ X, const double* __restrict__ Jb,
-                               const double* __restrict__ Vo, const double* __restrict__ Wo,
+__global__ void k_adj_residual(int n, const int* __restrict__ act, int ld, int N, Coll co,
+                               AdjIonic ion, int reaction_implicit,
+                               const double* __restrict__ X, const double* __restrict__ Vo,
+                               const double* __restrict__ Wo, const double* __restrict__ Vn,
                                const double* __restrict__ mass, double* __restrict__ Vb,
                                double* __restrict__ Wb, double* __restrict__ lv0,
-                               double* __restrict__ ffull, double* __restrict__ part3) {
+                               double* __restrict__ bfull, double* __restrict__ ffull,
+                               double* __restrict__ part3) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    double gga = 0.0, ggs = 0.0, ga_ = 0.0;
+    double gga = 0.0, ga_ = 0.0;
     if (p < n) {
         const int g = act ? sdc_idx(act[p], N, 204) : p;
         const double mi = mass[g];
-        double rb[M], fb[M];
+        double rb[M], fb[M], jb[M];
         double rsum = 0.0;
 #pragma unroll
         for (int m = 0; m < M; ++m) {
             rb[m] = X[(size_t)m * ld + p];
+            bfull[(size_t)g * M + m] = rb[m];
             rsum += rb[m];
             fb[m] = 0.0;
+            jb[m] = 0.0;
         }
-        lv0[g] += mi * rsum;
+        lv0[g] = fma(mi, rsum, lv0[g]);
 #pragma unroll
-        for (int m = 0; m < M; ++m)
+        for (int m = 0; m < M; ++m) {
 #pragma unroll
-            for (int j = 0; j < M; ++j) fb[j] += dt * co.Q[m * kMaxM + j] * rb[m];
+            for (int j = 0; j < M; ++j) fb[j] = fma(co.Q[m * kMaxM + j], rb[m], fb[j]);
+            if (reaction_implicit) {
+#pragma unroll
+                for (int j = 0; j <= m; ++j) jb[j] = fma(-co.Qh[m * kMaxM + j], rb[m], jb[j]);
+            }
+        }
 #pragma unroll
         for (int j = 0; j < M; ++j) {
-            const ApDer d = ap_der(ion, Vo[(size_t)g * M + j], Wo[(size_t)g * M + j]);
-            const double jb = reaction_implicit ? Jb[(size_t)j * ld + p] : 0.0;
-            // r_j = ... - mass V_j ;  f_j = -K V_j - mass (I - stim) ;  J_j = dI/dv
-            Vb[(size_t)g * M + j] += -mi * rb[j] - mi * d.Iv * fb[j] + jb * d.Ivv;
-            Wb[(size_t)g * M + j] += -mi * d.Iw * fb[j] + jb * d.Ivw;
-            gga += -mi * d.I_ga * fb[j] + jb * d.Iv_ga;
-            ga_ += -mi * d.I_a * fb[j] + jb * d.Iv_a;
-            ffull[(size_t)j * N + g] = fb[j];
+            const double v = Vo[(size_t)g * M + j], w = Wo[(size_t)g * M + j];
+            if (reaction_implicit) jb[j] *= Vn[(size_t)g * M + j] - v;
+            // I = ga v (v - a)(v - 1) + v w; r_j = ... - mass V_j,
+            // f_j = -K V_j - mass (I - stim), J_j = dI/dv
+            const double vv = v * (v - 1.0);
+            const double c1 = fma(3.0, v, -2.0 * ion.a1);
+            const double Iv_ga = fma(v, c1, ion.a);
+            const double Iv = fma(ion.ga, Iv_ga, w);
+            const double Ivv = fma(ion.ga6, v, ion.gaq);
+            Vb[(size_t)g * M + j] =
+                fma(mi, fma(jb[j], Ivv, -fma(Iv, fb[j], rb[j])), Vb[(size_t)g * M + j]);
+            Wb[(size_t)g * M + j] = fma(mi, fma(-v, fb[j], jb[j]), Wb[(size_t)g * M + j]);
+            gga = fma(jb[j], Iv_ga, fma(-vv * (v - ion.a), fb[j], gga));
+            ga_ = fma(jb[j], fma(-2.0, v, 1.0), fma(vv, fb[j], ga_));
+            ffull[(size_t)g * M + j] = fb[j];
         }
+        gga *= mi;
+        ga_ *= ion.ga * mi;
     }
-    block_sum3(gga, ggs, ga_, part3);
+    block_add3(gga, 0.0, ga_, part3);
 }
 
-// Vb_j -= K fbar_j over every row (fbar is zero off the active set).
+// Over every row: Vb_j -= K fbar_j (fbar is zero off the active set), and for the conductivity
+// gradient the field that bbar_m is paired with in every element,
+//   z_m = - dt sum_{j<=m} Qh_mj (V'_j - V_j) - dt sum_j Q_mj V_j
+// (the node solves' - K dt Qhat D and, with fbar_j = dt sum_m Q_mj bbar_m, the residual's
+// - fbar_j^T K V_j; V' = V off the active set).
 template <int M>
 __global__ void k_adj_kfull(int N, const double* __restrict__ kval, const int* __restrict__ kcol,
                             const int* __restrict__ klen, int ldk, const double* __restrict__ kdiag,
-                            const double* __restrict__ ffull, double* __restrict__ Vb) {
+                            const double* __restrict__ ffull, double* __restrict__ Vb, Coll co,
+                            const double* __restrict__ Vo, const double* __restrict__ Vn,
+                            double* __restrict__ z) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     double acc[M];
 #pragma unroll
-    for (int m = 0; m < M; ++m) acc[m] = kdiag[i] * ffull[(size_t)m * N + i];
+    for (int m = 0; m < M; ++m) acc[m] = kdiag[i] * ffull[(size_t)i * M + m];
     const int len = klen[i];
     for (int t = 0; t < len; ++t) {
         const double a = kval[(size_t)t * ldk + i];
         const int j = sdc_idx(kcol[(size_t)t * ldk + i], N, 205);
 #pragma unroll
-        for (int m = 0; m < M; ++m) acc[m] += a * ffull[(size_t)m * N + j];
+        for (int m = 0; m < M; ++m) acc[m] += a * ffull[(size_t)j * M + m];
     }
 #pragma unroll
     for (int m = 0; m < M; ++m) Vb[(size_t)i * M + m] -= acc[m];
+    if (!z) return;
+#pragma unroll
+    for (int m = 0; m < M; ++m) acc[m] = 0.0;
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+        const double v = Vo[(size_t)i * M + j], d = Vn[(size_t)i * M + j] - v;
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+            acc[m] = fma(-co.Q[m * kMaxM + j], v, acc[m]);
+            if (j <= m) acc[m] = fma(-co.Qh[m * kMaxM + j], d, acc[m]);
+        }
+    }
+#pragma unroll
+    for (int m = 0; m < M; ++m) z[(size_t)i * M + m] = acc[m];
 }
 
-// dL/dsbar_e += sum_m bbar_m^T Khat_e vk_m - sum_j fbar_j^T Khat_e V_j
-template <int M>
-__global__ void k_adj_elem(int NE, int dim, const double* __restrict__ xyz,
-                           const int* __restrict__ elem, const double* __restrict__ sig9,
-                           const double* __restrict__ esig9, int N,
-                           const double* __restrict__ bfull, const double* __restrict__ vkfull,
-                           const double* __restrict__ ffull, const double* __restrict__ Vo,
-                           double* __restrict__ ge) {
+// dL/dsbar_e += sum_m bbar_m^T Khat_e z_m.  The rows and columns of Khat_e sum to zero, so
+// with differences to the element's first vertex (u_a = bbar_a - bbar_0, likewise z)
+//   sum_m bbar_m^T Khat_e z_m = sum_{a,b>=1} (Khat_e)_ab T_ab,  T_ab = sum_m u_a,m z_b,m .
+// T is kept over the sweeps (first: it starts from zero; last: it is contracted with Khat_e),
+// so the geometry is formed once per adjoint and not in every sweep, and one pair of fields
+// per node is gathered where there were two: 15 FP64 operations per element and node, 115
+// for the geometry, where each sweep took 40 a node and 160.  The FP64 pipe bounds both.
+template <int DIM, int M>
+__global__ void k_adj_elem(int NE, const double* __restrict__ xyz, const int* __restrict__ elem,
+                           const double* __restrict__ sig9, const double* __restrict__ esig9,
+                           const double* __restrict__ bfull, const double* __restrict__ z,
+                           int first, int last, double* __restrict__ T, double* __restrict__ ge) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= NE) return;
-    const int nv = dim + 1;
-    const int* vt = elem + (size_t)e * nv;
-    double grad[4][3], vol;
-    if (!p1_gradients(dim, xyz, vt, grad, vol)) return;
-    const double* Dm = esig9 ? esig9 + (size_t)e * 9 : sig9;
-    double Ke[4][4];
-    for (int a = 0; a < nv; ++a) {
-        double Dg[3] = {0, 0, 0};
-        for (int r = 0; r < dim; ++r)
-            for (int c = 0; c < dim; ++c) Dg[c] += grad[a][r] * Dm[r * 3 + c];
-        for (int b = 0; b < nv; ++b) {
-            double s = 0.0;
-            for (int c = 0; c < dim; ++c) s += Dg[c] * grad[b][c];
-            Ke[a][b] = vol * s;
+    constexpr int NV = DIM + 1;
+    int vt[NV];
+#pragma unroll
+    for (int a = 0; a < NV; ++a) vt[a] = elem[(size_t)e * NV + a];
+    double u[NV][M];
+    long long any = 0;
+#pragma unroll
+    for (int a = 0; a < NV; ++a)
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+            u[a][m] = bfull[(size_t)vt[a] * M + m];
+            any |= __double_as_longlong(u[a][m]) & 0x7fffffffffffffffll;
+        }
+    if (!any && !first && !last) return;   // no active vertex
+    double t[DIM][DIM];
+#pragma unroll
+    for (int a = 0; a < DIM; ++a)
+#pragma unroll
+        for (int b = 0; b < DIM; ++b)
+            t[a][b] = first ? 0.0 : T[(size_t)(a * DIM + b) * NE + e];
+    if (any) {
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+            double dz[DIM];
+            const double z0 = z[(size_t)vt[0] * M + m];
+#pragma unroll
+            for (int b = 0; b < DIM; ++b) dz[b] = z[(size_t)vt[b + 1] * M + m] - z0;
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) {
+                const double du = u[a + 1][m] - u[0][m];
+#pragma unroll
+                for (int b = 0; b < DIM; ++b) t[a][b] = fma(du, dz[b], t[a][b]);
+            }
         }
     }
+    if (!last) {
+#pragma unroll
+        for (int a = 0; a < DIM; ++a)
+#pragma unroll
+            for (int b = 0; b < DIM; ++b) T[(size_t)(a * DIM + b) * NE + e] = t[a][b];
+        return;
+    }
+    double grad[4][3], vol;
+    if (!p1_gradients(DIM, xyz, vt, grad, vol)) return;
+    const double* Dm = esig9 ? esig9 + (size_t)e * 9 : sig9;
+    // sum_ab t_ab grad_a . D grad_b = sum_r (sum_a grad_a,r sum_b t_ab (D grad_b)_r)
     double acc = 0.0;
 #pragma unroll
-    for (int m = 0; m < M; ++m) {
-        for (int a = 0; a < nv; ++a) {
-            const double ub = bfull[(size_t)m * N + vt[a]];
-            const double uf = ffull[(size_t)m * N + vt[a]];
-            if (ub == 0.0 && uf == 0.0) continue;
-            double kb = 0.0, kf = 0.0;
-            for (int b = 0; b < nv; ++b) {
-                kb += Ke[a][b] * vkfull[(size_t)m * N + vt[b]];
-                kf += Ke[a][b] * Vo[(size_t)vt[b] * M + m];
-            }
-            acc += ub * kb - uf * kf;
+    for (int r = 0; r < DIM; ++r) {
+        double Dg[DIM];
+#pragma unroll
+        for (int b = 0; b < DIM; ++b) {
+            Dg[b] = 0.0;
+#pragma unroll
+            for (int c = 0; c < DIM; ++c) Dg[b] = fma(Dm[r * 3 + c], grad[b + 1][c], Dg[b]);
+        }
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+            double s = 0.0;
+#pragma unroll
+            for (int b = 0; b < DIM; ++b) s = fma(t[a][b], Dg[b], s);
+            acc = fma(grad[a + 1][r], s, acc);
         }
     }
-    ge[e] += acc;
+    ge[e] = fma(vol, acc, ge[e]);
 }
 
 // dL/ds_a += sum over elements e containing a of dL/dsbar_e / (d + 1)
@@ -444,7 +475,15 @@ int adjoint_step(const AdjointArgs& a, StepBuffers& B, AdjointBuffers& W, cudaSt
     const int N = B.N, M = B.M, ld = B.ld;
     const MeshDev& md = *a.mesh;
     const Ell& K = *a.K;
+    const AdjIonic ion = fold_adjoint(a.ion);
+    Coll co = a.co;   // times dt
+    for (int k = 0; k < kMaxM * kMaxM; ++k) {
+        co.Q[k] *= a.dt;
+        co.Qh[k] *= a.dt;
+    }
+    bool first = true;   // no element term yet
     cudaMemsetAsync(W.iacc, 0, 3 * sizeof(double), s);
+    cudaMemsetAsync(W.part3, 0, 3 * (size_t)nb(N, kAdjBlock) * sizeof(double), s);
     if (a.grad_scale) cudaMemsetAsync(W.ge, 0, (size_t)md.n_elems * sizeof(double), s);
     k_adj_init<<<nb(N, kAdjBlock), kAdjBlock, 0, s>>>(N, M, a.lam_v, a.lam_w, W.Vb, W.Wb,
                                                      a.lam_v0, a.lam_w0);
@@ -470,18 +509,15 @@ int adjoint_step(const AdjointArgs& a, StepBuffers& B, AdjointBuffers& W, cudaSt
         }
         dispatch_M(M, [&](auto mc) {
             constexpr int MM = decltype(mc)::value;
-            if (!a.w_frozen) {
-                k_adj_wsweep<MM><<<nbk, kAdjBlock, 0, s>>>(n, act, Vn, Wo, Wn, a.dt, a.ion, a.co,
-                                                           W.Vb, W.Wb, a.lam_w0, W.part3, N);
-                k_sum3<<<1, 32, 0, s>>>(nbk, W.part3, W.iacc);
-            }
-            k_adj_prep<MM><<<nbk, kAdjBlock, 0, s>>>(n, act, Vo, Wo, Vn, a.kdiag, a.mass, W.Vb,
-                                                     a.ion, a.reaction_implicit, ld, B.J, B.D,
-                                                     B.mc, B.kdc, B.R, W.Jb, N);
+            k_adj_prep<MM><<<nbk, kAdjBlock, 0, s>>>(n, act, Vo, Wo, Vn, Wn, a.kdiag, a.mass, ion,
+                                                     co, a.w_frozen, a.reaction_implicit, ld, W.Vb,
+                                                     W.Wb, a.lam_w0, W.part3, B.J, B.mc, B.kdc,
+                                                     B.R, N);
         });
-        cudaMemsetAsync(W.bfull, 0, (size_t)M * N * sizeof(double), s);
-        cudaMemsetAsync(W.vkfull, 0, (size_t)M * N * sizeof(double), s);
-        cudaMemsetAsync(W.ffull, 0, (size_t)M * N * sizeof(double), s);
+        if (n < N) {   // zero off the active set
+            cudaMemsetAsync(W.bfull, 0, (size_t)M * N * sizeof(double), s);
+            cudaMemsetAsync(W.ffull, 0, (size_t)M * N * sizeof(double), s);
+        }
         for (int m = M - 1; m >= 0 && status == SDC_OK; --m) {
             PcgRole role{};
             role.b = B.R + (size_t)m * ld;            // dvbar_m (coupled)
@@ -500,30 +536,29 @@ int adjoint_step(const AdjointArgs& a, StepBuffers& B, AdjointBuffers& W, cudaSt
                 status = SDC_E_CUDA;
                 break;
             }
-            dispatch_M(M, [&](auto mc) {
-                constexpr int MM = decltype(mc)::value;
-                k_adj_node_post<MM><<<nbk, kAdjBlock, 0, s>>>(n, act, m, a.dt, a.co, ld, N,
-                                                              W.X + (size_t)m * ld, B.D, B.mc,
-                                                              W.Jb, W.bfull, W.vkfull);
-            });
         }
         if (status != SDC_OK) break;
         dispatch_M(M, [&](auto mc) {
             constexpr int MM = decltype(mc)::value;
-            k_adj_residual<MM><<<nbk, kAdjBlock, 0, s>>>(n, act, ld, N, a.dt, a.co, a.ion,
-                                                         a.reaction_implicit, W.X, W.Jb, Vo, Wo,
-                                                         a.mass, W.Vb, W.Wb, a.lam_v0, W.ffull,
-                                                         W.part3);
-            k_sum3<<<1, 32, 0, s>>>(nbk, W.part3, W.iacc);
-            k_adj_kfull<MM><<<nb(N, kAdjBlock), kAdjBlock, 0, s>>>(N, K.val, K.col, K.len, K.ld,
-                                                                  a.kdiag, W.ffull, W.Vb);
-            if (a.grad_scale)
-                k_adj_elem<MM><<<nb(md.n_elems, 128), 128, 0, s>>>(
-                    md.n_elems, md.dim, md.xyz, md.elem, md.sig, md.esig, N, W.bfull, W.vkfull,
-                    W.ffull, Vo, W.ge);
+            k_adj_residual<MM><<<nbk, kAdjBlock, 0, s>>>(n, act, ld, N, co, ion,
+                                                         a.reaction_implicit, W.X, Vo, Wo, Vn,
+                                                         a.mass, W.Vb, W.Wb, a.lam_v0, W.bfull,
+                                                         W.ffull, W.part3);
+            k_adj_kfull<MM><<<nb(N, kAdjBlock), kAdjBlock, 0, s>>>(
+                N, K.val, K.col, K.len, K.ld, a.kdiag, W.ffull, W.Vb, co, Vo, Vn,
+                a.grad_scale ? W.z : nullptr);
+            if (a.grad_scale) {
+                // without the sweeps' T (no memory for it) each sweep is contracted by itself
+                const int f = first || !W.T, l = k == 0 || !W.T;
+                auto* kern = md.dim == 2 ? k_adj_elem<2, MM> : k_adj_elem<3, MM>;
+                kern<<<nb(md.n_elems, 128), 128, 0, s>>>(md.n_elems, md.xyz, md.elem, md.sig,
+                                                         md.esig, W.bfull, W.z, f, l, W.T, W.ge);
+                first = false;
+            }
         });
     }
     if (status != SDC_OK) return status;
+    k_sum3<<<1, 256, 0, s>>>(nb(N, kAdjBlock), W.part3, W.iacc);
     k_adj_spread_back<<<nb(N, kAdjBlock), kAdjBlock, 0, s>>>(N, M, W.Vb, W.Wb, a.lam_v0,
                                                             a.lam_w0);
     if (a.grad_scale)

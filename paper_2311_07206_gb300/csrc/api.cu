@@ -281,8 +281,8 @@ bool ensure_adjoint(sdc_ctx* c) {
     if (W.Vb) return true;
     const size_t NM = (size_t)c->N * c->M, MLD = (size_t)c->M * c->B.ld;
     return ensure_pos(c) && dalloc(&W.Vb, NM) && dalloc(&W.Wb, NM) && dalloc(&W.V0, NM) &&
-           dalloc(&W.W0, NM) && dalloc(&W.X, MLD) && dalloc(&W.Jb, MLD) &&
-           dalloc(&W.bfull, NM) && dalloc(&W.vkfull, NM) && dalloc(&W.ffull, NM) &&
+           dalloc(&W.W0, NM) && dalloc(&W.X, MLD) &&
+           dalloc(&W.bfull, NM) && dalloc(&W.z, NM) && dalloc(&W.ffull, NM) &&
            dalloc(&W.ge, (size_t)c->K.mesh.n_elems) &&
            dalloc(&W.part3, 3 * (size_t)((c->N + 255) / 256)) && dalloc(&W.iacc, 3) &&
            dalloc(&W.iters, (size_t)SDC_MAX_SWEEPS * kMaxM) &&
@@ -290,7 +290,7 @@ bool ensure_adjoint(sdc_ctx* c) {
 }
 
 void free_adjoint(AdjointBuffers& W) {
-    double* dp[] = {W.Vb, W.Wb, W.V0, W.W0, W.X, W.Jb, W.bfull, W.vkfull, W.ffull, W.ge,
+    double* dp[] = {W.Vb, W.Wb, W.V0, W.W0, W.X, W.bfull, W.z, W.ffull, W.ge, W.T,
                     W.part3, W.iacc, W.relres};
     for (double* p : dp) cudaFree(p);
     cudaFree(W.pos);
@@ -1658,6 +1658,13 @@ static sdc_status step_adjoint_body(sdc_ctx* c, const sdc_tape* tape, const doub
     if (tape->n_active[0] != c->N)
         return fail(c, SDC_E_INVALID, "sdc_step_adjoint: the first sweep must cover every dof");
     if (!ensure_adjoint(c)) return fail(c, SDC_E_NOMEM, "adjoint workspace allocation failed");
+    if (d_grad_scale && !c->AW.T) {   // optional: without it every sweep forms the geometry
+        const size_t dd = (size_t)c->K.mesh.dim * c->K.mesh.dim;
+        if (!dalloc(&c->AW.T, dd * (size_t)c->K.mesh.n_elems)) {
+            cudaGetLastError();
+            c->AW.T = nullptr;
+        }
+    }
     cudaStream_t s = c->stream;
     AdjointArgs a;
     a.mesh = &c->K.mesh;

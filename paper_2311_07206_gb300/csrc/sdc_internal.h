@@ -364,9 +364,10 @@ struct AdjointArgs {
 };
 struct AdjointBuffers {
     double *Vb = nullptr, *Wb = nullptr, *V0 = nullptr, *W0 = nullptr;
-    double *X = nullptr, *Jb = nullptr;                       // [M][ld]
-    double *bfull = nullptr, *vkfull = nullptr, *ffull = nullptr;   // [M][N]
-    double *ge = nullptr;                                     // [n_elems]
+    double* X = nullptr;                                      // [M][ld]
+    double *bfull = nullptr, *z = nullptr, *ffull = nullptr;  // [N][M]
+    double* ge = nullptr;                                     // [n_elems]
+    double* T = nullptr;   // [dim * dim][n_elems] element sums over the sweeps, or null
     double *part3 = nullptr, *iacc = nullptr;                 // block partials, 3 accumulators
     int* pos = nullptr;                                       // [N], -1 outside a list
     int* iters = nullptr;                                     // [SDC_MAX_SWEEPS * kMaxM]
