@@ -28,7 +28,7 @@
 namespace sdc {
 namespace {
 
-constexpr int kAdjBlock = 256;
+constexpr int kAdjBlock = 128;
 
 inline int nb(int n, int b) { return (n + b - 1) / b; }
 

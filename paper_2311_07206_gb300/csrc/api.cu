@@ -284,7 +284,7 @@ bool ensure_adjoint(sdc_ctx* c) {
            dalloc(&W.W0, NM) && dalloc(&W.X, MLD) &&
            dalloc(&W.bfull, NM) && dalloc(&W.z, NM) && dalloc(&W.ffull, NM) &&
            dalloc(&W.ge, (size_t)c->K.mesh.n_elems) &&
-           dalloc(&W.part3, 3 * (size_t)((c->N + 255) / 256)) && dalloc(&W.iacc, 3) &&
+           dalloc(&W.part3, 3 * (size_t)((c->N + 127) / 128)) && dalloc(&W.iacc, 3) &&
            dalloc(&W.iters, (size_t)SDC_MAX_SWEEPS * kMaxM) &&
            dalloc(&W.relres, (size_t)SDC_MAX_SWEEPS * kMaxM);
 }

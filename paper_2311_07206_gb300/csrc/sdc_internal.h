@@ -11,7 +11,7 @@
 namespace sdc {
 
 constexpr int kMaxM = SDC_MAX_M;
-constexpr int kUpdateBlock = 256;   // block size of the update / scatter kernels
+constexpr int kUpdateBlock = 128;   // block size of the update / scatter kernels
 
 // Aliev-Panfilov parameters as passed to kernels (Sec. 5.1.1).
 struct Ionic {
