@@ -775,8 +775,8 @@ __device__ __forceinline__ void cgc_flow(const CgParams& P, const FlowParams& Q,
             wb[l] = r;
             ss[l] = s;
         });
-        if (wid == 0) flow_next(S, P.rtol);
         __syncthreads();
+        if (wid == 0) flow_next(S, P.rtol);
         // (the thread that writes the row's product over r_old)
         if (!late) flow_rows(nl, [&](int l) { px_row(rb, l); });
         ga = de = 0.0;
@@ -1188,7 +1188,6 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc2_flow(CgParams P, FlowParams Q,
             ss[l] = s;
             sr[l] -= alpha * s;
         });
-        if (wid == 0) flow_next(S, P.rtol);
         __syncthreads();
         const unsigned utag = Q.id + (unsigned)it + 1;
         ulonglong2* const pub = Q.pub + (size_t)(it & 1) * ld + r0;
@@ -1198,6 +1197,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc2_flow(CgParams P, FlowParams Q,
             pub_store(pub + l, u, utag);
         });
         __syncthreads();
+        // (after the barrier: in front of it the other warps waited for its 400 cycles)
+        if (wid == 0) flow_next(S, P.rtol);
         if (!late) flow_rows(nl, [&](int l) { px_row(ub, l); });
         // u <- w's place; the next w goes into the third buffer (two: u_old's place)
         double* const o = ub;
