@@ -380,7 +380,7 @@ __device__ __forceinline__ bool flow_window(double a, double b, FlowShared& S, u
 // before the first is used.  The product of a CTA with many rows is bound by instruction
 // issue, not by FP64 or latency (two padded slots more per row: 442k rows 13.5 -> 15.2 us per
 // iteration), so a slot is kept to a dozen instructions.
-template <int CH>
+template <int CH, bool NC = true>
 __device__ __forceinline__ double flow_row_dot(double acc, int len, const int* __restrict__ c, int ld,
                                                const double* v, int vs, int ncol, int r0, int nl,
                                                unsigned own, const ulonglong2* pub, unsigned tag,
@@ -392,7 +392,8 @@ __device__ __forceinline__ double flow_row_dot(double acc, int len, const int* _
         for (int k = 0; k < CH; ++k) {
             j[k] = r0;
             if (k0 + k < len) {
-                j[k] = sdc_idx(__ldg(c + (size_t)k * ld), ncol, site);
+                const int* const q = c + (size_t)k * ld;
+                j[k] = sdc_idx(NC ? __ldg(q) : *q, ncol, site);
                 a[k] = v[(size_t)k * vs];
             }
         }
@@ -859,6 +860,7 @@ struct CoarseFlowParams {
     const double* Einv;       // [q][q]
     ulonglong2* words;        // [2][pstride] published piece sums
     int pstride;
+    int width;                // (matrix rows on chip) slots of a row
 };
 
 // gamma = r.u is a sum of terms that cancel against each other within a block, so its window
@@ -872,6 +874,10 @@ __host__ __device__ inline size_t coarse_flow_smem(int L, int vectors, int qn, i
     return (size_t)vectors * L * 8 + (size_t)(3 * qn + ptot + npmax) * 8 +
            (size_t)((L + 31) / 32 + npmax) * 16 + 16 + (size_t)(2 * qn + 1 + 5 * npmax) * 4 +
            (size_t)L * 4;
+}
+// columns and values of a CTA's rows
+__host__ __device__ inline size_t coarse_flow_matrix(int L, int width) {
+    return 8 + (size_t)L * width * 12;
 }
 
 __device__ __forceinline__ void flow_bar_sync(int id, int n) {
@@ -919,7 +925,12 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc2_flow(CgParams P, FlowParams Q,
     unsigned short* const plen = pid + L;                                            // [L]
     const bool has_rows = wid != 0 || nw <= nch;
     const int e0 = C.tp[blockIdx.x], np = C.tp[blockIdx.x + 1] - e0;
-    double* const vb = P.sval + r0;
+    // the CTA's matrix rows, on chip as well where there is room (see coarse_flow_fit)
+    double* const sv = reinterpret_cast<double*>(
+        (reinterpret_cast<uintptr_t>(plen + L) + 7) & ~(uintptr_t)7);   // [width][L]
+    double* const vb = Q.v_smem ? sv : P.sval + r0;
+    int* const cb = Q.v_smem ? reinterpret_cast<int*>(sv + (size_t)C.width * L) : C.pcol + r0;
+    const int ms = Q.v_smem ? L : ld;
     unsigned epoch = 0, gen = 0;
     flow_scalars_init(S);
     if (t == 0) {
@@ -1081,8 +1092,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc2_flow(CgParams P, FlowParams Q,
         for (int k = 0; k < len; ++k) {
             const size_t e = (size_t)k * ld;
             const int j = sdc_idx(C.ipos[sdc_idx(P.acol[e + i], P.n, 71)], P.n, 72);
-            C.pcol[e + r0 + l] = j;
-            vb[e + l] = csi * P.aval[e + i] * __ldcg(P.sv + j);
+            cb[(size_t)k * ms + l] = j;
+            vb[(size_t)k * ms + l] = csi * P.aval[e + i] * __ldcg(P.sv + j);
         }
     });
     if (wid != 0) coarse_in(C.words, Q.id + 1);
@@ -1123,8 +1134,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc2_flow(CgParams P, FlowParams Q,
                 double v = 0.0;
                 if (l < nl) {
                     const double u = ub[l];
-                    const double w = flow_row_dot<FlowChunk<MAXT>::value>(
-                        u, plen[l], C.pcol + r0 + l, ld, vb + l, ld, P.n, r0, nl, smem_addr(ub), pub,
+                    const double w = flow_row_dot<FlowChunk<MAXT>::value, false>(
+                        u, plen[l], cb + l, ms, vb + l, ms, P.n, r0, nl, smem_addr(ub), pub,
                         tag, 76, S, P.budget, P.err);
                     wb[l] = w;
                     ga += sr[l] * u;

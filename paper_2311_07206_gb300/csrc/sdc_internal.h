@@ -292,7 +292,7 @@ struct CoarseDev {
     int pstride = 0;
     unsigned wraps = 0;                  // the flow_wraps the words were last cleared at
     int flow = 0;                        // this sweep's solves run in it
-    int L = 0, block = 0, nbuf = 0, x_smem = 0;
+    int L = 0, block = 0, nbuf = 0, x_smem = 0, m_smem = 0;
     size_t smem = 0;
 };
 // Shape of the on-chip form for n rows: rows per CTA (0: none); then, with the pieces known,

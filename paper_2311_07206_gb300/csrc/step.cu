@@ -2175,7 +2175,11 @@ bool coarse_flow_fit(CoarseDev& C) {
         C.nbuf = v >= 7 ? 3 : 2;
         C.x_smem = v == 8;
         C.smem = coarse_flow_smem(C.L, v, C.qn, C.ptot, C.pmax);
-        if (C.smem <= (size_t)kFlowSmemBytes) return true;
+        if (C.smem > (size_t)kFlowSmemBytes) continue;
+        const size_t m = coarse_flow_matrix(C.L, C.width);
+        C.m_smem = C.smem + m <= (size_t)kFlowSmemBytes;
+        if (C.m_smem) C.smem += m;
+        return true;
     }
     return false;
 }
@@ -2225,6 +2229,7 @@ int launch_pcg_coarse(int n, const Ell& A, const PcgRole& role, double rtol, int
         }
         Q.x_smem = C.x_smem;
         Q.nbuf = C.nbuf;
+        Q.v_smem = C.m_smem;
         Q.iters_out = P.iters_out;
         Q.relres_out = P.relres_out;
         P.L = C.L;
@@ -2243,6 +2248,7 @@ int launch_pcg_coarse(int n, const Ell& A, const PcgRole& role, double rtol, int
         F.Einv = C.Einv;
         F.words = reinterpret_cast<ulonglong2*>(C.words);
         F.pstride = C.pstride;
+        F.width = C.width;
         void* fa[] = {&P, &Q, &F};
         const void* k = C.block > 768   ? (const void*)k_cgc2_flow<1024>
                         : C.block > 512 ? (const void*)k_cgc2_flow<768>
