@@ -654,23 +654,28 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
             }
         }
         __syncthreads();
-        if (!S.ok) return;
-        if (S.state == 3) {
-            if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, kFlowSumHead, P.budget, P.err)) return;
-            if (S.state == 0) {
-                exact = redo = true;
-                continue;
+        // (read together: one after the other they cost three shared-memory latencies)
+        alpha = S.alpha;
+        beta = S.beta;
+        if (S.ok - 1 | S.state) {
+            if (!S.ok) return;
+            if (S.state == 3) {
+                if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, kFlowSumHead, P.budget,
+                                 P.err))
+                    return;
+                if (S.state == 0) {
+                    exact = redo = true;
+                    continue;
+                }
             }
+            break;
         }
         exact = redo = false;
-        if (S.state != 0) break;
         if (it >= P.maxit) {
             if (blockIdx.x == 0 && t == 0) raise_error(P.err, SDC_E_CG_NOCONV);
             break;
         }
         ++it;
-        alpha = S.alpha;
-        beta = S.beta;
         if (t == 0) S.next = 0;
         if (wid == 0) flow_next(S, P.rtol);
         const unsigned tag = Q.id + (unsigned)it + 1;
@@ -750,23 +755,28 @@ __device__ __forceinline__ void cgc_flow(const CgParams& P, const FlowParams& Q,
         ++npub;
         if (late && it > 0 && !redo) flow_rows_px(nl, [&](int l) { px_row(fb, l); });
         __syncthreads();
-        if (!S.ok) return;
-        if (S.state == 3) {
-            if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, kFlowSumHead, P.budget, P.err)) return;
-            if (S.state == 0) {
-                exact = redo = true;
-                continue;
+        // (read together: one after the other they cost three shared-memory latencies)
+        alpha = S.alpha;
+        beta = S.beta;
+        if (S.ok - 1 | S.state) {
+            if (!S.ok) return;
+            if (S.state == 3) {
+                if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, kFlowSumHead, P.budget,
+                                 P.err))
+                    return;
+                if (S.state == 0) {
+                    exact = redo = true;
+                    continue;
+                }
             }
+            break;
         }
         exact = redo = false;
-        if (S.state != 0) break;
         if (it >= P.maxit) {
             if (Q.bidx == 0 && t == 0) raise_error(P.err, SDC_E_CG_NOCONV);
             break;
         }
         ++it;
-        alpha = S.alpha;
-        beta = S.beta;
         const unsigned tag = Q.id + (unsigned)it + 1;
         ulonglong2* const pub = Q.pub + (size_t)(it & 1) * ld;
         flow_rows(nl, [&](int l) {
@@ -1185,8 +1195,6 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc2_flow(CgParams P, FlowParams Q,
             break;
         }
         ++it;
-        alpha = S.alpha;
-        beta = S.beta;
         for (int m = B - 1 - t; m < C.qn; m += B) {
             const double sa = tw[m] + beta * ts[m];
             ts[m] = sa;
