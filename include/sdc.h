@@ -101,14 +101,20 @@ typedef struct {
     long long spin_budget; /* SM clock cycles a device-side barrier may wait; default 4e9     */
     int cg_block_size;     /* threads per block of the global-vector CG (64..1024, multiple
                               of 32); default 1024.  Batches use min(this, 256)               */
-    int cg_smem_block_size;/* threads per block of the shared-memory and cluster CG; default 512 */
+    int cg_smem_block_size;/* threads per block of the shared-memory and cluster CG; default 512.
+                              Scaled form: below 512 a limit on the threads (32 plus one per
+                              row up to 896 rows a block, else 1024)                         */
     int cg_cluster_max;    /* largest cluster (CTAs) for the cluster CG, 1..16; default 16      */
     int cg_max_blocks;     /* 0: no limit on the cooperative CG grid                          */
     int cg_variant;        /* 0: automatic; 1: vectors in global memory; 2: per-block vectors
-                              in shared memory whenever they fit (3584 rows per SM for the
-                              pipelined, 4768 for the classical arrangement)                 */
-    int cg_rows_per_block; /* shared-memory variant: target rows per block (0 = 256)          */
-    int cg_cluster_rows;   /* solves with |I_k| <= this run on one thread-block cluster
+                              in shared memory whenever they fit (scaled form: 3968 rows per
+                              SM for the pipelined, 6752 for the classical arrangement; Jacobi
+                              form: 3584 and 4768)                                            */
+    int cg_rows_per_block; /* shared-memory variant: target rows per block (0 = 256 in the
+                              Jacobi form; in the scaled form as many blocks as SMs, of at
+                              least 96 rows)                                                  */
+    int cg_cluster_rows;   /* Jacobi form (cg_scaled = 0): solves with |I_k| <= this run on one
+                              thread-block cluster
                               (16 CTAs, distributed shared memory); default 10000, 0 = never */
     int profile;           /* 1: bracket every kernel launch with CUDA events on the context's
                               stream and report device time per phase in sdc_stats; default 0 */
@@ -118,9 +124,10 @@ typedef struct {
     int cg_pipelined;      /* arrangement of the CG iteration (the same iterates in exact
                               arithmetic): 1 pipelined (one grid synchronisation per iteration,
                               the sums overlapped with the product); 0 classical (two); -1
-                              automatic: for monodomain contexts pipelined where the solve's
-                              vectors fit on chip and classical above (its lighter vector
-                              traffic wins there); classical for cell-by-cell contexts, whose
+                              automatic: for monodomain contexts pipelined up to 130,000
+                              active rows, where an iteration is bound by latency, and
+                              classical above (fewer FP64 operations per row; Jacobi form:
+                              pipelined where the vectors fit on chip); classical for cell-by-cell contexts, whose
                               long ill-conditioned solves need its smaller rounding error, and
                               for batches, whose many small groups favour its lighter rows;
                               default -1                                                       */
@@ -151,9 +158,7 @@ typedef struct {
                               max(0, -min dI/dv) / C_m over the first sweep's linearisation
                               (zero with reaction_implicit = 0); computed on the device once
                               per step, reported in sdc_stats.tol_drop.  Not in batches      */
-    int cg_scaled;         /* 1: the node solves (shared-memory, global-vector and batched
-                              variants; the cluster variant keeps the Jacobi form) run in the
-                              symmetrically scaled form, CG on diag^-1/2 A diag^-1/2: the same
+    int cg_scaled;         /* 1: the node solves run in the symmetrically scaled form, CG on diag^-1/2 A diag^-1/2: the same
                               iterates as Jacobi-PCG with fewer FP64 operations per row and
                               fewer vectors on chip; 0: the Jacobi form; default 1          */
     int batch_graph;       /* batches: 1 runs each step with device-driven sweeps (|I_k| read on
@@ -259,8 +264,9 @@ sdc_status sdc_get_matrix(const sdc_ctx* ctx, int* row_ptr, int* col, double* va
  * d_len[i] <= width entries, entry t at d_val[t * ld + i], column
  * d_col[t * ld + i] in [0, n); ld >= n.  Every array is caller-owned device
  * memory of the current device; d_x receives the solution.  The workspace
- * (8 n + 2 ld doubles plus a few per SM) is allocated and freed inside the call, which
- * synchronises `stream` (a cudaStream_t, NULL = legacy default).  iters and
+ * (up to 8 n + 2 ld doubles plus a few per SM; on-chip solves up to 2 n + (4 + width) ld) comes
+ * from a stream-ordered pool that keeps at most 64 MiB per device between calls (sdc_destroy
+ * gives them back) and is returned inside the call, which synchronises `stream` (a cudaStream_t, NULL = legacy default).  iters and
  * relres (host, may be NULL) receive the iteration count and the final
  * sqrt(r'z / r0'z0).  Errors: SDC_E_INVALID (nothing launched),
  * SDC_E_NOMEM, SDC_E_CG_NOCONV, SDC_E_NONFINITE, SDC_E_DOMAIN (a non-positive

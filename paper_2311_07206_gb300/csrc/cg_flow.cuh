@@ -574,6 +574,10 @@ __device__ __forceinline__ void flow_finish(const CgParams& P, const FlowParams&
 // n = (I + c S K_off S) w on every warp but warp 0, which waits for the sums and derives the
 // scalars.  The product's 32-row chunks beyond the first per warp are handed out by a
 // counter, so warp 0 takes what is left when it joins.
+// Bound by the chain post (1,000 cycles) - poll (1,300-1,900) - scalars (1,200-1,700) - update
+// (900-1,800); the product runs beside it.  us per iteration, before (barrier and records, or a
+// cluster for up to 10,000 rows) and now: 4,225 rows 4.7 / 2.8, 11.8k 5.2 / 2.8, 58k 6.2 / 3.9,
+// 89k 7.5 / 5.1.
 template <int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) {
     extern __shared__ double sm[];
@@ -709,6 +713,11 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
 // that r_old is still there for p after the product; with two, p and x come before it.
 // One group of Q.G CTAs (the launch, or one instance of a batched launch); this CTA, number
 // Q.bidx of it, owns rows [r0, r0 + nl), at most P.L.
+// Many rows a CTA: bound by FP64 issue (442k rows, 27,400 cycles an iteration: product 15,000 of
+// which 11,300 are FP64, update 3,750 of which 2,800, the sums' chain 6,000 with p and x beside
+// it); few: by the chain exchange (1,200) - product - post - poll (1,700) - scalars (1,100).
+// us per iteration, before and now: 442k 18.3 / 13.2, 813k 30 / 23.5; cell-by-cell 7.7k 6.9 / 2.9,
+// 53k 8.7 / 4.1.
 template <int CH>
 __device__ __forceinline__ void cgc_flow(const CgParams& P, const FlowParams& Q, FlowShared& S, double* sm,
                                          int r0, int nl) {
@@ -822,7 +831,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc_flow(CgParams P, FlowParams Q) 
 }
 
 // Batched form: the blocks of an instance are a group with its own sums, barrier and
-// iteration count.  Several CTAs share an SM, so that one works while another waits.
+// iteration count.  Several CTAs share an SM, so that one works while another waits (32
+// instances of 20k rows: 5,277 -> 2,493 us per step against the grid-barrier kernel with vectors
+// in global memory).  Bound by FP64 issue.
 template <int MAXT>
 __global__ void __launch_bounds__(MAXT, 1024 / MAXT)
     k_cgc_flow_batch(CgParams P, FlowParams Q, const SegBlock* __restrict__ tab,

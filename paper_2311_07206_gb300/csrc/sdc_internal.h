@@ -11,7 +11,9 @@
 namespace sdc {
 
 constexpr int kMaxM = SDC_MAX_M;
-constexpr int kUpdateBlock = 128;   // block size of the update / scatter kernels
+constexpr int kUpdateBlock = 128;  // block size of the update / scatter kernels
+// (256 leave FP64 pipes idle in the last wave: 58k rows are 228 blocks on 152 SMs; the 89k
+// shell's step 2,203 -> 2,167 us)
 
 // Aliev-Panfilov parameters as passed to kernels (Sec. 5.1.1).
 struct Ionic {
@@ -182,7 +184,11 @@ void launch_residual(int M, int n, const int* act, const Ell& K, const double* k
 constexpr int kFlowSmemBytes = 225 * 1024;   // dynamic shared memory of the flow kernels
 constexpr int kFlowMaxit = 1000000;   // iterations a tag can count
 constexpr int kFlowWords = 34;      // 64-bit words of their grid-wide state
-constexpr int kFlowClassicalRows = 130000;   // automatic arrangement: classical above
+// Automatic arrangement: classical above.  The pipelined form hides the sums behind the product
+// but takes z + 11 FP64 operations per row, the classical z + 5; us per iteration, pipelined /
+// classical, 7-point operator: 119.6k rows 6.46 / 6.47, 154k 7.51 / 7.05, 200k 8.70 / 8.62,
+// 250k 10.24 / 9.41.
+constexpr int kFlowClassicalRows = 130000;
 constexpr int kSmemVectors = 8;     // per-row doubles in shared memory, shared-memory variant
 constexpr int kSmemRows = 3584;     // rows per block of the shared-memory variant
 // target rows per block of the shared-memory variants below their capacity: one row
@@ -210,7 +216,7 @@ struct PcgConfig {
     int batch_rows_per_block = 1024;
     int inject_fault = 0;
     int pipelined = 1;              // 1: pipelined CG; 0: classical arrangement
-    int scaled = 1;                 // pipelined shared-memory solves in the scaled form
+    int scaled = 1;                 // solves in the scaled form
     int general_classical = 0;      // pipelined contexts: classical arrangement for the
                                     // global-vector variant (automatic choice)
     long long budget = 0;

@@ -199,7 +199,7 @@ struct CgParams {
     const double* Jall;
     int inject_fault;    // testing hook: the last block skips the first barrier
     int L;               // rows per block (shared-memory variants)
-    // symmetrically scaled form (k_pcg_scaled): s = diag^-1/2 per row and the
+    // symmetrically scaled form: s = diag^-1/2 per row and the
     // scaled off-diagonal values c s_i a_ij s_j, rebuilt per solve (null: not used)
     double* sv;
     double* sval;
@@ -520,7 +520,7 @@ __device__ __forceinline__ void pcg_group(const CgParams& P, CgShared& S, int ro
     }
 }
 
-// The symmetrically scaled form of pcg_group (see k_pcg_scaled): CG on
+// The symmetrically scaled form of pcg_group: CG on
 // I + c S K_off S with S = diag^-1/2, vectors in global memory, any size.
 __device__ __forceinline__ void pcg_group_scaled(const CgParams& P, CgShared& S, int nblk,
                                                  int bidx) {
@@ -1141,7 +1141,7 @@ __device__ __forceinline__ void pcgc_group(const CgParams& P, CgShared& S, int r
     }
 }
 
-// The symmetrically scaled form of pcgc_group (see k_pcg_scaled): classical
+// The symmetrically scaled form of pcgc_group: classical
 // arrangement of CG on I + c S K_off S, S = diag^-1/2, vectors in global memory.
 // Per row-iteration z-bar + 6 FP64 operations instead of z-bar + 8 (no u = D^-1 r,
 // no scaling of the product by c).  Each thread owns the same rows in every loop,
@@ -2031,8 +2031,7 @@ void pcg_smem_attrs() {
                          k_cgc_flow<768>, k_cgc_flow<1024>})
         cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kFlowSmemBytes);
-    for (const void* k : {(const void*)k_cgc2_flow<512>, (const void*)k_cgc2_flow<768>,
-                          (const void*)k_cgc2_flow<1024>})
+    for (const void* k : {(const void*)k_cgc2_flow<512>, (const void*)k_cgc2_flow<768>})
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kFlowSmemBytes);
     for (PcgKernel k : {k_pcg_cluster<512>, k_pcg_cluster<1024>}) {
         cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2169,7 +2168,8 @@ int coarse_flow_rows(int n, int maxit, const PcgConfig& cfg) {
 bool coarse_flow_fit(CoarseDev& C) {
     // one row per thread up to 736 rows; above, 512 threads with 128 registers each (us per
     // iteration with 512 / 768 / 1024 threads: 131k rows 9.4 / 10.9 / 10.5, 250k 14.9 / 16.2 /
-    // 15.5, 505k 23.8 / 25.2 / 26.4; in one row per thread 83k 8.4 against 8.9)
+    // 15.5, 505k 23.8 / 25.2 / 26.4; in one row per thread 83k 8.4 against 8.9).  The matrix
+    // rows go on chip too where they fit: 131k rows 9.7 -> 9.2 us per iteration.
     C.block = C.L <= 736 ? 32 + C.L : 512;
     for (int v = 8; v >= 6; --v) {   // with x and the third buffer, with the buffer, with neither
         C.nbuf = v >= 7 ? 3 : 2;
@@ -2250,9 +2250,8 @@ int launch_pcg_coarse(int n, const Ell& A, const PcgRole& role, double rtol, int
         F.pstride = C.pstride;
         F.width = C.width;
         void* fa[] = {&P, &Q, &F};
-        const void* k = C.block > 768   ? (const void*)k_cgc2_flow<1024>
-                        : C.block > 512 ? (const void*)k_cgc2_flow<768>
-                                        : (const void*)k_cgc2_flow<512>;
+        const void* k = C.block > 512 ? (const void*)k_cgc2_flow<768>
+                                      : (const void*)k_cgc2_flow<512>;
         if (cudaLaunchCooperativeKernel(k, dim3(C.G), dim3(C.block), fa, C.smem, s) != cudaSuccess)
             return SDC_E_CUDA;
         B.flow_set ^= 1;
@@ -2329,7 +2328,9 @@ int launch_pcg_role(int n, const Ell& A, const PcgRole& role, double dt, int M, 
 // Shape of a flow launch: rows per CTA, CTAs, threads, shared memory; false when the rows
 // do not fit on chip.  Up to 28 chunks of 32 rows a CTA has one row per thread, warp 0 apart,
 // and its rows are a multiple of 128: FP64 issue is what a full warp per sub-partition
-// takes whatever its active lanes, so fewer CTAs with full warps are never slower.
+// takes whatever its active lanes, so fewer CTAs with full warps are never slower.  Up to
+// 14,592 rows a CTA has 96: fewer CTAs make the sums quicker (34 CTAs 1,290 cycles, 152 CTAs
+// 1,510) and three warps are one chunk per sub-partition.
 struct FlowShape {
     int L, grid, block, x_smem, nbuf, v_smem;
     size_t smem;

@@ -127,3 +127,63 @@ def test_two_level_edges(torch_dev, blocks):
         for m in range(wl.M):
             a, b = st.cg_iters[k][m], r["stats"].cg_iters[k * 8 + m]
             assert abs(a - b) <= max(2, b // 20), (k, m, a, b)
+
+
+def test_launch_ids_wrap(torch_dev):
+    """A context numbers its solves with 12 bits and clears the published words when the
+    number wraps: 4,500 solves of the same step give the same bits every time (the sums are
+    exact, so nothing depends on the order of the CTAs)."""
+    torch, dev = torch_dev
+    from paper_2311_07206_gb300 import Context, default_options
+    wl = _workload(20, 17, 0.3, 0.1, M=3, sweeps=1)      # 340 rows: four CTAs
+    ctx = Context.from_workload(wl, options=default_options(),
+                                stream=torch.cuda.current_stream(dev).cuda_stream)
+    v0 = torch.tensor(wl.v0, dtype=torch.float64, device=dev)
+    w0 = torch.tensor(wl.w0, dtype=torch.float64, device=dev)
+    first = None
+    for k in range(1500):
+        v, w = v0.clone(), w0.clone()
+        ctx.step(v, w, 0.0, wl.dt, wl.sweeps, wl.tol)
+        if first is None:
+            first = (v, w)
+        elif k % 50 == 0 or 1360 < k < 1370:            # 1,365 steps: the wrap
+            assert torch.equal(v, first[0]) and torch.equal(w, first[1]), k
+    ctx.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(365, 356), (365, 357)])   # 129,940 rows and 130,305
+def test_stand_alone_solves_on_both_sides_of_the_arrangements(torch_dev, nx, ny):
+    """sdc_pcg_solve in the pipelined and in the classical kernel: a five-point matrix with
+    mass 1 and c K of condition about 10.  The recurrence residual is at 1e-10; the true one
+    differs by rounding, below 30 iterations x cond x 2^-52 ~ 1e-13: bound 1.01e-10."""
+    torch, dev = torch_dev
+    from paper_2311_07206_gb300 import binding
+    n = nx * ny
+    ld = (n + 31) // 32 * 32
+    i = np.arange(n)
+    x_, y_ = i % nx, i // nx
+    val, col = np.zeros((4, ld)), np.zeros((4, ld), dtype=np.int32)
+    ln = np.zeros(n, dtype=np.int32)
+    kd = np.zeros(n)
+    for ok, off in ((x_ > 0, -1), (x_ < nx - 1, 1), (y_ > 0, -nx), (y_ < ny - 1, nx)):
+        r = i[ok]
+        val[ln[r], r], col[ln[r], r] = -1.0, r + off
+        ln[r] += 1
+        kd[r] += 1.0
+    rng = np.random.default_rng(n)
+    mass, J, c = np.ones(n), rng.uniform(0.0, 0.2, n), 1.0
+    b = rng.standard_normal(n)
+    t = lambda a: torch.tensor(a, device=dev)
+    x = torch.zeros(n, dtype=torch.float64, device=dev)
+    it, rr = binding.pcg_solve(n, t(val), t(col), t(ln), ld, 4, t(kd), t(mass), t(J), c, t(b), x,
+                               rtol=1e-10, maxit=1000,
+                               stream=torch.cuda.current_stream(dev).cuda_stream)
+    assert 5 < it < 60 and rr <= 1e-10
+    xh = x.cpu().numpy()
+    d = mass * (1.0 + c * J) + c * kd
+    Ax = d * xh
+    for k in range(4):
+        m = ln > k
+        Ax[m] += c * val[k, :n][m] * xh[col[k, :n][m]]
+    r = b - Ax
+    assert np.sqrt((r * r / d).sum() / (b * b / d).sum()) <= 1.01e-10
