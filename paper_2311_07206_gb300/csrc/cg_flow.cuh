@@ -1190,17 +1190,22 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc2_flow(CgParams P, FlowParams Q,
         }
         ++npub;
         __syncthreads();
-        if (!S.ok) return;
-        if (S.state == 3) {
-            if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, kFlowSumHead, P.budget, P.err))
-                return;
-            if (S.state == 0) {
-                exact = redo = true;
-                continue;
+        alpha = S.alpha;
+        beta = S.beta;
+        if (S.ok - 1 | S.state) {
+            if (!S.ok) return;
+            if (S.state == 3) {
+                if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, kFlowSumHead, P.budget,
+                                 P.err))
+                    return;
+                if (S.state == 0) {
+                    exact = redo = true;
+                    continue;
+                }
             }
+            break;
         }
         exact = redo = false;
-        if (S.state != 0) break;
         if (it >= P.maxit) {
             if (blockIdx.x == 0 && t == 0) raise_error(P.err, SDC_E_CG_NOCONV);
             break;
