@@ -789,7 +789,7 @@ sdc_status step_batch_graph(sdc_ctx* c, double* d_v, double* d_w, double dt, int
             launch_select(N, act, next, B, s, nd);
             cudaMemcpyAsync(B.nk + k + 1, &B.sc->count, sizeof(int), cudaMemcpyDeviceToDevice, s);
             launch_seg_bounds(next, &B.sc->count, B, s, B.bounds_k + (size_t)(k + 1) * (nseg + 1));
-            L += 4;
+            L += 2 + select_launches(N);
             if (k + 1 < sweeps) {
                 Ell& An = B.A[cur];
                 launch_extract(N, *A, B.map, An, B, s, nd);
@@ -1019,7 +1019,8 @@ sdc_status step_core(sdc_ctx* c, double* d_v, double* d_w, double t, double dt, 
         int* next = (k + 1 < sweeps) ? c->act[k + 1] : c->act[0];
         const bool replay = tape && tape->mode == SDC_TAPE_REPLAY;
         if (!replay) {
-            run(SDC_PHASE_SELECT, 2, [&] { launch_select(n, act, next, B, s); });
+            run(SDC_PHASE_SELECT, select_launches(n),
+                [&] { launch_select(n, act, next, B, s); });
         } else {
             // the next set comes from the tape; the old->new row map from a position table
             const int nn = (k + 1 < sweeps) ? tape->n_active[k + 1] : 0;

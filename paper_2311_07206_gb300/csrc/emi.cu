@@ -519,7 +519,7 @@ int emi_step(const EmiStepArgs& a, double* d_u, double* d_w, double dt, int swee
                 });
         });
         int* next = (k + 1 < sweeps) ? (*a.act)[k + 1] : (*a.act)[0];
-        run(SDC_PHASE_SELECT, 3, [&] {
+        run(SDC_PHASE_SELECT, 1 + select_launches(n), [&] {
             if (act) launch_pos_set(n, act, E.pos, 1, B.N, s);
             else k_pos_identity<<<nbk(N, 256), 256, 0, s>>>(N, E.pos, 1);
             launch_select(n, act, next, B, s);

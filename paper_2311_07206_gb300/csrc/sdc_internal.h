@@ -423,6 +423,7 @@ void launch_drop_rule(int n, int M, const double* D, int ld, int nj, const doubl
                       double Cm, double rho, double TOL, double dt, StepBuffers& B,
                       cudaStream_t s);
 // n_dev: when set, |I_k| is read on the device and n only sizes the grid (captured steps)
+int select_launches(int n);
 void launch_select(int n, const int* act, int* act_next, StepBuffers& B, cudaStream_t s,
                    const int* n_dev = nullptr);
 void launch_extract(int n_old, const Ell& Aold, const int* map, Ell& Anew, StepBuffers& B,

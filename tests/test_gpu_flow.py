@@ -187,3 +187,18 @@ def test_stand_alone_solves_on_both_sides_of_the_arrangements(torch_dev, nx, ny)
         Ax[m] += c * val[k, :n][m] * xh[col[k, :n][m]]
     r = b - Ax
     assert np.sqrt((r * r / d).sum() / (b * b / d).sum()) <= 1.01e-10
+
+
+@pytest.mark.parametrize("nx,ny", [(512, 256), (331, 396)])   # 1,024 blocks of 128 rows, and 1,025
+def test_selection_on_both_sides_of_its_launch_rule(torch_dev, nx, ny):
+    """A front over a third of the grid: the rows far from it leave the set after a sweep.  The
+    sizes of the sets are the oracle's."""
+    torch, dev = torch_dev
+    wl = _workload(nx, ny, 0.3, 0.05, sweeps=3, tol=1e-4,
+                   v=lambda rng, n: (np.arange(n) < n // 3).astype(float))
+    st = _check(wl, torch, dev)
+    r = oracle.System.from_mesh(wl.mesh, wl.sigma).step(wl.ionic, wl.M, wl.v0, wl.w0, wl.dt,
+                                                        wl.sweeps, wl.tol, cg_maxit=20000)
+    n = list(st.n_active)[:wl.sweeps]
+    assert n == list(r["stats"].n_active)[:wl.sweeps]
+    assert 0 < n[1] < n[0]
