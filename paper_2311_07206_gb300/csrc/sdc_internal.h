@@ -183,7 +183,10 @@ void launch_residual(int M, int n, const int* act, const Ell& K, const double* k
 // Launch configuration of the restricted PCG solves.
 constexpr int kFlowSmemBytes = 225 * 1024;   // dynamic shared memory of the flow kernels
 constexpr int kFlowMaxit = 1000000;   // iterations a tag can count
-constexpr int kFlowWords = 34;      // 64-bit words of their grid-wide state
+// 64-bit words of their grid-wide state: 34, padded to whole 128-byte lines.  The second of two
+// adjacent sets of 34 had its sums across two lines, and every other solve took 1 to 4 % longer
+// (53k cell-by-cell dofs 26.60 -> 26.28 ms per step, 58k order 6 2,926 -> 2,906 us).
+constexpr int kFlowWords = 48;
 // Automatic arrangement: classical above.  The pipelined form hides the sums behind the product
 // but takes z + 11 FP64 operations per row, the classical z + 5; us per iteration, pipelined /
 // classical, 7-point operator: 119.6k rows 6.46 / 6.47, 154k 7.51 / 7.05, 200k 8.70 / 8.62,
