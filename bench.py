@@ -288,7 +288,7 @@ FP64_LANES_PER_CYCLE = 304          # whole GPU, ncu dfma peak_sustained on GB30
 FP64_ISSUE_FRACTION = 0.84
 SIZE_CLASSES = ((1, 10_000, "<=10k rows"), (10_001, 300_000, "10k-300k rows"),
                 (300_001, 1 << 62, ">300k rows"))
-CG_SOURCES = ("step.cu", "device_common.cuh")
+CG_SOURCES = ("step.cu", "cg_flow.cuh", "device_common.cuh")
 # DRAM traffic of the dominant kernel from one ncu capture (dram__bytes_read.sum +
 # dram__bytes_write.sum) of the first node solve of a slab step, all 442,401 rows, scaled to
 # the average launch by algorithmic bytes.  `source_sha` is the hash of the CG sources the
@@ -325,9 +325,9 @@ def interp_plain_ms(plain, err):
             return float(np.exp(np.log(m_lo) + f * np.log(m_hi / m_lo)))
     return None
 
-PCG_TRAFFIC = {"w1": {"dram_bytes": 64.25e6 + 10.65e6, "algorithmic_bytes": 1.735e9,
-                      "kernel": "k_pcg_scaled<1024>", "source_sha": "f6df4e0ce07892df",
-                      "capture": "profiles/pcg_scaled_w1_slab_full_solve.md"}}
+PCG_TRAFFIC = {"w1": {"dram_bytes": 64.34e6 + 12.56e6, "algorithmic_bytes": 2.479e9,
+                      "kernel": "k_cgc_flow<1024>", "source_sha": "70a061faac5c7e7e",
+                      "capture": "profiles/flow_kernels_slabs.md"}}
 
 
 def kernel_source_sha():
@@ -508,7 +508,7 @@ def run_gb300(args):
         ach_ops = agg["pcg_ops"] / pcg_s / 1e9 if pcg_s > 0 else None
         ach_gbs = agg["pcg_bytes"] / pcg_s / 1e9 if pcg_s > 0 else None
         avg_ms = agg["pcg_ms"] / launches
-        r = {"kernel": "k_pcg_scaled / k_pcg* (restricted Jacobi-PCG, symmetrically scaled "
+        r = {"kernel": "k_pcg_flow / k_cgc_flow (restricted Jacobi-PCG, symmetrically scaled "
                        "form, one cooperative launch per node solve)",
              "bound": "alu", "achieved": ach_ops, "peak": alu_peak, "unit": "G FP64 lane-op/s",
              "frac": ach_ops / alu_peak if ach_ops else None,
