@@ -290,7 +290,7 @@ SIZE_CLASSES = ((1, 10_000, "<=10k rows"), (10_001, 300_000, "10k-300k rows"),
                 (300_001, 1 << 62, ">300k rows"))
 CG_SOURCES = ("step.cu", "cg_flow.cuh", "device_common.cuh")
 # DRAM traffic of the dominant kernel from one ncu capture (dram__bytes_read.sum +
-# dram__bytes_write.sum) of the first node solve of a slab step, all 442,401 rows, scaled to
+# dram__bytes_write.sum) of a node solve of the slab, all 442,401 rows, scaled to
 # the average launch by algorithmic bytes.  `source_sha` is the hash of the CG sources the
 # capture was taken with (kernel_source_sha()); once they change, the figure is withheld.
 ERR_NORM = ("max over ten checkpoints evenly spaced in the window (the last step included) of "
