@@ -288,7 +288,7 @@ FP64_LANES_PER_CYCLE = 304          # whole GPU, ncu dfma peak_sustained on GB30
 FP64_ISSUE_FRACTION = 0.84
 SIZE_CLASSES = ((1, 10_000, "<=10k rows"), (10_001, 300_000, "10k-300k rows"),
                 (300_001, 1 << 62, ">300k rows"))
-CG_SOURCES = ("step.cu", "cg_flow.cuh", "device_common.cuh")
+CG_SOURCES = ("step.cu", "cg_flow.cuh", "cg_window.cuh", "device_common.cuh")
 # DRAM traffic of the dominant kernel from one ncu capture (dram__bytes_read.sum +
 # dram__bytes_write.sum) of a node solve of the slab, all 442,401 rows, scaled to
 # the average launch by algorithmic bytes.  `source_sha` is the hash of the CG sources the

@@ -24,20 +24,15 @@
 // Integer addition is exact, so a total does not depend on the order of the arrivals, and
 // every CTA reads the same total.  The window holds 103 bits from kFlowHead bits above
 // the previous gamma down; a partial sum above it, or a total more than kFlowDrop bits
-// below the previous one, repeats the exchange with the exact largest exponents (the
-// start of a solve finds its window the same way).
+// below the previous one, repeats the exchange once with the exact largest exponents (the
+// start of a solve finds its window the same way).  The windows: cg_window.cuh.
 #pragma once
 
+#include "cg_window.cuh"
 #include "device_common.cuh"
 
 namespace sdc {
 namespace {
-
-typedef unsigned long long u64;
-
-constexpr int kFlowHead = 10;    // growth of gamma over one iteration that fits the window
-constexpr int kFlowSumHead = 18; // total over largest partial sum (155,648 threads, 2^103 units)
-constexpr int kFlowDrop = 22;    // fall of gamma up to which the sum keeps 2^-54 of its value
 
 // A published word: value, tag (12 bits of launch, 20 of iteration; the host clears the words
 // when the launch count wraps), 32 spare bits.  Stored and loaded as one relaxed
@@ -104,24 +99,6 @@ struct FlowShared {
     int fmax[64];
 };
 
-// v against a window whose largest exponent field is `top`: |v| = sum_k l[k] 2^(26 k) units
-// of 2^(top - 1125), truncated; false when v lies above the window.
-__device__ __forceinline__ bool flow_limbs(double v, int top, int (&l)[4]) {
-    const u64 bits = (u64)__double_as_longlong(v);
-    const int f = (int)(bits >> 52) & 0x7ff;
-    const u64 mant = (bits & 0xfffffffffffffull) | (f > 0 ? (1ull << 52) : 0ull);
-    const int sh = min(max(f, 1) - top + 50, 50);
-    const u64 lo = sh >= 0 ? mant << sh : mant >> min(-sh, 63);
-    const u64 hi = sh > 0 ? mant >> (64 - sh) : 0ull;
-    const int s = (int)((long long)bits >> 63);   // 0 or -1
-    constexpr unsigned m = (1u << 26) - 1u;
-    l[0] = ((int)((unsigned)lo & m) ^ s) - s;
-    l[1] = ((int)((unsigned)(lo >> 26) & m) ^ s) - s;
-    l[2] = ((int)((unsigned)((lo >> 52) | (hi << 12)) & m) ^ s) - s;
-    l[3] = ((int)(unsigned)(hi >> 14) ^ s) - s;
-    return f <= top;
-}
-
 // Post the CTA's sums of a and b to the words acc[0..7]: every thread calls it; it holds
 // one CTA barrier, after which warp 0 adds the warps' limbs and posts them.  A warp without
 // rows (warp 0 of a CTA with one row per thread) leaves its zeros of flow_scalars_init.
@@ -165,7 +142,6 @@ __device__ __forceinline__ void flow_post(double a, double b, bool rows, FlowSha
 // The rare ends of the paths below, kept out of line so that none of their long sequences is
 // executed speculatively.
 __device__ __noinline__ double flow_divide(double n, double d) { return n / d; }
-__device__ __noinline__ double flow_ldexp(double v, int e) { return ldexp(v, e); }
 __device__ __noinline__ bool flow_sqrt_at_most(double g, double thresh) { return sqrt(g) <= thresh; }
 
 // Quotient by Newton's iteration from the hardware's reciprocal estimate y (relative error
@@ -184,28 +160,6 @@ __device__ __forceinline__ double flow_quot(double n, double d) {
     return q;
 }
 
-// Total of a value's four limb sums in units of 2^(top - 1125), rounded once: the digits are
-// carried into A 2^52 + B with |A| < 2^51 and 0 <= B < 2^52, which integer additions place in
-// the significands of 1.5 2^52 + A and 2^52 + B.  in: false when the total has grown out of
-// that range (2^103 units).
-__device__ __forceinline__ double flow_value(long long s0, long long s1, long long s2, long long s3,
-                                             int top, bool& in) {
-    constexpr long long m = (1ll << 26) - 1;
-    s1 += s0 >> 26;
-    s2 += s1 >> 26;
-    s3 += s2 >> 26;
-    in = s3 < (1ll << 24) && s3 >= -(1ll << 24);
-    const double a = __longlong_as_double(0x4338000000000000ll + ((s3 << 26) + (s2 & m)));
-    const double b = __longlong_as_double(0x4330000000000000ll + (((s1 & m) << 26) + (s0 & m)));
-    const double v = fma(a - 0x1.8p52, 0x1p52, b - 0x1p52);
-    // times 2^(top - 1125), in the exponent field where the result is normal
-    const long long w = __double_as_longlong(v);
-    const int f = (int)(w >> 52) & 0x7ff, g = f + top - 1125;
-    if (f == 0) return 0.0;
-    if (g >= 1 && g <= 2046) return __longlong_as_double(w + ((long long)(top - 1125) << 52));
-    return flow_ldexp(v, top - 1125);
-}
-
 __device__ __forceinline__ void flow_scalars_init(FlowShared& S) {
     FlowScalars& Z = S.z;
     for (int k = threadIdx.x; k < 256; k += blockDim.x) S.lim[k >> 3][k & 7] = 0;
@@ -222,10 +176,10 @@ __device__ __forceinline__ void flow_scalars_init(FlowShared& S) {
 
 // Warp 0: wait for the sums posted to set `set`, derive alpha and beta (cg_scalars'
 // recurrences, den_t = delta_t - beta_t gamma_t / alpha_{t-1}) and the next windows.
-// exact: the windows came from the exact exponents (no repeat for a fall of gamma).
+// redo: the sum is repeated, in windows from the exact exponents.
 // HEAD, DROP: kFlowHead and kFlowDrop.  arrived() runs once the wait is over.
 template <int HEAD, int DROP, class A>
-__device__ __forceinline__ void flow_totals(FlowShared& S, const u64* acc, int set, int G, bool exact,
+__device__ __forceinline__ void flow_totals(FlowShared& S, const u64* acc, int set, int G, bool redo,
                                             long long budget, int* err, A&& arrived) {
     const int lane = threadIdx.x & 31;
     FlowScalars& Z = S.z;
@@ -274,17 +228,8 @@ __device__ __forceinline__ void flow_totals(FlowShared& S, const u64* acc, int s
     const bool above = __any_sync(0xffffffffu, lane < 2 && (!in || ((d[0] >> 48) & 0xff) != 0));
     const double g = __shfl_sync(0xffffffffu, tot, 0), dl = __shfl_sync(0xffffffffu, tot, 1);
     const int fg = xs_field(g);
-    // the decisions compare bit patterns (g >= 0): an FP64 comparison has 65 cycles latency
-    const long long gb = __double_as_longlong(g);
-    int state = 0;
-    if (above) {
-        state = 3;
-    } else if (nsum == 0) {
-        state = gb == 0 ? 1 : 0;
-    } else if (gb < hi) {
-        state = gb <= lo || flow_sqrt_at_most(g, Z.thresh) ? 1 : 0;
-    }
-    if (state == 0 && !exact && fg < topa - HEAD - DROP) state = 3;
+    const int state = flow_decide(above, redo, nsum == 0, g, dl, topa, HEAD + DROP, lo, hi,
+                                  [&] { return flow_sqrt_at_most(g, Z.thresh); });
     const double beta = g * inv_g;
     const double den = fma(-beta, g * inv_a, dl);
     const double alpha = flow_quot(g, den);
@@ -297,7 +242,7 @@ __device__ __forceinline__ void flow_totals(FlowShared& S, const u64* acc, int s
             S.alpha = alpha;
             S.beta = beta;
             Z.den = den;
-            S.topa = S.topb = min(fg + HEAD, 2046);
+            S.topa = S.topb = flow_next_top(fg, HEAD);
         }
     }
     if (lane < 2) {
@@ -341,11 +286,11 @@ __device__ __forceinline__ void flow_next(FlowShared& S, double rtol) {
 
 // Windows from the exact largest exponents of the CTAs' partial sums, with a release /
 // acquire grid barrier that also publishes every global write before it.  emax words hold
-// (generation << 32) | field and only grow.  The windows leave room for the
-// total over the largest partial sum.  Returns false after a timeout.
+// (generation << 32) | field and only grow.  guess: b is not what the next sum adds as delta
+// (the first of a solve), see kFlowGuessHead.  Returns false after a timeout.
 __device__ __forceinline__ bool flow_window(double a, double b, FlowShared& S, u64* emax,
                                             unsigned* bar, int G, unsigned& epoch, unsigned gen,
-                                            int headb, long long budget, int* err) {
+                                            bool guess, long long budget, int* err) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int fa = __reduce_max_sync(0xffffffffu, xs_field(a));
     const int fb = __reduce_max_sync(0xffffffffu, xs_field(b));
@@ -364,8 +309,8 @@ __device__ __forceinline__ bool flow_window(double a, double b, FlowShared& S, u
             S.ok = barrier_arrive_wait(bar, epoch, budget, err);
             const int ga = (int)(unsigned)ld_relaxed64(emax), gb = (int)(unsigned)ld_relaxed64(emax + 1);
             S.state = ga >= 2047 || gb >= 2047 ? 2 : 0;
-            S.topa = min(ga + kFlowSumHead, 2046);
-            S.topb = min(gb + headb, 2046);
+            S.topa = flow_exact_top(ga);
+            S.topb = guess ? flow_guess_top(gb) : flow_exact_top(gb);
             S.ovf = 0;
         }
     }
@@ -489,8 +434,7 @@ __device__ __forceinline__ bool flow_start(const CgParams& P, const FlowParams& 
         if (G == 1 && t == 0) raise_error(P.err, SDC_E_TIMEOUT);
         return false;
     }
-    // delta's partial sums: |w.r| of a thread <= |A| gamma, gamma <= 2^17.3 largest partial
-    if (!flow_window(ga, ga, S, Q.emax, Q.bar, G, epoch, 1u, 22, P.budget, P.err)) return false;
+    if (!flow_window(ga, ga, S, Q.emax, Q.bar, G, epoch, 1u, true, P.budget, P.err)) return false;
     if (S.state == 2) {
         if (Q.bidx == 0 && t == 0) raise_error(P.err, SDC_E_NONFINITE);
         return false;
@@ -621,7 +565,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
         return;
     int it = 0;
     unsigned npub = 0;
-    bool exact = true, redo = false;
+    bool redo = false;
     auto update_px = [&]() {
         flow_rows_px(nl, [&](int l) {
             const double p = ro[l] + beta * sp[l];
@@ -633,7 +577,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
         u64* const acc = Q.acc + 8 * (npub & 1);
         flow_post(ga, de, has_rows, S, acc);
         if (wid == 0)
-            flow_totals<kFlowHead, kFlowDrop>(S, acc, npub & 1, G, exact, P.budget, P.err, [] {});
+            flow_totals<kFlowHead, kFlowDrop>(S, acc, npub & 1, G, redo, P.budget, P.err, [] {});
         ++npub;
         if (!redo) {
             if (it > 0) update_px();
@@ -664,17 +608,16 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
         if (S.ok - 1 | S.state) {
             if (!S.ok) return;
             if (S.state == 3) {
-                if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, kFlowSumHead, P.budget,
-                                 P.err))
+                if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, false, P.budget, P.err))
                     return;
                 if (S.state == 0) {
-                    exact = redo = true;
+                    redo = true;
                     continue;
                 }
             }
             break;
         }
-        exact = redo = false;
+        redo = false;
         if (it >= P.maxit) {
             if (blockIdx.x == 0 && t == 0) raise_error(P.err, SDC_E_CG_NOCONV);
             break;
@@ -750,7 +693,7 @@ __device__ __forceinline__ void cgc_flow(const CgParams& P, const FlowParams& Q,
         return;
     int it = 0;
     unsigned npub = 0;
-    bool exact = true, redo = false;
+    bool redo = false;
     auto px_row = [&](const double* r, int l) {
         const double p = r[l] + beta * sp[l];
         sp[l] = p;
@@ -760,7 +703,7 @@ __device__ __forceinline__ void cgc_flow(const CgParams& P, const FlowParams& Q,
         u64* const acc = Q.acc + 8 * (npub & 1);
         flow_post(ga, de, has_rows, S, acc);
         if (wid == 0)
-            flow_totals<kFlowHead, kFlowDrop>(S, acc, npub & 1, G, exact, P.budget, P.err, [] {});
+            flow_totals<kFlowHead, kFlowDrop>(S, acc, npub & 1, G, redo, P.budget, P.err, [] {});
         ++npub;
         if (late && it > 0 && !redo) flow_rows_px(nl, [&](int l) { px_row(fb, l); });
         __syncthreads();
@@ -770,17 +713,16 @@ __device__ __forceinline__ void cgc_flow(const CgParams& P, const FlowParams& Q,
         if (S.ok - 1 | S.state) {
             if (!S.ok) return;
             if (S.state == 3) {
-                if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, kFlowSumHead, P.budget,
-                                 P.err))
+                if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, false, P.budget, P.err))
                     return;
                 if (S.state == 0) {
-                    exact = redo = true;
+                    redo = true;
                     continue;
                 }
             }
             break;
         }
-        exact = redo = false;
+        redo = false;
         if (it >= P.maxit) {
             if (Q.bidx == 0 && t == 0) raise_error(P.err, SDC_E_CG_NOCONV);
             break;
@@ -1135,7 +1077,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc2_flow(CgParams P, FlowParams Q,
     __syncthreads();
     int it = 0;
     unsigned npub = 0;
-    bool exact = true, redo = false;
+    bool redo = false;
     double ga, de, alpha = 0.0, beta = 0.0;
     auto px_row = [&](const double* u, int l) {
         const double p = u[l] + beta * sp[l];
@@ -1168,8 +1110,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc2_flow(CgParams P, FlowParams Q,
             }
             if (it == 0) {
                 // the windows of the first sums, from the exact exponents
-                if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, kFlowSumHead, P.budget,
-                                 P.err))
+                if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, false, P.budget, P.err))
                     return;
                 if (S.state == 2) break;
             }
@@ -1177,7 +1118,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc2_flow(CgParams P, FlowParams Q,
         u64* const acc = Q.acc + 8 * (npub & 1);
         flow_post(ga, de, has_rows, S, acc);
         if (wid == 0) {
-            flow_totals<kCoarseHead, kCoarseDrop>(S, acc, npub & 1, G, exact, P.budget, P.err,
+            flow_totals<kCoarseHead, kCoarseDrop>(S, acc, npub & 1, G, redo, P.budget, P.err,
                                                   [&] { flow_bar_arrive(2, B); });
         } else {
             if (!redo) {
@@ -1195,17 +1136,16 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc2_flow(CgParams P, FlowParams Q,
         if (S.ok - 1 | S.state) {
             if (!S.ok) return;
             if (S.state == 3) {
-                if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, kFlowSumHead, P.budget,
-                                 P.err))
+                if (!flow_window(ga, de, S, Q.emax, Q.bar, G, epoch, ++gen, false, P.budget, P.err))
                     return;
                 if (S.state == 0) {
-                    exact = redo = true;
+                    redo = true;
                     continue;
                 }
             }
             break;
         }
-        exact = redo = false;
+        redo = false;
         if (it >= P.maxit) {
             if (blockIdx.x == 0 && t == 0) raise_error(P.err, SDC_E_CG_NOCONV);
             break;

@@ -1,0 +1,114 @@
+"""The sums of the on-chip node solves where the partial sums of more than 131,072 threads are
+close to each other (spatially uniform states, slow trends), and at the top of the FP64 range.
+
+Tolerance: that of the parity tests, 1e-10 relative in the max norm (both sides stop at
+rtol = 1e-10).  A spatially uniform state stays uniform (K 1 = 0), so its step is that of a
+small mesh.
+"""
+
+import numpy as np
+import pytest
+
+import oracle
+from workloads.configs import AP_BENCH, Workload
+from workloads.meshes import grid2d
+
+pytestmark = pytest.mark.gpu
+
+RTOL = 1e-10
+
+
+@pytest.fixture(scope="module")
+def torch_dev():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2311_07206_gb300 import build as b
+    b.build()
+    return torch, torch.device("cuda:0")
+
+
+def _workload(nx, ny, v0):
+    mesh = grid2d(nx, ny, 0.3)
+    return Workload("grid", mesh, np.diag([1.0, 0.5, 1.0]), dict(AP_BENCH), M=2, dt=0.1, sweeps=2,
+                    tol=0.0, steps=1, v0=v0(mesh), w0=np.zeros(mesh.n_nodes))
+
+
+def _context(wl, torch, dev, **opts):
+    from paper_2311_07206_gb300 import Context, default_options
+    return Context.from_workload(wl, options=default_options(**opts),
+                                 stream=torch.cuda.current_stream(dev).cuda_stream)
+
+
+def _step(ctx, wl, v0, torch, dev):
+    v = torch.tensor(v0, dtype=torch.float64, device=dev)
+    w = torch.tensor(wl.w0, dtype=torch.float64, device=dev)
+    ctx.step(v, w, 0.0, wl.dt, wl.sweeps, wl.tol)
+    return v.cpu().numpy(), w.cpu().numpy()
+
+
+@pytest.mark.parametrize("pipelined", [0, 1])
+@pytest.mark.parametrize("nx,ny", [(456, 342), (666, 665)])   # 155,952 and 442,890 rows
+def test_uniform_states(torch_dev, nx, ny, pipelined):
+    torch, dev = torch_dev
+    wl = _workload(nx, ny, lambda m: np.full(m.n_nodes, 0.5))
+    small = _workload(3, 3, lambda m: np.full(m.n_nodes, 0.5))
+    S = oracle.System.from_mesh(small.mesh, small.sigma)
+    ctx = _context(wl, torch, dev, cg_pipelined=pipelined)
+    for amp in np.exp(np.linspace(np.log(0.2), np.log(0.9), 12)):
+        v, w = _step(ctx, wl, np.full(wl.n, amp), torch, dev)
+        r = S.step(small.ionic, small.M, np.full(9, amp), np.zeros(9), small.dt, small.sweeps, 0.0)
+        assert r["status"] == 0
+        assert np.abs(v - r["v"][4]).max() <= RTOL and np.abs(w - r["w"][4]).max() <= RTOL
+    ctx.close()
+
+
+@pytest.mark.parametrize("pipelined", [0, 1])
+def test_linear_trend(torch_dev, pipelined):
+    torch, dev = torch_dev
+    wl = _workload(456, 342, lambda m: 0.4 + 0.02 * m.xyz[:, 0] / m.xyz[:, 0].max())
+    S = oracle.System.from_mesh(wl.mesh, wl.sigma)
+    ctx = _context(wl, torch, dev, cg_pipelined=pipelined)
+    for amp in (1.0, 1.2, 1.5):
+        v, w = _step(ctx, wl, amp * wl.v0, torch, dev)
+        r = S.step(wl.ionic, wl.M, amp * wl.v0, wl.w0, wl.dt, wl.sweeps, 0.0)
+        assert r["status"] == 0
+        assert np.abs(v - r["v"]).max() <= RTOL and np.abs(w - r["w"]).max() <= RTOL
+    ctx.close()
+
+
+def _diagonal_solve(n, b, torch, dev):
+    """sdc_pcg_solve with the identity: x = b after one iteration."""
+    from paper_2311_07206_gb300 import binding
+    t = lambda a: torch.tensor(a, device=dev)
+    x = torch.zeros(n, dtype=torch.float64, device=dev)
+    it, rr = binding.pcg_solve(n, t(np.zeros(n)), t(np.zeros(n, np.int32)),
+                               t(np.zeros(n, np.int32)), n, 1, t(np.zeros(n)), t(np.ones(n)),
+                               t(np.zeros(n)), 1.0, t(b), x, rtol=1e-10, maxit=50,
+                               stream=torch.cuda.current_stream(dev).cuda_stream)
+    return it, x.cpu().numpy()
+
+
+@pytest.mark.parametrize("n", [131_072, 155_648, 442_401])
+def test_equal_right_hand_sides(torch_dev, n):
+    torch, dev = torch_dev
+    for amp in np.exp(np.linspace(0.0, np.log(2.0), 12)):
+        it, x = _diagonal_solve(n, np.full(n, amp), torch, dev)
+        assert it == 1 and np.abs(x - amp).max() <= RTOL
+
+
+@pytest.mark.parametrize("n", [5, 4_000, 200_000])
+def test_top_of_the_range(torch_dev, n):
+    """b'b of 2^1022.5 and 2^1023.5 is solved as any other; above 2^1024 the solve ends as not
+    finite."""
+    torch, dev = torch_dev
+    from paper_2311_07206_gb300 import SdcError
+    from paper_2311_07206_gb300 import binding as B
+    for e in (1000.0, 1022.5, 1023.5):
+        b = np.full(n, 2.0 ** (e / 2.0) / np.sqrt(n))
+        it, x = _diagonal_solve(n, b, torch, dev)
+        assert it == 1 and np.abs(x / b - 1.0).max() <= RTOL
+    for e in (1024.5, 1030.0):
+        with pytest.raises(SdcError) as err:
+            _diagonal_solve(n, np.full(n, 2.0 ** (e / 2.0) / np.sqrt(n)), torch, dev)
+        assert err.value.status == B.SDC_E_NONFINITE
