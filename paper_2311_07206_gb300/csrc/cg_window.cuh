@@ -103,8 +103,9 @@ SDC_HD int flow_guess_top(int f) { return flow_min(f + kFlowGuessHead, 2046); }
 // 3 repeat the sum in the windows of the partial sums' exact exponents.  above: a partial sum or
 // a total lies above its window.  A sum is repeated once at most: in the exact windows nothing
 // finite lies above.  first: no bound on gamma yet, and no window to fall below.
-// close(): sqrt(g) against its bound, where g lies between lo and hi (bit patterns, as the
-// comparisons are of g >= 0: an FP64 comparison has 65 cycles latency).
+// close(): sqrt(g) against its bound, where g lies between lo and hi (bit patterns: an FP64
+// comparison has 65 cycles latency).  A negative g, which rounding or an indefinite coarse matrix
+// can give r.u, is no convergence.
 template <class C>
 SDC_HD int flow_decide(bool above, bool repeated, bool first, double g, double d, int topa,
                        int fall, long long lo, long long hi, C&& close) {
@@ -114,7 +115,7 @@ SDC_HD int flow_decide(bool above, bool repeated, bool first, double g, double d
     if (flow_max(fg, fd) == 0x7ff) return 2;
     if (first) {
         if (gb == 0) return 1;
-    } else if (gb < hi) {
+    } else if (gb >= 0 && gb < hi) {
         if (gb <= lo || close()) return 1;
     }
     if (!repeated && !first && flow_max(fg, 1) < topa - fall) return 3;

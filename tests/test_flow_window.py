@@ -68,6 +68,19 @@ extern "C" int solve_sum(const double* a, const double* b, long n, int first, in
     return -1;
 }
 
+// The decision on a total alone: sqrt(g) <= thresh, with the kernels' band around thresh^2.
+extern "C" int decide(double g, double d, int first, int topa, int fall, double thresh, int* asked) {
+    const double q = thresh * thresh;
+    const bool normal = q > 1e-280 && q < 1e280;
+    const double lo = normal ? q * (1.0 - 0x1p-50) : 0.0, hi = normal ? q * (1.0 + 0x1p-50) : INFINITY;
+    *asked = 0;
+    return flow_decide(false, false, first != 0, g, d, topa, fall, (long long)flow_bits(lo),
+                       (long long)flow_bits(hi), [&] {
+                           *asked = 1;
+                           return std::sqrt(g) <= thresh;
+                       });
+}
+
 extern "C" void constants(int* c) {
     c[0] = kFlowHead;
     c[1] = kFlowDrop;
@@ -183,3 +196,28 @@ def test_signed_partials(lib):
         for got, v in ((g, a), (d, b)):
             want = sum(Fraction(float(x)) for x in v)
             assert abs(Fraction(got) - want) <= len(v) * Fraction(2) ** (top - 1125) + abs(want) / 2 ** 53
+
+
+def test_stopping_decision(lib):
+    """Converged exactly where 0 <= g and sqrt(g) <= thresh: negative totals, zero, the bound and
+    its neighbours, squares beyond the normal range; and a start at gamma = 0 only."""
+    lib.decide.argtypes = [C.c_double, C.c_double, C.c_int, C.c_int, C.c_int, C.c_double, C.c_void_p]
+    asked = C.c_int()
+
+    def decide(g, thresh, first=False):
+        return lib.decide(g, 1.0, int(first), 1, 10_000, thresh, C.addressof(asked))
+
+    for thresh in (1e-10, 0.37, 3.0, 1e-150, 1e150):
+        q = thresh * thresh
+        gs = [0.0, q, q / 4, q * 4, 5e-324, 1e300]
+        for k in (-2, -1, 1, 2):
+            gs += [q * (1.0 + k * 2.0 ** -52), q * (1.0 + k * 2.0 ** -49)]
+        for g in gs:
+            assert decide(g, thresh) == (1 if math.sqrt(g) <= thresh else 0), (g, thresh)
+            if g > 0.0:
+                assert decide(-g, thresh) == 0, (-g, thresh)
+    assert decide(0.0, 0.0) == 1 and decide(1e-300, 0.0) == 0
+    for g in (-1.0, -1e-300, 1e-300, 1.0):
+        assert decide(g, 1e10, first=True) == 0
+    assert decide(0.0, 1e10, first=True) == 1
+    assert decide(math.inf, 1.0) == 2 and decide(math.inf, 1.0, first=True) == 2
