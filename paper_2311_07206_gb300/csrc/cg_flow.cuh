@@ -205,12 +205,12 @@ __device__ __forceinline__ void flow_totals(FlowShared& S, const u64* acc, int s
             for (int k = 0; k < 4; ++k) here = here && ((v[k] + d[k]) >> 56) == (u64)G;
         }
         if (__all_sync(0xffffffffu, here)) break;
-        if (clock64() - t0 > budget) {
+        // (a vote: the lanes read different clocks, and must leave the loop together)
+        if (__any_sync(0xffffffffu, clock64() - t0 > budget)) {
             ok = 0;
             break;
         }
     }
-    ok = __all_sync(0xffffffffu, ok);
     if (!ok && lane == 0) {
         raise_error(err, SDC_E_TIMEOUT);
         S.ok = 0;

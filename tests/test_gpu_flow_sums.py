@@ -112,3 +112,33 @@ def test_top_of_the_range(torch_dev, n):
         with pytest.raises(SdcError) as err:
             _diagonal_solve(n, np.full(n, 2.0 ** (e / 2.0) / np.sqrt(n)), torch, dev)
         assert err.value.status == B.SDC_E_NONFINITE
+
+
+@pytest.mark.parametrize("blocks", [0, 1])
+@pytest.mark.parametrize("pipelined", [0, 1])
+def test_waits_that_run_out(torch_dev, pipelined, blocks):
+    """Budgets from one cycle to more than an exchange takes, so that barrier, words and sums run
+    out of time here and there: a step either reports SDC_E_TIMEOUT or gives the full result, on
+    the same context, whatever the steps before it did."""
+    torch, dev = torch_dev
+    from paper_2311_07206_gb300 import SdcError
+    from paper_2311_07206_gb300 import binding as B
+    wl = _workload(41, 37, lambda m: 0.5 + 0.3 * np.sin(m.xyz[:, 0]))
+    r = oracle.System.from_mesh(wl.mesh, wl.sigma).step(wl.ionic, wl.M, wl.v0, wl.w0, wl.dt,
+                                                        wl.sweeps, 0.0)
+    assert r["status"] == 0
+    done = timeouts = 0
+    for budget in (1, 300, 1_000, 2_000, 4_000, 10_000, 4_000_000_000):
+        ctx = _context(wl, torch, dev, cg_pipelined=pipelined, cg_max_blocks=blocks,
+                       spin_budget=budget)
+        for _ in range(6):
+            try:
+                v, w = _step(ctx, wl, wl.v0, torch, dev)
+            except SdcError as e:
+                assert e.status == B.SDC_E_TIMEOUT and budget < 4_000_000_000
+                timeouts += 1
+                continue
+            done += 1
+            assert np.abs(v - r["v"]).max() <= RTOL and np.abs(w - r["w"]).max() <= RTOL
+        ctx.close()
+    assert done >= 6 and (timeouts >= 1 or blocks == 1)
