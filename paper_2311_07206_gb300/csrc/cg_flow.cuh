@@ -141,24 +141,7 @@ __device__ __forceinline__ void flow_post(double a, double b, bool rows, FlowSha
 
 // The rare ends of the paths below, kept out of line so that none of their long sequences is
 // executed speculatively.
-__device__ __noinline__ double flow_divide(double n, double d) { return n / d; }
 __device__ __noinline__ bool flow_sqrt_at_most(double g, double thresh) { return sqrt(g) <= thresh; }
-
-// Quotient by Newton's iteration from the hardware's reciprocal estimate y (relative error
-// 2^-20): n y (1 + e + e^2), e = 1 - d y, within an ulp of n / d.  Operands near the ends of
-// the exponent range take the division.  Four FP64 operations (65 cycles each) where the
-// division takes 570 cycles.
-__device__ __forceinline__ double flow_quot(double n, double d) {
-    const int f = (int)((u64)__double_as_longlong(d) >> 52) & 0x7ff;
-    const int fn = (int)((u64)__double_as_longlong(n) >> 52) & 0x7ff;
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-    const double e = fma(-d, y, 1.0), q0 = n * y;
-    const double e2 = fma(e, e, e);
-    const double q = fma(q0, e2, q0);
-    if (min(f, fn) < 200 || max(f, fn) > 1846 || abs(fn - f) > 800) return flow_divide(n, d);
-    return q;
-}
 
 __device__ __forceinline__ void flow_scalars_init(FlowShared& S) {
     FlowScalars& Z = S.z;
@@ -232,7 +215,7 @@ __device__ __forceinline__ void flow_totals(FlowShared& S, const u64* acc, int s
                                   [&] { return flow_sqrt_at_most(g, Z.thresh); });
     const double beta = g * inv_g;
     const double den = fma(-beta, g * inv_a, dl);
-    const double alpha = flow_quot(g, den);
+    const double alpha = quot(g, den);
     // (a non-finite alpha shows in the next sums, whose exact exponents end the solve)
     if (lane == 0) {
         S.state = state;
@@ -270,7 +253,7 @@ __device__ __forceinline__ void flow_next(FlowShared& S, double rtol) {
     const int lane = threadIdx.x & 31;
     FlowScalars& Z = S.z;
     const double g = Z.g, den = Z.den;
-    const double q = flow_quot(lane == 0 ? 1.0 : den, g);   // lane 0: 1 / gamma, lane 1: 1 / alpha
+    const double q = quot(lane == 0 ? 1.0 : den, g);   // lane 0: 1 / gamma, lane 1: 1 / alpha
     const double e = fma(S.alpha, g, Z.energy);             // x' A x = sum of alpha_t gamma_t
     const int nsum = Z.nsum;
     __syncwarp();
