@@ -809,9 +809,6 @@ struct CoarseFlowParams {
     int width;                // (matrix rows on chip) slots of a row
 };
 
-// gamma = r.u is a sum of terms that cancel against each other within a block, so its window
-// leaves more room above (and repeats for smaller falls).
-constexpr int kCoarseHead = 24, kCoarseDrop = 8;
 // A piece's window: room of the sum over its largest term, growth of the largest term since
 // the last sum, and its fall up to which the window keeps 57 bits of it.
 constexpr int kPieceHead = 16, kPieceGrow = 10, kPieceFall = 20;

@@ -25,7 +25,15 @@ constexpr int kFlowSumHead = 18; // total over largest partial sum: at most 2^18
                                  // of a window this far above the largest, so below 2^103
 constexpr int kFlowGuessHead = 22; // first delta over gamma's largest partial: |w.r| of a thread
                                    // <= |A| gamma, gamma <= 2^18 largest partials
-constexpr int kFlowDrop = 22;    // fall of gamma up to which the sum keeps 2^-54 of its value
+// Fall of gamma up to which its window serves.  2^17.3 partials truncated at 2^(head - 102) of the
+// gamma before it are off by 2^-74.7, and 2^-60.7 of a gamma 2^14 below it: less than the
+// partials' own rounding leaves in gamma, and in delta (2^-53 gamma over the root of the terms).
+// Slabs, squares and shells fall by 2^2 to 2^6 an iteration; no case took longer than with 2^22.
+constexpr int kFlowDrop = 14;
+// The same for the two-level solves' gamma = r.u, a sum of terms that cancel against each other
+// within a block: more room above, and a repeat for smaller falls (131k rows: no time, and the
+// same bits as with 24 and 8).
+constexpr int kCoarseHead = 20, kCoarseDrop = 4;
 
 SDC_HD u64 flow_bits(double v) {
 #ifdef __CUDA_ARCH__

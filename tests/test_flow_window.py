@@ -81,9 +81,21 @@ extern "C" int decide(double g, double d, int first, int topa, int fall, double 
                        });
 }
 
+// The limb sums of v in the window `top`: the total before it is rounded.
+extern "C" void limb_sums(const double* v, long n, int top, long long* s) {
+    for (int m = 0; m < 4; ++m) s[m] = 0;
+    for (long k = 0; k < n; ++k) {
+        int l[4];
+        flow_limbs(v[k], top, l);
+        for (int m = 0; m < 4; ++m) s[m] += l[m];
+    }
+}
+
 extern "C" void constants(int* c) {
     c[0] = kFlowHead;
     c[1] = kFlowDrop;
+    c[2] = kCoarseHead;
+    c[3] = kCoarseDrop;
 }
 """
 
@@ -99,14 +111,15 @@ def lib(tmp_path_factory):
     return C.CDLL(str(so))
 
 
-def _sum(lib, a, b, first=True, prev=0):
-    c = (C.c_int * 2)()
+def _sum(lib, a, b, first=True, prev=0, coarse=False):
+    c = (C.c_int * 4)()
     lib.constants(c)
     a = np.ascontiguousarray(a, dtype=np.float64)
     b = np.ascontiguousarray(b, dtype=np.float64)
     g, d, rep = C.c_double(), C.c_double(), C.c_int()
     p = lambda x: x.ctypes.data_as(C.c_void_p)
-    st = lib.solve_sum(p(a), p(b), C.c_long(len(a)), int(first), prev, c[0], c[1], C.byref(g),
+    st = lib.solve_sum(p(a), p(b), C.c_long(len(a)), int(first), prev, c[2 * coarse], c[2 * coarse + 1],
+                       C.byref(g),
                        C.byref(d), C.byref(rep))
     return st, g.value, d.value, rep.value
 
@@ -221,3 +234,27 @@ def test_stopping_decision(lib):
         assert decide(g, 1e10, first=True) == 0
     assert decide(0.0, 1e10, first=True) == 1
     assert decide(math.inf, 1.0) == 2 and decide(math.inf, 1.0, first=True) == 2
+
+
+@pytest.mark.parametrize("coarse", [False, True])
+def test_sums_after_a_fall_of_gamma(lib, coarse):
+    """gamma 2^1 to 2^40 below the one its window came from, partials over ten orders of
+    magnitude on the largest grid of each kernel.  Bound, before the total is rounded: a unit a
+    partial, 2^17.3 2^(10 - 102 + 14) = 2^-60.7 of the total for one row a thread, 2^16.8
+    2^(20 - 102 + 4) = 2^-61.2 for the two-level kernel; 2^-60."""
+    n = 111_872 if coarse else 155_648
+    rng = np.random.default_rng(5)
+    c = (C.c_int * 4)()
+    lib.constants(c)
+    for fall in (1, 3, 4, 5, 9, 13, 14, 15, 20, 21, 22, 23, 40):
+        a = np.exp(rng.uniform(-23.0, 0.0, n))
+        exact = sum(int(math.ldexp(x, 120)) for x in a)
+        prev = 1023 + int(math.floor(math.log2(exact))) - 120 + fall
+        st, g, d, rep = _sum(lib, a, -a, False, prev, coarse)
+        assert st == 0 and rep <= 1 and d == -g
+        assert abs(g - math.fsum(a)) <= np.spacing(g)
+        top = prev + c[2 * coarse] if rep == 0 else int(np.frexp(a.max())[1]) + 1022 + 18
+        limbs = (C.c_longlong * 4)()
+        lib.limb_sums(a.ctypes.data_as(C.c_void_p), C.c_long(n), top, limbs)
+        got = sum(x << (26 * k) for k, x in enumerate(limbs)) << (top - 1125 + 120)
+        assert 0 <= exact - got and (exact - got) << 60 <= exact, (fall, rep)
