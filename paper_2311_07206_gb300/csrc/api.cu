@@ -590,6 +590,12 @@ sdc_status create_impl(sdc_ctx** out, const sdc_mesh* mesh, const sdc_ionic* ion
             return fail(nullptr, (sdc_status)rc, "%s", why.c_str());
         }
     }
+    // what the node solves' launch rule asks of the matrix
+    c->pcg.row_slots = (double)(c->K.nnz - c->N) / c->N + (emi ? 2.0 * emi->n_pairs / c->N : 0.0);
+    unsigned long long* words = nullptr;
+    if (c->inst_off.empty() && c->N > kFlowClassicalRows && dalloc(&words, 2))
+        c->pcg.scattered = columns_scattered(c->N, c->K.K, c->pcg.sms, 1, words, c->stream);
+    cudaFree(words);
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) {
         sdc_status st = cuda_fail(nullptr, "sdc_create");
         free_all(c);
@@ -1403,16 +1409,25 @@ static sdc_status pcg_solve_body(int n, const double* d_val, const int* d_col, c
     int h[3] = {0, 0, 0};   // -, error, iterations
     double hr = 0.0;
     const size_t fd = pcg_standalone_flow_doubles(n, ld, width, maxit);
-    if (fd > 0) {
-        SolveWorkspace ws(fd * sizeof(double), s);
-        if (!ws.p) return fail(nullptr, SDC_E_NOMEM, "sdc_pcg_solve: workspace allocation failed");
+    const bool asks = fd > 0 && pcg_standalone_asks(n, width);
+    const int block = 256;
+    const int maxb = fd == 0 || asks ? pcg_max_blocks(block) : 0;
+    // workspace of the kernels with global vectors: 8 vectors of n, the published m in two
+    // buffers ld apart (the kernels offset the second by the matrix's ld), 12 * maxb for the
+    // partial-sum records (16-byte aligned: they are read with 16-byte loads), then the scalars
+    const size_t po = ((size_t)8 * n + 2 * (size_t)ld + 1) & ~(size_t)1;
+    const size_t nd = maxb > 0 ? po + 12 * (size_t)maxb + 2 + 8 : 0;
+    SolveWorkspace ws(std::max(fd, nd) * sizeof(double), s);
+    if (!ws.p) return fail(nullptr, SDC_E_NOMEM, "sdc_pcg_solve: workspace allocation failed");
+    double* v = (double*)ws.p;
+    if (fd > 0 &&
+        !(asks && columns_scattered(n, A, pcg_sm_count(), 64, (unsigned long long*)ws.p, s))) {
         double r[kStandaloneResults];
         if (launch_pcg_standalone_flow(n, A, d_kdiag, d_mass, d_J, c, d_b, d_x, rtol, maxit,
-                                       4000000000LL, (double*)ws.p, s) != SDC_OK) {
+                                       4000000000LL, v, s) != SDC_OK) {
             status = cuda_fail(nullptr, "sdc_pcg_solve launch");
         } else {
-            cudaMemcpyAsync(r, (double*)ws.p + fd - kStandaloneResults, sizeof r,
-                            cudaMemcpyDeviceToHost, s);
+            cudaMemcpyAsync(r, v + fd - kStandaloneResults, sizeof r, cudaMemcpyDeviceToHost, s);
             if (cudaStreamSynchronize(s) != cudaSuccess) {
                 status = cuda_fail(nullptr, "sdc_pcg_solve");
             } else {
@@ -1427,17 +1442,6 @@ static sdc_status pcg_solve_body(int n, const double* d_val, const int* d_col, c
         if (relres) *relres = hr;
         return (sdc_status)status;
     }
-    const int block = 256;
-    const int maxb = pcg_max_blocks(block);
-    // workspace: 8 vectors of n, the published m in two buffers ld apart (the kernels
-    // offset the second by the matrix's ld), 12 * maxb for the partial-sum records
-    // (16-byte aligned: they are read with 16-byte loads), then the scalars
-    const size_t po = ((size_t)8 * n + 2 * (size_t)ld + 1) & ~(size_t)1;
-    const size_t nd = po + 12 * (size_t)maxb + 2;
-    char* ws = nullptr;
-    if (cudaMalloc(&ws, nd * sizeof(double) + 64) != cudaSuccess)
-        return fail(nullptr, SDC_E_NOMEM, "sdc_pcg_solve: workspace allocation failed");
-    double* v = (double*)ws;
     PcgScratch w;
     w.r = v; w.u = v + n; w.p = v + 2 * (size_t)n; w.s = v + 3 * (size_t)n;
     w.w = v + 4 * (size_t)n; w.idA = v + 5 * (size_t)n;
@@ -1464,7 +1468,6 @@ static sdc_status pcg_solve_body(int n, const double* d_val, const int* d_col, c
     }
     if (iters) *iters = h[2];
     if (relres) *relres = hr;
-    cudaFree(ws);
     return (sdc_status)status;
 }
 

@@ -201,6 +201,7 @@ constexpr int kClusterVectors = 10; // per-row doubles in shared memory, cluster
 constexpr int kClusterRows = 2848;  // rows per CTA of the cluster variant
 constexpr int kSmemVectorsC = 6;    // classical arrangement, shared-memory form
 constexpr int kSmemRowsC = 4768;
+constexpr int kSmemVectorsCS = 4;   // the scaled classical shared-memory variant (kSmemRowsC rows)
 struct PcgConfig {
     int block = 256;                // block size of the general variant
     int max_blocks_general = 0;     // cooperative grid limit of the general variant
@@ -222,6 +223,8 @@ struct PcgConfig {
     int scaled = 1;                 // solves in the scaled form
     int general_classical = 0;      // pipelined contexts: classical arrangement for the
                                     // global-vector variant (automatic choice)
+    double row_slots = 0;           // off-diagonals of a row, on average
+    bool scattered = false;         // most columns lie outside their row's CTA (columns_scattered)
     long long budget = 0;
 };
 int launch_pcg(int n, const Ell& A, int m, double dt, const Coll& co, double rtol, int maxit,
@@ -411,6 +414,9 @@ int launch_pcg_standalone(int n, const Ell& A, const double* kdiag, const double
 // rows do not fit on chip; the last kStandaloneResults of them are the results: relres, then
 // error code and iterations (ints).
 constexpr int kStandaloneResults = 2;
+bool columns_scattered(int n, const Ell& A, int sms, int stride, unsigned long long* words,
+                       cudaStream_t s);
+bool pcg_standalone_asks(int n, int width);
 size_t pcg_standalone_flow_doubles(int n, int ld, int width, int maxit, size_t* zero_at = nullptr);
 int launch_pcg_standalone_flow(int n, const Ell& A, const double* kdiag, const double* mass,
                                const double* J, double c, const double* b, double* x, double rtol,

@@ -1609,6 +1609,136 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcgc_batch(CgParams P, const SegBlo
                seg_relres + g.seg);
 }
 
+// Shared-memory form of pcgc_group_scaled: rows as in k_pcgc_smem, r, p, s, w on
+// chip (four vectors), r published for the neighbours' products.
+template <int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) k_pcgc_scaled(CgParams P) {
+    extern __shared__ double sm[];
+    __shared__ CgShared S;
+    const int G = gridDim.x, B = blockDim.x, t = threadIdx.x;
+    const int L = P.L, ld = P.ld;
+    const int r0 = blockIdx.x * L;
+    const int nl = max(0, min(P.n - r0, L));
+    double* __restrict__ sr = sm;
+    double* __restrict__ sp = sm + L;
+    double* __restrict__ ss = sm + 2 * L;
+    double* __restrict__ sw = sm + 3 * L;
+    double* __restrict__ ug = P.u;
+    double* __restrict__ xg = P.x;
+    double* __restrict__ sg = P.sv;
+    double* __restrict__ sval = P.sval;
+    const double* __restrict__ aval = P.aval;
+    const int* __restrict__ acol = P.acol;
+    const int* __restrict__ alen = P.alen;
+    const double c = P.c;
+    unsigned epoch = 0;
+    int buf = 0;
+
+    for (int l = t; l < nl; l += B) {
+        const int i = r0 + l;
+        const double d = P.mc[i] * (1.0 + c * P.J[i]) + c * P.kdc[i];
+        double si = 0.0;
+        if (!isfinite(d)) raise_error(P.err, SDC_E_NONFINITE);
+        else if (!(d > 0.0)) raise_error(P.err, SDC_E_DOMAIN);
+        else si = rsqrt(d);
+        sg[i] = si;
+        const double r = si * P.b[i];
+        sr[l] = r;
+        ug[i] = r;
+        sp[l] = 0.0;
+        ss[l] = 0.0;
+        xg[i] = 0.0;
+    }
+    if (P.inject_fault && blockIdx.x == G - 1) {
+        if (G == 1 && t == 0) raise_error(P.err, SDC_E_TIMEOUT);
+        return;
+    }
+    if (!grid_barrier(P.bar, epoch, P.budget, P.err, &S.ok)) return;
+    // scaled rows: written and read back by the same thread (same row mapping in every loop)
+    for (int l = t; l < nl; l += B) {
+        const int i = r0 + l;
+        const int len = __ldg(alen + i);
+        const double csi = c * __ldcg(sg + i);
+        for (int k = 0; k < len; ++k) {
+            const size_t q = (size_t)k * ld + i;
+            sval[q] = csi * __ldg(aval + q) * __ldcg(sg + sdc_idx(__ldg(acol + q), P.n, 45));
+        }
+    }
+    XsRecord* const rec = reinterpret_cast<XsRecord*>(P.part);
+    int it = 0, nsum = 0;
+    while (true) {
+        double ga = 0.0, de = 0.0;
+        for (int l = t; l < nl; l += B) {
+            const int i = r0 + l;
+            const int len = __ldg(alen + i);
+            const double ri = sr[l];
+            double acc = ri;
+            for (int k = 0; k < len; ++k) {
+                const size_t q = (size_t)k * ld + i;
+                acc += sval[q] * __ldcg(ug + sdc_idx(__ldg(acol + q), P.n, 46));
+            }
+            sw[l] = acc;
+            ga += ri * ri;
+            de += acc * ri;
+        }
+        if (!cg_publish_arrive(ga, de, S, rec + buf * G, P.bar, G, (int)blockIdx.x, epoch,
+                               P.budget, P.err))
+            return;
+        if (t < 64) {
+            double g, d;
+            xs_group_total(G, [&](int k) { return xs_load_cg(rec + buf * G + k); }, S.xs, g, d);
+            if ((t & 31) == 0) cg_scalars(S, t >> 5, nsum, g, d, P.rtol);
+        }
+        __syncthreads();
+        ++nsum;
+        buf ^= 1;
+        if (S.state != 0) break;
+        if (it >= P.maxit) {
+            if (blockIdx.x == 0 && t == 0) raise_error(P.err, SDC_E_CG_NOCONV);
+            break;
+        }
+        ++it;
+        const double alpha = S.alpha, beta = S.beta;
+        for (int l = t; l < nl; l += B) {
+            const double ri = sr[l];
+            const double pi = ri + beta * sp[l];
+            const double s_i = sw[l] + beta * ss[l];
+            sp[l] = pi;
+            ss[l] = s_i;
+            xg[r0 + l] += alpha * pi;
+            const double r = ri - alpha * s_i;
+            sr[l] = r;
+            ug[r0 + l] = r;
+        }
+        if (!grid_barrier(P.bar, epoch, P.budget, P.err, &S.ok)) return;
+    }
+    if (S.state == 2) {
+        if (blockIdx.x == 0 && t == 0) raise_error(P.err, SDC_E_NONFINITE);
+        return;
+    }
+    if (blockIdx.x == 0 && t == 0) {
+        *P.iters_out = it;
+        *P.relres_out = cg_relres(S);
+        if (P.energy_out) *P.energy_out = S.energy;
+    }
+    for (int l = t; l < nl; l += B) {
+        const int i = r0 + l;
+        xg[i] = __ldcg(sg + i) * __ldcg(xg + i);
+    }
+    if (P.epi_lo < P.epi_hi) {
+        if (!grid_barrier(P.bar, epoch, P.budget, P.err, &S.ok)) return;
+        for (int l = t; l < nl; l += B) {
+            const int i = r0 + l;
+            const int len = __ldg(alen + i);
+            const double xi = __ldcg(xg + i);
+            double acc = 0.0;
+            for (int k = 0; k < len; ++k)
+                acc += __ldg(aval + (size_t)k * ld + i) * __ldcg(xg + sdc_idx(__ldg(acol + (size_t)k * ld + i), P.n, 47));
+            cg_couple_row(P, i, xi, acc);
+        }
+    }
+}
+
 // Shared-memory form of the classical arrangement (rows as in k_pcg_smem;
 // r, u, p, s, w and the reciprocal diagonal on chip, u published).
 template <int MAXT>
@@ -2018,6 +2148,9 @@ PcgKernel pcg_general_kernel(int block) {
     return block > 512 ? k_pcg<1024> : block > 256 ? k_pcg<512> : k_pcg<256>;
 }
 PcgKernel pcg_smem_kernel(int block) { return block > 512 ? k_pcg_smem<1024> : k_pcg_smem<512>; }
+PcgKernel pcgc_scaled_kernel(int block) {
+    return block > 512 ? k_pcgc_scaled<1024> : k_pcgc_scaled<512>;
+}
 using FlowKernel = void (*)(CgParams, FlowParams);
 FlowKernel flow_kernel(int block, bool classical) {
     if (classical)
@@ -2055,6 +2188,9 @@ void pcg_smem_attrs() {
     for (PcgKernel k : {k_pcgc_smem<512>, k_pcgc_smem<1024>})
         cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(kSmemVectorsC * kSmemRowsC * sizeof(double)));
+    for (PcgKernel k : {k_pcgc_scaled<512>, k_pcgc_scaled<1024>})
+        cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(kSmemVectorsCS * kSmemRowsC * sizeof(double)));
     for (FlowKernel k : {k_pcg_flow<512>, k_pcg_flow<768>, k_pcg_flow<1024>, k_cgc_flow<512>,
                          k_cgc_flow<768>, k_cgc_flow<1024>})
         cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2353,6 +2489,29 @@ int launch_pcg_role(int n, const Ell& A, const PcgRole& role, double dt, int M, 
     return launch_pcg_params(P, c2, B, s);
 }
 
+// What an iteration of the flow kernels reads again through L2: the matrix (12 bytes a slot) and
+// both buffers of published words.  Once that overflows L2 (129 MB in two halves) the kernels with
+// 8-byte words and nothing but vectors of their own are faster, the earlier the more columns
+// are other CTAs'.  us per iteration, full sets: classical flow / k_pcgc_scaled (to 724k rows) or
+// k_pcgcs (above), with the working set in MB:
+//   7-point slabs: 680k (70) 17.5 / 21.8, 834k (88) 27.2 / 28.9, 1.0M (103) 40.9 / 36.0
+//   full-tensor slabs: 442k (86) 20.8 / 21.2, 680k (132) 61.5 / 38.8, 1.0M (195) 80.5 / 56.3
+//   tissue meshes in Morton order: 376k (73) 21.2 / 21.5, 455k (88) 26.3 / 24.3, 497k (96) 38.4 / 30.3,
+//     550k (106) 51.7 / 30.0, 686k (133) 65.0 / 41.3, 1.0M (195) 91.2 / 57.8
+//   the same, randomly numbered: 376k (73) 29.9 / 30.2, 455k (88) 41.4 / 35.3, 686k (132) 125 / 57,
+//     1.0M (195) 177 / 76; cell-by-cell, 847k (90): 325 / 364 ms a step
+// The pipelined flow form, asked for, is the faster to its capacity but for scattered columns (455k
+// 22.4 / 29.5 in Morton order, 54.6 / 39.7 randomly numbered).  Scattered: three of four columns
+// further from the diagonal than a CTA's rows.
+constexpr double kFlowCache = 92e6, kFlowCacheWide = 80e6;   // wide rows or scattered columns
+double flow_working_set(int n, double row_slots) { return n * (12.0 * row_slots + 32.0); }
+bool flow_in_cache(int n, const PcgConfig& cfg) {
+    if (cfg.variant == 2) return true;   // on chip whenever the rows fit
+    if (cfg.pipelined && !cfg.general_classical && !cfg.scattered) return true;
+    return flow_working_set(n, cfg.row_slots) <=
+           (cfg.scattered || cfg.row_slots > 10.0 ? kFlowCacheWide : kFlowCache);
+}
+
 // Shape of a flow launch: rows per CTA, CTAs, threads, shared memory; false when the rows
 // do not fit on chip.  Up to 28 chunks of 32 rows a CTA has one row per thread, warp 0 apart,
 // and its rows are a multiple of 128: FP64 issue is what a full warp per sub-partition
@@ -2428,9 +2587,14 @@ int launch_pcg_params(CgParams& P, const PcgConfig& cfg, StepBuffers& B, cudaStr
     // the exact-sum records are read with 16-byte loads
     if (reinterpret_cast<uintptr_t>(P.part) % 16 != 0) return SDC_E_INVALID;
     FlowShape fs;
+    // (scattered columns: the pipelined form hides their latency; randomly numbered tissue, classical /
+    // pipelined: 140k 11.0 / 10.3, 212k 17.2 / 15.6, 302k 21.5 / 20.9, 376k 32.7 / 25.9)
     const bool flow_classical =
-        !cfg.pipelined || (cfg.general_classical && n > kFlowClassicalRows);
-    if (cfg.variant != 1 && cfg.scaled && P.sv && P.sval && B.pub && P.maxit < kFlowMaxit &&
+        !cfg.pipelined ||
+        (cfg.general_classical && n > kFlowClassicalRows && !cfg.scattered);
+    const bool scaled = cfg.scaled && P.sv && P.sval;
+    const bool in_cache = flow_in_cache(n, cfg);
+    if (cfg.variant != 1 && scaled && B.pub && P.maxit < kFlowMaxit && in_cache &&
         flow_shape(n, flow_classical, cfg, fs)) {
         unsigned long long* words = B.flow + (size_t)B.flow_set * kFlowWords;
         unsigned long long* other = B.flow + (size_t)(B.flow_set ^ 1) * kFlowWords;
@@ -2443,7 +2607,7 @@ int launch_pcg_params(CgParams& P, const PcgConfig& cfg, StepBuffers& B, cudaStr
     // automatic arrangement: the pipelined form pays off where the vectors live on chip;
     // for the global-vector variant (solves above the on-chip capacity) its extra vector
     // traffic outweighs the saved synchronisation
-    const bool on_chip = cfg.variant != 1 && n <= cfg.sms * kSmemRows;
+    const bool on_chip = cfg.variant != 1 && !(scaled && !in_cache) && n <= cfg.sms * kSmemRows;
     if (!cfg.pipelined || (cfg.general_classical && !on_chip)) {
         // classical arrangement: shared-memory form when it fits, else global vectors
         if (cfg.variant != 1 && n <= cfg.sms * kSmemRowsC) {
@@ -2456,8 +2620,9 @@ int launch_pcg_params(CgParams& P, const PcgConfig& cfg, StepBuffers& B, cudaStr
             const int blk = n >= cfg.big_rows ? 1024 : cfg.smem_block;
             pcg_smem_attrs();
             cudaError_t e = cudaLaunchCooperativeKernel(
-                (const void*)pcgc_smem_kernel(blk), dim3(grid), dim3(blk), args,
-                (size_t)kSmemVectorsC * P.L * sizeof(double), s);
+                (const void*)(scaled ? pcgc_scaled_kernel(blk) : pcgc_smem_kernel(blk)), dim3(grid),
+                dim3(blk), args,
+                (size_t)(scaled ? kSmemVectorsCS : kSmemVectorsC) * P.L * sizeof(double), s);
             return e == cudaSuccess ? SDC_OK : SDC_E_CUDA;
         }
         int grid = std::min(cfg.max_blocks_general, nblk(n, cfg.block));
@@ -2469,7 +2634,7 @@ int launch_pcg_params(CgParams& P, const PcgConfig& cfg, StepBuffers& B, cudaStr
         return e == cudaSuccess ? SDC_OK : SDC_E_CUDA;
     }
     // cluster variant: one cluster of cfg.cluster CTAs for small active sets
-    if (cfg.variant != 1 && cfg.cluster > 0 && !cfg.inject_fault && n <= cfg.cluster_rows &&
+    if (on_chip && cfg.cluster > 0 && !cfg.inject_fault && n <= cfg.cluster_rows &&
         n <= cfg.cluster * kClusterRows) {
         pcg_smem_attrs();
         // enough CTAs for the FP64 work, never more rows per CTA than fit
@@ -2493,8 +2658,7 @@ int launch_pcg_params(CgParams& P, const PcgConfig& cfg, StepBuffers& B, cudaStr
         return e == cudaSuccess ? SDC_OK : SDC_E_CUDA;
     }
     // shared-memory variant: one block per SM at most, each owning <= kSmemRows rows
-    const bool smem_ok = cfg.variant != 1 && n <= cfg.sms * kSmemRows;
-    if (smem_ok && cfg.variant != 1) {
+    if (on_chip) {
         const int rpb = cfg.rows_per_block > 0 ? cfg.rows_per_block : kSmemRowsDefault;
         int grid = std::max(nblk(n, kSmemRows), nblk(n, rpb));
         grid = std::min(grid, cfg.sms);
@@ -2859,6 +3023,47 @@ int launch_pcg_batch_planned(const Ell& A, int m, double dt, const Coll& co, dou
                                       cfg.scaled && P.sv && P.sval),
         dim3(G), dim3(cfg.batch_block), args, 0, s);
     return e == cudaSuccess ? SDC_OK : SDC_E_CUDA;
+}
+
+// Columns further than `far` from the diagonal, and all, over every stride-th row.
+__global__ void k_count_far(int n, const int* __restrict__ col, const int* __restrict__ len, int ld,
+                            int far, int stride, unsigned long long* __restrict__ out) {
+    const long long i = (long long)(blockIdx.x * blockDim.x + threadIdx.x) * stride;
+    int c = 0, all = 0;
+    if (i < n) {
+        const int l = len[i], step = (l + 15) / 16;   // up to sixteen slots of a row
+        for (int k = 0; k < l; k += step, ++all)
+            c += abs(col[(size_t)k * ld + i] - (int)i) >= far;
+    }
+    c = __reduce_add_sync(0xffffffffu, c);
+    all = __reduce_add_sync(0xffffffffu, all);
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(out, (unsigned long long)c);
+        atomicAdd(out + 1, (unsigned long long)all);
+    }
+}
+
+// Whether three of four columns lie further from the diagonal than the rows of one of `sms`
+// CTAs; words: two of device memory.  Synchronises the stream.
+bool columns_scattered(int n, const Ell& A, int sms, int stride, unsigned long long* words,
+                       cudaStream_t s) {
+    unsigned long long h[2] = {0, 0};
+    if (sms < 1 || cudaMemsetAsync(words, 0, sizeof h, s) != cudaSuccess) return false;
+    k_count_far<<<nblk(nblk(n, stride), 256), 256, 0, s>>>(n, A.col, A.len, A.ld, nblk(n, sms), stride,
+                                                          words);
+    if (cudaMemcpyAsync(h, words, sizeof h, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+        return false;
+    return 4 * h[0] > 3 * h[1];
+}
+
+// A stand-alone solve of this size asks columns_scattered: the kernel with global vectors is faster
+// for scattered ones then (randomly numbered tissue, us per iteration on chip / in global memory: 455k rows
+// 42.9 / 55.2, 550k 71.1 / 67.9, 686k 131 / 83, 1.0M 186 / 119; random rows of 32 slots, 300k
+// 66.1 / 63.1; full-tensor slabs 680k 61 / 72, 1.0M 84 / 109).  With few rows a CTA it is not: random rows
+// of 200 slots, 60k 76 / 94, of 600, 20k 128 / 236.
+bool pcg_standalone_asks(int n, int width) {
+    return n > 200000 && flow_working_set(n, width) > 100e6;
 }
 
 // Stand-alone solves run in the flow kernels while the rows fit on chip.
