@@ -1408,7 +1408,7 @@ static sdc_status pcg_solve_body(int n, const double* d_val, const int* d_col, c
     int status = SDC_OK;
     int h[3] = {0, 0, 0};   // -, error, iterations
     double hr = 0.0;
-    const size_t fd = pcg_standalone_flow_doubles(n, ld, width, maxit);
+    const size_t fd = pcg_standalone_flow_doubles(n, ld, width);
     const bool asks = fd > 0 && pcg_standalone_asks(n, width);
     const int block = 256;
     const int maxb = fd == 0 || asks ? pcg_max_blocks(block) : 0;

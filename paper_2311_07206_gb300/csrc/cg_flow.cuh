@@ -36,7 +36,9 @@ namespace {
 
 // A published word: value, tag (12 bits of launch, 20 of iteration; the host clears the words
 // when the launch count wraps), 32 spare bits.  Stored and loaded as one relaxed
-// single-copy-atomic 128-bit access.
+// single-copy-atomic 128-bit access.  The iteration may wrap: every word is overwritten two
+// iterations later, so the only stale one is that of k - 2.
+__device__ __forceinline__ unsigned flow_tag(unsigned id, unsigned k) { return id | (k & 0xfffffu); }
 __device__ __forceinline__ void pub_store(ulonglong2* p, double v, unsigned tag) {
     asm volatile("{ .reg .b128 t; mov.b128 t, {%1, %2}; st.relaxed.gpu.global.b128 [%0], t; }" ::"l"(p),
                  "l"((u64)__double_as_longlong(v)), "l"((u64)tag)
@@ -477,7 +479,7 @@ __device__ __forceinline__ void flow_finish(const CgParams& P, const FlowParams&
     }
     // the words of iteration it - 1, whose readers are done: their CTAs posted sum `it`
     ulonglong2* const pub = Q.pub + (size_t)((it + 1) & 1) * ld;
-    const unsigned tag = Q.id + (unsigned)it + 2;
+    const unsigned tag = flow_tag(Q.id, it + 2u);
     const bool couple = P.epi_lo < P.epi_hi;
     flow_rows(nl, [&](int l) {
         const int i = r0 + l;
@@ -564,7 +566,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
         ++npub;
         if (!redo) {
             if (it > 0) update_px();
-            const unsigned tag = Q.id + (unsigned)it + 1;
+            const unsigned tag = flow_tag(Q.id, it + 1u);
             const ulonglong2* const pub = Q.pub + (size_t)(it & 1) * ld;
             int c = wid - 1;
             while (true) {
@@ -608,7 +610,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcg_flow(CgParams P, FlowParams Q) 
         ++it;
         if (t == 0) S.next = 0;
         if (wid == 0) flow_next(S, P.rtol);
-        const unsigned tag = Q.id + (unsigned)it + 1;
+        const unsigned tag = flow_tag(Q.id, it + 1u);
         ulonglong2* const pub = Q.pub + (size_t)(it & 1) * ld + r0;
         ga = de = 0.0;
         flow_rows(nl, [&](int l) {
@@ -711,7 +713,7 @@ __device__ __forceinline__ void cgc_flow(const CgParams& P, const FlowParams& Q,
             break;
         }
         ++it;
-        const unsigned tag = Q.id + (unsigned)it + 1;
+        const unsigned tag = flow_tag(Q.id, it + 1u);
         ulonglong2* const pub = Q.pub + (size_t)(it & 1) * ld;
         flow_rows(nl, [&](int l) {
             const double s = wb[l] + beta * ss[l];
@@ -1065,11 +1067,11 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc2_flow(CgParams P, FlowParams Q,
         if (xs) xs[l] += alpha * p; else P.x[row_of(l)] += alpha * p;
     };
     while (true) {
-        const unsigned wtag = Q.id + (unsigned)it + 2;
+        const unsigned wtag = flow_tag(Q.id, it + 2u);
         ulonglong2* const words = C.words + (size_t)((it + 1) & 1) * C.pstride;
         if (!redo) {
             // w = (I + c S K_off S) u, r.u, w.u, Y' w
-            const unsigned tag = Q.id + (unsigned)it + 1;
+            const unsigned tag = flow_tag(Q.id, it + 1u);
             const ulonglong2* const pub = Q.pub + (size_t)(it & 1) * ld;
             ga = de = 0.0;
             for (int k = wid == 0 ? nw - 1 : wid - 1; k < nch; k += nw) {
@@ -1144,7 +1146,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cgc2_flow(CgParams P, FlowParams Q,
             sr[l] -= alpha * s;
         });
         __syncthreads();
-        const unsigned utag = Q.id + (unsigned)it + 1;
+        const unsigned utag = flow_tag(Q.id, it + 1u);
         ulonglong2* const pub = Q.pub + (size_t)(it & 1) * ld + r0;
         flow_rows(nl, [&](int l) {
             const double u = sr[l] + sy[l] * ysh[pid[l]];

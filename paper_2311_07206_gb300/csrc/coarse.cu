@@ -370,7 +370,7 @@ void coarse_free(CoarseDev& C) {
     C = CoarseDev{};
 }
 
-int coarse_sweep(CoarseDev& C, int n, const int* act, const int* pos, int maxit,
+int coarse_sweep(CoarseDev& C, int n, const int* act, const int* pos,
                  const PcgConfig& cfg, cudaStream_t s) {
     const int N = C.N, q = C.q, nc = nb(N, kChunk);
     if (n < 1) return SDC_OK;
@@ -416,7 +416,7 @@ int coarse_sweep(CoarseDev& C, int n, const int* act, const int* pos, int maxit,
         for (int b = 0; b < q; ++b) C.qn += C.h_blk_ptr[b + 1] > 0;
     };
     // on chip, one tile per CTA, where the rows and the coarse data fit
-    C.L = coarse_flow_rows(n, maxit, cfg);
+    C.L = coarse_flow_rows(n, cfg);
     C.flow = 0;
     if (C.L > 0) {
         cut(C.L, C.Gmax);

@@ -429,7 +429,7 @@ int emi_step(const EmiStepArgs& a, double* d_u, double* d_w, double dt, int swee
         if (coarse) {
             // the blocks of this sweep's active set: rows by block, CTA ownership
             int rc = SDC_OK;
-            run(SDC_PHASE_SELECT, 5, [&] { rc = coarse_sweep(*coarse, n, act, E.pos, a.opt->cg_maxit, *a.pcg, s); });
+            run(SDC_PHASE_SELECT, 5, [&] { rc = coarse_sweep(*coarse, n, act, E.pos, *a.pcg, s); });
             if (rc != SDC_OK) {
                 status = fail(rc, "two-level preconditioner: block ordering failed");
                 break;

@@ -134,7 +134,7 @@ extern "C" sdc_status sdc_pcg_solve_noalloc(int n, const double* d_val, const in
     A.width = width;
     int h[3] = {0, 0, 0};   // -, error, iterations
     double hr = 0.0;
-    const size_t fd = sdc::pcg_standalone_flow_doubles(n, ld, width, maxit);
+    const size_t fd = sdc::pcg_standalone_flow_doubles(n, ld, width);
     if (fd > 0 && fd <= kScratchDoubles) {
         if (sdc::launch_pcg_standalone_flow(n, A, d_kdiag, d_mass, d_J, c, d_b, d_x, rtol, maxit,
                                             4000000000LL, base, s) != SDC_OK)

@@ -182,7 +182,6 @@ void launch_residual(int M, int n, const int* act, const Ell& K, const double* k
                      const int* n_dev = nullptr);
 // Launch configuration of the restricted PCG solves.
 constexpr int kFlowSmemBytes = 225 * 1024;   // dynamic shared memory of the flow kernels
-constexpr int kFlowMaxit = 1000000;   // iterations a tag can count
 // 64-bit words of their grid-wide state: 34, padded to whole 128-byte lines.  The second of two
 // adjacent sets of 34 had its sums across two lines, and every other solve took 1 to 4 % longer
 // (53k cell-by-cell dofs 26.60 -> 26.28 ms per step, 58k order 6 2,926 -> 2,906 us).
@@ -309,7 +308,7 @@ struct CoarseDev {
 };
 // Shape of the on-chip form for n rows: rows per CTA (0: none); then, with the pieces known,
 // its buffers and shared memory (false: no room).
-int coarse_flow_rows(int n, int maxit, const PcgConfig& cfg);
+int coarse_flow_rows(int n, const PcgConfig& cfg);
 bool coarse_flow_fit(CoarseDev& C);
 // labels: host, N entries in [0, q).  Allocates and uploads; returns an sdc_status.
 int coarse_setup(CoarseDev& C, const int* h_lab, int N, int q, int ld, int width, int* err,
@@ -319,7 +318,7 @@ void coarse_free(CoarseDev& C);
 // pieces of the CG launch (tiles of kCoarseTile positions, round robin over the CTAs,
 // cut at blocks).  pos: dof -> compact row (-1 outside the active set).  Synchronises
 // the stream (reads the block ranges).
-int coarse_sweep(CoarseDev& C, int n, const int* act, const int* pos, int maxit,
+int coarse_sweep(CoarseDev& C, int n, const int* act, const int* pos,
                  const PcgConfig& cfg, cudaStream_t s);
 // Per node solve: E = Z' A Z of the operator diag(mc (1 + c J) + c kdc) + c A_off on the
 // active rows (exact fixed-point accumulation) and its inverse.
@@ -417,7 +416,7 @@ constexpr int kStandaloneResults = 2;
 bool columns_scattered(int n, const Ell& A, int sms, int stride, unsigned long long* words,
                        cudaStream_t s);
 bool pcg_standalone_asks(int n, int width);
-size_t pcg_standalone_flow_doubles(int n, int ld, int width, int maxit, size_t* zero_at = nullptr);
+size_t pcg_standalone_flow_doubles(int n, int ld, int width, size_t* zero_at = nullptr);
 int launch_pcg_standalone_flow(int n, const Ell& A, const double* kdiag, const double* mass,
                                const double* J, double c, const double* b, double* x, double rtol,
                                int maxit, long long budget, double* ws, cudaStream_t s);

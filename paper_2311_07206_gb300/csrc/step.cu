@@ -2321,8 +2321,8 @@ unsigned next_flow_id(StepBuffers& B, cudaStream_t s) {
     return B.flow_id;
 }
 
-int coarse_flow_rows(int n, int maxit, const PcgConfig& cfg) {
-    if (cfg.variant == 1 || !cfg.scaled || maxit >= kFlowMaxit) return 0;
+int coarse_flow_rows(int n, const PcgConfig& cfg) {
+    if (cfg.variant == 1 || !cfg.scaled) return 0;
     int gm = std::min(cfg.sms, 255);
     if (cfg.max_blocks > 0) gm = std::min(gm, cfg.max_blocks);
     const int l = nblk(n, gm);
@@ -2594,8 +2594,7 @@ int launch_pcg_params(CgParams& P, const PcgConfig& cfg, StepBuffers& B, cudaStr
         (cfg.general_classical && n > kFlowClassicalRows && !cfg.scattered);
     const bool scaled = cfg.scaled && P.sv && P.sval;
     const bool in_cache = flow_in_cache(n, cfg);
-    if (cfg.variant != 1 && scaled && B.pub && P.maxit < kFlowMaxit && in_cache &&
-        flow_shape(n, flow_classical, cfg, fs)) {
+    if (cfg.variant != 1 && scaled && B.pub && in_cache && flow_shape(n, flow_classical, cfg, fs)) {
         unsigned long long* words = B.flow + (size_t)B.flow_set * kFlowWords;
         unsigned long long* other = B.flow + (size_t)(B.flow_set ^ 1) * kFlowWords;
         const int rc = launch_flow(P, flow_classical, fs, B.pub, words, other, next_flow_id(B, s), s);
@@ -2928,7 +2927,7 @@ int launch_pcg_batch(int n, const Ell& A, int m, double dt, const Coll& co, doub
                      StepBuffers& B, cudaStream_t s) {
     const int nseg = (int)bounds.size() - 1;
     const BatchFlow& bf = batch_flow_shape(cfg, B);
-    if (bf.grid > 0 && maxit < kFlowMaxit) {
+    if (bf.grid > 0) {
         const int rpb = batch_flow_rows(bounds[nseg] - bounds[0], bf.grid, nseg, batch_flow_floor(cfg));
         std::vector<SegBlock> tab;
         for (int g = 0; g < nseg; ++g) {
@@ -2999,7 +2998,7 @@ int launch_pcg_batch_planned(const Ell& A, int m, double dt, const Coll& co, dou
     if (nseg < 1 || nseg > G || G > B.segtab_cap) return SDC_E_INVALID;
     SegBlock* tab = reinterpret_cast<SegBlock*>(B.segtab);
     const BatchFlow& bf = batch_flow_shape(cfg, B);
-    if (bf.grid > 0 && maxit < kFlowMaxit) {
+    if (bf.grid > 0) {
         if (plan)
             k_batch_plan_flow<<<1, 256, 0, s>>>(nseg, bounds_dev, bf.grid, batch_flow_floor(cfg), tab,
                                                 B.plan);
@@ -3077,10 +3076,10 @@ bool pcg_standalone_shape(int n, int width, FlowShape& f, bool& classical) {
     return true;
 }
 
-size_t pcg_standalone_flow_doubles(int n, int ld, int width, int maxit, size_t* zero_at) {
+size_t pcg_standalone_flow_doubles(int n, int ld, int width, size_t* zero_at) {
     FlowShape f;
     bool classical;
-    if (maxit >= kFlowMaxit || !pcg_standalone_shape(n, width, f, classical)) return 0;
+    if (!pcg_standalone_shape(n, width, f, classical)) return 0;
     // u, diag^-1/2, [scaled values], then from a 256-byte boundary on what starts at zero:
     // the published words, the sums, the results
     const size_t z = (2 * (size_t)n + (f.v_smem ? 0 : (size_t)width * ld) + 31) / 32 * 32;
@@ -3094,7 +3093,7 @@ int launch_pcg_standalone_flow(int n, const Ell& A, const double* kdiag, const d
     FlowShape f;
     bool classical;
     size_t z = 0;
-    const size_t total = pcg_standalone_flow_doubles(n, A.ld, A.width, maxit, &z);
+    const size_t total = pcg_standalone_flow_doubles(n, A.ld, A.width, &z);
     if (!total || !pcg_standalone_shape(n, A.width, f, classical) ||
         reinterpret_cast<uintptr_t>(ws) % 256 != 0)
         return SDC_E_INVALID;

@@ -142,3 +142,43 @@ def test_waits_that_run_out(torch_dev, pipelined, blocks):
             assert np.abs(v - r["v"]).max() <= RTOL and np.abs(w - r["w"]).max() <= RTOL
         ctx.close()
     assert done >= 6 and (timeouts >= 1 or blocks == 1)
+
+
+@pytest.mark.parametrize("pipelined", [-1, 0, 1])
+def test_a_high_iteration_limit_changes_nothing(torch_dev, pipelined):
+    """cg_maxit of 1,000,000 and above: the same kernels, the same bits."""
+    torch, dev = torch_dev
+    wl = _workload(67, 61, lambda m: 0.5 + 0.3 * np.sin(m.xyz[:, 0]))
+    out = []
+    for maxit in (10_000, 1_000_000, 2**31 - 1):
+        ctx = _context(wl, torch, dev, cg_pipelined=pipelined, cg_maxit=maxit)
+        out.append(_step(ctx, wl, wl.v0, torch, dev))
+        ctx.close()
+    for v, w in out[1:]:
+        assert np.array_equal(v, out[0][0]) and np.array_equal(w, out[0][1])
+
+
+def test_more_iterations_than_a_tag_counts(torch_dev):
+    """A chain of 1,000 links over thirteen decades does not converge in a million iterations;
+    the words' tags wrap at 2^20 on the way, and the solve ends at its limit, with no wait run
+    out."""
+    torch, dev = torch_dev
+    from paper_2311_07206_gb300 import SdcError
+    from paper_2311_07206_gb300 import binding as B
+    n, ld = 1_000, 1_024
+    rng = np.random.default_rng(1)
+    k = np.exp(30.0 * rng.uniform(0.0, 1.0, n - 1))
+    val, col, ln = np.zeros((2, ld)), np.zeros((2, ld), np.int32), np.zeros(n, np.int32)
+    for i in range(n):
+        for j in (i - 1, i + 1):
+            if 0 <= j < n:
+                val[ln[i], i], col[ln[i], i] = -k[min(i, j)], j
+                ln[i] += 1
+    kd = np.concatenate([k, [0.0]]) + np.concatenate([[0.0], k])
+    t = lambda a: torch.tensor(a, device=dev)
+    x = torch.zeros(n, dtype=torch.float64, device=dev)
+    with pytest.raises(SdcError) as e:
+        B.pcg_solve(n, t(val), t(col), t(ln), ld, 2, t(kd), t(np.full(n, 1e-6)), t(np.zeros(n)), 1.0,
+                    t(rng.uniform(-0.5, 0.5, n)), x, rtol=1e-14, maxit=1_060_000,
+                    stream=torch.cuda.current_stream(dev).cuda_stream)
+    assert e.value.status == B.SDC_E_CG_NOCONV
