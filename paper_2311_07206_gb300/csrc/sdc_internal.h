@@ -182,6 +182,7 @@ void launch_residual(int M, int n, const int* act, const Ell& K, const double* k
                      const int* n_dev = nullptr);
 // Launch configuration of the restricted PCG solves.
 constexpr int kFlowSmemBytes = 225 * 1024;   // dynamic shared memory of the flow kernels
+constexpr int kFlowMaxSlots = 65535;         // they keep a row's length in 16 bits
 // 64-bit words of their grid-wide state: 34, padded to whole 128-byte lines.  The second of two
 // adjacent sets of 34 had its sums across two lines, and every other solve took 1 to 4 % longer
 // (53k cell-by-cell dofs 26.60 -> 26.28 ms per step, 58k order 6 2,926 -> 2,906 us).

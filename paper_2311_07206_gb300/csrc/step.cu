@@ -2330,6 +2330,7 @@ int coarse_flow_rows(int n, const PcgConfig& cfg) {
     return 6 * L <= kFlowSmemBytes / 8 ? L : 0;
 }
 bool coarse_flow_fit(CoarseDev& C) {
+    if (C.width > kFlowMaxSlots) return false;
     // one row per thread up to 736 rows; above, 512 threads with 128 registers each (us per
     // iteration with 512 / 768 / 1024 threads: 131k rows 9.4 / 10.9 / 10.5, 250k 14.9 / 16.2 /
     // 15.5, 505k 23.8 / 25.2 / 26.4; in one row per thread 83k 8.4 against 8.9).  The matrix
@@ -2593,7 +2594,7 @@ int launch_pcg_params(CgParams& P, const PcgConfig& cfg, StepBuffers& B, cudaStr
         !cfg.pipelined ||
         (cfg.general_classical && n > kFlowClassicalRows && !cfg.scattered);
     const bool scaled = cfg.scaled && P.sv && P.sval;
-    const bool in_cache = flow_in_cache(n, cfg);
+    const bool in_cache = B.sval_width <= kFlowMaxSlots && flow_in_cache(n, cfg);
     if (cfg.variant != 1 && scaled && B.pub && in_cache && flow_shape(n, flow_classical, cfg, fs)) {
         unsigned long long* words = B.flow + (size_t)B.flow_set * kFlowWords;
         unsigned long long* other = B.flow + (size_t)(B.flow_set ^ 1) * kFlowWords;
@@ -2724,7 +2725,8 @@ const void* batch_flow_kernel(int block) {
 // CTAs per SM down; grid 0 when the rows do not fit.  Kept per launch configuration.
 const BatchFlow& batch_flow_shape(const PcgConfig& cfg, StepBuffers& B) {
     BatchFlow& f = B.bflow;
-    const bool on = cfg.variant != 1 && cfg.scaled && !cfg.batch_pipelined && B.pub && B.sval;
+    const bool on = cfg.variant != 1 && cfg.scaled && !cfg.batch_pipelined && B.pub && B.sval &&
+                    B.sval_width <= kFlowMaxSlots;
     if (f.block == cfg.batch_block && f.rpb == cfg.batch_rows_per_block &&
         f.max_blocks == cfg.max_blocks && f.on == on)
         return f;
@@ -3071,7 +3073,7 @@ bool pcg_standalone_shape(int n, int width, FlowShape& f, bool& classical) {
     cfg.sms = pcg_sm_count();
     cfg.smem_block = 512;
     classical = n > kFlowClassicalRows;
-    if (cfg.sms < 1 || !flow_shape(n, classical, cfg, f)) return false;
+    if (cfg.sms < 1 || width > kFlowMaxSlots || !flow_shape(n, classical, cfg, f)) return false;
     flow_values_on_chip(width, f);
     return true;
 }

@@ -182,3 +182,36 @@ def test_more_iterations_than_a_tag_counts(torch_dev):
                     t(rng.uniform(-0.5, 0.5, n)), x, rtol=1e-14, maxit=1_060_000,
                     stream=torch.cuda.current_stream(dev).cuda_stream)
     assert e.value.status == B.SDC_E_CG_NOCONV
+
+
+def test_a_row_longer_than_65535(torch_dev):
+    """An arrow matrix whose first row has 65,699 off-diagonals (52 GB of slots, nearly all
+    unused), against its Schur complement."""
+    torch, dev = torch_dev
+    from paper_2311_07206_gb300 import binding
+    n = 65_700
+    ld, width = (n + 31) // 32 * 32, n - 1
+    torch.cuda.empty_cache()
+    if torch.cuda.mem_get_info(dev)[0] < 80e9:
+        pytest.skip("not enough device memory")
+    rng = np.random.default_rng(7)
+    a = -rng.uniform(0.5, 1.5, n - 1)
+    kd = np.concatenate([[-a.sum()], -a])
+    b = rng.standard_normal(n)
+    t = lambda q: torch.tensor(q, device=dev)
+    val = torch.zeros((width, ld), dtype=torch.float64, device=dev)
+    col = torch.zeros((width, ld), dtype=torch.int32, device=dev)
+    val[:, 0], col[:, 0] = t(a), t(np.arange(1, n, dtype=np.int32))
+    val[0, 1:n] = t(a)
+    ln = np.ones(n, np.int32)
+    ln[0] = n - 1
+    x = torch.zeros(n, dtype=torch.float64, device=dev)
+    c = 0.5
+    binding.pcg_solve(n, val, col, t(ln), ld, width, t(kd), t(np.ones(n)), t(np.zeros(n)), c, t(b), x,
+                      rtol=1e-12, maxit=500, stream=torch.cuda.current_stream(dev).cuda_stream)
+    d = 1.0 + c * kd
+    x0 = (b[0] - (c * a * b[1:] / d[1:]).sum()) / (d[0] - (c * c * a * a / d[1:]).sum())
+    want = np.concatenate([[x0], (b[1:] - c * a * x0) / d[1:]])
+    assert np.abs(x.cpu().numpy() - want).max() <= RTOL * np.abs(want).max()
+    del val, col
+    torch.cuda.empty_cache()
