@@ -1359,13 +1359,18 @@ struct SolveWorkspace {
     void* p = nullptr;
     cudaStream_t s;
     bool pooled = false;
-    SolveWorkspace(size_t bytes, cudaStream_t stream) : s(stream) {
+    explicit SolveWorkspace(cudaStream_t stream) : s(stream) {}
+    bool get(size_t bytes) {
         if (cudaMemPool_t q = g_solve_pools.get())
             pooled = cudaMallocFromPoolAsync(&p, bytes, q, s) == cudaSuccess;
         if (!pooled) {
             cudaGetLastError();
-            if (cudaMalloc(&p, bytes) != cudaSuccess) p = nullptr;
+            if (cudaMalloc(&p, bytes) != cudaSuccess) {
+                cudaGetLastError();
+                p = nullptr;
+            }
         }
+        return p != nullptr;
     }
     ~SolveWorkspace() {
         if (pooled) cudaFreeAsync(p, s);
@@ -1408,17 +1413,24 @@ static sdc_status pcg_solve_body(int n, const double* d_val, const int* d_col, c
     int status = SDC_OK;
     int h[3] = {0, 0, 0};   // -, error, iterations
     double hr = 0.0;
-    const size_t fd = pcg_standalone_flow_doubles(n, ld, width);
+    size_t fd = pcg_standalone_flow_doubles(n, ld, width);
     const bool asks = fd > 0 && pcg_standalone_asks(n, width);
     const int block = 256;
-    const int maxb = fd == 0 || asks ? pcg_max_blocks(block) : 0;
+    int maxb = 0;
     // workspace of the kernels with global vectors: 8 vectors of n, the published m in two
     // buffers ld apart (the kernels offset the second by the matrix's ld), 12 * maxb for the
     // partial-sum records (16-byte aligned: they are read with 16-byte loads), then the scalars
     const size_t po = ((size_t)8 * n + 2 * (size_t)ld + 1) & ~(size_t)1;
-    const size_t nd = maxb > 0 ? po + 12 * (size_t)maxb + 2 + 8 : 0;
-    SolveWorkspace ws(std::max(fd, nd) * sizeof(double), s);
-    if (!ws.p) return fail(nullptr, SDC_E_NOMEM, "sdc_pcg_solve: workspace allocation failed");
+    auto global_doubles = [&] {
+        maxb = pcg_max_blocks(block);
+        return po + 12 * (size_t)maxb + 2 + 8;
+    };
+    SolveWorkspace ws(s);
+    // (the on-chip kernels' workspace grows with the width, the other's does not: without room
+    // for the first, the solve runs in the second)
+    if (fd > 0 && !ws.get(std::max(fd, asks ? global_doubles() : 0) * sizeof(double))) fd = 0;
+    if (!ws.p && !ws.get(global_doubles() * sizeof(double)))
+        return fail(nullptr, SDC_E_NOMEM, "sdc_pcg_solve: workspace allocation failed");
     double* v = (double*)ws.p;
     if (fd > 0 &&
         !(asks && columns_scattered(n, A, pcg_sm_count(), 64, (unsigned long long*)ws.p, s))) {

@@ -215,3 +215,32 @@ def test_a_row_longer_than_65535(torch_dev):
     assert np.abs(x.cpu().numpy() - want).max() <= RTOL * np.abs(want).max()
     del val, col
     torch.cuda.empty_cache()
+
+
+def test_no_room_for_the_on_chip_workspace(torch_dev):
+    """A tridiagonal matrix declared 65,000 slots wide: scaled values of every slot would take
+    364 GB; the solve runs in the kernels that keep none."""
+    torch, dev = torch_dev
+    linalg = pytest.importorskip("scipy.linalg")
+    from paper_2311_07206_gb300 import binding
+    n, width = 700_000, 65_000
+    ld = (n + 31) // 32 * 32
+    val, col = np.zeros((2, ld)), np.zeros((2, ld), np.int32)
+    i = np.arange(n)
+    val[:, :n] = -1.0
+    col[0, :n] = np.where(i > 0, i - 1, 1)
+    col[1, :n] = np.minimum(i + 1, n - 1)
+    ln = np.full(n, 2, np.int32)
+    ln[0] = ln[-1] = 1
+    kd = np.full(n, 2.0)
+    kd[0] = kd[-1] = 1.0
+    b = np.random.default_rng(8).standard_normal(n)
+    t = lambda a: torch.tensor(a, device=dev)
+    x = torch.zeros(n, dtype=torch.float64, device=dev)
+    it, rr = binding.pcg_solve(n, t(val), t(col), t(ln), ld, width, t(kd), t(np.ones(n)),
+                               t(np.zeros(n)), 1.0, t(b), x, rtol=1e-12, maxit=500,
+                               stream=torch.cuda.current_stream(dev).cuda_stream)
+    ab = np.zeros((3, n))
+    ab[0, 1:], ab[1], ab[2, :-1] = -1.0, 1.0 + kd, -1.0
+    want = linalg.solve_banded((1, 1), ab, b)
+    assert rr <= 1e-12 and np.abs(x.cpu().numpy() - want).max() <= RTOL * np.abs(want).max()
