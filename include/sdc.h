@@ -376,11 +376,12 @@ sdc_ctx* sdc_batch_context(sdc_batch* batch);
  * be adopted (each configuration is timed twice from the restored state, the
  * better run counting).  The state arrays are restored bitwise before returning.  Every
  * configuration computes the same iteration (results differ by rounding only).
- *   single context: cg_pipelined {1, 0}; cg_scaled {1, 0}; shared-memory block
- *     size {512, 1024}; rows from which the shared-memory variants use 1024
- *     threads {0, 100000, 300000, never}; general-variant block size {256, 512,
- *     1024}; cluster_rows {0, 2000, 5000, 10000, 20000 (within the cluster's
- *     capacity)};
+ *   single context: cg_pipelined {1, 0}; cg_scaled {1, 0}; then, where every solve
+ *     runs in the scaled form on chip, target rows per block {0, 128, 256, 512} (kept
+ *     in the context, not reported); else shared-memory block size {512, 1024}; rows
+ *     from which the shared-memory variants use 1024 threads {0, 100000, 300000,
+ *     never}; general-variant block size {256, 512, 1024}; cluster_rows {0, 2000,
+ *     5000, 10000, 20000 (within the cluster's capacity)};
  *   batch: arrangement {classical, pipelined}; cg_scaled {1, 0}; block size
  *     {256, 512, 1024}; target active rows per block {256, 512, 1024, 2048, 4096}.
  * Candidates whose cooperative grid would exceed the context's reserved

@@ -1835,20 +1835,36 @@ sdc_status autotune_impl(sdc_ctx* c, double* d_v, double* d_w, double t, double 
     if (!batch) {
         knobs.push_back({{1, 0}, [](PcgConfig& q, int v) { q.pipelined = v; return true; }});
         knobs.push_back({{1, 0}, [](PcgConfig& q, int v) { q.scaled = v; return true; }});
-        knobs.push_back({{512, 1024}, [](PcgConfig& q, int v) { q.smem_block = v; return true; }});
-        knobs.push_back({{0, 100000, 300000, 0x7fffffff},
-                         [](PcgConfig& q, int v) { q.big_rows = v; return true; }});
+        // a value that leaves every launch of the context as it is would be chosen by noise
+        StepBuffers& B = c->B;
+        auto flow = [&B](const PcgConfig& q) { return all_solves_on_chip(q, B); };
+        auto threads = [flow](const PcgConfig& q) { return flow(q) && q.smem_block >= 512; };
+        knobs.push_back({{512, 1024}, [threads](PcgConfig& q, int v) {
+                             if (threads(q)) return false;
+                             q.smem_block = v;
+                             return true;
+                         }});
+        knobs.push_back({{0, 100000, 300000, 0x7fffffff}, [threads](PcgConfig& q, int v) {
+                             if (threads(q)) return false;
+                             q.big_rows = v;
+                             return true;
+                         }});
+        knobs.push_back({{0, 128, 256, 512}, [flow](PcgConfig& q, int v) {
+                             if (!flow(q)) return false;
+                             q.rows_per_block = v;
+                             return true;
+                         }});
         const int cap = c->B.max_blocks;
-        knobs.push_back({{256, 512, 1024}, [cap](PcgConfig& q, int v) {
+        knobs.push_back({{256, 512, 1024}, [cap, flow](PcgConfig& q, int v) {
                              const int g = pcg_max_blocks(v);
-                             if (g < 1 || g > cap) return false;
+                             if (flow(q) || g < 1 || g > cap) return false;
                              q.block = v;
                              q.max_blocks_general = q.max_blocks > 0 ? std::min(g, q.max_blocks) : g;
                              return true;
                          }});
         const int ccap = P.cluster * kClusterRows;
-        knobs.push_back({{0, 2000, 5000, 10000, 20000}, [ccap](PcgConfig& q, int v) {
-                             if (v > ccap) return false;
+        knobs.push_back({{0, 2000, 5000, 10000, 20000}, [ccap, flow](PcgConfig& q, int v) {
+                             if (flow(q) || v > ccap) return false;
                              q.cluster_rows = v;
                              return true;
                          }});

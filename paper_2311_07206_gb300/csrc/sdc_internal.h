@@ -229,6 +229,7 @@ struct PcgConfig {
 };
 int launch_pcg(int n, const Ell& A, int m, double dt, const Coll& co, double rtol, int maxit,
                int sweep, const PcgConfig& cfg, StepBuffers& B, cudaStream_t s);
+bool all_solves_on_chip(const PcgConfig& cfg, const StepBuffers& B);
 int pcg_sm_count();
 // dof permutation (perm[new] = old): dst[i] = src[perm[i]] / dst[perm[i]] = src[i]
 void launch_perm_gather(int N, const int* perm, const double* src, double* dst, cudaStream_t s);

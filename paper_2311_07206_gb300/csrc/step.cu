@@ -2559,6 +2559,23 @@ bool flow_values_on_chip(int width, FlowShape& f) {
     return true;
 }
 
+bool flow_classical_at(int n, const PcgConfig& cfg) {
+    // (scattered columns: the pipelined form hides their latency; randomly numbered tissue, classical /
+    // pipelined: 140k 11.0 / 10.3, 212k 17.2 / 15.6, 302k 21.5 / 20.9, 376k 32.7 / 25.9)
+    return !cfg.pipelined ||
+           (cfg.general_classical && n > kFlowClassicalRows && !cfg.scattered);
+}
+
+// Whether a solve of n rows runs in the flow kernels, and its shape there.
+bool flow_takes(int n, const PcgConfig& cfg, const StepBuffers& B, FlowShape& f) {
+    return cfg.variant != 1 && cfg.scaled && B.pub && B.sval_width <= kFlowMaxSlots &&
+           flow_in_cache(n, cfg) && flow_shape(n, flow_classical_at(n, cfg), cfg, f);
+}
+bool all_solves_on_chip(const PcgConfig& cfg, const StepBuffers& B) {
+    FlowShape f;
+    return flow_takes(B.N, cfg, B, f);
+}
+
 // words: kFlowWords words, zero; zero: the next launch's, to be cleared (or null); pub: tags
 // of other launches only
 int launch_flow(CgParams& P, bool classical, const FlowShape& f, void* pub,
@@ -2588,14 +2605,9 @@ int launch_pcg_params(CgParams& P, const PcgConfig& cfg, StepBuffers& B, cudaStr
     // the exact-sum records are read with 16-byte loads
     if (reinterpret_cast<uintptr_t>(P.part) % 16 != 0) return SDC_E_INVALID;
     FlowShape fs;
-    // (scattered columns: the pipelined form hides their latency; randomly numbered tissue, classical /
-    // pipelined: 140k 11.0 / 10.3, 212k 17.2 / 15.6, 302k 21.5 / 20.9, 376k 32.7 / 25.9)
-    const bool flow_classical =
-        !cfg.pipelined ||
-        (cfg.general_classical && n > kFlowClassicalRows && !cfg.scattered);
     const bool scaled = cfg.scaled && P.sv && P.sval;
-    const bool in_cache = B.sval_width <= kFlowMaxSlots && flow_in_cache(n, cfg);
-    if (cfg.variant != 1 && scaled && B.pub && in_cache && flow_shape(n, flow_classical, cfg, fs)) {
+    if (P.sv && P.sval && flow_takes(n, cfg, B, fs)) {
+        const bool flow_classical = flow_classical_at(n, cfg);
         unsigned long long* words = B.flow + (size_t)B.flow_set * kFlowWords;
         unsigned long long* other = B.flow + (size_t)(B.flow_set ^ 1) * kFlowWords;
         const int rc = launch_flow(P, flow_classical, fs, B.pub, words, other, next_flow_id(B, s), s);
@@ -2607,7 +2619,7 @@ int launch_pcg_params(CgParams& P, const PcgConfig& cfg, StepBuffers& B, cudaStr
     // automatic arrangement: the pipelined form pays off where the vectors live on chip;
     // for the global-vector variant (solves above the on-chip capacity) its extra vector
     // traffic outweighs the saved synchronisation
-    const bool on_chip = cfg.variant != 1 && !(scaled && !in_cache) && n <= cfg.sms * kSmemRows;
+    const bool on_chip = cfg.variant != 1 && !scaled && n <= cfg.sms * kSmemRows;
     if (!cfg.pipelined || (cfg.general_classical && !on_chip)) {
         // classical arrangement: shared-memory form when it fits, else global vectors
         if (cfg.variant != 1 && n <= cfg.sms * kSmemRowsC) {
