@@ -178,8 +178,8 @@ def test_more_iterations_than_a_tag_counts(torch_dev):
     t = lambda a: torch.tensor(a, device=dev)
     x = torch.zeros(n, dtype=torch.float64, device=dev)
     with pytest.raises(SdcError) as e:
-        B.pcg_solve(n, t(val), t(col), t(ln), ld, 2, t(kd), t(np.full(n, 1e-6)), t(np.zeros(n)), 1.0,
-                    t(rng.uniform(-0.5, 0.5, n)), x, rtol=1e-14, maxit=1_060_000,
+        B.pcg_solve(n, t(val), t(col), t(ln), ld, 2, t(kd), t(np.full(n, 1e-6)), t(np.zeros(n)),
+                    1.0, t(rng.uniform(-0.5, 0.5, n)), x, rtol=1e-14, maxit=1_060_000,
                     stream=torch.cuda.current_stream(dev).cuda_stream)
     assert e.value.status == B.SDC_E_CG_NOCONV
 
@@ -207,8 +207,8 @@ def test_a_row_longer_than_65535(torch_dev):
     ln[0] = n - 1
     x = torch.zeros(n, dtype=torch.float64, device=dev)
     c = 0.5
-    binding.pcg_solve(n, val, col, t(ln), ld, width, t(kd), t(np.ones(n)), t(np.zeros(n)), c, t(b), x,
-                      rtol=1e-12, maxit=500, stream=torch.cuda.current_stream(dev).cuda_stream)
+    binding.pcg_solve(n, val, col, t(ln), ld, width, t(kd), t(np.ones(n)), t(np.zeros(n)), c, t(b),
+                      x, rtol=1e-12, maxit=500, stream=torch.cuda.current_stream(dev).cuda_stream)
     d = 1.0 + c * kd
     x0 = (b[0] - (c * a * b[1:] / d[1:]).sum()) / (d[0] - (c * c * a * a / d[1:]).sum())
     want = np.concatenate([[x0], (b[1:] - c * a * x0) / d[1:]])
@@ -244,3 +244,80 @@ def test_no_room_for_the_on_chip_workspace(torch_dev):
     ab[0, 1:], ab[1], ab[2, :-1] = -1.0, 1.0 + kd, -1.0
     want = linalg.solve_banded((1, 1), ab, b)
     assert rr <= 1e-12 and np.abs(x.cpu().numpy() - want).max() <= RTOL * np.abs(want).max()
+
+
+def _grid_ell(nx, ny):
+    n = nx * ny
+    ld = (n + 31) // 32 * 32
+    i = np.arange(n)
+    val, col = np.zeros((4, ld)), np.zeros((4, ld), np.int32)
+    ln, kd = np.zeros(n, np.int32), np.zeros(n)
+    for ok, off in ((i % nx > 0, -1), (i % nx < nx - 1, 1), (i >= nx, -nx), (i < n - nx, nx)):
+        r = i[ok]
+        val[ln[r], r], col[ln[r], r] = -1.0, r + off
+        ln[r] += 1
+        kd[r] += 1.0
+    return n, ld, val, col, ln, kd
+
+
+@pytest.mark.parametrize("case", ["rise", "fall"])
+def test_repeated_sums_in_the_pipelined_arrangement(torch_dev, case):
+    """One to four iterations of a stand-alone solve (pipelined at this size) against the same
+    iterates of plain CG.  Rise: the lowest mode with a trace of others, gamma grows by 2^11
+    in the first iteration.  Fall: an almost diagonal matrix, 2^-30 an iteration."""
+    torch, dev = torch_dev
+    from paper_2311_07206_gb300 import SdcError
+    from paper_2311_07206_gb300 import binding as B
+    n, ld, val, col, ln, kd = _grid_ell(61, 53)
+    rng = np.random.default_rng(9)
+    c, mass = (1.0, np.full(n, 1e-4)) if case == "rise" else (1e-5, np.ones(n))
+    d = mass + c * kd
+
+    def A(x):
+        y = d * x
+        for k in range(4):
+            m = ln > k
+            y[m] += c * val[k, :n][m] * x[col[k, :n][m]]
+        return y
+    b = d * (1.0 + 5e-3 * rng.standard_normal(n)) if case == "rise" else rng.standard_normal(n)
+    t = lambda a: torch.tensor(a, device=dev)
+    x, r = np.zeros(n), b.copy()
+    p, g, ratio = np.zeros(n), 1.0, []
+    for it in range(1, 5):
+        g1 = r @ (r / d)
+        p = r / d + (g1 / g if it > 1 else 0.0) * p
+        q = A(p)
+        a = g1 / (p @ q)
+        x, r, g = x + a * p, r - a * q, g1
+        ratio.append((r @ (r / d)) / g)
+        dx = torch.zeros(n, dtype=torch.float64, device=dev)
+        with pytest.raises(SdcError) as e:
+            B.pcg_solve(n, t(val), t(col), t(ln), ld, 4, t(kd), t(mass), t(np.zeros(n)), c, t(b),
+                        dx, rtol=1e-150, maxit=it, stream=torch.cuda.current_stream(dev).cuda_stream)
+        assert e.value.status == B.SDC_E_CG_NOCONV
+        assert np.abs(dx.cpu().numpy() - x).max() <= RTOL * np.abs(x).max(), it
+    assert ratio[0] > 2.0**11 if case == "rise" else max(ratio[:2]) < 2.0**-25
+
+
+def test_repeated_sums_in_the_two_level_solves(torch_dev):
+    """Every dof a block of its own: the coarse matrix is the operator, and gamma falls by
+    2^4 and more an iteration."""
+    torch, dev = torch_dev
+    from paper_2311_07206_gb300 import Context, default_options
+    from workloads.emi import emi_tiny
+    wl = emi_tiny("two_cells")
+    lab = np.arange(wl.n, dtype=np.int32)
+    r = oracle.System.from_mesh(wl.mesh).step_emi(wl, wl.u0, wl.w0, coarse=lab)
+    assert r["status"] == 0
+    for blocks in (0, 1, 3):
+        ctx = Context.from_emi(wl, options=default_options(cg_max_blocks=blocks),
+                               stream=torch.cuda.current_stream(dev).cuda_stream)
+        ctx.set_coarse_blocks(lab)
+        u = torch.tensor(wl.u0, dtype=torch.float64, device=dev)
+        w = torch.tensor(wl.w0, dtype=torch.float64, device=dev)
+        st = ctx.step(u, w, 0.0, wl.dt, wl.sweeps, wl.tol)
+        ctx.close()
+        for a, b in ((u, r["u"]), (w, r["w"])):
+            assert np.abs(a.cpu().numpy() - b).max() <= RTOL * max(1.0, np.abs(b).max())
+        for m in range(wl.M):
+            assert st.cg_iters[0][m] <= 20 and abs(st.cg_iters[0][m] - r["stats"].cg_iters[m]) <= 2
