@@ -103,13 +103,18 @@ typedef struct {
                               of 32); default 1024.  Batches use min(this, 256)               */
     int cg_smem_block_size;/* threads per block of the shared-memory and cluster CG; default 512.
                               Scaled form: below 512 a limit on the threads (32 plus one per
-                              row up to 896 rows a block, else 1024)                         */
+                              row of a block, at most 1024)                                   */
     int cg_cluster_max;    /* largest cluster (CTAs) for the cluster CG, 1..16; default 16      */
     int cg_max_blocks;     /* 0: no limit on the cooperative CG grid                          */
     int cg_variant;        /* 0: automatic; 1: vectors in global memory; 2: per-block vectors
                               in shared memory whenever they fit (scaled form: 3968 rows per
                               SM for the pipelined, 6752 for the classical arrangement; Jacobi
-                              form: 3584 and 4768)                                            */
+                              form: 3584 and 4768).  Automatic in the scaled form: the same
+                              while the matrix and the published vectors stay in L2, 12 bytes
+                              per stored off-diagonal and 32 per row up to 92 MB (80 MB with more
+                              than ten off-diagonals a row or a numbering that scatters most
+                              columns; a pipelined arrangement that was asked for heeds only
+                              the last)                                                       */
     int cg_rows_per_block; /* shared-memory variant: target rows per block (0 = 256 in the
                               Jacobi form; in the scaled form as many blocks as SMs, of at
                               least 96 rows)                                                  */
@@ -126,11 +131,12 @@ typedef struct {
                               the sums overlapped with the product); 0 classical (two); -1
                               automatic: for monodomain contexts pipelined up to 130,000
                               active rows, where an iteration is bound by latency, and
-                              classical above (fewer FP64 operations per row; Jacobi form:
-                              pipelined where the vectors fit on chip); classical for cell-by-cell contexts, whose
-                              long ill-conditioned solves need its smaller rounding error, and
-                              for batches, whose many small groups favour its lighter rows;
-                              default -1                                                       */
+                              classical above (fewer FP64 operations per row), unless the
+                              numbering scatters most columns; Jacobi form: pipelined where
+                              the vectors fit on chip.  Classical for cell-by-cell contexts,
+                              whose long ill-conditioned solves need its smaller rounding
+                              error, and for batches, whose many small groups favour its
+                              lighter rows; default -1                                         */
     int energy_stop;       /* 1: end the sweeps of a step once the energy norm of the sweep's
                               corrections, E_k = sum_m dv_m' A~_m dv_m with A~_m the node system
                               matrix, is at most ((1 - rho) / rho * TOL)^2 (Sec. 3.2); `sweeps`
@@ -158,9 +164,10 @@ typedef struct {
                               max(0, -min dI/dv) / C_m over the first sweep's linearisation
                               (zero with reaction_implicit = 0); computed on the device once
                               per step, reported in sdc_stats.tol_drop.  Not in batches      */
-    int cg_scaled;         /* 1: the node solves run in the symmetrically scaled form, CG on diag^-1/2 A diag^-1/2: the same
-                              iterates as Jacobi-PCG with fewer FP64 operations per row and
-                              fewer vectors on chip; 0: the Jacobi form; default 1          */
+    int cg_scaled;         /* 1: the node solves run in the symmetrically scaled form, CG on
+                              diag^-1/2 A diag^-1/2: the same iterates as Jacobi-PCG with fewer
+                              FP64 operations per row and fewer vectors on chip; 0: the Jacobi
+                              form; default 1                                                 */
     int batch_graph;       /* batches: 1 runs each step with device-driven sweeps (|I_k| read on
                               the device, the batched solves' block plan built on the device)
                               captured once per (state arrays, dt, sweeps, TOL, stimulus on or
@@ -264,10 +271,11 @@ sdc_status sdc_get_matrix(const sdc_ctx* ctx, int* row_ptr, int* col, double* va
  * d_len[i] <= width entries, entry t at d_val[t * ld + i], column
  * d_col[t * ld + i] in [0, n); ld >= n.  Every array is caller-owned device
  * memory of the current device; d_x receives the solution.  The workspace
- * (up to 8 n + 2 ld doubles plus a few per SM; on-chip solves up to 2 n + (4 + width) ld) comes
- * from a stream-ordered pool that keeps at most 64 MiB per device between calls (sdc_destroy
- * gives them back) and is returned inside the call, which synchronises `stream` (a cudaStream_t, NULL = legacy default).  iters and
- * relres (host, may be NULL) receive the iteration count and the final
+ * (on-chip solves up to 2 n + (4 + width) ld doubles; the others, and those without room
+ * for that, 8 n + 2 ld and a few per SM) comes from a stream-ordered pool that keeps at most
+ * 64 MiB per device between calls (sdc_destroy gives them back) and is returned inside the
+ * call, which synchronises `stream` (a cudaStream_t, NULL = legacy default).  iters and relres
+ * (host, may be NULL) receive the iteration count and the final
  * sqrt(r'z / r0'z0).  Errors: SDC_E_INVALID (nothing launched),
  * SDC_E_NOMEM, SDC_E_CG_NOCONV, SDC_E_NONFINITE, SDC_E_DOMAIN (a non-positive
  * diagonal); details from sdc_last_error(NULL) on the calling thread. */
@@ -312,7 +320,10 @@ sdc_status sdc_step_taped(sdc_ctx* ctx, double* d_v, double* d_w, double t, doub
  * d_grad_scale (device, n_nodes; may be NULL), s being the per-node
  * conductivity scale, and adds dL/d(ga, gs, a) to grad_ionic[3] (host; may be
  * NULL).  The reverse node solves use the forward's Jacobi-PCG with the
- * context's cg_rtol.  Synchronises the stream.  Not available for batches. */
+ * context's cg_rtol.  Synchronises the stream.  Not available for batches.  The
+ * first call allocates workspace that the context keeps: 7 M + 1 doubles per node (and M more
+ * per row), one per element, and, with d_grad_scale, dim^2 doubles per element (72 bytes a
+ * tetrahedron; without room for them every sweep forms the elements' geometry). */
 sdc_status sdc_step_adjoint(sdc_ctx* ctx, const sdc_tape* tape, const double* d_v0,
                             const double* d_w0, double dt, const double* d_lam_v,
                             const double* d_lam_w, double* d_lam_v0, double* d_lam_w0,
