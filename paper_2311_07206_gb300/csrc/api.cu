@@ -280,13 +280,18 @@ bool ensure_adjoint(sdc_ctx* c) {
     AdjointBuffers& W = c->AW;
     if (W.Vb) return true;
     const size_t NM = (size_t)c->N * c->M, MLD = (size_t)c->M * c->B.ld;
-    return ensure_pos(c) && dalloc(&W.Vb, NM) && dalloc(&W.Wb, NM) && dalloc(&W.V0, NM) &&
-           dalloc(&W.W0, NM) && dalloc(&W.X, MLD) &&
-           dalloc(&W.bfull, NM) && dalloc(&W.z, NM) && dalloc(&W.ffull, NM) &&
-           dalloc(&W.ge, (size_t)c->K.mesh.n_elems) &&
-           dalloc(&W.part3, 3 * (size_t)((c->N + 127) / 128)) && dalloc(&W.iacc, 3) &&
-           dalloc(&W.iters, (size_t)SDC_MAX_SWEEPS * kMaxM) &&
-           dalloc(&W.relres, (size_t)SDC_MAX_SWEEPS * kMaxM);
+    const bool ok =
+        ensure_pos(c) && dalloc(&W.Vb, NM) && dalloc(&W.Wb, NM) && dalloc(&W.V0, NM) &&
+        dalloc(&W.W0, NM) && dalloc(&W.X, MLD) && dalloc(&W.bfull, NM) && dalloc(&W.z, NM) &&
+        dalloc(&W.ffull, NM) && dalloc(&W.ge, (size_t)c->K.mesh.n_elems) &&
+        dalloc(&W.part3, 3 * (size_t)((c->N + 127) / 128)) && dalloc(&W.iacc, 3) &&
+        dalloc(&W.iters, (size_t)SDC_MAX_SWEEPS * kMaxM) &&
+        dalloc(&W.relres, (size_t)SDC_MAX_SWEEPS * kMaxM);
+    if (!ok) {   // all or nothing: a later call starts over
+        cudaGetLastError();
+        free_adjoint(W);
+    }
+    return ok;
 }
 
 void free_adjoint(AdjointBuffers& W) {
