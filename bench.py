@@ -325,8 +325,8 @@ def interp_plain_ms(plain, err):
             return float(np.exp(np.log(m_lo) + f * np.log(m_hi / m_lo)))
     return None
 
-PCG_TRAFFIC = {"w1": {"dram_bytes": 64.34e6 + 12.56e6, "algorithmic_bytes": 2.479e9,
-                      "kernel": "k_cgc_flow<1024>", "source_sha": "70a061faac5c7e7e",
+PCG_TRAFFIC = {"w1": {"dram_bytes": 65.25e6 + 13.38e6, "algorithmic_bytes": 2.479e9,
+                      "kernel": "k_cgc_flow<1024>", "source_sha": "0dbf339a1ede4805",
                       "capture": "profiles/flow_kernels_slabs.md"}}
 
 

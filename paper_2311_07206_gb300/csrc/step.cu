@@ -1610,7 +1610,10 @@ __global__ void __launch_bounds__(MAXT, 1) k_pcgc_batch(CgParams P, const SegBlo
 }
 
 // Shared-memory form of pcgc_group_scaled: rows as in k_pcgc_smem, r, p, s, w on
-// chip (four vectors), r published for the neighbours' products.
+// chip (four vectors), r published for the neighbours' products. Solves of up to
+// 724k rows whose matrix and words overflow L2 (flow_in_cache): 8-byte words, two grid barriers and
+// x in global memory.  Bound by L2's misses there: 550k rows of 13.4 slots 30.0 us per iteration
+// against 51.7 in k_cgc_flow, 686k 41.3 / 65.0.
 template <int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) k_pcgc_scaled(CgParams P) {
     extern __shared__ double sm[];
