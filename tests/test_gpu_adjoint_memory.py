@@ -39,8 +39,14 @@ def test_adjoint_after_a_shortage(torch_dev):
         if short:
             torch.cuda.synchronize(dev)
             torch.cuda.empty_cache()
-            free = torch.cuda.mem_get_info(dev)[0]
-            fill = torch.empty(free - (24 << 20), dtype=torch.uint8, device=dev)
+            fill, chunk = [], torch.cuda.mem_get_info(dev)[0]
+            while chunk >= 1 << 21:      # all but about 24 MB, in as many pieces as it takes
+                chunk = min(chunk, torch.cuda.mem_get_info(dev)[0] - (24 << 20))
+                try:
+                    if chunk >= 1 << 21:
+                        fill.append(torch.empty(chunk, dtype=torch.uint8, device=dev))
+                except torch.cuda.OutOfMemoryError:
+                    chunk //= 2
             with pytest.raises(SdcError) as e:
                 run()
             assert e.value.status == B.SDC_E_NOMEM
